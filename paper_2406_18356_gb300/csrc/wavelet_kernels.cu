@@ -382,7 +382,9 @@ __device__ __forceinline__ void synth_stage(const R* plane, const R* llp, int N,
   const int nch = (ncol + V - 1) / V;
   // rows lie in [-7, h), columns in [-8, h): one conditional wrap when h >= 8
   const bool cheap = h >= kMaxTaps / 2;
-  if (base_c >= 0 && base_c + nch * V <= h) {
+  // whole chunks: no column wraps, and every subband row of the window starts
+  // on a 16-byte boundary (h = 30, tiles of 4: neither holds)
+  if (base_c >= 0 && base_c + nch * V <= h && base_c % V == 0 && h % V == 0) {
     const int per_sub = cnt * nch;
     for (int e = threadIdx.x; e < 4 * per_sub; e += G::Threads) {
       const int sb = e / per_sub, rem = e - sb * per_sub;
@@ -572,7 +574,8 @@ __device__ __forceinline__ void synth_item(unsigned char* smem_raw, const R* __r
   constexpr int V = Tab::V;
   const int nch = (cnt + 1 + V - 1) / V;
   const int base_r = r0 / 2 - (kMaxTaps / 2 - 1), base_c = c0 / 2 - kMaxTaps / 2;
-  const bool table = sum_bases && m_hi - m_lo > 1 && base_c >= 0 && base_c + nch * V <= h;
+  const bool table = sum_bases && m_hi - m_lo > 1 && base_c >= 0 && base_c + nch * V <= h &&
+                     base_c % V == 0 && h % V == 0;
   if (table) {
     const int per_sub = cnt * nch;
     const bool cheap = h >= kMaxTaps / 2;
