@@ -561,9 +561,24 @@ __device__ __forceinline__ void dft_reg(C2<R> (&v)[Rd]) {
 
 // one Stockham stage (radix Rd after sub-transforms of size NS) of the
 // calling thread's sequence; src / dst already offset to the sequence
-template <typename R, int LOGN, int Rd, int NS, bool INV>
+// threads of one sequence of length 2^LOGN at radix 2^LRAD
+__host__ __device__ constexpr int fft_threads(int logn, int lrad) {
+  return logn > lrad ? 1 << (logn - lrad) : 1;
+}
+// log2 of the largest radix.  FP32: 8 (fewest stages).  FP64: a warp
+// instruction holds its scheduler's FP64 pipe (2 lanes a cycle per SM) for 64
+// cycles, so the time of a short transform is the instructions of its busiest
+// warp: radix 2 spreads them over 4 times the warps up to length 256, radix 4
+// over twice as many above (its stages take about as many operations per
+// point as radix 8's); radix 8 where a sequence would pass 1024 threads.
+// Measured at 128 px, FP64 (with the blocks per launch below): row R2C 36.8 ->
+// 5.3 us, column step 22.8 -> 11.5 us, row C2R 34.2 -> 5.0 us.
+__host__ __device__ constexpr int fft_lrad(size_t rsz, int logn) {
+  return rsz == 4 ? 3 : (logn <= 8 ? 1 : (logn <= 11 ? 2 : 3));
+}
+template <typename R, int LOGN, int Rd, int NS, int TPS, bool INV>
 __device__ __forceinline__ void stage_ct(const C2<R>* src, C2<R>* dst, const C2<R>* tw, int tid) {
-  constexpr int N = 1 << LOGN, nj = N / Rd, TPS = N / 8;
+  constexpr int N = 1 << LOGN, nj = N / Rd;
 #pragma unroll
   for (int j0 = 0; j0 < nj; j0 += TPS) {
     const int j = j0 + tid;
@@ -589,18 +604,20 @@ __device__ __forceinline__ void stage_ct(const C2<R>* src, C2<R>* dst, const C2<
   }
 }
 
-// the stages from sub-transform size 2^DONE on; data in (cur ? b1 : b0),
-// result in (cur ? b1 : b0) on return; a block barrier after every stage
-template <typename R, int LOGN, int DONE, bool INV>
+// the stages from sub-transform size 2^DONE on, of radix up to 2^LRAD; data
+// in (cur ? b1 : b0), result in (cur ? b1 : b0) on return; a block barrier
+// after every stage
+template <typename R, int LOGN, int LRAD, int DONE, bool INV>
 __device__ __forceinline__ void stages_ct(C2<R>* b0, C2<R>* b1, int& cur, const C2<R>* tw, int tid,
                                           bool active) {
   if constexpr (DONE < LOGN) {
-    constexpr int LR = LOGN - DONE >= 3 ? 3 : LOGN - DONE;
+    constexpr int LR = LOGN - DONE >= LRAD ? LRAD : LOGN - DONE;
     if (active)
-      stage_ct<R, LOGN, 1 << LR, 1 << DONE, INV>(cur ? b1 : b0, cur ? b0 : b1, tw, tid);
+      stage_ct<R, LOGN, 1 << LR, 1 << DONE, fft_threads(LOGN, LRAD), INV>(
+          cur ? b1 : b0, cur ? b0 : b1, tw, tid);
     __syncthreads();
     cur ^= 1;
-    stages_ct<R, LOGN, DONE + LR, INV>(b0, b1, cur, tw, tid, active);
+    stages_ct<R, LOGN, LRAD, DONE + LR, INV>(b0, b1, cur, tw, tid, active);
   }
 }
 
@@ -613,6 +630,10 @@ __host__ __device__ constexpr int seq_pitch(int n) { return padi(n) + 8; }
 // the shared memory would pass kColSmemCap) and PF, the prefetch of the
 // block's X^_{k-1}, B^ and K^ when it fits.
 constexpr size_t kColSmemCap = 200 * 1024;
+#ifndef MS_COL_BLOCKS_MIN
+#define MS_COL_BLOCKS_MIN 128
+#endif
+constexpr int kColBlocksMin = MS_COL_BLOCKS_MIN;
 #ifndef MS_COL_ROW_BYTES
 #define MS_COL_ROW_BYTES 32
 #endif
@@ -622,6 +643,9 @@ constexpr size_t col_smem_c(int n, int cb, size_t cbytes, bool pf) {
 }
 constexpr int col_cb_c(int n, size_t cbytes, bool pf) {
   int cb = (int)(MS_COL_ROW_BYTES / cbytes) > 4 ? 4 : (int)(MS_COL_ROW_BYTES / cbytes);
+  // (short transforms: a block for every SM before whole sectors; FP32 at
+  // 512 px, 65 -> 129 blocks: 7.2 us either way)
+  while (cb > 1 && (n / 2 + 1 + cb - 1) / cb < kColBlocksMin) cb /= 2;
   if (cb < 1) cb = 1;
   while (cb > 1 && col_smem_c(n, cb, cbytes, pf) > kColSmemCap) cb /= 2;
   return cb;
@@ -631,7 +655,8 @@ template <typename R, int LOGN> struct ColCfg {
   static constexpr size_t CBY = sizeof(C2<R>);
   static constexpr bool PF = col_smem_c(N, col_cb_c(N, CBY, true), CBY, true) <= kColSmemCap;
   static constexpr int CB = col_cb_c(N, CBY, PF);
-  static constexpr int TPS = N / 8;
+  static constexpr int LRAD = fft_lrad(sizeof(R), LOGN);
+  static constexpr int TPS = fft_threads(LOGN, LRAD);
   static constexpr int THREADS = CB * TPS < 32 ? 32 : CB * TPS;
   static constexpr size_t SMEM = col_smem_c(N, CB, CBY, PF);
   static_assert(THREADS <= 1024 && THREADS % 32 == 0, "column block");
@@ -747,7 +772,7 @@ __global__ void __launch_bounds__(ColCfg<R, LOGN>::THREADS, 1) spec_col_kernel(
   int cur = 0;
   C2<R>* c_b0 = b0 + (active ? ccol : 0) * P;
   C2<R>* c_b1 = b1 + (active ? ccol : 0) * P;
-  stages_ct<R, LOGN, 0, false>(c_b0, c_b1, cur, tw, tcol, active);
+  stages_ct<R, LOGN, Cfg::LRAD, 0, false>(c_b0, c_b1, cur, tw, tcol, active);
   if (PF) cp_async_wait<0>();   // this thread's own prefetched elements
   C2<R>* X = cur ? b1 : b0;
   R s0 = 0, cc0 = 0, s1 = 0, cc1 = 0;
@@ -811,7 +836,7 @@ __global__ void __launch_bounds__(ColCfg<R, LOGN>::THREADS, 1) spec_col_kernel(
     }
   }
   __syncthreads();
-  stages_ct<R, LOGN, 0, true>(c_b0, c_b1, cur, tw, tcol, active);
+  stages_ct<R, LOGN, Cfg::LRAD, 0, true>(c_b0, c_b1, cur, tw, tcol, active);
   const C2<R>* Y = cur ? b1 : b0;
   for (int e = threadIdx.x; e < N * CB; e += T) {
     const int r = e / CB, c = e - r * CB;
@@ -847,15 +872,22 @@ __global__ void __launch_bounds__(ColCfg<R, LOGN>::THREADS, 1) spec_col_kernel(
 // forms Z'_k = (X_k + conj X_(M-k)) + i W_N^-k (X_k - conj X_(M-k)), k < M,
 // and x_2n + i x_2n+1 = sum_k Z'_k W_M^-kn.  One row per M/8 threads, RB
 // rows per block.
+#ifndef MS_ROW_BLOCKS_MIN
+#define MS_ROW_BLOCKS_MIN 128
+#endif
 #ifndef MS_ROW_THREADS
 #define MS_ROW_THREADS 512   // threads per block of the row transforms (rows x N/16)
 #endif
 template <typename R, int LOGN> struct RowCfg {
   static constexpr int N = 1 << LOGN, M = N / 2;
-  static constexpr int TPS = M / 8 > 0 ? M / 8 : 1;
-  static constexpr int RB = MS_ROW_THREADS / TPS < 1
-                                ? 1
-                                : (MS_ROW_THREADS / TPS > N ? N : MS_ROW_THREADS / TPS);
+  static constexpr int LRAD = fft_lrad(sizeof(R), LOGN - 1);
+  static constexpr int TPS = fft_threads(LOGN - 1, LRAD);
+  // rows per block: MS_ROW_THREADS threads, fewer rows where that would
+  // leave less than about a block per SM (FP32 at 512 px, 32 -> 128 blocks:
+  // row R2C 3.9 -> 2.7 us)
+  static constexpr int RBT = MS_ROW_THREADS / TPS < 1 ? 1 : MS_ROW_THREADS / TPS;
+  static constexpr int RBN = N / MS_ROW_BLOCKS_MIN < 1 ? 1 : N / MS_ROW_BLOCKS_MIN;
+  static constexpr int RB = RBT < RBN ? RBT : RBN;
   static constexpr int THREADS = RB * TPS < 32 ? 32 : RB * TPS;
   // two buffers of RB rows, the M-point twiddle table W_M^m = W_N^2m
   // (padded) and W_N^k, k <= M, for the packing step
@@ -904,7 +936,7 @@ __global__ void __launch_bounds__(RowCfg<R, LOGN>::THREADS) row_r2c_kernel(
   cp_async_wait<0>();
   __syncthreads();
   int cur = 0;
-  stages_ct<R, LOGN - 1, 0, false>(b0 + (active ? rr : 0) * P, b1 + (active ? rr : 0) * P, cur,
+  stages_ct<R, LOGN - 1, Cfg::LRAD, 0, false>(b0 + (active ? rr : 0) * P, b1 + (active ? rr : 0) * P, cur,
                                    tw, t, active);
   if (!active) return;
   const C2<R>* Zs = (cur ? b1 : b0) + rr * P;
@@ -1037,7 +1069,7 @@ __global__ void __launch_bounds__(RowCfg<R, LOGN>::THREADS) row_c2r_kernel(
   }
   __syncthreads();
   int cur = 0;
-  stages_ct<R, LOGN - 1, 0, true>(b0 + (active ? rr : 0) * P, b1 + (active ? rr : 0) * P, cur,
+  stages_ct<R, LOGN - 1, Cfg::LRAD, 0, true>(b0 + (active ? rr : 0) * P, b1 + (active ? rr : 0) * P, cur,
                                   tw, t, active);
   if (!active) return;
   const C2<R>* zs = (cur ? b1 : b0) + rr * P;
