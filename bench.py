@@ -377,12 +377,11 @@ def record_traffic(paths, precision):
             for m in ("dram__bytes_read.sum", "dram__bytes_write.sum"):
                 b += float(r[idx[m]].replace(",", "")) * scale[units[idx[m]]]
             launches.append((name, b))
-    # (levels J..2 are one cooperative launch, or one launch per level)
+    # (one launch per level, in order)
     syn = [b for n, b in launches
-           if "synthesis_level_kernel" in n or "coarse_synthesis_kernel" in n]
+           if "synthesis_level_kernel" in n or "fine_synthesis" in n]
     ana = [b for n, b in launches
-           if "analysis_level_kernel" in n or "analysis_l1_tile_kernel" in n
-           or "coarse_analysis_kernel" in n]
+           if "analysis_level_kernel" in n or "fine_analysis_kernel" in n]
     if syn:
         fams["synth"], fams["synth_l1"] = sum(syn[:-1]), syn[-1]
     if ana:
@@ -893,7 +892,7 @@ def kernel_source_digest(fam):
     import hashlib
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2406_18356_gb300", "csrc")
-    extra = ("coarse_levels.cuh",) if FAMILY_SOURCE[fam] == "wavelet_kernels.cu" else ()
+    extra = ("fine_levels.cuh",) if FAMILY_SOURCE[fam] == "wavelet_kernels.cu" else ()
     for f in (FAMILY_SOURCE[fam], "common.cuh") + extra:
         with open(os.path.join(csrc, f), "rb") as fh:
             h.update(fh.read())

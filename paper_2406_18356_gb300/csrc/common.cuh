@@ -273,23 +273,16 @@ void set_wavelet_filters(const double* h, const int* len, int nbases);   // host
 struct WaveletGeom {
   int N, J, M;
 };
-// coef3 / B3 / Yh2 are DEVICE arrays of pointers; with a FistaCtl the kernels
-// pick buffer k % 3 (and k % 2) from it and skip all work once ctl->done is set
+// x = W coef and coef = W^H x; tmp: M N^2 elements
 template <typename R>
-void launch_synthesis3(const R* const* coef3_dev, R* x, R* tmp, WaveletGeom g,
-                       const FistaCtl* ctl, cudaStream_t s, int only_level = 0);
+cudaError_t launch_synthesis(const R* coef, R* x, R* tmp, WaveletGeom g, cudaStream_t s);
 template <typename R>
-void launch_analysis(const R* x, R* coef, R* tmp, WaveletGeom g, cudaStream_t s);
+cudaError_t launch_analysis(const R* x, R* coef, R* tmp, WaveletGeom g, cudaStream_t s);
 // Buffers of one minor-cycle pass, passed by value to the persistent pass
 // kernels: the coefficient ring B0..B2 (B[k % 3] is current), the gradient
 // image 2 (K W alpha_k - b) written by the inverse FFT, the synthesized image
 // x = W B_k, the approximation ping-pong, the control block and the per-block
 // partial sums of ||B_{k+1}||_1.
-// CTAs of each basis's group in the one-launch coarse levels: basis m owns
-// CTAs [first[m], first[m + 1]).
-struct CoarseGroups {
-  int first[kMaxBases + 1];
-};
 // Batched minor cycles: `jobs` independent FISTA problems whose state lives
 // in arrays of equal per-job slices; a kernel's blockIdx.z is its job, and
 // each buffer of job z starts z times its stride (elements) after job 0's.
@@ -315,11 +308,7 @@ template <typename R> struct FistaPass {
   FistaCtl* ctl;
   double* l1_parts;
   int N, J, M;
-  int coarse_ctas;     // CTAs of the one-launch coarse levels (0: one launch per level)
-  int coarse_budget;   // their shared-memory budget per CTA (bytes)
-  CoarseGroups coarse_groups;
-  int* coarse_bar;     // group barrier state, two ints per basis, zero at rest
-  JobStride js{};      // batched minor cycles (coarse_ctas must then be 0)
+  JobStride js{};      // batched minor cycles
 };
 
 // this block's job's view of a (batched) pass
@@ -347,7 +336,7 @@ cudaError_t launch_synthesis_pass(const FistaPass<R>& a, cudaStream_t s, int onl
 template <typename R>
 cudaError_t launch_analysis_pass(const FistaPass<R>& a, const CUtensorMap* grad_map,
                                  cudaStream_t s, int only_level = 0);
-int analysis_prox_partials(WaveletGeom g);
+int analysis_prox_partials(WaveletGeom g, size_t rsz);
 void analysis_window_box(unsigned* cols, unsigned* rows);
 
 // iuwt_kernels.cu: the IUWT dictionary W = T^H (J levels, J + 1 planes).
@@ -361,14 +350,6 @@ template <typename R>
 cudaError_t launch_iuwt_analysis(const FistaPass<R>* fp, const R* img, R* alpha, R* work, int N,
                                  int J, cudaStream_t s);
 int iuwt_prox_partials(int J);
-// The one-launch coarse levels (2..J of both transforms, one cooperative
-// launch per transform) on the current device: the CTAs of each basis's
-// group (in proportion to its filter length) and the shared-memory budget
-// per CTA with which all of them are resident at once.  Returns the number
-// of CTAs, or 0 when the geometry needs the per-level kernels (N not a power
-// of two, N < 256, N >> J < 8, J < 2) or no such launch fits.
-int coarse_groups(WaveletGeom g, size_t rsz, CoarseGroups* groups, int* budget);
-
 // spectral_kernels.cu
 int spectral_partials(int N);
 template <typename R>

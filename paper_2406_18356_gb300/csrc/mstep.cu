@@ -155,12 +155,6 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-__global__ void set_ptrs_kernel(void** dst, void* a, void* b, void* c) {
-  dst[0] = a;
-  dst[1] = b;
-  dst[2] = c;
-}
-
 __global__ void init_ctl_kernel(FistaCtl* ctl, int max_iters, double rel_tol, double lam,
                                 int set_lam, double sigma2, double eta2, int set_noise) {
   ctl->k = 0;
@@ -301,7 +295,6 @@ struct ms_plan {
   void *F[2] = {};   // FISTA spectra X^_k / X^_{k-1} (ping-pong by pass parity)
   void *spec = nullptr, *spec2 = nullptr, *Ks = nullptr, *Bs = nullptr;
   void *gl2 = nullptr, *gh2 = nullptr, *wtmp = nullptr;
-  void** api3_dev = nullptr;   // pointer table of the one-shot synthesis calls
   CUtensorMap grad_map{};   // TMA descriptor of the gradient image (ywork)
   bool have_grad_map = false;
   FistaCtl* ctl = nullptr;
@@ -310,10 +303,6 @@ struct ms_plan {
   double* l1parts = nullptr;   // per-block |B_k+1| partials of the analysis levels
   int n_l1 = 0;                // their number
   int dict = MS_DICT_DAUBECHIES;   // minor-cycle dictionary
-  int coarse_ctas = 0;         // CTAs of the one-launch coarse levels (0: one launch per level)
-  int coarse_budget = 0;       // their shared-memory budget per CTA
-  CoarseGroups coarse_gr{};    // their split over the bases
-  int* coarse_bar = nullptr;   // their group barrier state
   int32_t* tickets = nullptr;
   double* scal = nullptr;
   int32_t* err = nullptr;
@@ -679,10 +668,6 @@ template <typename R> FistaPass<R> fista_pass_args(ms_plan* p) {
   a.N = p->N;
   a.J = p->J;
   a.M = p->M;
-  a.coarse_ctas = p->coarse_ctas;
-  a.coarse_budget = p->coarse_budget;
-  a.coarse_groups = p->coarse_gr;
-  a.coarse_bar = p->coarse_bar;
   return a;
 }
 
@@ -900,9 +885,8 @@ template <typename R> void dict_synthesis(ms_plan* p, const R* alpha, R* x) {
        "IUWT synthesis");
     return;
   }
-  set_ptrs_kernel<<<1, 1, 0, p->ps>>>(p->api3_dev, (void*)alpha, (void*)alpha, (void*)alpha);
-  launch_synthesis3<R>((const R* const*)p->api3_dev, x, (R*)p->wtmp,
-                       WaveletGeom{p->N, p->J, p->M}, nullptr, p->ps);
+  ck(launch_synthesis<R>(alpha, x, (R*)p->wtmp, WaveletGeom{p->N, p->J, p->M}, p->ps),
+     "synthesis");
 }
 template <typename R> void dict_analysis(ms_plan* p, const R* x, R* alpha) {
   if (p->dict == MS_DICT_IUWT) {
@@ -910,7 +894,8 @@ template <typename R> void dict_analysis(ms_plan* p, const R* x, R* alpha) {
        "IUWT analysis");
     return;
   }
-  launch_analysis<R>(x, alpha, (R*)p->wtmp, WaveletGeom{p->N, p->J, p->M}, p->ps);
+  ck(launch_analysis<R>(x, alpha, (R*)p->wtmp, WaveletGeom{p->N, p->J, p->M}, p->ps),
+     "analysis");
 }
 
 // The normal operator of the current problem with the linear PSF operator,
@@ -1066,9 +1051,6 @@ void run_fista(ms_plan* p, int step, PartDev& pd, const void* residual, const vo
   ck(cudaMemcpyAsync(p->B[2], p->B[0], sizeof(R) * ncoef, cudaMemcpyDeviceToDevice, p->ps),
      "copy");
   set_target_kernel<<<1, 1, 0, p->ps>>>(p->ctl, p->obj_target);
-  // the coarse levels' group barriers start at rest (a wait that ran out
-  // may have left a count behind)
-  ck(cudaMemsetAsync(p->coarse_bar, 0, sizeof(int) * 2 * kMaxBases, p->ps), "memset");
   const bool poll = rel_tol > 0 || std::isfinite(p->obj_target);
   // ||B_0||_1 enters the first objective through the analysis partials
   ck(cudaMemsetAsync(p->l1parts, 0, sizeof(double) * p->n_l1, p->ps), "memset");
@@ -1164,7 +1146,7 @@ void warm_start_beta(ms_plan* p, ms_unet* net, const void* low, const void* res,
     throw Fail{st, std::string("warm start network: ") + ms_unet_last_error(net)};
   ws_output_kernel<R><<<nb, 256, 0, p->ps>>>(p->ws_out, p->ctl, n2, x0);
   WaveletGeom g{p->N, p->J, p->M};
-  launch_analysis<R>(x0, (R*)beta, (R*)p->wtmp, g, p->ps);
+  ck(launch_analysis<R>(x0, (R*)beta, (R*)p->wtmp, g, p->ps), "analysis");
   launch_axpby<R>((const R*)beta, nullptr, (R*)beta, 1.0 / p->M, 0.0, (int64_t)p->M * n2,
                   p->ps);
   ck(cudaGetLastError(), "warm start kernels");
@@ -1478,18 +1460,13 @@ template <typename R> void build_plan(ms_plan* p, const ms_plan_desc* d) {
   p->gh2 = p->alloc<R>(nspec, "filter");
   // two LL buffers of M (N/2)^2 (Daubechies), or three work images (IUWT)
   p->wtmp = p->alloc<R>(std::max<int64_t>(ncoef, 3 * n2), "wavelet tmp");
-  p->api3_dev = p->alloc<void*>(3, "ptrs");
   p->ctl = p->alloc<FistaCtl>(1, "ctl");
   p->parts = p->alloc<double>(std::max(4096, 3 * spec_col_warps(N, sizeof(C2<R>))), "partials");
   if (p->dict == MS_DICT_IUWT) {
     p->n_l1 = iuwt_prox_partials(p->J);
   } else {
-    p->n_l1 = analysis_prox_partials(WaveletGeom{N, p->J, p->M});
-    p->coarse_ctas =
-        coarse_groups(WaveletGeom{N, p->J, p->M}, sizeof(R), &p->coarse_gr, &p->coarse_budget);
+    p->n_l1 = analysis_prox_partials(WaveletGeom{N, p->J, p->M}, sizeof(R));
   }
-  p->coarse_bar = p->alloc<int>(2 * kMaxBases, "coarse barrier");
-  ck(cudaMemset(p->coarse_bar, 0, sizeof(int) * 2 * kMaxBases), "memset");
   p->l1parts = p->alloc<double>(p->n_l1, "partials");
   p->tickets = p->alloc<int32_t>(16, "tickets");
   p->scal = p->alloc<double>(16, "scalars");
@@ -1570,10 +1547,10 @@ template <typename R> void build_plan(ms_plan* p, const ms_plan_desc* d) {
         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) throw Fail{MS_ERR_CUDA, "cuTensorMapEncodeTiled failed"};
     // gradient image of the minor cycle: {N, N}, box = the analysis input
-    // window {80, 78}; only images at least one window wide use it
+    // window {80, 78}, for the wide tiles of FP64 level 1
     unsigned bc = 0, br = 0;
     analysis_window_box(&bc, &br);
-    if ((unsigned)N >= bc) {
+    if (sizeof(R) == 8 && (unsigned)N >= bc) {
       cuuint64_t gd[2] = {(cuuint64_t)N, (cuuint64_t)N};
       cuuint64_t gs[1] = {(cuuint64_t)N * sizeof(R)};
       cuuint32_t gb[2] = {bc, br};
@@ -1967,7 +1944,6 @@ template <typename R> PassView<R> batch_view(ms_plan* p, int jobs) {
   v.a.tmp = (R*)F.tmp;
   v.a.ctl = F.ctl;
   v.a.l1_parts = F.l1;
-  v.a.coarse_ctas = 0;   // per-level launches: a cooperative launch cannot hold every job
   JobStride& js = v.a.js;
   js.jobs = jobs;
   js.coef = (int64_t)p->M * n2;

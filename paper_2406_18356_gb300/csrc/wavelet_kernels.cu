@@ -11,13 +11,15 @@
 // rows [h,n) x cols [0,h) high-y/low-x, [h,n)^2 high/high, h = n/2.
 // Synthesis is the transpose X = T^T Y T.
 //
-// Both directions are register-blocked: a thread slides over 8 outputs of one
-// row or column with its inputs held in registers, and each basis is a
-// separate template instance so the filter taps are compile-time constant-bank
-// operands.  Global traffic goes through shared memory in whole rows: input
-// windows arrive by TMA (level-1 analysis) or cp.async (the next basis's
-// subband windows are prefetched while the current one is filtered), and
-// results leave as 16-byte vector stores.
+// Most levels run in small tiles, one block per (tile, basis)
+// (fine_levels.cuh).  The kernels of this file serve what is left: level 1 of
+// the FP32 synthesis (a block sums the bases of a 32 or 64 pixel tile, the
+// next basis's subband windows prefetched while the current one is filtered),
+// the analysis levels of FP64 images of more than 512 pixels, and subbands
+// whose side is no multiple of four.  They are register-blocked: a thread
+// slides over 8 outputs of one row or column with its inputs held in
+// registers.  Each basis is a separate template instance so the filter taps
+// are compile-time constant-bank operands.
 //
 // The analysis kernel of the minor cycle also does FISTA's step (Algorithm 1):
 // its level-1 input is the gradient image 2 (K W alpha_k - b) of the
@@ -35,8 +37,6 @@ namespace ms {
 
 __constant__ double c_hd[kMaxBases][kMaxTaps];
 __constant__ double c_gd[kMaxBases][kMaxTaps];
-__constant__ float c_hf[kMaxBases][kMaxTaps];
-__constant__ float c_gf[kMaxBases][kMaxTaps];
 // FP32 coefficient pairs for the packed filters: (h_k, g_k) of the analysis
 // tap k, (h_2m, h_2m+1) and (g_2m, g_2m+1) of the synthesis output pair
 __constant__ float2 c_hg2[kMaxBases][kMaxTaps];
@@ -56,8 +56,6 @@ void set_wavelet_filters(const double* h, const int* len, int nbases) {
   }
   cudaMemcpyToSymbol(c_hd, hd, sizeof(hd));
   cudaMemcpyToSymbol(c_gd, gd, sizeof(gd));
-  cudaMemcpyToSymbol(c_hf, hf, sizeof(hf));
-  cudaMemcpyToSymbol(c_gf, gf, sizeof(gf));
   float2 hg[kMaxBases][kMaxTaps] = {}, hh[kMaxBases][kMaxTaps / 2] = {},
          gg[kMaxBases][kMaxTaps / 2] = {};
   for (int m = 0; m < kMaxBases; ++m)
@@ -74,13 +72,6 @@ void set_wavelet_filters(const double* h, const int* len, int nbases) {
 }
 
 namespace {
-template <typename R> __device__ __forceinline__ R fh(int m, int k);
-template <typename R> __device__ __forceinline__ R fg(int m, int k);
-template <> __device__ __forceinline__ float fh<float>(int m, int k) { return c_hf[m][k]; }
-template <> __device__ __forceinline__ float fg<float>(int m, int k) { return c_gf[m][k]; }
-template <> __device__ __forceinline__ double fh<double>(int m, int k) { return c_hd[m][k]; }
-template <> __device__ __forceinline__ double fg<double>(int m, int k) { return c_gd[m][k]; }
-
 // Filter pairs on the FP32 pipe's packed form (fma.rn.f32x2: two lanes of
 // FP32 fused multiply-add per instruction, each lane rounded as fmaf): the
 // two outputs of a filter step that share their input (analysis: the low and
@@ -90,9 +81,6 @@ template <> __device__ __forceinline__ double fg<double>(int m, int k) { return 
 // Measured at 1024^2 (FP32, M = 8, J = 4), per FISTA iteration: synthesis
 // levels 4..2 29.8 -> 26.8 us, level 1 36.0 -> 33.3 us, analysis levels 2..4
 // 35.5 -> 33.6 us, level 1 37.1 -> 35.1 us (144.9 -> 136.0 us in all).
-#ifndef MS_PACKED_F32
-#define MS_PACKED_F32 1
-#endif
 // (d.x, d.y) = (c.x x + acc.x, c.y x + acc.y), c a coefficient pair read from
 // constant memory as one 64-bit operand
 __device__ __forceinline__ float2 ffma2_cx(const float2& c, float x, float2 acc) {
@@ -106,36 +94,33 @@ __device__ __forceinline__ float2 ffma2_cx(const float2& c, float x, float2 acc)
   return d;
 }
 // analysis tap k of basis MB on input x: (a, d) += (h_k, g_k) x
-template <typename R, int MB, bool PACK>
+template <typename R, int MB>
 __device__ __forceinline__ void tap_hg(int k, R x, R& a, R& d) {
-  if constexpr (sizeof(R) == 4 && MS_PACKED_F32 && PACK) {
+  if constexpr (sizeof(R) == 4) {
     const float2 r = ffma2_cx(c_hg2[MB][k], x, make_float2(a, d));
     a = r.x;
     d = r.y;
   } else {
-    a = fma(fh<R>(MB, k), x, a);
-    d = fma(fg<R>(MB, k), x, d);
+    a = fma(c_hd[MB][k], x, a);
+    d = fma(c_gd[MB][k], x, d);
   }
 }
 // synthesis taps 2m, 2m + 1 of basis MB on low input x and high input y:
 // (e, o) += (h_2m, h_2m+1) x, then (e, o) += (g_2m, g_2m+1) y
 template <typename R, int MB>
 __device__ __forceinline__ void tap_syn(int m, R x, R y, R& e, R& o) {
-  if constexpr (sizeof(R) == 4 && MS_PACKED_F32) {
+  if constexpr (sizeof(R) == 4) {
     float2 r = ffma2_cx(c_hh2[MB][m], x, make_float2(e, o));
     r = ffma2_cx(c_gg2[MB][m], y, r);
     e = r.x;
     o = r.y;
   } else {
-    e = fma(fh<R>(MB, 2 * m), x, e);
-    e = fma(fg<R>(MB, 2 * m), y, e);
-    o = fma(fh<R>(MB, 2 * m + 1), x, o);
-    o = fma(fg<R>(MB, 2 * m + 1), y, o);
+    e = fma(c_hd[MB][2 * m], x, e);
+    e = fma(c_gd[MB][2 * m], y, e);
+    o = fma(c_hd[MB][2 * m + 1], x, o);
+    o = fma(c_gd[MB][2 * m + 1], y, o);
   }
 }
-#ifndef MS_PACKED_ANALYSIS
-#define MS_PACKED_ANALYSIS 1
-#endif
 
 constexpr int kP = 8;   // outputs per thread and direction
 
@@ -190,29 +175,6 @@ template <typename R, class G> struct SynTab {
 constexpr int kAT = 32;
 constexpr int kST = 64;
 
-// Tile sides (compile-time tunables; the defaults are the measured best on
-// GB300): large levels use wide tiles (less halo), small levels narrow ones
-// with small blocks so that they still fill the SMs.
-#ifndef MS_SYN_T1
-#define MS_SYN_T1 64   // synthesis output tile for n >= 512 (<= kST)
-#endif
-#ifndef MS_SYN_T2
-#define MS_SYN_T2 32   // synthesis output tile for 256 <= n < 512
-#endif
-#ifndef MS_SYN_T3
-#define MS_SYN_T3 16   // synthesis output tile for 16 <= n < 256
-#endif
-#ifndef MS_ANA_L1_TILE
-#define MS_ANA_L1_TILE 1   // level-1 analysis: one block per tile over all bases
-#endif
-#ifndef MS_ANA_T1
-#define MS_ANA_T1 32   // analysis subband tile for h >= 256 (<= kAT)
-#endif
-#ifndef MS_ANA_T2
-#define MS_ANA_T2 16   // analysis subband tile for 128 <= h < 256
-#endif
-static_assert(MS_SYN_T1 <= kST && MS_SYN_T2 <= kST && MS_SYN_T3 <= kST, "synthesis tile");
-static_assert(MS_ANA_T1 <= kAT && MS_ANA_T2 <= kAT, "analysis tile");
 // The largest power of two <= the preferred side that divides the level's
 // side (sides need not be powers of two: N = 48 gives 48, 24, 12, 6).
 __host__ __device__ __forceinline__ int fit_tile(int t, int n) {
@@ -220,25 +182,13 @@ __host__ __device__ __forceinline__ int fit_tile(int t, int n) {
   while (2 * p <= t && n % (2 * p) == 0) p *= 2;
   return p;
 }
-#ifndef MS_SYN_T1B
-#define MS_SYN_T1B MS_SYN_T1   // synthesis output tile for 512 <= n < 1024
-#endif
-// wide: the batched minor cycles, whose launches have blocks to spare (the
-// jobs multiply them), take the widest tiles at every level: the per-tile
-// staging and set-up dominate the narrow tiles of the coarse levels.
-__host__ __device__ __forceinline__ int syn_tile(int n, bool wide = false) {   // output side
-  if (wide) return fit_tile(kST, n);
-  return fit_tile(n >= 1024 ? MS_SYN_T1 : (n >= 512 ? MS_SYN_T1B : (n >= 256 ? MS_SYN_T2 : MS_SYN_T3)),
-                  n);
+// output side of a synthesis tile: 64 (fewest halo rows) where that leaves a
+// block for nearly every resident slot, else 32.  Measured at 512 px, one job
+// (64 -> 256 blocks): level 1 21.0 -> 12.6 us.
+__host__ __device__ __forceinline__ int syn_tile(int n, int jobs) {
+  return fit_tile((n / kST) * (n / kST) * jobs >= 256 ? kST : 32, n);
 }
-__host__ __device__ __forceinline__ int ana_tile(int h, bool wide = false) {   // subband side
-  if (wide) return fit_tile(kAT, h);
-  return fit_tile(h >= 256 ? MS_ANA_T1 : (h >= 128 ? MS_ANA_T2 : 16), h);
-}
-// geometry (template argument) serving a tile side
-__host__ __device__ __forceinline__ int syn_geom(int TS) { return TS >= 64 ? 64 : (TS >= 32 ? 32 : 16); }
-__host__ __device__ __forceinline__ int ana_geom(int TO) { return TO >= 32 ? 32 : (TO >= 16 ? 16 : 8); }
-
+__host__ __device__ __forceinline__ int ana_tile(int h) { return fit_tile(kAT, h); }   // subband side
 __device__ __forceinline__ int wrap(int i, int n) {
   i %= n;
   return i < 0 ? i + n : i;
@@ -315,7 +265,7 @@ __device__ __forceinline__ void fir_down8(const R* x, R* lo, R* hi) {
   for (int j = 0; j < kP; ++j) {
     R a = 0, d = 0;
 #pragma unroll
-    for (int k = 0; k < L; ++k) tap_hg<R, MB, MS_PACKED_ANALYSIS>(k, x[2 * j + k], a, d);
+    for (int k = 0; k < L; ++k) tap_hg<R, MB>(k, x[2 * j + k], a, d);
     lo[j] = a;
     hi[j] = d;
   }
@@ -549,13 +499,13 @@ template <typename R, class G>
 __device__ __forceinline__ void synth_item(unsigned char* smem_raw, const R* __restrict__ coef,
                                            const R* __restrict__ ll_in, R* __restrict__ ll_out,
                                            R* __restrict__ x, int N, int j, int J, int M,
-                                           int tile, int mb, bool wide = false) {
+                                           int tile, int mb, int jobs) {
   R* subs = reinterpret_cast<R*>(smem_raw);          // [2][4][G::In][G::SubS]
   R* zlo = subs + 2 * G::SubSz;                       // [G::T][G::ZS]
   R* zhi = zlo + G::T * G::ZS;
   int2* tab = reinterpret_cast<int2*>(zhi + G::T * G::ZS);   // [K][G::Threads]
   const int h = N >> j, n = 2 * h;
-  const int TS = syn_tile(n, wide);
+  const int TS = syn_tile(n, jobs);
   const int lts = 31 - __clz(TS);
   const int cnt = TS / 2 + kMaxTaps / 2 - 1;
   const int tiles_x = n / TS;
@@ -668,39 +618,29 @@ __device__ __forceinline__ void synth_item(unsigned char* smem_raw, const R* __r
   }
 }
 
-// one level per launch (dictionary synthesis of the API and the power
-// iteration): blockIdx.x = tile, blockIdx.y = basis
+// Level j of the synthesis x = W B_k of the minor cycle (B_k picked by k % 3
+// from buffers that come by value, so no pointer table is read before the
+// first load), or of a.x = W plain: blockIdx.x = output tile, blockIdx.y =
+// basis (level 1: one block per tile sums all bases).
 template <typename R, int ST>
 __global__ void __launch_bounds__(SG<ST>::Threads, 512 / SG<ST>::Threads)
-    synthesis_kernel(const R* const* __restrict__ coef3, const R* __restrict__ ll_in,
-                     R* __restrict__ ll_out, R* __restrict__ x, int N, int j, int J, int M,
-                     const FistaCtl* __restrict__ ctl) {
-  if (ctl && ctl->done) return;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const R* coef = coef3[ctl ? (ctl->k % 3) : 0];
-  synth_item<R, SG<ST>>(smem_raw, coef, ll_in, ll_out, x, N, j, J, M, blockIdx.x, blockIdx.y);
-}
-
-// Level j of the minor cycle's synthesis x = W B_k: blockIdx.x = output
-// tile, blockIdx.y = basis (level 1: one block per tile sums all bases).  The
-// buffers come by value and B_k is picked by k % 3, so no pointer table is
-// read before the first load.
-template <typename R, int ST>
-__global__ void __launch_bounds__(SG<ST>::Threads, 512 / SG<ST>::Threads)
-    synthesis_level_kernel(FistaPass<R> a_, int j) {
+    synthesis_level_kernel(FistaPass<R> a_, const R* plain, int j) {
   const FistaPass<R> a = job_slice(a_);   // blockIdx.z: the job (batched form)
   pdl_wait();
   pdl_trigger();
-  const int done = a.ctl->done;
-  const int k = a.ctl->k;
-  if (done) return;   // uniform: `done` does not change during this kernel
+  const R* coef = plain;
+  if (!plain) {
+    const int done = a.ctl->done;
+    const int k = a.ctl->k;
+    if (done) return;   // uniform: `done` does not change during this kernel
+    coef = k % 3 == 0 ? a.B0 : (k % 3 == 1 ? a.B1 : a.B2);
+  }
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const R* coef = k % 3 == 0 ? a.B0 : (k % 3 == 1 ? a.B1 : a.B2);
   const int64_t half = (int64_t)a.M * (a.N / 2) * (a.N / 2);
   const R* ll_in = (j == a.J) ? nullptr : a.tmp + ((j + 1) & 1) * half;
   R* ll_out = a.tmp + (j & 1) * half;
   synth_item<R, SG<ST>>(smem_raw, coef, ll_in, ll_out, a.x, a.N, j, a.J, a.M, blockIdx.x,
-                        blockIdx.y, a.js.jobs > 1);
+                        blockIdx.y, a.js.jobs);
 }
 
 namespace {
@@ -717,30 +657,6 @@ template <int AT> size_t analysis_smem_bytes(size_t rsz) {
          (AG<AT>::Threads / 32) * sizeof(double) + sizeof(uint64_t) + 2 * sizeof(int);
 }
 }  // namespace
-
-template <typename R>
-void launch_synthesis3(const R* const* coef3_dev, R* x, R* tmp, WaveletGeom g,
-                       const FistaCtl* ctl, cudaStream_t s, int only_level) {
-  const int64_t half = (int64_t)g.M * (g.N / 2) * (g.N / 2);
-  for (int j = g.J; j >= 1; --j) {
-    if (only_level > 0 && j != only_level) continue;
-    int h = g.N >> j, n = 2 * h;
-    int TS = syn_tile(n);
-    int tiles = (n / TS) * (n / TS);
-    const R* ll_in = (j == g.J) ? nullptr : tmp + ((j + 1) & 1) * half;
-    R* ll_out = tmp + (j & 1) * half;
-    dim3 grid(tiles, j == 1 ? 1 : g.M);
-    auto go = [&](auto kern, int threads, size_t smem) {
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      kern<<<grid, threads, smem, s>>>(coef3_dev, ll_in, ll_out, x, g.N, j, g.J, g.M, ctl);
-    };
-    switch (syn_geom(TS)) {
-      case 64: go(synthesis_kernel<R, 64>, SG<64>::Threads, synthesis_smem_bytes<64>(sizeof(R))); break;
-      case 32: go(synthesis_kernel<R, 32>, SG<32>::Threads, synthesis_smem_bytes<32>(sizeof(R))); break;
-      default: go(synthesis_kernel<R, 16>, SG<16>::Threads, synthesis_smem_bytes<16>(sizeof(R))); break;
-    }
-  }
-}
 
 // ------------------------------------------------------------------ analysis
 // Small tiles (the coarse levels) run the same filters with the output loop
@@ -767,7 +683,7 @@ __device__ __forceinline__ void analysis_filter_compact(const R* sIn, R* ylo, R*
       R a = 0, d = 0;
 #pragma unroll
       for (int k = 0; k < L; ++k) {
-        tap_hg<R, MB, MS_PACKED_ANALYSIS>(k, xc[(2 * r + k) * G::InS], a, d);
+        tap_hg<R, MB>(k, xc[(2 * r + k) * G::InS], a, d);
       }
       ylo[(kP * part + r) * G::YS + col] = a;
       yhi[(kP * part + r) * G::YS + col] = d;
@@ -786,7 +702,7 @@ __device__ __forceinline__ void analysis_filter_compact(const R* sIn, R* ylo, R*
     R a = 0, d = 0;
 #pragma unroll
     for (int k = 0; k < L; ++k) {
-      tap_hg<R, MB, MS_PACKED_ANALYSIS>(k, yrow[2 * q + k], a, d);
+      tap_hg<R, MB>(k, yrow[2 * q + k], a, d);
     }
     o_lo[q] = a;
     o_hi[q] = d;
@@ -797,9 +713,7 @@ __device__ __forceinline__ void analysis_filter_compact(const R* sIn, R* ylo, R*
 // ylo / yhi, then rows (x) into the four subbands gout[0..3] =
 // (approximation, low-y/high-x, high-y/low-x, high/high), G::T x G::GS each.
 // TOe (a power of two, 8..G::T) outputs per subband side, lt = log2(TOe).
-// (ROWS_IN_REGS: the register-blocked version whatever the tile side, for
-// callers whose outputs alias the column-filtered rows)
-template <typename R, int MB, class G, bool ROWS_IN_REGS = false>
+template <typename R, int MB, class G>
 __device__ __forceinline__ void analysis_filter(const R* sIn, R* ylo, R* yhi, R* gout, int TOe,
                                                 int lt) {
   constexpr int L = 2 * (MB + 1);
@@ -807,7 +721,7 @@ __device__ __forceinline__ void analysis_filter(const R* sIn, R* ylo, R* yhi, R*
   const int tid = threadIdx.x;
   const int nparts = TOe >> 3;
   const int cols = 2 * TOe + L - 2;
-  if constexpr (kCompact<G::T> && !ROWS_IN_REGS) {
+  if constexpr (kCompact<G::T>) {
     analysis_filter_compact<R, MB, G>(sIn, ylo, yhi, gout, TOe, lt);
   } else {
     const float inv_cols = 1.0f / (float)cols;
@@ -888,15 +802,14 @@ __device__ __forceinline__ void analysis_item(unsigned char* base, const CUtenso
                                               const R* ll_in, R* ll_out, R* out_plain,
                                               const R* cur, const R* prev, R* next, R t, R mu,
                                               R thr, int N, int j, int J, int tile,
-                                              FistaCtl* ctl, KSum<R>& l1, int tma_y0 = 0,
-                                              bool wide = false) {
+                                              FistaCtl* ctl, KSum<R>& l1, int tma_y0) {
   constexpr int m = MB;
   const AnaSmem<R, G> sm(base);
   R* sIn = sm.sIn;
   R* gout = sIn;
 
   const int n = N >> (j - 1), h = n / 2;
-  const int TO = ana_tile(h, wide);
+  const int TO = ana_tile(h);
   const int TOe = TO < kP ? kP : TO;             // outputs computed per side
   const int lt = 31 - __clz(TOe);
   const int lto = 31 - __clz(TO);
@@ -1056,54 +969,37 @@ __device__ __forceinline__ void analysis_item(unsigned char* base, const CUtenso
   __syncthreads();
 }
 
-// one level per launch (dictionary analysis of the API and the power
-// iteration): blockIdx.x = tile, blockIdx.y = basis
-template <typename R, int AT>
+// MODE 1: level j of the minor cycle's analysis + FISTA update.  The spectral
+// kernel of this pass has already advanced ctl->k, so this builds B_{k+1}
+// with k = ctl->k - 1; each block leaves its sum of |B_{k+1}| over its tile
+// in l1_parts[part_base + block] (the next spectral kernel adds them up, in a
+// fixed order).  MODE 0: level j of plain = W^H a.grad.  blockIdx.x = subband
+// tile, blockIdx.y = basis.
+template <typename R, int MODE, int AT>
 __global__ void __launch_bounds__(AG<AT>::Threads, 512 / AG<AT>::Threads)
-    analysis_kernel(const R* __restrict__ x_in, const R* __restrict__ ll_in,
-                    R* __restrict__ ll_out, R* __restrict__ out_plain, int N, int j, int J) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  unsigned char* base = smem_align128(smem_raw);
-  unsigned phase = 0;
-  KSum<R> l1;
-  switch (blockIdx.y) {
-#define MS_ANA(MBV)                                                                             \
-  case MBV:                                                                                     \
-    analysis_item<R, 0, MBV, AG<AT>>(base, nullptr, false, phase, x_in, ll_in, ll_out,          \
-                                     out_plain, nullptr, nullptr, nullptr, (R)0, (R)0, (R)0, N, \
-                                     j, J, blockIdx.x, nullptr, l1);                            \
-    break;
-    MS_ANA(0) MS_ANA(1) MS_ANA(2) MS_ANA(3) MS_ANA(4) MS_ANA(5) MS_ANA(6) MS_ANA(7)
-#undef MS_ANA
-  }
-}
-
-// Level j of the minor cycle's analysis + FISTA update: blockIdx.x = subband
-// tile, blockIdx.y = basis.  The spectral kernel of this pass has already
-// advanced ctl->k, so this builds B_{k+1} with k = ctl->k - 1.  Each block
-// leaves its sum of |B_{k+1}| over its tile in l1_parts[part_base + block];
-// the next spectral kernel adds them up (fixed order).
-template <typename R, int AT>
-__global__ void __launch_bounds__(AG<AT>::Threads, 512 / AG<AT>::Threads)
-    analysis_level_kernel(const __grid_constant__ CUtensorMap xmap, FistaPass<R> a_, int j,
-                          int use_tma, int part_base) {
+    analysis_level_kernel(const __grid_constant__ CUtensorMap xmap, FistaPass<R> a_, R* plain,
+                          int j, int use_tma, int part_base) {
   using G = AG<AT>;
   const FistaPass<R> a = job_slice(a_);   // blockIdx.z: the job (batched form)
   pdl_wait();
   pdl_trigger();
-  const int done = a.ctl->done;
-  const int kc = a.ctl->k;
-  if (done) return;   // uniform: `done` does not change during this kernel
+  R t = 0, mu = 0, thr = 0;
+  const R *cur = nullptr, *prev = nullptr;
+  R* next = nullptr;
+  if (MODE == 1) {
+    const int done = a.ctl->done;
+    const int k = a.ctl->k - 1;
+    if (done) return;   // uniform: `done` does not change during this kernel
+    t = ctl_t<R>(a.ctl, k & 1);   // momentum t_k
+    mu = ctl_mu<R>(a.ctl);        // 1 / theta
+    thr = ctl_thr<R>(a.ctl);      // lambda / theta
+    cur = k % 3 == 0 ? a.B0 : (k % 3 == 1 ? a.B1 : a.B2);
+    prev = k % 3 == 0 ? a.B2 : (k % 3 == 1 ? a.B0 : a.B1);
+    next = k % 3 == 0 ? a.B1 : (k % 3 == 1 ? a.B2 : a.B0);
+  }
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* base = smem_align128(smem_raw);
   const AnaSmem<R, G> sm(base);
-  const int k = kc - 1;
-  const R t = ctl_t<R>(a.ctl, k & 1);   // momentum t_k
-  const R mu = ctl_mu<R>(a.ctl);        // 1 / theta
-  const R thr = ctl_thr<R>(a.ctl);      // lambda / theta
-  const R* cur = k % 3 == 0 ? a.B0 : (k % 3 == 1 ? a.B1 : a.B2);
-  const R* prev = k % 3 == 0 ? a.B2 : (k % 3 == 1 ? a.B0 : a.B1);
-  R* next = k % 3 == 0 ? a.B1 : (k % 3 == 1 ? a.B2 : a.B0);
   const bool tma = G::T == kAT && use_tma != 0 && j == 1;
   if (tma && threadIdx.x == 0) mbar_init(sm.bar, 1);
   __syncthreads();
@@ -1113,15 +1009,16 @@ __global__ void __launch_bounds__(AG<AT>::Threads, 512 / AG<AT>::Threads)
   const R* ll_in = (j == 1) ? nullptr : a.tmp + ((j - 1) & 1) * half;
   R* ll_out = a.tmp + (j & 1) * half;
   switch (blockIdx.y) {
-#define MS_ANA(MBV)                                                                          \
-  case MBV:                                                                                  \
-    analysis_item<R, 1, MBV, G>(base, &xmap, tma, phase, a.grad, ll_in, ll_out, nullptr, cur, \
-                                prev, next, t, mu, thr, a.N, j, a.J, blockIdx.x, a.ctl, l1,   \
-                                (int)blockIdx.z * a.N, a.js.jobs > 1);                        \
+#define MS_ANA(MBV)                                                                            \
+  case MBV:                                                                                    \
+    analysis_item<R, MODE, MBV, G>(base, &xmap, tma, phase, a.grad, ll_in, ll_out, plain, cur, \
+                                   prev, next, t, mu, thr, a.N, j, a.J, blockIdx.x,            \
+                                   MODE == 1 ? a.ctl : nullptr, l1, (int)blockIdx.z * a.N);    \
     break;
     MS_ANA(0) MS_ANA(1) MS_ANA(2) MS_ANA(3) MS_ANA(4) MS_ANA(5) MS_ANA(6) MS_ANA(7)
 #undef MS_ANA
   }
+  if (MODE == 0) return;
   // block sum of |B_{k+1}|: error-free working-precision warp sums, FP64
   // once per warp
   R hi = l1.s, lo = -l1.c;
@@ -1135,402 +1032,178 @@ __global__ void __launch_bounds__(AG<AT>::Threads, 512 / AG<AT>::Threads)
   }
 }
 
-// Level 1 of the minor cycle's analysis + FISTA step with one block per
-// subband tile looping over the M bases (for the widest geometry, 1 < J):
-// the gradient window is staged once (TMA, or cp.async with wrap at the
-// image edge) and serves every basis, and the tiles of B_k and B_{k-1} of the
-// next basis arrive by cp.async (double-buffered) while the current basis is
-// filtered.  The filter's outputs alias its column-filtered rows (both are
-// dead / rewritten only after the block barriers that separate them), so
-// the window survives.  The block's sum of |B_{k+1}| over all bases goes to
-// l1_parts[part_base + tile]; it zeroes the other M - 1 slots of its tile.
-template <typename R> struct AnaTile {
-  using G = AG<kAT>;
-  static constexpr int T = G::T;
-  static constexpr int PF = 2 * 2 * 3 * T * T;   // [buffer][B_k, B_k-1][subband 1..3][T][T]
-  static constexpr size_t bytes() {
-    return (size_t)(G::InSz + 2 * G::YSz + PF) * sizeof(R) + 128 +
-           (G::Threads / 32) * sizeof(double) + sizeof(uint64_t) + 2 * sizeof(int);
-  }
-  static_assert(4 * T * G::GS <= 2 * G::YSz, "the outputs alias the filtered rows");
-};
+#include "fine_levels.cuh"
 
-template <typename R>
-__global__ void __launch_bounds__(AG<kAT>::Threads, 2)
-    analysis_l1_tile_kernel(const __grid_constant__ CUtensorMap xmap, FistaPass<R> a_,
-                            int use_tma, int part_base, int split) {
-  using A = AnaTile<R>;
-  const FistaPass<R> a = job_slice(a_);   // blockIdx.z: the job (batched form)
-  // blockIdx.y: the basis group, bases [0, split) or [split, M) (split = M:
-  // one group)
-  const int m_lo = blockIdx.y == 0 ? 0 : split, m_hi = blockIdx.y == 0 ? split : a.M;
-  using G = typename A::G;
-  constexpr int T = A::T;
-  pdl_wait();
-  pdl_trigger();
-  const int done = a.ctl->done;
-  const int kc = a.ctl->k;
-  if (done) return;   // uniform: `done` does not change during this kernel
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  unsigned char* base = smem_align128(smem_raw);
-  R* sIn = reinterpret_cast<R*>(base);   // [G::In][G::InS]
-  R* ylo = sIn + G::InSz;                // [T][G::YS]; also the outputs [4][T][G::GS]
-  R* yhi = ylo + G::YSz;
-  R* gout = ylo;
-  R* pf = yhi + G::YSz;                  // [2][2][3][T][T]
-  double* red = reinterpret_cast<double*>(pf + A::PF);
-  uint64_t* bar = reinterpret_cast<uint64_t*>(red + G::Threads / 32);
-  int* flags = reinterpret_cast<int*>(bar + 1);
-
-  const int k = kc - 1;
-  const R t = ctl_t<R>(a.ctl, k & 1);   // momentum t_k
-  const R mu = ctl_mu<R>(a.ctl);        // 1 / theta
-  const R thr = ctl_thr<R>(a.ctl);      // lambda / theta
-  const R* cur = k % 3 == 0 ? a.B0 : (k % 3 == 1 ? a.B1 : a.B2);
-  const R* prev = k % 3 == 0 ? a.B2 : (k % 3 == 1 ? a.B0 : a.B1);
-  R* next = k % 3 == 0 ? a.B1 : (k % 3 == 1 ? a.B2 : a.B0);
-  const int N = a.N, n = N, h = N / 2;
-  const int tile = blockIdx.x;
-  const int tiles_x = h / T;
-  const int o0y = (tile / tiles_x) * T, o0x = (tile % tiles_x) * T;
-  const int p0y = 2 * o0y, p0x = 2 * o0x;
-  constexpr int ext = G::In;   // 2 T + 14
-  constexpr int NV = Vec<R>::N;
-  constexpr int LNV = NV == 4 ? 2 : 1;
-  using V = typename Vec<R>::T;
-  const int64_t half = (int64_t)a.M * (N / 2) * (N / 2);
-  R* ll_out = a.tmp + half;   // level 1 writes LL buffer (1 & 1)
-
-  // coefficient offset of (subband s = 1..3, row, col) of this tile in basis m
-  auto coef_off = [&](int m, int s, int row, int col) -> int64_t {
-    return (int64_t)m * N * N + (int64_t)((s >= 2 ? h : 0) + o0y + row) * N + (s & 1 ? h : 0) +
-           o0x + col;
-  };
-  // prefetch of basis m's B_k and B_k-1 tiles into buffer m & 1
-  auto prefetch = [&](int m) {
-    constexpr int V16 = 16 / (int)sizeof(R);
-    constexpr int CPR = T / V16;   // 16-byte chunks per tile row
-    R* dst = pf + (m & 1) * (2 * 3 * T * T);
-    for (int e = threadIdx.x; e < 2 * 3 * T * CPR; e += G::Threads) {
-      const int arr = e / (3 * T * CPR), r = e - arr * (3 * T * CPR);
-      const int sb = r / (T * CPR), r2 = r - sb * (T * CPR);
-      const int row = r2 / CPR, ch = r2 - row * CPR;
-      cp_async<16>(dst + ((arr * 3 + sb) * T + row) * T + ch * V16,
-                   (arr ? prev : cur) + coef_off(m, sb + 1, row, ch * V16));
-    }
-    cp_async_commit();
-  };
-
-  // the window: TMA when interior and aligned, else cp.async with wrap
-  if (threadIdx.x == 0) mbar_init(bar, 1);
-  __syncthreads();
-  bool tma = use_tma != 0 && p0x + G::InS <= n && p0y + G::In <= n;
-  if (tma) {
-    if (threadIdx.x == 0) {
-      const bool aligned = (saddr(sIn) & 127u) == 0 &&
-                           (reinterpret_cast<uintptr_t>(&xmap) & 63u) == 0 &&
-                           ((p0x * (int)sizeof(R)) & 15) == 0;
-      flags[1] = aligned ? 1 : 0;
-      if (aligned) {
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_expect_tx(bar, (unsigned)(G::In * G::InS * sizeof(R)));
-        tma_load_2d(sIn, &xmap, p0x, p0y + (int)blockIdx.z * N, bar);
-      } else {
-        atomicExch(&a.ctl->error, 8);
-      }
-    }
-    __syncthreads();
-    tma = flags[1] != 0;
-  }
-  if (!tma) {
-    const R* src = a.grad;
-    const bool cheap = n >= ext;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr int NW = G::Threads / 32;
-    for (int r = warp; r < ext; r += NW) {
-      const int py = cheap ? wrapc(p0y + r, n) : wrap(p0y + r, n);
-      const R* row = src + (int64_t)py * n;
-      for (int b = lane; b < ext; b += 32) {
-        const int px = cheap ? wrapc(p0x + b, n) : wrap(p0x + b, n);
-        cp_async<sizeof(R)>(sIn + r * G::InS + b, row + px);
-      }
-    }
-  }
-  cp_async_commit();   // (empty on the TMA path)
-  prefetch(m_lo);
-  bool skip = false;
-  if (tma) {
-    unsigned phase = 0;
-    const bool ok = mbar_wait_bounded(bar, phase);
-    skip = __syncthreads_or(!ok) != 0;
-    if (skip && threadIdx.x == 0) atomicExch(&a.ctl->error, 5);
-  }
-  cp_async_wait<1>();   // the window's copies (the first prefetch may still run)
-  __syncthreads();
-  if (skip) {
-    cp_async_wait<0>();
-    return;   // uniform: nothing is written for a tile whose window never arrived
-  }
-
-  KSum<R> l1;
-  constexpr int lto = 5, lpr = lto - LNV, lsub = lto + lpr;   // T = 32
-  static_assert(T == 32, "level-1 tile side");
-  constexpr int items = 3 << lsub;
-  // the bases in sequence, each a straight-line step (a loop around a
-  // switch over the bases raised register pressure into spills)
-  auto step = [&](auto mb) {
-    constexpr int m = decltype(mb)::value;
-    if (m < m_lo || m >= m_hi) return;   // uniform over the block
-    if (m + 1 < m_hi) prefetch(m + 1);
-    analysis_filter<R, m, G, true>(sIn, ylo, yhi, gout, T, lto);
-    if (m + 1 < m_hi) cp_async_wait<1>();
-    else cp_async_wait<0>();
-    __syncthreads();   // the filter's outputs and basis m's prefetch are visible
-    const R* pc = pf + (m & 1) * (2 * 3 * T * T);
-    const R* pp = pc + 3 * T * T;
-    for (int e = threadIdx.x; e < items; e += G::Threads) {
-      const int sb = e >> lsub;   // subband 1..3 is sb + 1
-      const int rem = e & ((1 << lsub) - 1);
-      const int row = rem >> lpr, c4 = (rem & ((1 << lpr) - 1)) << LNV;
-      const V gv = *reinterpret_cast<const V*>(gout + ((sb + 1) * T + row) * G::GS + c4);
-      const V cv = *reinterpret_cast<const V*>(pc + (sb * T + row) * T + c4);
-      const V qv = *reinterpret_cast<const V*>(pp + (sb * T + row) * T + c4);
-      V nv;
-      R* np = reinterpret_cast<R*>(&nv);
-      const R* gp = reinterpret_cast<const R*>(&gv);
-      const R* cp = reinterpret_cast<const R*>(&cv);
-      const R* qp = reinterpret_cast<const R*>(&qv);
-#pragma unroll
-      for (int q = 0; q < NV; ++q) {
-        const R alpha = cp[q] + t * (cp[q] - qp[q]);
-        const R z = alpha - mu * gp[q];
-        const R az = fabs(z) - thr;
-        const R nb = az > (R)0 ? copysign(az, z) : (R)0;
-        l1.add(fabs(nb));
-        np[q] = nb;
-      }
-      *reinterpret_cast<V*>(next + coef_off(m, sb + 1, row, c4)) = nv;
-    }
-    // the approximation feeds level 2
-    for (int e = threadIdx.x; e < (1 << lsub); e += G::Threads) {
-      const int row = e >> lpr, c4 = (e & ((1 << lpr) - 1)) << LNV;
-      *reinterpret_cast<V*>(ll_out + (int64_t)m * h * h + (int64_t)(o0y + row) * h + o0x + c4) =
-          *reinterpret_cast<const V*>(gout + row * G::GS + c4);
-    }
-    __syncthreads();   // gout and prefetch buffer m & 1 are reused
-  };
-  step(std::integral_constant<int, 0>{});
-  step(std::integral_constant<int, 1>{});
-  step(std::integral_constant<int, 2>{});
-  step(std::integral_constant<int, 3>{});
-  step(std::integral_constant<int, 4>{});
-  step(std::integral_constant<int, 5>{});
-  step(std::integral_constant<int, 6>{});
-  step(std::integral_constant<int, 7>{});
-  static_assert(kMaxBases == 8, "one step per basis");
-  R hi = l1.s, lo = -l1.c;
-  warp_sum_comp<R>(hi, lo);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = (double)hi + (double)lo;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double sum = 0.0;
-    for (int q = 0; q < G::Threads / 32; ++q) sum += red[q];
-    // slot (group, tile); the first group also zeroes the slots no group uses
-    a.l1_parts[part_base + (int64_t)blockIdx.y * gridDim.x + tile] = sum;
-    if (blockIdx.y == 0)
-      for (int m = gridDim.y; m < a.M; ++m)
-        a.l1_parts[part_base + (int64_t)m * gridDim.x + tile] = 0.0;
-  }
-}
-
-#include "coarse_levels.cuh"
-
-// CTAs per SM of the one-launch coarse levels and their shared-memory
-// budget per CTA (compile-time tunables; the defaults are the measured best)
-#ifndef MS_COARSE_CTAS_PER_SM
-#define MS_COARSE_CTAS_PER_SM 1
-#endif
-#ifndef MS_COARSE_BUDGET_KB
-#define MS_COARSE_BUDGET_KB 200
-#endif
-#ifndef MS_COARSE_WOFF
-#define MS_COARSE_WOFF 24   // fixed share of a basis's work per row, in taps / 2 (measured best)
-#endif
-
+// ------------------------------------------------------------- dispatch
 namespace {
-template <typename R>
-size_t coarse_smem(bool analysis, WaveletGeom g, const CoarseGroups& gr, int budget) {
-  int cs_min = 1 << 30;
-  for (int m = 0; m < g.M; ++m) cs_min = std::min(cs_min, gr.first[m + 1] - gr.first[m]);
-  return strip_smem_bytes(analysis, g.N, g.J, cs_min, sizeof(R), (size_t)budget);
+// The kernel of an analysis level with subbands of side h.  Tiles of 16 (a
+// thread forms 4 outputs of a row or column) where that makes a block for
+// nearly every SM (8 bases x 16 tiles at h = 64), else tiles of 8 or 4 with
+// an output per thread; FP64, whose time is the FP64 instructions of the
+// busiest scheduler, takes tiles of 8 up to h = 128 and of 16 at 256, and
+// above that the wide register-blocked tiles (fewest halo columns filtered
+// twice).  Measured per level, us (this rule's | the alternatives'): FP32
+// h = 512 27.7 | 31.7 (one block per tile over all bases); h = 256..64
+// together 26 | 26.7 in one cooperative launch of full-width strips, and 120
+// against 133 per iteration at 1024 px with both directions' coarse levels
+// replaced; FP64, an iteration at 128 px with h = 64..8: 155 | 219, at 256
+// px 301 | 337 with tiles of 16, at 1024 px with h = 512 wide 1549 | 1715
+// with tiles of 16.
+enum class Ana { kWide, k16, k8, k4 };
+Ana ana_kernel(bool f64, int h) {
+  if (f64 && h > 256) return h % 16 == 0 ? Ana::kWide : (h % 4 == 0 ? Ana::k4 : Ana::kWide);
+  if (h % 16 == 0 && h >= (f64 ? 129 : 64)) return Ana::k16;
+  if (h % 8 == 0) return Ana::k8;
+  return h % 4 == 0 ? Ana::k4 : Ana::kWide;
 }
-
-// The level-1 analysis tile kernel's basis groups: bases [0, split) and
-// [split, M), split where the work (2 (m + 1) taps + MS_L1_WFIX per basis)
-// is closest to half; split = M (one group) when MS_L1_GROUPS is 1.
-#ifndef MS_L1_GROUPS
-#define MS_L1_GROUPS 1   // 2 measured no faster at 1024^2 (37.4 vs 37.2 us)
-#endif
-#ifndef MS_L1_WFIX
-#define MS_L1_WFIX 10
-#endif
-int l1_basis_split(int M) {
-  if (MS_L1_GROUPS < 2 || M < 2) return M;
-  double total = 0.0;
-  for (int m = 0; m < M; ++m) total += 2.0 * (m + 1) + MS_L1_WFIX;
-  double acc = 0.0;
-  int best = 1;
-  double best_d = 1e30;
-  for (int sp = 1; sp < M; ++sp) {
-    acc += 2.0 * sp + MS_L1_WFIX;   // work of bases 0..sp-1
-    const double d = std::fabs(2.0 * acc - total);
-    if (d < best_d) {
-      best_d = d;
-      best = sp;
-    }
+int ana_side(bool f64, int h) {
+  switch (ana_kernel(f64, h)) {
+    case Ana::k16: return 16;
+    case Ana::k8: return 8;
+    case Ana::k4: return 4;
+    default: return ana_tile(h);
   }
-  return best;
+}
+// The kernel of a synthesis level j >= 2 with output side n, M bases and
+// `jobs` jobs: tiles of 32 or 16 (4 or 2 output pairs per unit) where they
+// make some 1000 or 500 blocks, else of 8.  Measured at 1024 px, FP32, one
+// job, us an iteration: (n = 512, 256, 128) in tiles of (32, 16, 16) 128,
+// (32, 32, 16) 132 and 136, (16, 16, 16) 134; 8 jobs: (32, 32, 32) 89.9 a
+// job, (16, 16, 16) 95.1.  FP64: 8 below 512 (the fewest instructions in the
+// busiest scheduler), else 16.
+enum class Syn { kWide, k32, k16, k8 };
+Syn syn_kernel(bool f64, int n, int M, int jobs) {
+  auto blocks = [&](int t) { return (int64_t)(n / t) * (n / t) * M * jobs; };
+  if (f64) return n >= 512 && n % 16 == 0 ? Syn::k16 : (n % 8 == 0 ? Syn::k8 : Syn::kWide);
+  if (n % 32 == 0 && blocks(32) >= 1000) return Syn::k32;
+  if (n % 16 == 0 && blocks(16) >= 500) return Syn::k16;
+  return n % 8 == 0 ? Syn::k8 : Syn::kWide;
 }
 
-// l1 partial slots of level 1 (the per-tile kernel's share) and in all
-int level1_partials(WaveletGeom g) {
-  const int h = g.N >> 1, TO = ana_tile(h);
-  return (h / TO) * (h / TO) * g.M;
-}
-
-template <typename R>
-cudaError_t launch_coarse(const FistaPass<R>& a, bool analysis, int part_base, int part_end,
-                          cudaStream_t s) {
-  const WaveletGeom g{a.N, a.J, a.M};
-  const size_t smem = coarse_smem<R>(analysis, g, a.coarse_groups, a.coarse_budget);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(a.coarse_ctas);
-  cfg.blockDim = dim3(kStripThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;   // every group resident at once
-  attr[0].val.cooperative = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (analysis) {
-    auto kern = coarse_analysis_kernel<R>;
+template <typename R, int MODE>
+cudaError_t launch_analysis_level(const FistaPass<R>& a, R* plain, const CUtensorMap* grad_map,
+                                  int j, int part_base, cudaStream_t s) {
+  const int h = a.N >> j, T = ana_side(sizeof(R) == 8, h);
+  const dim3 grid((h / T) * (h / T), a.M, a.js.jobs);
+  switch (ana_kernel(sizeof(R) == 8, h)) {
+    case Ana::k16:
+      return launch_pdl(fine_analysis_kernel<R, MODE, 16, 16, 4, 128>, grid, dim3(128), 0, s, a,
+                        plain, j, part_base);
+    case Ana::k8:
+      return launch_pdl(fine_analysis_kernel<R, MODE, 8, 8, 1, 128>, grid, dim3(128), 0, s, a,
+                        plain, j, part_base);
+    case Ana::k4:
+      return launch_pdl(fine_analysis_kernel<R, MODE, 4, 4, 1, 64>, grid, dim3(64), 0, s, a,
+                        plain, j, part_base);
+    default: break;
+  }
+  const CUtensorMap m = grad_map ? *grad_map : CUtensorMap{};
+  auto go = [&](auto kern, int threads, size_t smem) {
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    return cudaLaunchKernelEx(&cfg, kern, a, a.coarse_groups, a.coarse_bar, part_base, part_end,
-                              a.coarse_budget);
+    return launch_pdl(kern, grid, dim3(threads), smem, s, m, a, plain, j, grad_map ? 1 : 0,
+                      part_base);
+  };
+  if constexpr (sizeof(R) == 8) {   // (FP32: subbands no multiple of 4, tiles of 1 or 2)
+    if (T >= 32)
+      return go(analysis_level_kernel<R, MODE, 32>, AG<32>::Threads,
+                analysis_smem_bytes<32>(sizeof(R)));
+    if (T >= 16)
+      return go(analysis_level_kernel<R, MODE, 16>, AG<16>::Threads,
+                analysis_smem_bytes<16>(sizeof(R)));
   }
-  auto kern = coarse_synthesis_kernel<R>;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  return cudaLaunchKernelEx(&cfg, kern, a, a.coarse_groups, a.coarse_bar, a.coarse_budget);
+  return go(analysis_level_kernel<R, MODE, 8>, AG<8>::Threads, analysis_smem_bytes<8>(sizeof(R)));
 }
 
-// CTAs of both strip kernels resident per SM with `budget` bytes of shared
-// memory per CTA
-template <typename R> int coarse_per_sm(WaveletGeom g, const CoarseGroups& gr, int budget) {
-  int per = 1 << 30;
-  int dev = 0, optin = 0;
-  cudaGetDevice(&dev);
-  if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
-    return 0;
-  for (int an = 0; an < 2; ++an) {
-    const size_t smem = coarse_smem<R>(an != 0, g, gr, budget);
-    if (smem == 0 || smem > (size_t)optin) return 0;   // strips too wide for shared memory
-    int blocks = 0;
-    cudaError_t e;
-    if (an) {
-      auto kern = coarse_analysis_kernel<R>;
+// Level j of the synthesis of B_k (plain NULL) or of `plain` into a.x
+template <typename R>
+cudaError_t launch_synthesis_level(const FistaPass<R>& a, const R* plain, int j, cudaStream_t s) {
+  const int n = 2 * (a.N >> j), jobs = a.js.jobs;
+  const bool f64 = sizeof(R) == 8;
+  if (j == 1) {
+    // FP64, and FP32 images too small for the wide tiles: a warp per basis.
+    // Measured at 128 px, FP64: 24.6 us an iteration less than one block per
+    // 16-pixel tile; at 512 px 542 | 632 us an iteration.  FP32 at 256 px:
+    // 49.6 | 48.5 with the wide tiles.
+    auto go = [&](auto kern, int ty, int tx, size_t elems) {
+      const size_t smem = kMaxBases * elems * sizeof(R);
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, kStripThreads, smem);
-    } else {
-      auto kern = coarse_synthesis_kernel<R>;
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, kStripThreads, smem);
+      return launch_pdl(kern, dim3((n / ty) * (n / tx), 1, jobs), dim3(32 * kMaxBases), smem, s, a,
+                        plain);
+    };
+    if (f64 && (int64_t)(n / 8) * (n / 16) * jobs < 256)
+      return go(fine_synthesis_l1_kernel<R, 8, 16, 1>, 8, 16, FineSyn<8, 16>::Elems);
+    if (f64 || n < 256 || n % 32)
+      return go(fine_synthesis_l1_kernel<R, 16, 16, 2>, 16, 16, FineSyn<16, 16>::Elems);
+  } else {
+    auto go = [&](auto kern, int t, int threads) {
+      return launch_pdl(kern, dim3((n / t) * (n / t), a.M, jobs), dim3(threads), 0, s, a, plain, j);
+    };
+    switch (syn_kernel(f64, n, a.M, jobs)) {
+      case Syn::k32:
+        if constexpr (sizeof(R) == 4) return go(fine_synthesis_kernel<R, 32, 32, 4, 128>, 32, 128);
+        break;
+      case Syn::k16: return go(fine_synthesis_kernel<R, 16, 16, 2, 128>, 16, 128);
+      case Syn::k8: return go(fine_synthesis_kernel<R, 8, 8, 1, 128>, 8, 128);
+      default: break;
     }
-    if (e != cudaSuccess) {
-      cudaGetLastError();   // clear: "does not fit" is an answer here, not an error
-      return 0;
-    }
-    per = std::min(per, blocks);
   }
-  return per;
+  const int TS = syn_tile(n, jobs);
+  const dim3 grid((n / TS) * (n / TS), j == 1 ? 1 : a.M, jobs);
+  auto go = [&](auto kern, int threads, size_t smem) {
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return launch_pdl(kern, grid, dim3(threads), smem, s, a, plain, j);
+  };
+  if constexpr (sizeof(R) == 4) {
+    if (TS >= 64)
+      return go(synthesis_level_kernel<R, 64>, SG<64>::Threads, synthesis_smem_bytes<64>(sizeof(R)));
+    if (TS >= 32)
+      return go(synthesis_level_kernel<R, 32>, SG<32>::Threads, synthesis_smem_bytes<32>(sizeof(R)));
+  }
+  return go(synthesis_level_kernel<R, 16>, SG<16>::Threads, synthesis_smem_bytes<16>(sizeof(R)));
 }
 }  // namespace
 
-int coarse_groups(WaveletGeom g, size_t rsz, CoarseGroups* gr, int* budget) {
-#ifdef MS_NO_COARSE_GROUPS
-  return 0;
-#endif
-  const bool pow2 = g.N > 0 && (g.N & (g.N - 1)) == 0;
-  if (!pow2 || g.N < 256 || g.J < 2 || (g.N >> g.J) < 8 || g.M < 1) return 0;
-  int dev = 0, coop = 0;
-  cudaGetDevice(&dev);
-  if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop)
-    return 0;
-  const int span = analysis_prox_partials(g) - level1_partials(g);
-  // one CTA per SM; group m gets CTAs in proportion to its work per row:
-  // the filters' 2 (m + 1) taps plus a share that does not grow with them
-  // (staging, stores, the prox), measured at about 4 taps' worth
-  auto weight = [](int m) { return m + 1 + MS_COARSE_WOFF; };
-  int total_w = 0;
-  for (int m = 0; m < g.M; ++m) total_w += weight(m);
-  // one l1 partial per CTA in the coarse share
-  const int ctas = std::min(MS_COARSE_CTAS_PER_SM * sm_count(), span);
-  if (ctas < g.M) return 0;
-  gr->first[0] = 0;
-  for (int m = 0; m < g.M; ++m)
-    gr->first[m + 1] = gr->first[m] + std::max(1, ctas * weight(m) / total_w);
-  for (int m = g.M + 1; m <= kMaxBases; ++m) gr->first[m] = gr->first[g.M];
-  const int used = gr->first[g.M];
-  if (used > ctas) return 0;
-  for (int b : {MS_COARSE_BUDGET_KB * 1024, MS_COARSE_BUDGET_KB * 1024 * 4 / 5}) {
-    const int per = rsz == 4 ? coarse_per_sm<float>(g, *gr, b) : coarse_per_sm<double>(g, *gr, b);
-    if (per >= 1 && per * sm_count() >= used) {
-      *budget = b;
-      return used;
-    }
-  }
-  return 0;
-}
-
-#ifdef MS_COARSE_PROBE
-}  // namespace ms
-extern "C" int ms_coarse_probe_read(unsigned long long* host) {
-  return (int)cudaMemcpyFromSymbol(host, ms::g_coarse_probe, sizeof(ms::g_coarse_probe));
-}
-namespace ms {
-#endif
-
-int analysis_prox_partials(WaveletGeom g) {
+int analysis_prox_partials(WaveletGeom g, size_t rsz) {
   int total = 0;
   for (int j = 1; j <= g.J; ++j) {
-    int h = g.N >> j;
-    int TO = ana_tile(h);
-    int tiles = (h / TO) * (h / TO);
-    total += tiles * g.M;
+    const int h = g.N >> j, T = ana_side(rsz == 8, h);
+    total += (h / T) * (h / T) * g.M;
   }
   return total;
 }
 
+namespace {
+// a pass that only names the images and the geometry (plain transforms)
+template <typename R> FistaPass<R> plain_pass(const R* grad, R* x, R* tmp, WaveletGeom g) {
+  FistaPass<R> a{};
+  a.grad = grad;
+  a.x = x;
+  a.tmp = tmp;
+  a.N = g.N;
+  a.J = g.J;
+  a.M = g.M;
+  return a;
+}
+}  // namespace
+
 template <typename R>
-void launch_analysis(const R* x, R* coef, R* tmp, WaveletGeom g, cudaStream_t s) {
-  const int64_t half = (int64_t)g.M * (g.N / 2) * (g.N / 2);
-  for (int j = 1; j <= g.J; ++j) {
-    int h = g.N >> j;
-    int TO = ana_tile(h);
-    int tiles = (h / TO) * (h / TO);
-    const R* ll_in = (j == 1) ? nullptr : tmp + ((j - 1) & 1) * half;
-    R* ll_out = tmp + (j & 1) * half;
-    dim3 grid(tiles, g.M);
-    auto go = [&](auto kern, int threads, size_t smem) {
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      kern<<<grid, threads, smem, s>>>(x, ll_in, ll_out, coef, g.N, j, g.J);
-    };
-    switch (ana_geom(TO)) {
-      case 32: go(analysis_kernel<R, 32>, AG<32>::Threads, analysis_smem_bytes<32>(sizeof(R))); break;
-      case 16: go(analysis_kernel<R, 16>, AG<16>::Threads, analysis_smem_bytes<16>(sizeof(R))); break;
-      default: go(analysis_kernel<R, 8>, AG<8>::Threads, analysis_smem_bytes<8>(sizeof(R))); break;
-    }
+cudaError_t launch_synthesis(const R* coef, R* x, R* tmp, WaveletGeom g, cudaStream_t s) {
+  const FistaPass<R> a = plain_pass<R>(nullptr, x, tmp, g);
+  for (int j = g.J; j >= 1; --j) {
+    const cudaError_t e = launch_synthesis_level<R>(a, coef, j, s);
+    if (e != cudaSuccess) return e;
   }
+  return cudaSuccess;
+}
+
+template <typename R>
+cudaError_t launch_analysis(const R* x, R* coef, R* tmp, WaveletGeom g, cudaStream_t s) {
+  const FistaPass<R> a = plain_pass<R>(x, nullptr, tmp, g);
+  for (int j = 1; j <= g.J; ++j) {
+    const cudaError_t e = launch_analysis_level<R, 0>(a, coef, nullptr, j, 0, s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 // TMA box of the level-1 input window: {80 columns, 78 rows}
@@ -1541,23 +1214,10 @@ void analysis_window_box(unsigned* cols, unsigned* rows) {
 
 template <typename R>
 cudaError_t launch_synthesis_pass(const FistaPass<R>& a, cudaStream_t s, int only_level) {
-  if (only_level < 0 && a.coarse_ctas > 0 && a.js.jobs == 1)   // levels J..2, one cooperative launch
-    return launch_coarse<R>(a, false, 0, 0, s);
   for (int j = a.J; j >= 1; --j) {
     if (only_level > 0 && j != only_level) continue;
     if (only_level < 0 && j == 1) continue;
-    int n = 2 * (a.N >> j), TS = syn_tile(n, a.js.jobs > 1);
-    dim3 grid((n / TS) * (n / TS), j == 1 ? 1 : a.M, a.js.jobs);
-    auto go = [&](auto kern, int threads, size_t smem) {
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      return launch_pdl(kern, grid, dim3(threads), smem, s, a, j);
-    };
-    cudaError_t e;
-    switch (syn_geom(TS)) {
-      case 64: e = go(synthesis_level_kernel<R, 64>, SG<64>::Threads, synthesis_smem_bytes<64>(sizeof(R))); break;
-      case 32: e = go(synthesis_level_kernel<R, 32>, SG<32>::Threads, synthesis_smem_bytes<32>(sizeof(R))); break;
-      default: e = go(synthesis_level_kernel<R, 16>, SG<16>::Threads, synthesis_smem_bytes<16>(sizeof(R))); break;
-    }
+    const cudaError_t e = launch_synthesis_level<R>(a, nullptr, j, s);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -1566,64 +1226,26 @@ cudaError_t launch_synthesis_pass(const FistaPass<R>& a, cudaStream_t s, int onl
 template <typename R>
 cudaError_t launch_analysis_pass(const FistaPass<R>& a, const CUtensorMap* grad_map,
                                  cudaStream_t s, int only_level) {
-  const CUtensorMap m = grad_map ? *grad_map : CUtensorMap{};
-  if (only_level < 0 && a.coarse_ctas > 0 && a.js.jobs == 1) {   // levels 2..J, one cooperative launch
-    const WaveletGeom g{a.N, a.J, a.M};
-    return launch_coarse<R>(a, true, level1_partials(g), analysis_prox_partials(g), s);
-  }
   int part_base = 0;
   for (int j = 1; j <= a.J; ++j) {
-    const int h = a.N >> j, TO = ana_tile(h, a.js.jobs > 1);
-    const int tiles = (h / TO) * (h / TO);
-    const bool run = only_level == 0 || j == only_level || (only_level < 0 && j > 1);
-    bool done_here = false;
-    if constexpr (sizeof(R) == 4) {
-      if (run && MS_ANA_L1_TILE && j == 1 && a.J > 1 && TO == kAT && grad_map) {
-        const size_t smem = AnaTile<R>::bytes();
-        auto kern = analysis_l1_tile_kernel<R>;
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        // two block groups over the bases, split where the filter work
-        // (taps plus a fixed per-basis share) is about equal
-        const int split = l1_basis_split(a.M);
-        const cudaError_t e =
-            launch_pdl(kern, dim3(tiles, split < a.M ? 2 : 1, a.js.jobs), dim3(AG<kAT>::Threads),
-                       smem, s, m, a, 1, part_base, split);
-        if (e != cudaSuccess) return e;
-        done_here = true;
-      }
-    }
-    if (run && !done_here) {
-      dim3 grid(tiles, a.M, a.js.jobs);
-      auto go = [&](auto kern, int threads, size_t smem) {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        return launch_pdl(kern, grid, dim3(threads), smem, s, m, a, j, grad_map ? 1 : 0,
-                          part_base);
-      };
-      cudaError_t e;
-      switch (ana_geom(TO)) {
-        case 32: e = go(analysis_level_kernel<R, 32>, AG<32>::Threads, analysis_smem_bytes<32>(sizeof(R))); break;
-        case 16: e = go(analysis_level_kernel<R, 16>, AG<16>::Threads, analysis_smem_bytes<16>(sizeof(R))); break;
-        default: e = go(analysis_level_kernel<R, 8>, AG<8>::Threads, analysis_smem_bytes<8>(sizeof(R))); break;
-      }
+    const int h = a.N >> j, T = ana_side(sizeof(R) == 8, h);
+    if (only_level == 0 || j == only_level || (only_level < 0 && j > 1)) {
+      const cudaError_t e = launch_analysis_level<R, 1>(a, nullptr, grad_map, j, part_base, s);
       if (e != cudaSuccess) return e;
     }
-    part_base += tiles * a.M;
+    part_base += (h / T) * (h / T) * a.M;
   }
   return cudaSuccess;
 }
 
-template void launch_synthesis3<float>(const float* const*, float*, float*, WaveletGeom,
-                                       const FistaCtl*, cudaStream_t, int);
-template void launch_synthesis3<double>(const double* const*, double*, double*, WaveletGeom,
-                                        const FistaCtl*, cudaStream_t, int);
-template void launch_analysis<float>(const float*, float*, float*, WaveletGeom, cudaStream_t);
-template void launch_analysis<double>(const double*, double*, double*, WaveletGeom,
-                                      cudaStream_t);
-template cudaError_t launch_synthesis_pass<float>(const FistaPass<float>&, cudaStream_t, int);
-template cudaError_t launch_synthesis_pass<double>(const FistaPass<double>&, cudaStream_t, int);
-template cudaError_t launch_analysis_pass<float>(const FistaPass<float>&, const CUtensorMap*,
-                                                 cudaStream_t, int);
-template cudaError_t launch_analysis_pass<double>(const FistaPass<double>&, const CUtensorMap*,
-                                                  cudaStream_t, int);
+#define MS_INST(R)                                                                              \
+  template cudaError_t launch_synthesis<R>(const R*, R*, R*, WaveletGeom, cudaStream_t);        \
+  template cudaError_t launch_analysis<R>(const R*, R*, R*, WaveletGeom, cudaStream_t);         \
+  template cudaError_t launch_synthesis_pass<R>(const FistaPass<R>&, cudaStream_t, int);        \
+  template cudaError_t launch_analysis_pass<R>(const FistaPass<R>&, const CUtensorMap*,         \
+                                               cudaStream_t, int);
+MS_INST(float)
+MS_INST(double)
+#undef MS_INST
 
 }  // namespace ms

@@ -45,3 +45,31 @@ def test_transforms_on_odd_coarse_levels(ms, N, J, precision, tol):
     got = plan.dictionary_analysis(torch.from_numpy(x).to("cuda", dt)).double().cpu().numpy()
     assert rel(got, W.analysis(x)) <= tol
     plan.close()
+
+
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-9), ("fp32", 2e-5)])
+@pytest.mark.parametrize("N,J", [(176, 4), (480, 4), (96, 4)])
+def test_fista_on_odd_coarse_levels(ms, N, J, precision, tol):
+    """Three iterations of step one's problem (the prox fused into the level
+    kernels), started from given coefficients."""
+    import torch
+    from oracle.gridding import GriddedOperator, partition
+    from oracle.solver import Problem, fista, psf_spectrum
+    w = synth.tiny(npix=32)
+    dl = w.pixel_size * 32 / N
+    ell, delta = 0.1 * N, 3.0
+    plan = ms.Plan(w.u[0], w.v[0], N, dl, ell, delta, precision=precision, levels=J)
+    dt = torch.float64 if precision == "fp64" else torch.float32
+    rng = np.random.default_rng(N)
+    res, start = rng.standard_normal((N, N)), rng.standard_normal((8, N, N))
+    in_l, _ = partition(w.u[0], w.v[0], N, dl, ell, delta)
+    A = GriddedOperator(w.u[0][in_l], w.v[0][in_l], N, dl)
+    lam = 0.5
+    prob = Problem("low", Dictionary(N, 8, J), psf_spectrum(A.psf()), res, lam)
+    ref = fista(prob, 3, beta0=start)
+    beta = torch.from_numpy(start).to("cuda", dt)
+    model, st = plan.minor_cycle("low", torch.from_numpy(res).to("cuda", dt), lam, 3, beta=beta)
+    assert st.iterations == 3
+    assert rel(beta.double().cpu().numpy(), ref.beta) <= tol
+    assert rel(model.double().cpu().numpy(), prob.W.synth(ref.beta)) <= tol
+    plan.close()
