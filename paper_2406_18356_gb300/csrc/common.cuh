@@ -19,6 +19,20 @@ constexpr int kMaxBases = 8;   // db1 .. db8
 constexpr int kMaxTaps = 16;   // db8 has 16 taps
 constexpr int kMaxLevels = 8;
 
+// The gridding kernel: its shape and, for FP64 plans, the device tables of
+// its taps' weights (nullptr: evaluated directly): kEsSegs segments of the
+// inner taps (5 x 7 polynomial coefficients, the segment's centre, one pad),
+// then of the outer taps (9 coefficients, the centre, one pad).  Odd strides,
+// so that lanes in different segments read different banks.
+struct EsKernel {
+  double beta = 0;
+  const double* tab = nullptr;
+};
+constexpr int kEsSegs = 64, kEsInner = 37, kEsOuter = 11;
+constexpr int kEsTable = kEsSegs * (kEsInner + kEsOuter);
+constexpr double kEsOuterRange = 0.7;   // of v = sqrt(1 - z^2) at |z| >= 5/7
+constexpr double kEsMaxBeta = 32.0;     // the tables' accuracy holds up to here
+
 // One unit of (de)gridding work: `count` sorted rows starting at `start`
 // that all anchor in grid tile `tile`.
 struct WorkItem {
@@ -233,11 +247,11 @@ void launch_crop(const C2<R>* grid, const R* psi, int npix, int Ng, double scale
 template <typename R>
 void launch_degrid(const CUtensorMap* tmap, const C2<R>* grid, const WorkItem* items,
                    int nitems, const uint32_t* cell, const C2<R>* frac, const C2<R>* obs,
-                   C2<R>* out, int Ng, int tile, int ntx, double beta, int32_t* err,
+                   C2<R>* out, int Ng, int tile, int ntx, const EsKernel& es, int32_t* err,
                    cudaStream_t s);
 template <typename R, bool KAHAN>
 void launch_grid(const WorkItem* items, int nitems, const uint32_t* cell, const C2<R>* frac,
-                 const C2<R>* vis, void* scratch, int Ng, int tile, int ntx, double beta,
+                 const C2<R>* vis, void* scratch, int Ng, int tile, int ntx, const EsKernel& es,
                  cudaStream_t s);
 template <typename R, bool KAHAN>
 void launch_fold(const void* scratch, const int32_t* tile_items, int Ng, int tile, int ntx,
@@ -253,14 +267,14 @@ template <typename R>
 void launch_batch_scatter(const BatchJob<R>* jobs, int njobs, int64_t max_n, cudaStream_t s);
 template <typename R, bool KAHAN>
 void launch_grid_batch(const BatchJob<R>* jobs, const int32_t* job_of, int total_items,
-                       void* scratch, int tile, int ntx, double beta, cudaStream_t s);
+                       void* scratch, int tile, int ntx, const EsKernel& es, cudaStream_t s);
 template <typename R, bool KAHAN>
 void launch_fold_batch(const BatchJob<R>* jobs, int njobs, const void* scratch, int Ng,
                        int tile, int ntx, cudaStream_t s);
 template <typename R>
 void launch_degrid_batch(const CUtensorMap* tmap, const BatchJob<R>* jobs,
                          const int32_t* job_of, int total_items, bool has_obs, int Ng, int tile,
-                         int ntx, double beta, int32_t* err, cudaStream_t s);
+                         int ntx, const EsKernel& es, int32_t* err, cudaStream_t s);
 template <typename R>
 void launch_pad_batch(const BatchJob<R>* jobs, int njobs, const R* psi, int npix, int Ng,
                       cudaStream_t s);

@@ -121,6 +121,85 @@ __device__ __forceinline__ void es_weights<float>(float f, float beta, float* w)
     w[i] = exp2_approx(nb * z2 * rcp_approx(1.0f + sqrt_approx(s)));
   }
 }
+
+// FP64 weights from the plan's tables (EsKernel): the inner five taps are
+// degree-6 polynomials of f on 64 segments of its range, the outer two
+// exp(beta (v - 1)), a degree-8 polynomial on 64 segments of v = sqrt(1 - z^2)
+// in [0, 0.7) (smooth there; in f they have a square-root end point).  Their
+// errors are below 1e-16 of the kernel's peak.  A scheduler issues one FP64
+// instruction per 76 cycles, and the library's exp, sqrt and division spend
+// most of the operator's on the 14 weights of a row: some 170 of them this
+// way.  Measured at 128 px, 31,744 rows (with the smaller work items): the
+// residual image 374 -> 203 us, degridding 20.9 and gridding 30.9 us of it;
+// 5.9M rows 16.1 -> 9.0 ms.
+__device__ __forceinline__ void es_weights_tab(double f, const double* tab, double* w) {
+  const int seg = min(max((int)(((float)f + 0.5f) * kEsSegs), 0), kEsSegs - 1);
+  const double* c = tab + seg * kEsInner;
+  const double x = f - c[kEsInner - 2];
+#pragma unroll
+  for (int i = 1; i < kW - 1; ++i) {
+    const double* q = c + (i - 1) * 7;
+    double a = q[6];
+#pragma unroll
+    for (int k = 5; k >= 0; --k) a = fma(a, x, q[k]);
+    w[i] = a;
+  }
+#pragma unroll
+  for (int i = 0; i < kW; i += kW - 1) {
+    const double t = f + (double)(kHalfW - i);
+    double s = fma(t * (-4.0 / (kW * kW)), t, 1.0);
+    s = s > 0.0 ? s : 0.0;
+    const double v = sqrt(s);
+    const double* q = tab + kEsSegs * kEsInner +
+                      min((int)((float)v * (float)(kEsSegs / kEsOuterRange)), kEsSegs - 1) * kEsOuter;
+    const double y = v - q[kEsOuter - 2];
+    double a = q[8];
+#pragma unroll
+    for (int k = 7; k >= 0; --k) a = fma(a, y, q[k]);
+    w[i] = a;
+  }
+}
+
+// the weights of one axis: FP64 from the tables where the plan has them
+// (staged in shared memory), else directly
+template <typename R> struct EsWeights {
+  R beta;
+  const double* tab;
+  __device__ __forceinline__ void operator()(R f, R* w) const {
+    if constexpr (sizeof(R) == 8) {
+      if (tab) {   // uniform over the grid
+        es_weights_tab(f, tab, w);
+        return;
+      }
+    }
+    es_weights<R>(f, beta, w);
+  }
+};
+// stages the tables at dst (16-byte aligned; the caller joins the block
+// before using them)
+template <typename R>
+__device__ __forceinline__ EsWeights<R> stage_es(R beta, const double* tab, void* dst) {
+  if constexpr (sizeof(R) == 8) {
+    if (tab) {
+      double2* d = static_cast<double2*>(dst);
+      const double2* g = reinterpret_cast<const double2*>(tab);
+      for (int k = threadIdx.x; k < kEsTable / 2; k += blockDim.x) d[k] = g[k];
+      return EsWeights<R>{beta, static_cast<const double*>(dst)};
+    }
+  }
+  return EsWeights<R>{beta, nullptr};
+}
+template <typename R> size_t es_smem(const EsKernel& es) {
+  return sizeof(R) == 8 && es.tab ? kEsTable * sizeof(double) + 16 : 0;
+}
+__device__ __forceinline__ unsigned char* align16(void* p) {
+  return static_cast<unsigned char*>(p) + ((16u - (smem_addr(p) & 15u)) & 15u);
+}
+// threads of a degridding block: an FP64 work item has few rows (see
+// ms_plan_create)
+template <typename R> __host__ __device__ constexpr int degrid_threads() {
+  return sizeof(R) == 8 ? 128 : kThreads;
+}
 }  // namespace
 
 // ------------------------------------------------------------------ pad / crop
@@ -193,7 +272,8 @@ __device__ __forceinline__ void degrid_item(const CUtensorMap* tmap, int tma_y0,
                                             const C2<R>* __restrict__ frac,
                                             const C2<R>* __restrict__ obs,
                                             C2<R>* __restrict__ out, int Ng, int T, int ntx,
-                                            R beta, int32_t* __restrict__ err) {
+                                            R beta, const double* __restrict__ es_tab,
+                                            int32_t* __restrict__ err) {
   // the tile sits at a 128-byte-aligned shared address (TMA destination rule),
   // the mbarrier and a flag after it, all in the dynamic allocation
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -202,6 +282,7 @@ __device__ __forceinline__ void degrid_item(const CUtensorMap* tmap, int tma_y0,
   const int S = T + kW - 1;
   uint64_t& bar = *reinterpret_cast<uint64_t*>(tile + S * S);
   int& use_tma = *reinterpret_cast<int*>(&bar + 1);
+  const EsWeights<R> es = stage_es<R>(beta, es_tab, align16(&bar + 2));
   const int tx = it.tile % ntx, ty = it.tile / ntx;
   const int ox = tx * T, oy = ty * T;
   bool edge = (ox + S > Ng) || (oy + S > Ng);
@@ -228,6 +309,7 @@ __device__ __forceinline__ void degrid_item(const CUtensorMap* tmap, int tma_y0,
       mbar_expect_tx(&bar, (unsigned)(S * S * sizeof(C2<R>)));
       tma_load_2d(tile, tmap, 2 * ox, tma_y0 + oy, &bar);
     }
+    if (sizeof(R) == 8) __syncthreads();   // the tables
     ok = mbar_wait_bounded(&bar, 0);
     if (!ok) {
       if (threadIdx.x == 0) atomicExch(err, 5);
@@ -251,8 +333,8 @@ __device__ __forceinline__ void degrid_item(const CUtensorMap* tmap, int tma_y0,
     int lv = (int)(pc >> 16) - oy;
     C2<R> f = frac[k];
     R wu[kW], wv[kW];
-    es_weights<R>(f.x, beta, wu);
-    es_weights<R>(f.y, beta, wv);
+    es(f.x, wu);
+    es(f.y, wv);
     R accr = 0, acci = 0;
     if constexpr (sizeof(R) == 4 && MS_DEGRID_PACKED) {
       // the real and imaginary chains as packed FP32 pairs (same operations)
@@ -297,49 +379,50 @@ __device__ __forceinline__ void degrid_item(const CUtensorMap* tmap, int tma_y0,
 
 
 template <typename R, bool HAS_OBS>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(degrid_threads<R>())
     degrid_kernel(const __grid_constant__ CUtensorMap tmap, const C2<R>* __restrict__ grid,
                   const WorkItem* __restrict__ items, const uint32_t* __restrict__ cell,
                   const C2<R>* __restrict__ frac, const C2<R>* __restrict__ obs,
                   C2<R>* __restrict__ out, int Ng, int T, int ntx, R beta,
-                  int32_t* __restrict__ err) {
+                  const double* __restrict__ es_tab, int32_t* __restrict__ err) {
   degrid_item<R, HAS_OBS>(&tmap, 0, grid, items[blockIdx.x], cell, frac, obs, out, Ng, T, ntx,
-                          beta, err);
+                          beta, es_tab, err);
 }
 
 // Stacked form: one block per work item of all jobs; job_of[item] names the
 // job, whose grid is row block job * Ng of the stacked TMA descriptor.
 template <typename R, bool HAS_OBS>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(degrid_threads<R>())
     degrid_batch_kernel(const __grid_constant__ CUtensorMap tmap,
                         const BatchJob<R>* __restrict__ jobs, const int32_t* __restrict__ job_of,
-                        int Ng, int T, int ntx, R beta, int32_t* __restrict__ err) {
+                        int Ng, int T, int ntx, R beta, const double* __restrict__ es_tab,
+                        int32_t* __restrict__ err) {
   const int j = job_of[blockIdx.x];
   const BatchJob<R> jb = jobs[j];
   const WorkItem it = jb.items[blockIdx.x - jb.item_base];
   degrid_item<R, HAS_OBS>(&tmap, j * Ng, jb.grid, it, jb.cell, jb.frac, jb.sorted_in,
-                          jb.sorted_out, Ng, T, ntx, beta, err);
+                          jb.sorted_out, Ng, T, ntx, beta, es_tab, err);
 }
 
 template <typename R>
 void launch_degrid(const CUtensorMap* tmap, const C2<R>* grid, const WorkItem* items,
                    int nitems, const uint32_t* cell, const C2<R>* frac, const C2<R>* obs,
-                   C2<R>* out, int Ng, int tile, int ntx, double beta, int32_t* err,
+                   C2<R>* out, int Ng, int tile, int ntx, const EsKernel& es, int32_t* err,
                    cudaStream_t s) {
   if (nitems <= 0) return;
   const int S = tile + kW - 1;
-  // tile + alignment slack + mbarrier + flag
-  size_t smem = (size_t)S * S * sizeof(C2<R>) + 128 + sizeof(uint64_t) + sizeof(int) + 4;
+  // tile + alignment slack + mbarrier + flag + tables
+  const size_t smem = (size_t)S * S * sizeof(C2<R>) + 128 + 16 + es_smem<R>(es);
   if (obs) {
     auto k = degrid_kernel<R, true>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<nitems, kThreads, smem, s>>>(*tmap, grid, items, cell, frac, obs, out, Ng, tile, ntx,
-                                     (R)beta, err);
+    k<<<nitems, degrid_threads<R>(), smem, s>>>(*tmap, grid, items, cell, frac, obs, out, Ng, tile,
+                                                ntx, (R)es.beta, es.tab, err);
   } else {
     auto k = degrid_kernel<R, false>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<nitems, kThreads, smem, s>>>(*tmap, grid, items, cell, frac, obs, out, Ng, tile, ntx,
-                                     (R)beta, err);
+    k<<<nitems, degrid_threads<R>(), smem, s>>>(*tmap, grid, items, cell, frac, obs, out, Ng, tile,
+                                                ntx, (R)es.beta, es.tab, err);
   }
 }
 
@@ -353,6 +436,11 @@ size_t grid_scratch_cell_bytes(int precision) { return precision == 1 ? 8 : 16; 
 
 template <typename R, bool KAHAN> __host__ __device__ constexpr int grid_warps() {
   return (KAHAN || sizeof(R) == 8) ? 4 : 8;
+}
+
+// values staged per row: w_u, w_v and the visibility, or w_u and w_v v
+template <bool KAHAN> __host__ __device__ constexpr int grid_stage_values() {
+  return KAHAN ? 2 * kW + 2 : 3 * kW;
 }
 
 // Adds v (and, compensated, its correction) to a tile cell.
@@ -379,18 +467,17 @@ __device__ __forceinline__ void cell_add(C2<R>* my, C2<R>* myc, int c, C2<R> v) 
 // Kahan form).
 template <typename R, bool KAHAN> struct TapSum {
   R sr = 0, si = 0, cr = 0, ci = 0;
-  __device__ __forceinline__ void add(R w, C2<R> v) {
-    if (KAHAN) {
-      const R yr = w * v.x - cr, yi = w * v.y - ci;
-      const R tr = sr + yr, ti = si + yi;
-      cr = (tr - sr) - yr;
-      ci = (ti - si) - yi;
-      sr = tr;
-      si = ti;
-    } else {
-      sr = fma(w, v.x, sr);
-      si = fma(w, v.y, si);
-    }
+  __device__ __forceinline__ void add(R w, C2<R> v) {   // compensated
+    const R yr = w * v.x - cr, yi = w * v.y - ci;
+    const R tr = sr + yr, ti = si + yi;
+    cr = (tr - sr) - yr;
+    ci = (ti - si) - yi;
+    sr = tr;
+    si = ti;
+  }
+  __device__ __forceinline__ void add(R w, R pr, R pi) {   // plain, w_v v given
+    sr = fma(w, pr, sr);
+    si = fma(w, pi, si);
   }
   __device__ __forceinline__ C2<R> value() const {
     C2<R> o;
@@ -409,7 +496,9 @@ template <typename R, bool KAHAN> struct TapSum {
 // when the anchor changes, the lanes add their sums to the 49 distinct cells
 // of the footprint in the warp's own sub-tile (no atomics) and __syncwarp
 // orders that update before the next.  The rows' ES weights, values and
-// anchors are staged 32 at a time in shared memory.  The compensated form
+// anchors are staged 32 at a time in shared memory; the plain form stages the
+// seven products w_v[j] v with them, so a tap is two multiply-adds (of 6 FP64
+// instructions a row in the lanes' two taps, 4 remain).  The compensated form
 // sums each run with Kahan compensation and adds it into compensated cells.
 // At the end the warps' sub-tiles are summed in a fixed order into the
 // item's scratch tile.
@@ -419,17 +508,19 @@ __device__ __forceinline__ void grid_item(const WorkItem it, const uint32_t* __r
                                           const C2<R>* __restrict__ frac,
                                           const C2<R>* __restrict__ vis,
                                           typename ScratchOf<R, KAHAN>::T* __restrict__ scratch,
-                                          int64_t scratch_tile, int T, int ntx, R beta) {
+                                          int64_t scratch_tile, int T, int ntx, R beta,
+                                          const double* __restrict__ es_tab) {
   using Acc = typename ScratchOf<R, KAHAN>::T;
   constexpr int NW = grid_warps<R, KAHAN>();
+  constexpr int SW = grid_stage_values<KAHAN>();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int S = T + kW - 1;
   const int cells = S * S;
   C2<R>* tiles = reinterpret_cast<C2<R>*>(smem_raw);                  // [NW][cells]
   C2<R>* comps = tiles + (KAHAN ? NW * cells : 0);                     // [NW][cells]
-  R* stage_w = reinterpret_cast<R*>(tiles + (KAHAN ? 2 : 1) * NW * cells);  // [NW][32][14]
-  C2<R>* stage_v = reinterpret_cast<C2<R>*>(stage_w + NW * 32 * 2 * kW);     // [NW][32]
-  int* stage_c = reinterpret_cast<int*>(stage_v + NW * 32);                  // [NW][32]
+  R* stage_w = reinterpret_cast<R*>(tiles + (KAHAN ? 2 : 1) * NW * cells);  // [NW][32][SW]
+  int* stage_c = reinterpret_cast<int*>(stage_w + NW * 32 * SW);             // [NW][32]
+  const EsWeights<R> es = stage_es<R>(beta, es_tab, align16(stage_c + NW * 32));
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ox = (it.tile % ntx) * T, oy = (it.tile / ntx) * T;
@@ -445,8 +536,7 @@ __device__ __forceinline__ void grid_item(const WorkItem it, const uint32_t* __r
 
   C2<R>* my = tiles + warp * cells;
   C2<R>* myc = comps + warp * cells;
-  R* sw = stage_w + warp * 32 * 2 * kW;
-  C2<R>* sv = stage_v + warp * 32;
+  R* sw = stage_w + warp * 32 * SW;
   int* sc = stage_c + warp * 32;
   const int i1 = lane % kW, j1 = lane / kW;
   const int i2 = (lane + 32) % kW, j2 = (lane + 32) / kW;
@@ -466,9 +556,22 @@ __device__ __forceinline__ void grid_item(const WorkItem it, const uint32_t* __r
       int lu = (int)(pc & 0xffffu) - ox;
       int lv = (int)(pc >> 16) - oy;
       C2<R> f = frac[k];
-      es_weights<R>(f.x, beta, sw + lane * 2 * kW);
-      es_weights<R>(f.y, beta, sw + lane * 2 * kW + kW);
-      sv[lane] = vis[k];
+      // w_u, then w_v and v (compensated) or w_v Re v and w_v Im v
+      R wu[kW], wv[kW];
+      es(f.x, wu);
+      es(f.y, wv);
+      const C2<R> v = vis[k];
+      R* d = sw + lane * SW;
+#pragma unroll
+      for (int i = 0; i < kW; ++i) {
+        d[i] = wu[i];
+        d[kW + i] = KAHAN ? wv[i] : wv[i] * v.x;
+        if (!KAHAN) d[2 * kW + i] = wv[i] * v.y;
+      }
+      if (KAHAN) {
+        d[2 * kW] = v.x;
+        d[2 * kW + 1] = v.y;
+      }
       sc[lane] = lv * S + lu;
     }
     __syncwarp();
@@ -485,10 +588,17 @@ __device__ __forceinline__ void grid_item(const WorkItem it, const uint32_t* __r
         t1.clear();
         t2.clear();
       }
-      const R* w = sw + sidx * 2 * kW;
-      const C2<R> val = sv[sidx];
-      t1.add(w[i1] * w[kW + j1], val);
-      if (two) t2.add(w[i2] * w[kW + j2], val);
+      const R* w = sw + sidx * SW;
+      if constexpr (KAHAN) {
+        C2<R> val;
+        val.x = w[2 * kW];
+        val.y = w[2 * kW + 1];
+        t1.add(w[i1] * w[kW + j1], val);
+        if (two) t2.add(w[i2] * w[kW + j2], val);
+      } else {
+        t1.add(w[i1], w[kW + j1], w[2 * kW + j1]);
+        if (two) t2.add(w[i2], w[kW + j2], w[2 * kW + j2]);
+      }
     }
     __syncwarp();   // the staging buffers are rewritten
   }
@@ -710,25 +820,27 @@ template <typename R, bool KAHAN> __host__ __device__ constexpr int grid_block_t
 template <typename R, bool KAHAN> __host__ __device__ constexpr int grid_min_blocks() {
   return grid_lane_rows<R, KAHAN>() ? MS_GRID_LANE_MINB : 1;
 }
-template <typename R, bool KAHAN> size_t grid_smem_bytes(int tile) {
+template <typename R, bool KAHAN> size_t grid_smem_bytes(int tile, const EsKernel& es) {
   const int S = tile + kW - 1;
   if (grid_lane_rows<R, KAHAN>()) return grid_lanes_smem(S);
   constexpr int NW = grid_warps<R, KAHAN>();
   return (size_t)NW * S * S * sizeof(C2<R>) * (KAHAN ? 2 : 1) +
-         (size_t)NW * 32 * (2 * kW * sizeof(R) + sizeof(C2<R>) + sizeof(int));
+         (size_t)NW * 32 * (grid_stage_values<KAHAN>() * sizeof(R) + sizeof(int)) +
+         es_smem<R>(es);
 }
 
 template <typename R, bool KAHAN>
 __device__ __forceinline__ void grid_any_item(const WorkItem it, const uint32_t* cell,
                                               const C2<R>* frac, const C2<R>* vis,
                                               typename ScratchOf<R, KAHAN>::T* scratch,
-                                              int64_t scratch_tile, int T, int ntx, R beta) {
+                                              int64_t scratch_tile, int T, int ntx, R beta,
+                                              const double* es_tab) {
   if constexpr (grid_lane_rows<R, KAHAN>())
     grid_item_lanes(it, cell, reinterpret_cast<const float2*>(frac),
                     reinterpret_cast<const float2*>(vis), reinterpret_cast<float2*>(scratch),
                     scratch_tile, T, ntx, (float)beta);
   else
-    grid_item<R, KAHAN>(it, cell, frac, vis, scratch, scratch_tile, T, ntx, beta);
+    grid_item<R, KAHAN>(it, cell, frac, vis, scratch, scratch_tile, T, ntx, beta, es_tab);
 }
 
 template <typename R, bool KAHAN>
@@ -736,8 +848,9 @@ __global__ void __launch_bounds__(grid_block_threads<R, KAHAN>(), grid_min_block
     grid_kernel(const WorkItem* __restrict__ items, const uint32_t* __restrict__ cell,
                 const C2<R>* __restrict__ frac, const C2<R>* __restrict__ vis,
                 typename ScratchOf<R, KAHAN>::T* __restrict__ scratch, int Ng, int T, int ntx,
-                R beta) {
-  grid_any_item<R, KAHAN>(items[blockIdx.x], cell, frac, vis, scratch, blockIdx.x, T, ntx, beta);
+                R beta, const double* __restrict__ es_tab) {
+  grid_any_item<R, KAHAN>(items[blockIdx.x], cell, frac, vis, scratch, blockIdx.x, T, ntx, beta,
+                          es_tab);
 }
 
 // Stacked form: one block per work item of all jobs (scratch tile = the
@@ -746,23 +859,23 @@ template <typename R, bool KAHAN>
 __global__ void __launch_bounds__(grid_block_threads<R, KAHAN>(), grid_min_blocks<R, KAHAN>())
     grid_batch_kernel(const BatchJob<R>* __restrict__ jobs, const int32_t* __restrict__ job_of,
                       typename ScratchOf<R, KAHAN>::T* __restrict__ scratch, int T, int ntx,
-                      R beta) {
+                      R beta, const double* __restrict__ es_tab) {
   const BatchJob<R> jb = jobs[job_of[blockIdx.x]];
   grid_any_item<R, KAHAN>(jb.items[blockIdx.x - jb.item_base], jb.cell, jb.frac, jb.sorted_in,
-                      scratch, blockIdx.x, T, ntx, beta);
+                          scratch, blockIdx.x, T, ntx, beta, es_tab);
 }
 
 template <typename R, bool KAHAN>
 void launch_grid(const WorkItem* items, int nitems, const uint32_t* cell, const C2<R>* frac,
-                 const C2<R>* vis, void* scratch, int Ng, int tile, int ntx, double beta,
+                 const C2<R>* vis, void* scratch, int Ng, int tile, int ntx, const EsKernel& es,
                  cudaStream_t s) {
   if (nitems <= 0) return;
-  const size_t smem = grid_smem_bytes<R, KAHAN>(tile);
+  const size_t smem = grid_smem_bytes<R, KAHAN>(tile, es);
   auto k = grid_kernel<R, KAHAN>;
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   k<<<nitems, grid_block_threads<R, KAHAN>(), smem, s>>>(items, cell, frac, vis,
                                  reinterpret_cast<typename ScratchOf<R, KAHAN>::T*>(scratch),
-                                 Ng, tile, ntx, (R)beta);
+                                 Ng, tile, ntx, (R)es.beta, es.tab);
 }
 
 // Cells are walked x-stride over the whole grid (dense tiles, with many
@@ -946,14 +1059,14 @@ void launch_batch_scatter(const BatchJob<R>* jobs, int njobs, int64_t max_n, cud
 
 template <typename R, bool KAHAN>
 void launch_grid_batch(const BatchJob<R>* jobs, const int32_t* job_of, int total_items,
-                       void* scratch, int tile, int ntx, double beta, cudaStream_t s) {
+                       void* scratch, int tile, int ntx, const EsKernel& es, cudaStream_t s) {
   if (total_items <= 0) return;
-  const size_t smem = grid_smem_bytes<R, KAHAN>(tile);
+  const size_t smem = grid_smem_bytes<R, KAHAN>(tile, es);
   auto k = grid_batch_kernel<R, KAHAN>;
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   k<<<total_items, grid_block_threads<R, KAHAN>(), smem, s>>>(
       jobs, job_of, reinterpret_cast<typename ScratchOf<R, KAHAN>::T*>(scratch), tile, ntx,
-      (R)beta);
+      (R)es.beta, es.tab);
 }
 
 template <typename R, bool KAHAN>
@@ -967,18 +1080,20 @@ void launch_fold_batch(const BatchJob<R>* jobs, int njobs, const void* scratch, 
 template <typename R>
 void launch_degrid_batch(const CUtensorMap* tmap, const BatchJob<R>* jobs,
                          const int32_t* job_of, int total_items, bool has_obs, int Ng, int tile,
-                         int ntx, double beta, int32_t* err, cudaStream_t s) {
+                         int ntx, const EsKernel& es, int32_t* err, cudaStream_t s) {
   if (total_items <= 0) return;
   const int S = tile + kW - 1;
-  size_t smem = (size_t)S * S * sizeof(C2<R>) + 128 + sizeof(uint64_t) + sizeof(int) + 4;
+  const size_t smem = (size_t)S * S * sizeof(C2<R>) + 128 + 16 + es_smem<R>(es);
   if (has_obs) {
     auto k = degrid_batch_kernel<R, true>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<total_items, kThreads, smem, s>>>(*tmap, jobs, job_of, Ng, tile, ntx, (R)beta, err);
+    k<<<total_items, degrid_threads<R>(), smem, s>>>(*tmap, jobs, job_of, Ng, tile, ntx,
+                                                     (R)es.beta, es.tab, err);
   } else {
     auto k = degrid_batch_kernel<R, false>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<total_items, kThreads, smem, s>>>(*tmap, jobs, job_of, Ng, tile, ntx, (R)beta, err);
+    k<<<total_items, degrid_threads<R>(), smem, s>>>(*tmap, jobs, job_of, Ng, tile, ntx,
+                                                     (R)es.beta, es.tab, err);
   }
 }
 
@@ -1001,7 +1116,7 @@ void launch_crop_batch(const BatchJob<R>* jobs, int njobs, const R* psi, int npi
   template void launch_batch_gather<R>(const BatchJob<R>*, int, int64_t, cudaStream_t);         \
   template void launch_batch_scatter<R>(const BatchJob<R>*, int, int64_t, cudaStream_t);        \
   template void launch_degrid_batch<R>(const CUtensorMap*, const BatchJob<R>*, const int32_t*,  \
-                                       int, bool, int, int, int, double, int32_t*,             \
+                                       int, bool, int, int, int, const EsKernel&, int32_t*,             \
                                        cudaStream_t);                                           \
   template void launch_pad_batch<R>(const BatchJob<R>*, int, const R*, int, int, cudaStream_t); \
   template void launch_crop_batch<R>(const BatchJob<R>*, int, const R*, int, int, cudaStream_t);
@@ -1009,11 +1124,11 @@ MS_BATCH_INST(float)
 MS_BATCH_INST(double)
 #undef MS_BATCH_INST
 template void launch_grid_batch<float, false>(const BatchJob<float>*, const int32_t*, int, void*,
-                                              int, int, double, cudaStream_t);
+                                              int, int, const EsKernel&, cudaStream_t);
 template void launch_grid_batch<float, true>(const BatchJob<float>*, const int32_t*, int, void*,
-                                             int, int, double, cudaStream_t);
+                                             int, int, const EsKernel&, cudaStream_t);
 template void launch_grid_batch<double, false>(const BatchJob<double>*, const int32_t*, int,
-                                               void*, int, int, double, cudaStream_t);
+                                               void*, int, int, const EsKernel&, cudaStream_t);
 template void launch_fold_batch<float, false>(const BatchJob<float>*, int, const void*, int, int,
                                               int, cudaStream_t);
 template void launch_fold_batch<float, true>(const BatchJob<float>*, int, const void*, int, int,
@@ -1030,18 +1145,18 @@ template void launch_crop<double>(const double2*, const double*, int, int, doubl
                                   cudaStream_t);
 template void launch_degrid<float>(const CUtensorMap*, const float2*, const WorkItem*, int,
                                    const uint32_t*, const float2*, const float2*, float2*, int,
-                                   int, int, double, int32_t*, cudaStream_t);
+                                   int, int, const EsKernel&, int32_t*, cudaStream_t);
 template void launch_degrid<double>(const CUtensorMap*, const double2*, const WorkItem*, int,
                                     const uint32_t*, const double2*, const double2*, double2*,
-                                    int, int, int, double, int32_t*, cudaStream_t);
+                                    int, int, int, const EsKernel&, int32_t*, cudaStream_t);
 template void launch_grid<float, false>(const WorkItem*, int, const uint32_t*, const float2*,
-                                        const float2*, void*, int, int, int, double,
+                                        const float2*, void*, int, int, int, const EsKernel&,
                                         cudaStream_t);
 template void launch_grid<float, true>(const WorkItem*, int, const uint32_t*, const float2*,
-                                       const float2*, void*, int, int, int, double,
+                                       const float2*, void*, int, int, int, const EsKernel&,
                                        cudaStream_t);
 template void launch_grid<double, false>(const WorkItem*, int, const uint32_t*, const double2*,
-                                         const double2*, void*, int, int, int, double,
+                                         const double2*, void*, int, int, int, const EsKernel&,
                                          cudaStream_t);
 template void launch_fold<float, false>(const void*, const int32_t*, int, int, int, float2*,
                                         cudaStream_t);

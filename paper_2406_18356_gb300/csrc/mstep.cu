@@ -150,6 +150,75 @@ void gauss_legendre(int n, std::vector<double>& x, std::vector<double>& w) {
   }
 }
 
+// Matrix [n][n] from the values of a function at the n Chebyshev nodes x_i =
+// cos(pi (2i + 1) / 2n) of [-1, 1] to the monomial coefficients of its
+// interpolating polynomial (Newton's divided differences of unit vectors).
+std::vector<double> chebyshev_fit(int n, std::vector<double>* nodes) {
+  const long double pi = 3.141592653589793238462643383279502884L;
+  std::vector<long double> x(n);
+  for (int i = 0; i < n; ++i) x[i] = std::cos(pi * (2 * i + 1) / (2.0L * n));
+  if (n % 2) x[n / 2] = 0.0L;
+  nodes->assign(x.begin(), x.end());
+  std::vector<double> m(n * n);
+  for (int u = 0; u < n; ++u) {
+    std::vector<long double> d(n, 0.0L), p(n, 0.0L);
+    d[u] = 1.0L;
+    for (int k = 1; k < n; ++k)
+      for (int i = n - 1; i >= k; --i) d[i] = (d[i] - d[i - 1]) / (x[i] - x[i - k]);
+    for (int i = n - 1; i >= 0; --i) {   // p <- p (x - x_i) + d_i
+      for (int k = n - 1; k >= 1; --k) p[k] = p[k - 1] - x[i] * p[k];
+      p[0] = d[i] - x[i] * p[0];
+    }
+    for (int k = 0; k < n; ++k) m[k * n + u] = (double)p[k];
+  }
+  return m;
+}
+
+// The FP64 weight tables (see EsKernel) of the ES kernel with shape beta.  A
+// segment's polynomial interpolates the differences from its centre value
+// (relative to it, through expm1, so that they keep their digits); the inner
+// taps i and 6 - i mirror each other, and the outer function's segments are
+// one polynomial of exp(beta x) times their centre values.
+std::vector<double> es_tables(double beta) {
+  std::vector<double> t(kEsTable, 0.0), x7, x9;
+  const std::vector<double> f7 = chebyshev_fit(7, &x7), f9 = chebyshev_fit(9, &x9);
+  const double c2 = 4.0 / (kW * kW), h = 0.5 / kEsSegs, ho = 0.5 * kEsOuterRange / kEsSegs;
+  // out[k] = a c_k / h^k, c the fit of d (d = 0 at the centre), out[0] = a
+  auto put = [](const std::vector<double>& fit, int n, const double* d, double a, double h,
+                double* out) {
+    double hk = 1.0;
+    out[0] = a;
+    for (int k = 1; k < n; ++k) {
+      double s = 0.0;
+      hk *= h;
+      for (int i = 0; i < n; ++i) s += fit[k * n + i] * d[i];
+      out[k] = a * s / hk;
+    }
+  };
+  double d9[9];
+  for (int i = 0; i < 9; ++i) d9[i] = std::expm1(beta * ho * x9[i]);
+  for (int g = 0; g < kEsSegs; ++g) {
+    const double c = -0.5 + (2 * g + 1) * h;
+    double* q = &t[g * kEsInner];
+    q[kEsInner - 2] = c;
+    for (int i = 1; i <= kHalfW; ++i) {
+      const double tc = c + (kHalfW - i), z2 = tc * tc * c2, sc = std::sqrt(1.0 - z2);
+      double d[7];
+      for (int n = 0; n < 7; ++n) {
+        const double x = h * x7[n], ds = -c2 * x * (2.0 * tc + x);   // s(tc + x) - s(tc)
+        d[n] = std::expm1(beta * ds / (std::sqrt(1.0 - z2 + ds) + sc));
+      }
+      put(f7, 7, d, std::exp(-beta * z2 / (1.0 + sc)), h, q + (i - 1) * 7);
+      double* mirror = &t[(kEsSegs - 1 - g) * kEsInner] + (kW - 2 - i) * 7;
+      for (int k = 0; k < 7 && i < kHalfW; ++k) mirror[k] = (k & 1 ? -1 : 1) * q[(i - 1) * 7 + k];
+    }
+    double* o = &t[kEsSegs * kEsInner + g * kEsOuter];
+    o[kEsOuter - 2] = (2 * g + 1) * ho;
+    put(f9, 9, d9, std::exp(beta * (o[kEsOuter - 2] - 1.0)), ho, o);
+  }
+  return t;
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
                                   const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
                                   const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -278,6 +347,7 @@ struct ms_plan {
   int chunk = 0;
   size_t rsz = 8;
   double beta = 0;
+  EsKernel es;      // beta and, for FP64, the weight tables
   std::vector<ChanDev> ch;
   std::vector<void*> allocs;
   cudaStream_t ps = nullptr;
@@ -565,7 +635,7 @@ void degrid_sorted(ms_plan* p, PartDev& pd, const void* obs_sorted, void* out_so
     KSpan k(p, MS_K_DEGRID);
     launch_degrid<R>(&p->tmap, (const C2<R>*)p->grid, pd.items, pd.nitems, pd.cell,
                      (const C2<R>*)pd.frac, (const C2<R>*)obs_sorted, (C2<R>*)out_sorted, p->Ng,
-                     p->T, p->ntx, p->beta, p->err, p->ps);
+                     p->T, p->ntx, p->es, p->err, p->ps);
   }
   if (tm) tm->spans[0].push_back({a, tm->mark()});
 }
@@ -582,7 +652,7 @@ void grid_sorted(ms_plan* p, PartDev& pd, const void* vis_sorted, void* image, T
       KSpan k(p, MS_K_GRID);
       launch_grid<float, true>(pd.items, pd.nitems, pd.cell, (const float2*)pd.frac,
                                (const float2*)vis_sorted, scratch, p->Ng, p->T, p->ntx,
-                               p->beta, p->ps);
+                               p->es, p->ps);
     }
     KSpan k(p, MS_K_FOLD);
     launch_fold<float, true>(scratch, pd.tile_items, p->Ng, p->T, p->ntx, (float2*)p->grid,
@@ -591,7 +661,7 @@ void grid_sorted(ms_plan* p, PartDev& pd, const void* vis_sorted, void* image, T
     {
       KSpan k(p, MS_K_GRID);
       launch_grid<R, false>(pd.items, pd.nitems, pd.cell, (const C2<R>*)pd.frac,
-                            (const C2<R>*)vis_sorted, scratch, p->Ng, p->T, p->ntx, p->beta,
+                            (const C2<R>*)vis_sorted, scratch, p->Ng, p->T, p->ntx, p->es,
                             p->ps);
     }
     KSpan k(p, MS_K_FOLD);
@@ -1357,6 +1427,13 @@ template <typename R> void build_plan(ms_plan* p, const ms_plan_desc* d) {
     cudaFree(dw);
     cudaFree(psi);
   }
+  p->es.beta = p->beta;
+  if (sizeof(R) == 8 && p->beta <= kEsMaxBeta) {
+    const std::vector<double> t = es_tables(p->beta);
+    double* d_tab = p->alloc<double>(t.size(), "kernel tables");
+    ck(cudaMemcpy(d_tab, t.data(), sizeof(double) * t.size(), cudaMemcpyHostToDevice), "copy");
+    p->es.tab = d_tab;
+  }
   // per channel: classify, sort, work items
   double* du = dalloc<double>(nvis, "u");
   double* dv = dalloc<double>(nvis, "v");
@@ -1823,10 +1900,10 @@ void grid_batch(ms_plan* p, int njobs, const int32_t* chans, const int32_t* part
     KSpan k(p, MS_K_GRID);
     if (p->prec == MS_FP32_KAHAN)
       launch_grid_batch<float, true>((const BatchJob<float>*)jd, p->batch.job_of, (int)sh.items,
-                                     p->batch.scratch, p->T, p->ntx, p->beta, p->ps);
+                                     p->batch.scratch, p->T, p->ntx, p->es, p->ps);
     else
       launch_grid_batch<R, false>(jd, p->batch.job_of, (int)sh.items, p->batch.scratch, p->T,
-                                  p->ntx, p->beta, p->ps);
+                                  p->ntx, p->es, p->ps);
   }
   {
     KSpan k(p, MS_K_FOLD);
@@ -1872,7 +1949,7 @@ void degrid_batch(ms_plan* p, int njobs, const int32_t* chans, const int32_t* pa
   {
     KSpan k(p, MS_K_DEGRID);
     launch_degrid_batch<R>(&p->batch.tmap, jd, p->batch.job_of, (int)sh.items, vis_obs != nullptr,
-                           p->Ng, p->T, p->ntx, p->beta, p->err, p->ps);
+                           p->Ng, p->T, p->ntx, p->es, p->err, p->ps);
   }
   launch_batch_scatter<R>(jd, njobs, sh.max_n, p->ps);
 }
@@ -2148,7 +2225,7 @@ void residual_batch(ms_plan* p, int njobs, const int32_t* chans, const int32_t* 
   {
     KSpan k(p, MS_K_DEGRID);
     launch_degrid_batch<R>(&p->batch.tmap, jd, p->batch.job_of, (int)sh.items, true, p->Ng,
-                           p->T, p->ntx, p->beta, p->err, p->ps);
+                           p->T, p->ntx, p->es, p->err, p->ps);
   }
   // grid the residual rows obs - A x where the degridding left them
   for (auto& b : jobs) std::swap(b.sorted_in, b.sorted_out);
@@ -2159,10 +2236,10 @@ void residual_batch(ms_plan* p, int njobs, const int32_t* chans, const int32_t* 
     KSpan k(p, MS_K_GRID);
     if (p->prec == MS_FP32_KAHAN)
       launch_grid_batch<float, true>((const BatchJob<float>*)jd, p->batch.job_of, (int)sh.items,
-                                     p->batch.scratch, p->T, p->ntx, p->beta, p->ps);
+                                     p->batch.scratch, p->T, p->ntx, p->es, p->ps);
     else
       launch_grid_batch<R, false>(jd, p->batch.job_of, (int)sh.items, p->batch.scratch, p->T,
-                                  p->ntx, p->beta, p->ps);
+                                  p->ntx, p->es, p->ps);
   }
   {
     KSpan k(p, MS_K_FOLD);
@@ -2665,7 +2742,14 @@ ms_status ms_plan_create(const ms_plan_desc* d, ms_plan** out) {
     } else {
       const int64_t per = (int64_t)sm_count() * 8;   // about 8 work items per SM
       int64_t c = (d->nvis + per - 1) / per;
-      p->chunk = (int)std::min<int64_t>(std::max<int64_t>(c, 512), 8192);
+      // at least 512 rows (an FP32 lane then sums runs of a few rows), or in
+      // FP64 the 128 that give each of a block's warps one batch, so that
+      // small observations use every SM's FP64 pipe (31,744 rows: 62 -> 304
+      // work items)
+      // while any partition's tiles still fit the static scratch
+      const bool fits = ((int64_t)p->ntiles + per + 1) * p->S * p->S * 16 <= 64 << 20;
+      const int64_t least = p->prec == MS_FP64 && fits ? 128 : 512;
+      p->chunk = (int)std::min<int64_t>(std::max<int64_t>(c, least), 8192);
     }
     ck(cudaStreamCreateWithFlags(&p->ps, cudaStreamNonBlocking), "stream");
     ck(cudaEventCreateWithFlags(&p->ev_in, cudaEventDisableTiming), "event");

@@ -1,0 +1,344 @@
+// The 2-D transforms of the measurement operator (Sect. 2: F Z D and Z^H D^H
+// F^H) for image sides N a power of two, 16..4096, on the Ng = 2N grid.
+//
+// An image is real and fills a quarter of its padded grid, its grid is
+// Hermitian, and visibilities reach only cells within `ext` of the origin
+// (the plan's longest baseline).  So:
+//   forward   N real rows (deapodized, padded) -> columns 0..ext of the half
+//             plane; each column's transform of its N nonzero rows, written
+//             to rows -ext..ext and, conjugated, to the column's mirror;
+//   adjoint   Re(F^H g) needs the Hermitian part only: column u and the mirror
+//             of column -u are added as they are read, transformed, and the N
+//             image rows of the result kept; N real rows from the half plane,
+//             cropped, deapodized and scaled as they are written.
+// Each grid cell is written or read once, by lanes that cover 32-byte sectors;
+// padding, cropping, deapodization and the grid's centring (cell k at index k
+// + Ng / 2) cost no pass of their own.  A complex transform of the whole grid (2-D cuFFT between a padding
+// and a cropping pass) moves 4 to 9 times the bytes.  MEAS_FFT
+//
+// A sequence of 2^LOGN elements is held by 2^(LOGN - LE) threads, 2^LE
+// elements each, through Stockham stages of radix up to 2^LE: inputs of the
+// first stage come from global memory, outputs of the last one go there, and
+// the stages between exchange through one padded shared-memory buffer
+// (written and read on opposite sides of a barrier, so that four 4096-point
+// columns fit a block).  LE is 4 for long FP32 sequences (fewest exchanges);
+// FP64, bound by the FP64 instructions of its busiest warp at short lengths,
+// spreads them over more threads (see fft_lrad of the spectral kernels).
+#include <algorithm>
+
+#include "common.cuh"
+#include "fft_radix.cuh"
+
+namespace ms {
+namespace {
+
+// one sequence: v holds the inputs of the stage after sub-transforms of size
+// 2^DONE; store(index, value) receives the outputs of the last stage
+template <typename R, int LOGN, int LE, int DONE, bool INV, class Store>
+__device__ __forceinline__ void run_stages(C2<R> (&v)[1 << LE], C2<R>* buf,
+                                           const C2<R>* __restrict__ tw, int tw_step, int t,
+                                           const Store& store) {
+  constexpr int N = 1 << LOGN, TPS = N >> LE, EPT = 1 << LE;
+  constexpr int LR = LOGN - DONE >= LE ? LE : LOGN - DONE;
+  constexpr int Rd = 1 << LR, NS = 1 << DONE;
+#pragma unroll
+  for (int q = 0; q < EPT / Rd; ++q) {
+    const int j = t + q * TPS, js = j & (NS - 1);
+    C2<R> w[Rd];
+#pragma unroll
+    for (int r = 0; r < Rd; ++r) w[r] = v[q * Rd + r];
+    if (NS > 1) {
+      const int unit = js * (N / (NS * Rd)) * tw_step;
+#pragma unroll
+      for (int r = 1; r < Rd; ++r) {
+        C2<R> z = tw[r * unit];
+        if (INV) z.y = -z.y;
+        const C2<R> x = w[r];
+        w[r].x = x.x * z.x - x.y * z.y;
+        w[r].y = x.x * z.y + x.y * z.x;
+      }
+    }
+    dft_reg<R, Rd, INV>(w);
+    const int d0 = (j - js) * Rd + js;
+#pragma unroll
+    for (int r = 0; r < Rd; ++r) {
+      if constexpr (DONE + LR == LOGN)
+        store(d0 + r * NS, w[r]);
+      else
+        buf[padi(d0 + r * NS)] = w[r];
+    }
+  }
+  if constexpr (DONE + LR < LOGN) {
+    __syncthreads();
+    constexpr int LR2 = LOGN - DONE - LR >= LE ? LE : LOGN - DONE - LR;
+    constexpr int Rd2 = 1 << LR2;
+#pragma unroll
+    for (int q = 0; q < EPT / Rd2; ++q)
+#pragma unroll
+      for (int r = 0; r < Rd2; ++r) v[q * Rd2 + r] = buf[padi(t + q * TPS + r * (N / Rd2))];
+    __syncthreads();
+    run_stages<R, LOGN, LE, DONE + LR, INV>(v, buf, tw, tw_step, t, store);
+  }
+}
+
+// transform of one sequence, load(index) -> store(index, value); tw[m
+// tw_step] = exp(-2 pi i m / 2^LOGN)
+template <typename R, int LOGN, int LE, bool INV, class Load, class Store>
+__device__ __forceinline__ void transform(C2<R>* buf, const C2<R>* __restrict__ tw, int tw_step,
+                                          int t, const Load& load, const Store& store) {
+  constexpr int N = 1 << LOGN, TPS = N >> LE, EPT = 1 << LE;
+  constexpr int Rd = LOGN >= LE ? EPT : N;
+  static_assert(LOGN >= LE, "a thread's elements");
+  C2<R> v[EPT];
+#pragma unroll
+  for (int r = 0; r < Rd; ++r) v[r] = load(t + r * TPS);
+  run_stages<R, LOGN, LE, 0, INV>(v, buf, tw, tw_step, t, store);
+}
+
+// log2 of the elements per thread of a sequence of length 2^logn
+constexpr int elems_log(size_t rsz, int logn) {
+  return rsz == 4 ? (logn >= 11 ? 4 : (logn >= 6 ? 3 : 2))
+                  : (logn <= 9 ? 1 : (logn <= 11 ? 2 : 3));
+}
+// sequences of length 2^logn of a block and its shared memory.  Columns: a
+// 32-byte sector of each row, fewer for short columns (a block per SM) and
+// where 1024 threads or the shared memory set the limit.  Rows: some 256
+// threads, at most N / 128 rows.
+template <typename R, int LOGN> struct Seq {
+  static constexpr int LE = elems_log(sizeof(R), LOGN);
+  static constexpr int TPS = 1 << (LOGN - LE);
+  static constexpr int P = padi(1 << LOGN) + 4;   // so that 4 columns' elements share no banks
+};
+template <typename R, int LOGN> struct ColBlock {
+  using S = Seq<R, LOGN>;
+  static constexpr int kWant = sizeof(R) == 4 ? (LOGN >= 11 ? 4 : (LOGN == 10 ? 2 : 1))
+                                              : (LOGN >= 10 ? 2 : 1);
+  static constexpr int kMax = 1024 / S::TPS;
+  static constexpr int CB0 = kWant < kMax ? kWant : kMax;
+  static constexpr int CB = S::TPS * CB0 < 32 ? 32 / S::TPS : CB0;
+  static constexpr int THREADS = CB * S::TPS;
+  static constexpr size_t SMEM = (size_t)CB * S::P * sizeof(C2<R>);
+};
+template <typename R, int LOGM> struct RowBlock {
+  using S = Seq<R, LOGM>;
+  static constexpr int N = 1 << LOGM;
+  static constexpr int kThreads = 256 / S::TPS < 1 ? 1 : 256 / S::TPS;
+  static constexpr int kRows = N / 128 < 1 ? 1 : N / 128;
+  static constexpr int RB0 = kThreads < kRows ? kThreads : kRows;
+  static constexpr int RB = S::TPS * RB0 < 32 ? 32 / S::TPS : RB0;
+  static constexpr int THREADS = RB * S::TPS;
+  static constexpr size_t SMEM = (size_t)RB * S::P * sizeof(C2<R>);
+  static_assert(RB <= N, "rows of a block");
+};
+
+// the job of this block: blockIdx.y of the device table, or the one given
+template <typename R> __device__ __forceinline__ OpFftJob<R> pick_job(const OpFftArgs<R>& a) {
+  if (!a.jobs) return a.one;
+  const BatchJob<R>& b = a.jobs[blockIdx.y];
+  OpFftJob<R> o;
+  o.image_in = b.image_in;
+  o.image_out = b.image_out;
+  o.grid = b.grid;
+  o.scale = b.inv_n;
+  o.half = a.one.half + (int64_t)blockIdx.y * a.N * a.pitch;
+  return o;
+}
+
+// image row p, deapodized and centred -> its half-plane spectrum 0..ext
+template <typename R, int LOGM>
+__global__ void __launch_bounds__(RowBlock<R, LOGM>::THREADS) op_row_forward_kernel(OpFftArgs<R> a) {
+  using B = RowBlock<R, LOGM>;
+  using S = typename B::S;
+  constexpr int M = 1 << LOGM, N = M, H = N / 2;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const OpFftJob<R> jb = pick_job(a);
+  const int rr = threadIdx.x / S::TPS, t = threadIdx.x - rr * S::TPS;
+  const int p = blockIdx.x * B::RB + rr;
+  C2<R>* buf = reinterpret_cast<C2<R>*>(smem_raw) + rr * S::P;
+  const R* row = jb.image_in + (int64_t)p * N;
+  const R dp = a.psi[p];
+  // z_n = x_2n + i x_2n+1 of the padded row; image column q sits at q - H mod 2N
+  auto load = [&](int n) {
+    C2<R> z;
+    z.x = z.y = (R)0;
+    if (n < H / 2 || n >= M - H / 2) {
+      const int q = n < H / 2 ? 2 * n + H : 2 * n - (2 * N - H);
+      z.x = row[q] / (dp * a.psi[q]);
+      z.y = row[q + 1] / (dp * a.psi[q + 1]);
+    }
+    return z;
+  };
+  auto keep = [&](int k, C2<R> z) { buf[padi(k)] = z; };
+  transform<R, LOGM, S::LE, false>(buf, a.tw, 2, t, load, keep);
+  __syncthreads();
+  // X_k = E_k + W^k O_k, E, O the transforms of the even and odd elements
+  C2<R>* out = jb.half + (int64_t)p * a.pitch;
+  for (int k = t; k <= a.ext; k += S::TPS) {
+    const C2<R> zk = buf[padi(k == M ? 0 : k)], zm = buf[padi(k == 0 ? 0 : M - k)];
+    const R ex = (R)0.5 * (zk.x + zm.x), ey = (R)0.5 * (zk.y - zm.y);
+    const R ox = (R)0.5 * (zk.y + zm.y), oy = (R)-0.5 * (zk.x - zm.x);
+    const C2<R> w = a.tw[k];
+    C2<R> X;
+    X.x = ex + (w.x * ox - w.y * oy);
+    X.y = ey + (w.x * oy + w.y * ox);
+    out[k] = X;
+  }
+}
+
+// columns u of the half plane -> grid columns u and -u, rows -ext..ext
+template <typename R, int LOGG>
+__global__ void __launch_bounds__(ColBlock<R, LOGG>::THREADS) op_col_forward_kernel(OpFftArgs<R> a) {
+  using B = ColBlock<R, LOGG>;
+  using S = typename B::S;
+  constexpr int Ng = 1 << LOGG, N = Ng / 2, H = N / 2;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const OpFftJob<R> jb = pick_job(a);
+  const int c = threadIdx.x % B::CB, t = threadIdx.x / B::CB;
+  const int u = blockIdx.x * B::CB + c;
+  const bool live = u <= a.ext;
+  C2<R>* buf = reinterpret_cast<C2<R>*>(smem_raw) + c * S::P;
+  const C2<R>* col = jb.half + u;
+  auto load = [&](int n) {
+    C2<R> z;
+    z.x = z.y = (R)0;
+    if (live && (n < H || n >= Ng - H)) z = col[(int64_t)(n < H ? n + H : n - (Ng - H)) * a.pitch];
+    return z;
+  };
+  C2<R>* g = jb.grid;
+  const int iu = (N + u) & (Ng - 1), mu = N - u;   // grid columns of u and -u
+  auto store = [&](int v, C2<R> z) {
+    if (!live || (v > a.ext && v < Ng - a.ext)) return;
+    g[(int64_t)((N + v) & (Ng - 1)) * Ng + iu] = z;
+    if (mu != iu) {
+      z.y = -z.y;
+      g[(int64_t)((N - v) & (Ng - 1)) * Ng + mu] = z;
+    }
+  };
+  transform<R, LOGG, S::LE, false>(buf, a.tw, 1, t, load, store);
+}
+
+// grid columns u and -u (their Hermitian part, doubled), rows -ext..ext -> the
+// N image rows of the column's inverse transform
+template <typename R, int LOGG>
+__global__ void __launch_bounds__(ColBlock<R, LOGG>::THREADS) op_col_adjoint_kernel(OpFftArgs<R> a) {
+  using B = ColBlock<R, LOGG>;
+  using S = typename B::S;
+  constexpr int Ng = 1 << LOGG, N = Ng / 2, H = N / 2;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const OpFftJob<R> jb = pick_job(a);
+  const int c = threadIdx.x % B::CB, t = threadIdx.x / B::CB;
+  const int u = blockIdx.x * B::CB + c;
+  const bool live = u <= a.ext;
+  C2<R>* buf = reinterpret_cast<C2<R>*>(smem_raw) + c * S::P;
+  const C2<R>* g = jb.grid;
+  const int iu = (N + u) & (Ng - 1), mu = N - u;   // grid columns of u and -u
+  auto load = [&](int v) {
+    C2<R> z;
+    z.x = z.y = (R)0;
+    if (live && (v <= a.ext || v >= Ng - a.ext)) {
+      const C2<R> x = g[(int64_t)((N + v) & (Ng - 1)) * Ng + iu];
+      const C2<R> y = g[(int64_t)((N - v) & (Ng - 1)) * Ng + mu];
+      z.x = x.x + y.x;
+      z.y = x.y - y.y;
+    }
+    return z;
+  };
+  C2<R>* col = jb.half + u;
+  auto store = [&](int n, C2<R> z) {
+    if (live && (n < H || n >= Ng - H)) col[(int64_t)(n < H ? n + H : n - (Ng - H)) * a.pitch] = z;
+  };
+  transform<R, LOGG, S::LE, true>(buf, a.tw, 1, t, load, store);
+}
+
+// half-plane row p (0..ext) -> image row p: cropped, deapodized, scaled
+template <typename R, int LOGM>
+__global__ void __launch_bounds__(RowBlock<R, LOGM>::THREADS) op_row_adjoint_kernel(OpFftArgs<R> a) {
+  using B = RowBlock<R, LOGM>;
+  using S = typename B::S;
+  constexpr int M = 1 << LOGM, N = M, H = N / 2;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const OpFftJob<R> jb = pick_job(a);
+  const int rr = threadIdx.x / S::TPS, t = threadIdx.x - rr * S::TPS;
+  const int p = blockIdx.x * B::RB + rr;
+  C2<R>* buf = reinterpret_cast<C2<R>*>(smem_raw) + rr * S::P;
+  const C2<R>* in = jb.half + (int64_t)p * a.pitch;
+  auto at = [&](int k) {
+    C2<R> z;
+    z.x = z.y = (R)0;
+    if (k <= a.ext) z = in[k];
+    if (k == 0 || k == M) z.y = (R)0;   // real up to rounding
+    return z;
+  };
+  // Z'_k = (X_k + conj X_(M-k)) + i W^-k (X_k - conj X_(M-k))
+  auto load = [&](int k) {
+    const C2<R> x = at(k), y = at(M - k), w = a.tw[k];
+    const R sx = x.x + y.x, sy = x.y - y.y, dx = x.x - y.x, dy = x.y + y.y;
+    const R fx = w.x * dx + w.y * dy, fy = w.x * dy - w.y * dx;
+    C2<R> z;
+    z.x = sx - fy;
+    z.y = sy + fx;
+    return z;
+  };
+  R* row = jb.image_out + (int64_t)p * N;
+  const R dp = a.psi[p], sc = (R)(0.5 * jb.scale);   // (the columns were doubled)
+  auto store = [&](int n, C2<R> z) {
+    if (n >= H / 2 && n < M - H / 2) return;
+    const int q = n < H / 2 ? 2 * n + H : 2 * n - (2 * N - H);
+    row[q] = z.x * sc / (dp * a.psi[q]);
+    row[q + 1] = z.y * sc / (dp * a.psi[q + 1]);
+  };
+  transform<R, LOGM, S::LE, true>(buf, a.tw, 2, t, load, store);
+}
+
+template <typename R, int LOGG>
+cudaError_t go(const OpFftArgs<R>& a, bool forward, int njobs, cudaStream_t s) {
+  using C = ColBlock<R, LOGG>;
+  using W = RowBlock<R, LOGG - 1>;
+  auto run = [&](auto kern, int blocks, int threads, size_t smem) {
+    if (smem > 48 * 1024) {
+      const cudaError_t e =
+          cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+    }
+    kern<<<dim3(blocks, njobs), threads, smem, s>>>(a);
+    return cudaGetLastError();
+  };
+  const int rows = W::N / W::RB, cols = a.ext / C::CB + 1;
+  cudaError_t e;
+  if (forward) {
+    e = run(op_row_forward_kernel<R, LOGG - 1>, rows, W::THREADS, W::SMEM);
+    if (e == cudaSuccess) e = run(op_col_forward_kernel<R, LOGG>, cols, C::THREADS, C::SMEM);
+  } else {
+    e = run(op_col_adjoint_kernel<R, LOGG>, cols, C::THREADS, C::SMEM);
+    if (e == cudaSuccess) e = run(op_row_adjoint_kernel<R, LOGG - 1>, rows, W::THREADS, W::SMEM);
+  }
+  return e;
+}
+}  // namespace
+
+bool op_fft_supported(int N) { return N >= 16 && N <= 4096 && (N & (N - 1)) == 0; }
+
+// row pitch of the half plane: whole 32-byte sectors
+int op_fft_pitch(int N) { return N + 4; }
+
+template <typename R>
+cudaError_t launch_op_fft(const OpFftArgs<R>& a, bool forward, int njobs, cudaStream_t s) {
+  int l = 0;
+  while ((1 << l) < 2 * a.N) ++l;
+  switch (l) {
+    case 5: return go<R, 5>(a, forward, njobs, s);
+    case 6: return go<R, 6>(a, forward, njobs, s);
+    case 7: return go<R, 7>(a, forward, njobs, s);
+    case 8: return go<R, 8>(a, forward, njobs, s);
+    case 9: return go<R, 9>(a, forward, njobs, s);
+    case 10: return go<R, 10>(a, forward, njobs, s);
+    case 11: return go<R, 11>(a, forward, njobs, s);
+    case 12: return go<R, 12>(a, forward, njobs, s);
+    case 13: return go<R, 13>(a, forward, njobs, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+template cudaError_t launch_op_fft<float>(const OpFftArgs<float>&, bool, int, cudaStream_t);
+template cudaError_t launch_op_fft<double>(const OpFftArgs<double>&, bool, int, cudaStream_t);
+
+}  // namespace ms
