@@ -65,6 +65,24 @@ template <typename R> struct BatchJob {
   double inv_n;               // 1 / n (dirty-image scale; 0 when n = 0)
 };
 
+// Operands of the operator's own transforms (operator_fft.cu): one call's
+// buffers, or (jobs set) a batch's, whose half planes follow one another.
+template <typename R> struct OpFftJob {
+  const R* image_in;    // forward
+  R* image_out;         // adjoint, times scale
+  C2<R>* grid;
+  C2<R>* half;          // N rows of the half plane, `pitch` values each
+  double scale;
+};
+template <typename R> struct OpFftArgs {
+  const BatchJob<R>* jobs;
+  OpFftJob<R> one;
+  const R* psi;
+  const C2<R>* tw;      // exp(-2 pi i m / Ng), m < Ng
+  int N, pitch;
+  int ext;              // cells beyond +-ext are neither written nor read (<= Ng / 2)
+};
+
 // Device-side state of a minor cycle, one per plan.  Read and written only by
 // the library's kernels; the host reads it back after a cycle.
 struct FistaCtl {
@@ -209,6 +227,9 @@ void launch_classify(const double* u, const double* v, const uint8_t* flags, int
                      int Ng, int npix, double dl, double ell, double delta, int tile,
                      int ntx, uint32_t* cell, double2* frac, uint32_t* tile_id,
                      uint8_t* member, cudaStream_t s);
+// *ext = max(*ext, the largest |cell| that a footprint of a kept row touches)
+void launch_extent(const uint32_t* cell, const uint8_t* member, int64_t n, int Ng, int32_t* ext,
+                   cudaStream_t s);
 void launch_make_keys(const uint32_t* tile_id, const uint32_t* cell, const uint8_t* member,
                       int64_t n, uint8_t mask, int log2_tile, uint32_t sentinel, uint32_t* keys,
                       int32_t* vals, cudaStream_t s);
@@ -253,8 +274,9 @@ template <typename R, bool KAHAN>
 void launch_grid(const WorkItem* items, int nitems, const uint32_t* cell, const C2<R>* frac,
                  const C2<R>* vis, void* scratch, int Ng, int tile, int ntx, const EsKernel& es,
                  cudaStream_t s);
+// (ext: cells within +-ext of the origin only, Ng / 2 = all)
 template <typename R, bool KAHAN>
-void launch_fold(const void* scratch, const int32_t* tile_items, int Ng, int tile, int ntx,
+void launch_fold(const void* scratch, const int32_t* tile_items, int Ng, int tile, int ntx, int ext,
                  C2<R>* grid, cudaStream_t s);
 size_t grid_scratch_cell_bytes(int precision);
 // batched form (all launches take the device job table)
@@ -270,7 +292,7 @@ void launch_grid_batch(const BatchJob<R>* jobs, const int32_t* job_of, int total
                        void* scratch, int tile, int ntx, const EsKernel& es, cudaStream_t s);
 template <typename R, bool KAHAN>
 void launch_fold_batch(const BatchJob<R>* jobs, int njobs, const void* scratch, int Ng,
-                       int tile, int ntx, cudaStream_t s);
+                       int tile, int ntx, int ext, cudaStream_t s);
 template <typename R>
 void launch_degrid_batch(const CUtensorMap* tmap, const BatchJob<R>* jobs,
                          const int32_t* job_of, int total_items, bool has_obs, int Ng, int tile,
@@ -281,6 +303,12 @@ void launch_pad_batch(const BatchJob<R>* jobs, int njobs, const R* psi, int npix
 template <typename R>
 void launch_crop_batch(const BatchJob<R>* jobs, int njobs, const R* psi, int npix, int Ng,
                        cudaStream_t s);
+
+// operator_fft.cu: image -> grid (forward) or grid -> image, N a power of two
+bool op_fft_supported(int N);
+int op_fft_pitch(int N);
+template <typename R>
+cudaError_t launch_op_fft(const OpFftArgs<R>& a, bool forward, int njobs, cudaStream_t s);
 
 // wavelet_kernels.cu
 void set_wavelet_filters(const double* h, const int* len, int nbases);   // host -> __constant__

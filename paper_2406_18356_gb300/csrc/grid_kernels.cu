@@ -878,92 +878,100 @@ void launch_grid(const WorkItem* items, int nitems, const uint32_t* cell, const 
                                  Ng, tile, ntx, (R)es.beta, es.tab);
 }
 
-// Cells are walked x-stride over the whole grid (dense tiles, with many
-// items, spread over all blocks); a cell's items are read four at a time
-// (independent loads in flight) and added in item order.
+// Every grid cell within +-ext of the origin (index Ng / 2) sums, in a fixed
+// order, the scratch tiles of all work items of the (up to four) tiles whose
+// footprint region covers it: its own tile and, within W - 1 cells of a tile
+// edge, the tiles to the left and above (periodically).  Each cell is written
+// once, so the grid needs no clearing.  A thread per cell, a block per 256
+// cells of a row (a row of cells shares its tile row, so the branch on it is
+// uniform); a cell's items are read four at a time (independent loads in
+// flight) and added in item order.  Bound by the latency of the tile and
+// scratch loads.
 template <typename R, bool KAHAN>
-__device__ __forceinline__ void fold_cells(const typename ScratchOf<R, KAHAN>::T* __restrict__ scratch,
-                                           const int32_t* __restrict__ tile_items, int Ng, int T,
-                                           int ntx, C2<R>* __restrict__ grid) {
+__device__ __forceinline__ void fold_cell(const typename ScratchOf<R, KAHAN>::T* __restrict__ scratch,
+                                          const int32_t* __restrict__ tile_items, int Ng, int T,
+                                          int ntx, int first, int side, C2<R>* __restrict__ grid) {
   using Acc = typename ScratchOf<R, KAHAN>::T;
   const int S = T + kW - 1;
   const int cells = S * S;
   const int lt = __ffs(T) - 1;   // T is a power of two
-  const int total = Ng * Ng;     // < 2^31 (Ng <= 32768)
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < total; k += gridDim.x * blockDim.x) {
-    const int cv = k / Ng, cu = k - cv * Ng;
-    const int tx = cu >> lt, ty = cv >> lt, ou = cu & (T - 1), ov = cv & (T - 1);
-    Acc sum;
-    sum.x = 0;
-    sum.y = 0;
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  if (x >= side) return;
+  const int cu = first + x, cv = first + blockIdx.y;
+  const int tx = cu >> lt, ty = cv >> lt, ou = cu & (T - 1), ov = cv & (T - 1);
+  Acc sum;
+  sum.x = 0;
+  sum.y = 0;
 #pragma unroll
-    for (int dy = 0; dy < 2; ++dy) {
-      if (dy && ov >= kW - 1) break;
+  for (int dy = 0; dy < 2; ++dy) {
+    if (dy && ov >= kW - 1) break;
 #pragma unroll
-      for (int dx = 0; dx < 2; ++dx) {
-        if (dx && ou >= kW - 1) break;
-        int stx = tx - dx, sty = ty - dy;
-        stx += stx < 0 ? ntx : 0;
-        sty += sty < 0 ? ntx : 0;
-        const int t = sty * ntx + stx;
-        const int off = (ov + dy * T) * S + (ou + dx * T);
-        const int e = tile_items[t + 1];
-        int i = tile_items[t];
-        for (; i + 4 <= e; i += 4) {
-          Acc a[4];
+    for (int dx = 0; dx < 2; ++dx) {
+      if (dx && ou >= kW - 1) break;
+      int stx = tx - dx, sty = ty - dy;
+      stx += stx < 0 ? ntx : 0;
+      sty += sty < 0 ? ntx : 0;
+      const int t = sty * ntx + stx;
+      const int off = (ov + dy * T) * S + (ou + dx * T);
+      const int e = tile_items[t + 1];
+      int i = tile_items[t];
+      for (; i + 4 <= e; i += 4) {
+        Acc a[4];
 #pragma unroll
-          for (int u = 0; u < 4; ++u) a[u] = scratch[(int64_t)(i + u) * cells + off];
+        for (int u = 0; u < 4; ++u) a[u] = scratch[(int64_t)(i + u) * cells + off];
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            sum.x += a[u].x;
-            sum.y += a[u].y;
-          }
-        }
-        for (; i < e; ++i) {
-          const Acc a = scratch[(int64_t)i * cells + off];
-          sum.x += a.x;
-          sum.y += a.y;
+        for (int u = 0; u < 4; ++u) {
+          sum.x += a[u].x;
+          sum.y += a[u].y;
         }
       }
+      for (; i < e; ++i) {
+        const Acc a = scratch[(int64_t)i * cells + off];
+        sum.x += a.x;
+        sum.y += a.y;
+      }
     }
-    C2<R> o;
-    o.x = (R)sum.x;
-    o.y = (R)sum.y;
-    grid[k] = o;
   }
+  C2<R> o;
+  o.x = (R)sum.x;
+  o.y = (R)sum.y;
+  grid[(int64_t)cv * Ng + cu] = o;
 }
 
-// Every grid cell sums, in a fixed order, the scratch tiles of all work items
-// of the (up to four) tiles whose footprint region covers it: its own tile
-// and, within W - 1 cells of a tile edge, the tiles to the left and above
-// (periodically).  Each cell is written once, so the grid needs no clearing.
 template <typename R, bool KAHAN>
 __global__ void fold_kernel(const typename ScratchOf<R, KAHAN>::T* __restrict__ scratch,
                             const int32_t* __restrict__ tile_items, int Ng, int T, int ntx,
-                            C2<R>* __restrict__ grid) {
-  fold_cells<R, KAHAN>(scratch, tile_items, Ng, T, ntx, grid);
+                            int first, int side, C2<R>* __restrict__ grid) {
+  fold_cell<R, KAHAN>(scratch, tile_items, Ng, T, ntx, first, side, grid);
 }
 
-// stacked form: blockIdx.y = job (its tiles start at its first item)
+// stacked form: blockIdx.z = job (its tiles start at its first item)
 template <typename R, bool KAHAN>
 __global__ void fold_batch_kernel(const BatchJob<R>* __restrict__ jobs,
                                   const typename ScratchOf<R, KAHAN>::T* __restrict__ scratch,
-                                  int Ng, int T, int ntx) {
-  const BatchJob<R> jb = jobs[blockIdx.y];
+                                  int Ng, int T, int ntx, int first, int side) {
+  const BatchJob<R>& jb = jobs[blockIdx.z];
   const int S = T + kW - 1;
-  fold_cells<R, KAHAN>(scratch + jb.item_base * (int64_t)(S * S), jb.tile_items, Ng, T, ntx,
-                       jb.grid);
+  fold_cell<R, KAHAN>(scratch + jb.item_base * (int64_t)(S * S), jb.tile_items, Ng, T, ntx, first,
+                      side, jb.grid);
 }
 
+namespace {
+// first index and side of the square of cells within +-ext of the origin
+void fold_region(int Ng, int ext, int* first, int* side) {
+  *first = ext >= Ng / 2 ? 0 : Ng / 2 - ext;
+  *side = ext >= Ng / 2 ? Ng : 2 * ext + 1;
+}
+}  // namespace
+
 template <typename R, bool KAHAN>
-void launch_fold(const void* scratch, const int32_t* tile_items, int Ng, int tile, int ntx,
+void launch_fold(const void* scratch, const int32_t* tile_items, int Ng, int tile, int ntx, int ext,
                  C2<R>* grid, cudaStream_t s) {
-  int64_t total = (int64_t)Ng * Ng;
-  int blocks = (int)((total + kThreads - 1) / kThreads);
-  if (blocks > sm_count() * 32) blocks = sm_count() * 32;
-  fold_kernel<R, KAHAN><<<blocks, kThreads, 0, s>>>(
+  int first, side;
+  fold_region(Ng, ext, &first, &side);
+  fold_kernel<R, KAHAN><<<dim3((side + kThreads - 1) / kThreads, side), kThreads, 0, s>>>(
       reinterpret_cast<const typename ScratchOf<R, KAHAN>::T*>(scratch), tile_items, Ng, tile,
-      ntx, grid);
+      ntx, first, side, grid);
 }
 
 // ---------------------------------------------------------------- instances
@@ -1071,10 +1079,13 @@ void launch_grid_batch(const BatchJob<R>* jobs, const int32_t* job_of, int total
 
 template <typename R, bool KAHAN>
 void launch_fold_batch(const BatchJob<R>* jobs, int njobs, const void* scratch, int Ng,
-                       int tile, int ntx, cudaStream_t s) {
-  fold_batch_kernel<R, KAHAN><<<dim3(blocks_for((int64_t)Ng * Ng, sm_count() * 8), njobs), kThreads, 0,
-                                s>>>(
-      jobs, reinterpret_cast<const typename ScratchOf<R, KAHAN>::T*>(scratch), Ng, tile, ntx);
+                       int tile, int ntx, int ext, cudaStream_t s) {
+  int first, side;
+  fold_region(Ng, ext, &first, &side);
+  fold_batch_kernel<R, KAHAN>
+      <<<dim3((side + kThreads - 1) / kThreads, side, njobs), kThreads, 0, s>>>(
+          jobs, reinterpret_cast<const typename ScratchOf<R, KAHAN>::T*>(scratch), Ng, tile, ntx,
+          first, side);
 }
 
 template <typename R>
@@ -1130,11 +1141,11 @@ template void launch_grid_batch<float, true>(const BatchJob<float>*, const int32
 template void launch_grid_batch<double, false>(const BatchJob<double>*, const int32_t*, int,
                                                void*, int, int, const EsKernel&, cudaStream_t);
 template void launch_fold_batch<float, false>(const BatchJob<float>*, int, const void*, int, int,
-                                              int, cudaStream_t);
+                                              int, int, cudaStream_t);
 template void launch_fold_batch<float, true>(const BatchJob<float>*, int, const void*, int, int,
-                                             int, cudaStream_t);
-template void launch_fold_batch<double, false>(const BatchJob<double>*, int, const void*, int,
-                                               int, int, cudaStream_t);
+                                              int, int, cudaStream_t);
+template void launch_fold_batch<double, false>(const BatchJob<double>*, int, const void*, int, int,
+                                              int, int, cudaStream_t);
 
 template void launch_pad<float>(const float*, const float*, int, int, float2*, cudaStream_t);
 template void launch_pad<double>(const double*, const double*, int, int, double2*,
@@ -1158,11 +1169,11 @@ template void launch_grid<float, true>(const WorkItem*, int, const uint32_t*, co
 template void launch_grid<double, false>(const WorkItem*, int, const uint32_t*, const double2*,
                                          const double2*, void*, int, int, int, const EsKernel&,
                                          cudaStream_t);
-template void launch_fold<float, false>(const void*, const int32_t*, int, int, int, float2*,
+template void launch_fold<float, false>(const void*, const int32_t*, int, int, int, int, float2*,
                                         cudaStream_t);
-template void launch_fold<float, true>(const void*, const int32_t*, int, int, int, float2*,
+template void launch_fold<float, true>(const void*, const int32_t*, int, int, int, int, float2*,
                                        cudaStream_t);
-template void launch_fold<double, false>(const void*, const int32_t*, int, int, int, double2*,
+template void launch_fold<double, false>(const void*, const int32_t*, int, int, int, int, double2*,
                                          cudaStream_t);
 
 }  // namespace ms

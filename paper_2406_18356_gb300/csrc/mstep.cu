@@ -378,6 +378,11 @@ struct ms_plan {
   int32_t* err = nullptr;
   int trace_cap = 0;
   cufftHandle c2c = 0, r2c = 0, c2r = 0;
+  // the operator's own transforms (N a power of two up to 4096; else cuFFT):
+  // half-plane rows, twiddles of length Ng, and the cells in use
+  bool own_fft = false;
+  void *half = nullptr, *otw = nullptr;
+  int ext = 0;
   // fused spectral step (N a power of two whose blocks fit in shared
   // memory): the row-transform buffer and the twiddles
   bool fused_spec = false;
@@ -432,6 +437,7 @@ struct ms_plan {
     void* jobs = nullptr;       // BatchJob<R>[cap_jobs]
     int32_t* job_of = nullptr;  // [cap_items]
     void* grids = nullptr;      // cap_jobs Ng^2 complex
+    void* half = nullptr;       // cap_jobs half planes of the own transforms
     void* scratch = nullptr;    // cap_items tiles
     void* rows_a = nullptr;     // cap_rows complex (inputs in plan order)
     void* rows_b = nullptr;     // cap_rows complex (outputs in plan order)
@@ -613,16 +619,34 @@ template <typename R> void exec_c2r(cufftHandle h, void* in, void* out) {
     ckf(cufftExecC2R(h, (cufftComplex*)in, (cufftReal*)out), "C2R");
 }
 
+template <typename R> OpFftArgs<R> op_fft_args(ms_plan* p) {
+  OpFftArgs<R> a{};
+  a.one.grid = (C2<R>*)p->grid;
+  a.one.half = (C2<R>*)p->half;
+  a.psi = (const R*)p->psi;
+  a.tw = (const C2<R>*)p->otw;
+  a.N = p->N;
+  a.pitch = op_fft_pitch(p->N);
+  a.ext = p->ext;
+  return a;
+}
+
 // model grid = F Z D image (centred)
 template <typename R> void image_to_grid(ms_plan* p, const void* image, Timer* tm) {
-  {
+  if (!p->own_fft) {
     KSpan k(p, MS_K_PAD_CROP);
     launch_pad<R>((const R*)image, (const R*)p->psi, p->N, p->Ng, (C2<R>*)p->grid, p->ps);
   }
   int a = tm ? tm->mark() : 0;
   {
     KSpan k(p, MS_K_FFT_GRID);
-    fft_c2c<R>(p, CUFFT_FORWARD);
+    if (p->own_fft) {
+      OpFftArgs<R> o = op_fft_args<R>(p);
+      o.one.image_in = (const R*)image;
+      ck(launch_op_fft<R>(o, true, 1, p->ps), "operator transform");
+    } else {
+      fft_c2c<R>(p, CUFFT_FORWARD);
+    }
   }
   if (tm) tm->spans[1].push_back({a, tm->mark()});
 }
@@ -655,7 +679,7 @@ void grid_sorted(ms_plan* p, PartDev& pd, const void* vis_sorted, void* image, T
                                p->es, p->ps);
     }
     KSpan k(p, MS_K_FOLD);
-    launch_fold<float, true>(scratch, pd.tile_items, p->Ng, p->T, p->ntx, (float2*)p->grid,
+    launch_fold<float, true>(scratch, pd.tile_items, p->Ng, p->T, p->ntx, p->ext, (float2*)p->grid,
                              p->ps);
   } else {
     {
@@ -665,17 +689,25 @@ void grid_sorted(ms_plan* p, PartDev& pd, const void* vis_sorted, void* image, T
                             p->ps);
     }
     KSpan k(p, MS_K_FOLD);
-    launch_fold<R, false>(scratch, pd.tile_items, p->Ng, p->T, p->ntx, (C2<R>*)p->grid,
+    launch_fold<R, false>(scratch, pd.tile_items, p->Ng, p->T, p->ntx, p->ext, (C2<R>*)p->grid,
                           p->ps);
   }
   int b = tm ? tm->mark() : 0;
   if (tm) tm->spans[0].push_back({a, b});
+  const double sc = pd.n > 0 ? 1.0 / (double)pd.n : 0.0;
   {
     KSpan k(p, MS_K_FFT_GRID);
-    fft_c2c<R>(p, CUFFT_INVERSE);
+    if (p->own_fft) {
+      OpFftArgs<R> o = op_fft_args<R>(p);
+      o.one.image_out = (R*)image;
+      o.one.scale = sc;
+      ck(launch_op_fft<R>(o, false, 1, p->ps), "operator transform");
+    } else {
+      fft_c2c<R>(p, CUFFT_INVERSE);
+    }
   }
   if (tm) tm->spans[1].push_back({b, tm->mark()});
-  double sc = pd.n > 0 ? 1.0 / (double)pd.n : 0.0;
+  if (p->own_fft) return;
   KSpan k(p, MS_K_PAD_CROP);
   launch_crop<R>((const C2<R>*)p->grid, (const R*)p->psi, p->N, p->Ng, sc, (R*)image, p->ps);
 }
@@ -1458,6 +1490,8 @@ template <typename R> void build_plan(ms_plan* p, const ms_plan_desc* d) {
   while ((1u << bits) <= (unsigned)p->ntiles) ++bits;
   bits = ((bits + 2 * lg_t + 7) / 8) * 8;
   const uint32_t sentinel = (uint32_t)p->ntiles << (2 * lg_t);
+  int32_t* d_ext = dalloc<int32_t>(1, "extent");
+  ck(cudaMemsetAsync(d_ext, 0, sizeof(int32_t), s), "memset");
   const uint8_t masks[3] = {4 | 1, 4 | 2, 4};
   p->ch.resize(d->nchan);
   for (int c = 0; c < d->nchan; ++c) {
@@ -1470,6 +1504,7 @@ template <typename R> void build_plan(ms_plan* p, const ms_plan_desc* d) {
          "copy flags");
     launch_classify(du, dv, dfl, nvis, Ng, N, d->pixel_size, d->ell_px, d->delta_px, p->T,
                     p->ntx, cell_all, frac_all, tile_id, member, s);
+    launch_extent(cell_all, member, nvis, Ng, d_ext, s);
     for (int pt = 0; pt < 3; ++pt) {
       PartDev& pd = p->ch[c].part[pt];
       launch_make_keys(tile_id, cell_all, member, nvis, masks[pt], lg_t, sentinel, keys, vals, s);
@@ -1509,8 +1544,9 @@ template <typename R> void build_plan(ms_plan* p, const ms_plan_desc* d) {
     ChanDev& cd = p->ch[c];
     cd.counts[2] = cd.counts[0] + cd.counts[1] - cd.counts[3];
   }
+  ck(cudaMemcpyAsync(&p->ext, d_ext, sizeof(int32_t), cudaMemcpyDeviceToHost, s), "copy");
   ck(cudaStreamSynchronize(s), "plan");
-  for (void* q : {(void*)du, (void*)dv, (void*)dfl, (void*)cell_all, (void*)frac_all,
+  for (void* q : {(void*)d_ext, (void*)du, (void*)dv, (void*)dfl, (void*)cell_all, (void*)frac_all,
                   (void*)tile_id, (void*)member, (void*)keys, (void*)vals, (void*)ktmp,
                   (void*)vtmp, (void*)hist, (void*)counts, (void*)tstart, (void*)nch})
     if (q) cudaFree(q);
@@ -1556,10 +1592,25 @@ template <typename R> void build_plan(ms_plan* p, const ms_plan_desc* d) {
   cufftType tc = sizeof(R) == 8 ? CUFFT_Z2Z : CUFFT_C2C;
   cufftType tr = sizeof(R) == 8 ? CUFFT_D2Z : CUFFT_R2C;
   cufftType ti = sizeof(R) == 8 ? CUFFT_Z2D : CUFFT_C2R;
-  ckf(cufftPlan2d(&p->c2c, Ng, Ng, tc), "plan C2C");
+  p->own_fft = op_fft_supported(N);
+  if (p->own_fft) {
+    p->half = p->alloc<C2<R>>((size_t)N * op_fft_pitch(N), "half plane");
+    std::vector<C2<R>> tw(Ng);   // exp(-2 pi i m / Ng) in FP64
+    for (int m = 0; m < Ng; ++m) {
+      const double ang = -2.0 * M_PI * (double)m / (double)Ng;
+      tw[m].x = (R)std::cos(ang);
+      tw[m].y = (R)std::sin(ang);
+    }
+    p->otw = p->alloc<C2<R>>(Ng, "twiddles");
+    ck(cudaMemcpy(p->otw, tw.data(), sizeof(C2<R>) * Ng, cudaMemcpyHostToDevice), "twiddles");
+  } else {
+    p->ext = Ng / 2;   // cuFFT transforms the whole grid
+    ckf(cufftPlan2d(&p->c2c, Ng, Ng, tc), "plan C2C");
+    ckf(cufftSetStream(p->c2c, s), "set stream");
+  }
   ckf(cufftPlan2d(&p->r2c, N, N, tr), "plan R2C");
   ckf(cufftPlan2d(&p->c2r, N, N, ti), "plan C2R");
-  for (cufftHandle h : {p->c2c, p->r2c, p->c2r}) ckf(cufftSetStream(h, s), "set stream");
+  for (cufftHandle h : {p->r2c, p->c2r}) ckf(cufftSetStream(h, s), "set stream");
   if (p->conv == MS_CONV_LINEAR) {
     const int64_t n4 = 4 * n2, s2 = (int64_t)2 * N * (N + 1);
     p->lp = p->alloc<R>(n4, "linear pad");
@@ -1721,7 +1772,7 @@ void destroy(ms_plan* p) {
     if (h) cufftDestroy(h);
   for (void* a : p->allocs) cudaFree(a);
   if (p->batch.fft) cufftDestroy(p->batch.fft);
-  for (void* a : {p->batch.jobs, (void*)p->batch.job_of, p->batch.grids, p->batch.scratch,
+  for (void* a : {p->batch.jobs, (void*)p->batch.job_of, p->batch.grids, p->batch.half, p->batch.scratch,
                   p->batch.rows_a, p->batch.rows_b})
     if (a) cudaFree(a);
   for (auto e : p->tev) cudaEventDestroy(e);
@@ -1801,6 +1852,8 @@ template <typename R> void batch_reserve(ms_plan* p, const BatchShape& sh) {
   if (sh.njobs > B.cap_jobs) {
     grow(B.jobs, sizeof(BatchJob<R>) * sh.njobs, "batch jobs");
     grow(B.grids, sizeof(C2<R>) * (size_t)Ng * Ng * sh.njobs, "batch grids");
+    if (p->own_fft)
+      grow(B.half, sizeof(C2<R>) * (size_t)p->N * op_fft_pitch(p->N) * sh.njobs, "batch spectra");
     B.cap_jobs = sh.njobs;
     B.tmap_jobs = 0;   // the stacked-grid descriptor names the old buffer
     if (B.fft) cufftDestroy(B.fft);
@@ -1821,7 +1874,7 @@ template <typename R> void batch_reserve(ms_plan* p, const BatchShape& sh) {
     grow(B.rows_b, sizeof(C2<R>) * std::max<int64_t>(sh.rows, 1), "batch rows");
     B.cap_rows = sh.rows;
   }
-  if (B.fft_jobs != sh.njobs) {
+  if (!p->own_fft && B.fft_jobs != sh.njobs) {
     if (B.fft) cufftDestroy(B.fft);
     B.fft = 0;
     int n[2] = {Ng, Ng};
@@ -1870,15 +1923,36 @@ void batch_upload(ms_plan* p, const BatchShape& sh, std::vector<BatchJob<R>>& jo
   launch_job_of<R>((const BatchJob<R>*)B.jobs, sh.njobs, sh.max_items, B.job_of, p->ps);
 }
 
-template <typename R> void batch_fft(ms_plan* p, int dir) {
-  if (sizeof(R) == 8)
-    ckf(cufftExecZ2Z(p->batch.fft, (cufftDoubleComplex*)p->batch.grids,
-                     (cufftDoubleComplex*)p->batch.grids, dir),
-        "batched Z2Z");
-  else
-    ckf(cufftExecC2C(p->batch.fft, (cufftComplex*)p->batch.grids,
-                     (cufftComplex*)p->batch.grids, dir),
-        "batched C2C");
+// the jobs' images -> their grids, and their grids -> dirty images
+template <typename R> void batch_fft(ms_plan* p, const BatchJob<R>* jd, int njobs, bool forward) {
+  if (p->own_fft) {
+    KSpan k(p, MS_K_FFT_GRID);
+    OpFftArgs<R> o = op_fft_args<R>(p);
+    o.jobs = jd;
+    o.one.half = (C2<R>*)p->batch.half;
+    ck(launch_op_fft<R>(o, forward, njobs, p->ps), "operator transform");
+    return;
+  }
+  if (forward) {
+    KSpan k(p, MS_K_PAD_CROP);
+    launch_pad_batch<R>(jd, njobs, (const R*)p->psi, p->N, p->Ng, p->ps);
+  }
+  {
+    KSpan k(p, MS_K_FFT_GRID);
+    const int dir = forward ? CUFFT_FORWARD : CUFFT_INVERSE;
+    if (sizeof(R) == 8)
+      ckf(cufftExecZ2Z(p->batch.fft, (cufftDoubleComplex*)p->batch.grids,
+                       (cufftDoubleComplex*)p->batch.grids, dir),
+          "batched Z2Z");
+    else
+      ckf(cufftExecC2C(p->batch.fft, (cufftComplex*)p->batch.grids,
+                       (cufftComplex*)p->batch.grids, dir),
+          "batched C2C");
+  }
+  if (!forward) {
+    KSpan k(p, MS_K_PAD_CROP);
+    launch_crop_batch<R>(jd, njobs, (const R*)p->psi, p->N, p->Ng, p->ps);
+  }
 }
 
 template <typename R>
@@ -1909,16 +1983,12 @@ void grid_batch(ms_plan* p, int njobs, const int32_t* chans, const int32_t* part
     KSpan k(p, MS_K_FOLD);
     if (p->prec == MS_FP32_KAHAN)
       launch_fold_batch<float, true>((const BatchJob<float>*)jd, njobs, p->batch.scratch, p->Ng,
-                                     p->T, p->ntx, p->ps);
+                                     p->T, p->ntx, p->ext, p->ps);
     else
-      launch_fold_batch<R, false>(jd, njobs, p->batch.scratch, p->Ng, p->T, p->ntx, p->ps);
+      launch_fold_batch<R, false>(jd, njobs, p->batch.scratch, p->Ng, p->T, p->ntx, p->ext,
+                                  p->ps);
   }
-  {
-    KSpan k(p, MS_K_FFT_GRID);
-    batch_fft<R>(p, CUFFT_INVERSE);
-  }
-  KSpan k(p, MS_K_PAD_CROP);
-  launch_crop_batch<R>(jd, njobs, (const R*)p->psi, p->N, p->Ng, p->ps);
+  batch_fft<R>(p, jd, njobs, false);
 }
 
 template <typename R>
@@ -1938,14 +2008,7 @@ void degrid_batch(ms_plan* p, int njobs, const int32_t* chans, const int32_t* pa
   batch_upload<R>(p, sh, jobs);
   const BatchJob<R>* jd = (const BatchJob<R>*)p->batch.jobs;
   if (vis_obs) launch_batch_gather<R>(jd, njobs, sh.max_n, p->ps);
-  {
-    KSpan k(p, MS_K_PAD_CROP);
-    launch_pad_batch<R>(jd, njobs, (const R*)p->psi, p->N, p->Ng, p->ps);
-  }
-  {
-    KSpan k(p, MS_K_FFT_GRID);
-    batch_fft<R>(p, CUFFT_FORWARD);
-  }
+  batch_fft<R>(p, jd, njobs, true);
   {
     KSpan k(p, MS_K_DEGRID);
     launch_degrid_batch<R>(&p->batch.tmap, jd, p->batch.job_of, (int)sh.items, vis_obs != nullptr,
@@ -2214,14 +2277,7 @@ void residual_batch(ms_plan* p, int njobs, const int32_t* chans, const int32_t* 
   batch_upload<R>(p, sh, jobs);
   const BatchJob<R>* jd = (const BatchJob<R>*)p->batch.jobs;
   launch_batch_gather<R>(jd, njobs, sh.max_n, p->ps);
-  {
-    KSpan k(p, MS_K_PAD_CROP);
-    launch_pad_batch<R>(jd, njobs, (const R*)p->psi, p->N, p->Ng, p->ps);
-  }
-  {
-    KSpan k(p, MS_K_FFT_GRID);
-    batch_fft<R>(p, CUFFT_FORWARD);
-  }
+  batch_fft<R>(p, jd, njobs, true);
   {
     KSpan k(p, MS_K_DEGRID);
     launch_degrid_batch<R>(&p->batch.tmap, jd, p->batch.job_of, (int)sh.items, true, p->Ng,
@@ -2245,16 +2301,12 @@ void residual_batch(ms_plan* p, int njobs, const int32_t* chans, const int32_t* 
     KSpan k(p, MS_K_FOLD);
     if (p->prec == MS_FP32_KAHAN)
       launch_fold_batch<float, true>((const BatchJob<float>*)jd, njobs, p->batch.scratch, p->Ng,
-                                     p->T, p->ntx, p->ps);
+                                     p->T, p->ntx, p->ext, p->ps);
     else
-      launch_fold_batch<R, false>(jd, njobs, p->batch.scratch, p->Ng, p->T, p->ntx, p->ps);
+      launch_fold_batch<R, false>(jd, njobs, p->batch.scratch, p->Ng, p->T, p->ntx, p->ext,
+                                  p->ps);
   }
-  {
-    KSpan k(p, MS_K_FFT_GRID);
-    batch_fft<R>(p, CUFFT_INVERSE);
-  }
-  KSpan k(p, MS_K_PAD_CROP);
-  launch_crop_batch<R>(jd, njobs, (const R*)p->psi, p->N, p->Ng, p->ps);
+  batch_fft<R>(p, jd, njobs, false);
 }
 
 // One step of the method (as run_step) for several channels at once: the

@@ -78,6 +78,28 @@ void launch_classify(const double* u, const double* v, const uint8_t* flags, int
                                                     tile, ntx, cell, frac, tile_id, member);
 }
 
+// Largest distance of a footprint's cells from the grid's origin (cell k at
+// index k + Ng / 2; a footprint that wraps reaches Ng / 2), over the unflagged
+// rows.
+__global__ void extent_kernel(const uint32_t* __restrict__ cell, const uint8_t* __restrict__ member,
+                              int64_t n, int Ng, int32_t* __restrict__ ext) {
+  int most = 0;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    if (!(member[i] & 4)) continue;
+    const uint32_t c = cell[i];
+    const int u = (int)(c & 0xffffu) - Ng / 2, v = (int)(c >> 16) - Ng / 2;
+    most = max(most, max(max(abs(u), abs(u + kW - 1)), max(abs(v), abs(v + kW - 1))));
+  }
+  for (int o = 16; o > 0; o >>= 1) most = max(most, __shfl_down_sync(0xffffffffu, most, o));
+  if ((threadIdx.x & 31) == 0 && most > 0) atomicMax(ext, min(most, Ng / 2));
+}
+
+void launch_extent(const uint32_t* cell, const uint8_t* member, int64_t n, int Ng, int32_t* ext,
+                   cudaStream_t s) {
+  extent_kernel<<<grid_for(n, 256), 256, 0, s>>>(cell, member, n, Ng, ext);
+}
+
 // Sort key of a row: its tile, then its anchor cell inside the tile (row v,
 // then column u), so that rows sharing an anchor are adjacent in plan order;
 // rows outside the partition get the sentinel (after every tile).
