@@ -253,9 +253,6 @@ void launch_gather_geometry(const int32_t* idx, int64_t n, const uint32_t* cell_
 template <typename R>
 void launch_gather_vis(const int32_t* idx, int64_t n, const C2<R>* src, C2<R>* dst,
                        cudaStream_t s);
-template <typename R>
-void launch_scatter_vis(const int32_t* idx, int64_t n, const C2<R>* src, C2<R>* dst,
-                        cudaStream_t s);
 void launch_deapodization(int npix, int ngrid, double beta, const double* nodes,
                           const double* weights, int nq, double* psi, cudaStream_t s);
 
@@ -265,10 +262,12 @@ void launch_pad(const R* image, const R* psi, int npix, int Ng, C2<R>* grid, cud
 template <typename R>
 void launch_crop(const C2<R>* grid, const R* psi, int npix, int Ng, double scale, R* image,
                  cudaStream_t s);
+// Row k of the plan order reads obs[obs_idx[k]] and writes out[out_idx[k]]
+// (nullptr: position k).
 template <typename R>
 void launch_degrid(const CUtensorMap* tmap, const C2<R>* grid, const WorkItem* items,
                    int nitems, const uint32_t* cell, const C2<R>* frac, const C2<R>* obs,
-                   C2<R>* out, int Ng, int tile, int ntx, const EsKernel& es, int32_t* err,
+                   const int32_t* obs_idx, C2<R>* out, const int32_t* out_idx, int Ng, int tile, int ntx, const EsKernel& es, int32_t* err,
                    cudaStream_t s);
 template <typename R, bool KAHAN>
 void launch_grid(const WorkItem* items, int nitems, const uint32_t* cell, const C2<R>* frac,
@@ -285,18 +284,18 @@ void launch_job_of(const BatchJob<R>* jobs, int njobs, int max_items, int32_t* j
                    cudaStream_t s);
 template <typename R>
 void launch_batch_gather(const BatchJob<R>* jobs, int njobs, int64_t max_n, cudaStream_t s);
-template <typename R>
-void launch_batch_scatter(const BatchJob<R>* jobs, int njobs, int64_t max_n, cudaStream_t s);
 template <typename R, bool KAHAN>
 void launch_grid_batch(const BatchJob<R>* jobs, const int32_t* job_of, int total_items,
                        void* scratch, int tile, int ntx, const EsKernel& es, cudaStream_t s);
 template <typename R, bool KAHAN>
 void launch_fold_batch(const BatchJob<R>* jobs, int njobs, const void* scratch, int Ng,
                        int tile, int ntx, int ext, cudaStream_t s);
+// observed values from user_in, or (gathered) sorted_in; results to user_out
+// (user_order) or sorted_out
 template <typename R>
 void launch_degrid_batch(const CUtensorMap* tmap, const BatchJob<R>* jobs,
-                         const int32_t* job_of, int total_items, bool has_obs, int Ng, int tile,
-                         int ntx, const EsKernel& es, int32_t* err, cudaStream_t s);
+                         const int32_t* job_of, int total_items, bool has_obs, bool gathered,
+                         bool user_order, int Ng, int tile, int ntx, const EsKernel& es, int32_t* err, cudaStream_t s);
 template <typename R>
 void launch_pad_batch(const BatchJob<R>* jobs, int njobs, const R* psi, int npix, int Ng,
                       cudaStream_t s);

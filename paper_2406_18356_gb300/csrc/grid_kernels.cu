@@ -271,8 +271,10 @@ __device__ __forceinline__ void degrid_item(const CUtensorMap* tmap, int tma_y0,
                                             const uint32_t* __restrict__ cell,
                                             const C2<R>* __restrict__ frac,
                                             const C2<R>* __restrict__ obs,
-                                            C2<R>* __restrict__ out, int Ng, int T, int ntx,
-                                            R beta, const double* __restrict__ es_tab,
+                                            const int32_t* __restrict__ obs_idx,
+                                            C2<R>* __restrict__ out,
+                                            const int32_t* __restrict__ out_idx, int Ng, int T,
+                                            int ntx, R beta, const double* __restrict__ es_tab,
                                             int32_t* __restrict__ err) {
   // the tile sits at a 128-byte-aligned shared address (TMA destination rule),
   // the mbarrier and a flag after it, all in the dynamic allocation
@@ -332,6 +334,8 @@ __device__ __forceinline__ void degrid_item(const CUtensorMap* tmap, int tma_y0,
     int lu = (int)(pc & 0xffffu) - ox;
     int lv = (int)(pc >> 16) - oy;
     C2<R> f = frac[k];
+    C2<R> v{};
+    if (HAS_OBS) v = obs[obs_idx ? obs_idx[k] : k];   // in flight during the taps
     R wu[kW], wv[kW];
     es(f.x, wu);
     es(f.y, wv);
@@ -366,14 +370,16 @@ __device__ __forceinline__ void degrid_item(const CUtensorMap* tmap, int tma_y0,
     }
     C2<R> o;
     if (HAS_OBS) {
-      C2<R> v = obs[k];
       o.x = v.x - accr;
       o.y = v.y - acci;
     } else {
       o.x = accr;
       o.y = acci;
     }
-    out[k] = o;
+    // (straight to the caller's order: 8-byte writes beside the next rows'
+    // arithmetic, for a pass of their own; likewise the reads of obs.  16 jobs
+    // at 1024 px: 131 + 42 + 94 us in three passes, 158 in one)
+    out[out_idx ? out_idx[k] : k] = o;
   }
 }
 
@@ -383,10 +389,11 @@ __global__ void __launch_bounds__(degrid_threads<R>())
     degrid_kernel(const __grid_constant__ CUtensorMap tmap, const C2<R>* __restrict__ grid,
                   const WorkItem* __restrict__ items, const uint32_t* __restrict__ cell,
                   const C2<R>* __restrict__ frac, const C2<R>* __restrict__ obs,
-                  C2<R>* __restrict__ out, int Ng, int T, int ntx, R beta,
+                  const int32_t* __restrict__ obs_idx, C2<R>* __restrict__ out,
+                  const int32_t* __restrict__ out_idx, int Ng, int T, int ntx, R beta,
                   const double* __restrict__ es_tab, int32_t* __restrict__ err) {
-  degrid_item<R, HAS_OBS>(&tmap, 0, grid, items[blockIdx.x], cell, frac, obs, out, Ng, T, ntx,
-                          beta, es_tab, err);
+  degrid_item<R, HAS_OBS>(&tmap, 0, grid, items[blockIdx.x], cell, frac, obs, obs_idx, out,
+                          out_idx, Ng, T, ntx, beta, es_tab, err);
 }
 
 // Stacked form: one block per work item of all jobs; job_of[item] names the
@@ -395,19 +402,21 @@ template <typename R, bool HAS_OBS>
 __global__ void __launch_bounds__(degrid_threads<R>())
     degrid_batch_kernel(const __grid_constant__ CUtensorMap tmap,
                         const BatchJob<R>* __restrict__ jobs, const int32_t* __restrict__ job_of,
-                        int Ng, int T, int ntx, R beta, const double* __restrict__ es_tab,
-                        int32_t* __restrict__ err) {
+                        bool gathered, bool user_order, int Ng, int T, int ntx, R beta,
+                        const double* __restrict__ es_tab, int32_t* __restrict__ err) {
   const int j = job_of[blockIdx.x];
   const BatchJob<R> jb = jobs[j];
   const WorkItem it = jb.items[blockIdx.x - jb.item_base];
-  degrid_item<R, HAS_OBS>(&tmap, j * Ng, jb.grid, it, jb.cell, jb.frac, jb.sorted_in,
-                          jb.sorted_out, Ng, T, ntx, beta, es_tab, err);
+  degrid_item<R, HAS_OBS>(&tmap, j * Ng, jb.grid, it, jb.cell, jb.frac,
+                          gathered ? jb.sorted_in : jb.user_in, gathered ? nullptr : jb.idx,
+                          user_order ? jb.user_out : jb.sorted_out,
+                          user_order ? jb.idx : nullptr, Ng, T, ntx, beta, es_tab, err);
 }
 
 template <typename R>
 void launch_degrid(const CUtensorMap* tmap, const C2<R>* grid, const WorkItem* items,
                    int nitems, const uint32_t* cell, const C2<R>* frac, const C2<R>* obs,
-                   C2<R>* out, int Ng, int tile, int ntx, const EsKernel& es, int32_t* err,
+                   const int32_t* obs_idx, C2<R>* out, const int32_t* out_idx, int Ng, int tile, int ntx, const EsKernel& es, int32_t* err,
                    cudaStream_t s) {
   if (nitems <= 0) return;
   const int S = tile + kW - 1;
@@ -416,21 +425,52 @@ void launch_degrid(const CUtensorMap* tmap, const C2<R>* grid, const WorkItem* i
   if (obs) {
     auto k = degrid_kernel<R, true>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<nitems, degrid_threads<R>(), smem, s>>>(*tmap, grid, items, cell, frac, obs, out, Ng, tile,
-                                                ntx, (R)es.beta, es.tab, err);
+    k<<<nitems, degrid_threads<R>(), smem, s>>>(*tmap, grid, items, cell, frac, obs, obs_idx, out,
+                                                out_idx, Ng, tile, ntx, (R)es.beta, es.tab, err);
   } else {
     auto k = degrid_kernel<R, false>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<nitems, degrid_threads<R>(), smem, s>>>(*tmap, grid, items, cell, frac, obs, out, Ng, tile,
-                                                ntx, (R)es.beta, es.tab, err);
+    k<<<nitems, degrid_threads<R>(), smem, s>>>(*tmap, grid, items, cell, frac, obs, obs_idx, out,
+                                                out_idx, Ng, tile, ntx, (R)es.beta, es.tab, err);
   }
 }
 
 // ------------------------------------------------------------------ grid
 // Scratch holds one (T + W - 1)^2 tile per work item: float2 for the plain
-// FP32 form, double2 for FP64 and for the compensated FP32 form.
+// FP32 form, double2 for FP64, and FP32 pairs (Re hi, Re lo, Im hi, Im lo) for
+// the compensated FP32 form, whose sums over warps and work items are
+// error-free FP32 additions (TwoSum, the errors summed in lo): in FP64 the
+// conversions and additions of a tile's 484 cells took 6,900 cycles of an
+// SM's FP64 pipe per work item, most of the kernel (3.4M rows in 38,884 items
+// at 4096 px: 1168 -> 305 us, with the sub-tiles of idle warps left out).
 template <typename R, bool KAHAN> struct ScratchOf { using T = double2; };
 template <> struct ScratchOf<float, false> { using T = float2; };
+template <> struct ScratchOf<float, true> { using T = float4; };
+
+// s += a for a scratch cell
+__device__ __forceinline__ void cell_sum(float2& s, const float2& a) {
+  s.x += a.x;
+  s.y += a.y;
+}
+__device__ __forceinline__ void cell_sum(double2& s, const double2& a) {
+  s.x += a.x;
+  s.y += a.y;
+}
+__device__ __forceinline__ void cell_sum(float4& s, const float4& a) {
+  float h, e;
+  two_sum<float>(s.x, a.x, h, e);
+  s.x = h;
+  s.y += a.y + e;
+  two_sum<float>(s.z, a.z, h, e);
+  s.z = h;
+  s.w += a.w + e;
+}
+// the grid value of a summed cell
+__device__ __forceinline__ float2 cell_value(const float2& s) { return s; }
+__device__ __forceinline__ double2 cell_value(const double2& s) { return s; }
+__device__ __forceinline__ float2 cell_value(const float4& s) {
+  return make_float2(s.x + s.y, s.z + s.w);
+}
 
 size_t grid_scratch_cell_bytes(int precision) { return precision == 1 ? 8 : 16; }
 
@@ -525,7 +565,10 @@ __device__ __forceinline__ void grid_item(const WorkItem it, const uint32_t* __r
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ox = (it.tile % ntx) * T, oy = (it.tile / ntx) * T;
 
-  for (int c = threadIdx.x; c < NW * cells; c += blockDim.x) {
+  // warps with rows: a batch of 32 each, so that a small item (a sparse tile
+  // of a large grid holds some 90 rows) clears and sums fewer sub-tiles
+  const int used = min(NW, (it.count + 31) / 32);
+  for (int c = threadIdx.x; c < used * cells; c += blockDim.x) {
     C2<R> z;
     z.x = (R)0;
     z.y = (R)0;
@@ -543,10 +586,11 @@ __device__ __forceinline__ void grid_item(const WorkItem it, const uint32_t* __r
   const bool two = lane + 32 < kW * kW;
   const int off1 = j1 * S + i1, off2 = j2 * S + i2;
 
-  const int per = (it.count + NW - 1) / NW;
+  const int per = (it.count + used - 1) / used;
   const int ws = it.start + warp * per;
   int we = ws + per;
   if (we > it.start + it.count) we = it.start + it.count;
+  if (warp >= used) we = ws;
   TapSum<R, KAHAN> t1, t2;
   int run = -1;   // anchor (tile-local cell index) of the current run
   for (int base = ws; base < we; base += 32) {
@@ -609,19 +653,14 @@ __device__ __forceinline__ void grid_item(const WorkItem it, const uint32_t* __r
   __syncthreads();
   Acc* dst = scratch + scratch_tile * cells;
   for (int c = threadIdx.x; c < cells; c += blockDim.x) {
-    Acc s;
-    s.x = 0;
-    s.y = 0;
-#pragma unroll
-    for (int w = 0; w < NW; ++w) {
-      C2<R> a = tiles[w * cells + c];
-      if (KAHAN) {
-        C2<R> cp = comps[w * cells + c];
-        s.x += (double)a.x - (double)cp.x;
-        s.y += (double)a.y - (double)cp.y;
+    Acc s{};
+    for (int w = 0; w < used; ++w) {
+      const C2<R> a = tiles[w * cells + c];
+      if constexpr (KAHAN) {
+        const C2<R> cp = comps[w * cells + c];
+        cell_sum(s, make_float4(a.x, -cp.x, a.y, -cp.y));
       } else {
-        s.x += a.x;
-        s.y += a.y;
+        cell_sum(s, a);
       }
     }
     dst[c] = s;
@@ -884,9 +923,10 @@ void launch_grid(const WorkItem* items, int nitems, const uint32_t* cell, const 
 // edge, the tiles to the left and above (periodically).  Each cell is written
 // once, so the grid needs no clearing.  A thread per cell, a block per 256
 // cells of a row (a row of cells shares its tile row, so the branch on it is
-// uniform); a cell's items are read four at a time (independent loads in
-// flight) and added in item order.  Bound by the latency of the tile and
-// scratch loads.
+// uniform); a cell's items are read 16 (8) or 4 at a time (independent loads
+// in flight) and added in item order.  Bound by the latency of the tile and
+// scratch loads: the densest tile of a 9.27M-row observation has hundreds of
+// work items.
 template <typename R, bool KAHAN>
 __device__ __forceinline__ void fold_cell(const typename ScratchOf<R, KAHAN>::T* __restrict__ scratch,
                                           const int32_t* __restrict__ tile_items, int Ng, int T,
@@ -899,9 +939,8 @@ __device__ __forceinline__ void fold_cell(const typename ScratchOf<R, KAHAN>::T*
   if (x >= side) return;
   const int cu = first + x, cv = first + blockIdx.y;
   const int tx = cu >> lt, ty = cv >> lt, ou = cu & (T - 1), ov = cv & (T - 1);
-  Acc sum;
-  sum.x = 0;
-  sum.y = 0;
+  constexpr int U = sizeof(Acc) == 8 ? 16 : 8;   // loads in flight of a long item list
+  Acc sum{};
 #pragma unroll
   for (int dy = 0; dy < 2; ++dy) {
     if (dy && ov >= kW - 1) break;
@@ -915,27 +954,24 @@ __device__ __forceinline__ void fold_cell(const typename ScratchOf<R, KAHAN>::T*
       const int off = (ov + dy * T) * S + (ou + dx * T);
       const int e = tile_items[t + 1];
       int i = tile_items[t];
+      for (; i + U <= e; i += U) {
+        Acc a[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) a[u] = scratch[(int64_t)(i + u) * cells + off];
+#pragma unroll
+        for (int u = 0; u < U; ++u) cell_sum(sum, a[u]);
+      }
       for (; i + 4 <= e; i += 4) {
         Acc a[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) a[u] = scratch[(int64_t)(i + u) * cells + off];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          sum.x += a[u].x;
-          sum.y += a[u].y;
-        }
+        for (int u = 0; u < 4; ++u) cell_sum(sum, a[u]);
       }
-      for (; i < e; ++i) {
-        const Acc a = scratch[(int64_t)i * cells + off];
-        sum.x += a.x;
-        sum.y += a.y;
-      }
+      for (; i < e; ++i) cell_sum(sum, scratch[(int64_t)i * cells + off]);
     }
   }
-  C2<R> o;
-  o.x = (R)sum.x;
-  o.y = (R)sum.y;
-  grid[(int64_t)cv * Ng + cu] = o;
+  grid[(int64_t)cv * Ng + cu] = cell_value(sum);
 }
 
 template <typename R, bool KAHAN>
@@ -990,14 +1026,6 @@ __global__ void batch_gather_kernel(const BatchJob<R>* __restrict__ jobs) {
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < jb.n;
        k += (int64_t)gridDim.x * blockDim.x)
     jb.sorted_in[k] = jb.user_in[jb.idx[k]];
-}
-
-template <typename R>
-__global__ void batch_scatter_kernel(const BatchJob<R>* __restrict__ jobs) {
-  const BatchJob<R> jb = jobs[blockIdx.y];
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < jb.n;
-       k += (int64_t)gridDim.x * blockDim.x)
-    jb.user_out[jb.idx[k]] = jb.sorted_out[k];
 }
 
 template <typename R>
@@ -1060,11 +1088,6 @@ void launch_batch_gather(const BatchJob<R>* jobs, int njobs, int64_t max_n, cuda
   batch_gather_kernel<R><<<dim3(blocks_for(max_n, sm_count() * 4), njobs), kThreads, 0, s>>>(jobs);
 }
 
-template <typename R>
-void launch_batch_scatter(const BatchJob<R>* jobs, int njobs, int64_t max_n, cudaStream_t s) {
-  batch_scatter_kernel<R><<<dim3(blocks_for(max_n, sm_count() * 4), njobs), kThreads, 0, s>>>(jobs);
-}
-
 template <typename R, bool KAHAN>
 void launch_grid_batch(const BatchJob<R>* jobs, const int32_t* job_of, int total_items,
                        void* scratch, int tile, int ntx, const EsKernel& es, cudaStream_t s) {
@@ -1090,21 +1113,21 @@ void launch_fold_batch(const BatchJob<R>* jobs, int njobs, const void* scratch, 
 
 template <typename R>
 void launch_degrid_batch(const CUtensorMap* tmap, const BatchJob<R>* jobs,
-                         const int32_t* job_of, int total_items, bool has_obs, int Ng, int tile,
-                         int ntx, const EsKernel& es, int32_t* err, cudaStream_t s) {
+                         const int32_t* job_of, int total_items, bool has_obs, bool gathered,
+                         bool user_order, int Ng, int tile, int ntx, const EsKernel& es, int32_t* err, cudaStream_t s) {
   if (total_items <= 0) return;
   const int S = tile + kW - 1;
   const size_t smem = (size_t)S * S * sizeof(C2<R>) + 128 + 16 + es_smem<R>(es);
   if (has_obs) {
     auto k = degrid_batch_kernel<R, true>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<total_items, degrid_threads<R>(), smem, s>>>(*tmap, jobs, job_of, Ng, tile, ntx,
-                                                     (R)es.beta, es.tab, err);
+    k<<<total_items, degrid_threads<R>(), smem, s>>>(*tmap, jobs, job_of, gathered, user_order, Ng, tile,
+                                                     ntx, (R)es.beta, es.tab, err);
   } else {
     auto k = degrid_batch_kernel<R, false>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<total_items, degrid_threads<R>(), smem, s>>>(*tmap, jobs, job_of, Ng, tile, ntx,
-                                                     (R)es.beta, es.tab, err);
+    k<<<total_items, degrid_threads<R>(), smem, s>>>(*tmap, jobs, job_of, gathered, user_order, Ng, tile,
+                                                     ntx, (R)es.beta, es.tab, err);
   }
 }
 
@@ -1125,10 +1148,9 @@ void launch_crop_batch(const BatchJob<R>* jobs, int njobs, const R* psi, int npi
 #define MS_BATCH_INST(R)                                                                         \
   template void launch_job_of<R>(const BatchJob<R>*, int, int, int32_t*, cudaStream_t);         \
   template void launch_batch_gather<R>(const BatchJob<R>*, int, int64_t, cudaStream_t);         \
-  template void launch_batch_scatter<R>(const BatchJob<R>*, int, int64_t, cudaStream_t);        \
   template void launch_degrid_batch<R>(const CUtensorMap*, const BatchJob<R>*, const int32_t*,  \
-                                       int, bool, int, int, int, const EsKernel&, int32_t*,             \
-                                       cudaStream_t);                                           \
+                                       int, bool, bool, bool, int, int, int, const EsKernel&,   \
+                                       int32_t*, cudaStream_t);                                 \
   template void launch_pad_batch<R>(const BatchJob<R>*, int, const R*, int, int, cudaStream_t); \
   template void launch_crop_batch<R>(const BatchJob<R>*, int, const R*, int, int, cudaStream_t);
 MS_BATCH_INST(float)
@@ -1155,11 +1177,11 @@ template void launch_crop<float>(const float2*, const float*, int, int, double, 
 template void launch_crop<double>(const double2*, const double*, int, int, double, double*,
                                   cudaStream_t);
 template void launch_degrid<float>(const CUtensorMap*, const float2*, const WorkItem*, int,
-                                   const uint32_t*, const float2*, const float2*, float2*, int,
-                                   int, int, const EsKernel&, int32_t*, cudaStream_t);
+                                   const uint32_t*, const float2*, const float2*, const int32_t*,
+                                   float2*, const int32_t*, int, int, int, const EsKernel&, int32_t*, cudaStream_t);
 template void launch_degrid<double>(const CUtensorMap*, const double2*, const WorkItem*, int,
-                                    const uint32_t*, const double2*, const double2*, double2*,
-                                    int, int, int, const EsKernel&, int32_t*, cudaStream_t);
+                                    const uint32_t*, const double2*, const double2*,
+                                    const int32_t*, double2*, const int32_t*, int, int, int, const EsKernel&, int32_t*, cudaStream_t);
 template void launch_grid<float, false>(const WorkItem*, int, const uint32_t*, const float2*,
                                         const float2*, void*, int, int, int, const EsKernel&,
                                         cudaStream_t);

@@ -651,17 +651,40 @@ template <typename R> void image_to_grid(ms_plan* p, const void* image, Timer* t
   if (tm) tm->spans[1].push_back({a, tm->mark()});
 }
 
-// sorted visibilities -> model (or residual when obs given) with G
+// model (or residual when obs given) of the partition's rows with G: row k of
+// the plan order from obs[obs_idx[k]] to out[out_idx[k]] (NULL: position k)
 template <typename R>
-void degrid_sorted(ms_plan* p, PartDev& pd, const void* obs_sorted, void* out_sorted, Timer* tm) {
+void degrid_rows(ms_plan* p, PartDev& pd, const void* obs, const int32_t* obs_idx, void* out,
+                 const int32_t* out_idx, Timer* tm) {
   int a = tm ? tm->mark() : 0;
   {
     KSpan k(p, MS_K_DEGRID);
     launch_degrid<R>(&p->tmap, (const C2<R>*)p->grid, pd.items, pd.nitems, pd.cell,
-                     (const C2<R>*)pd.frac, (const C2<R>*)obs_sorted, (C2<R>*)out_sorted, p->Ng,
+                     (const C2<R>*)pd.frac, (const C2<R>*)obs, obs_idx, (C2<R>*)out, out_idx, p->Ng,
                      p->T, p->ntx, p->es, p->err, p->ps);
   }
   if (tm) tm->spans[0].push_back({a, tm->mark()});
+}
+
+// Whether a degridding call may read observed rows while it writes results
+// (each row by one thread, which reads before it writes): every job's obs is
+// its own out or lies apart from all outs.  Else (jobs that share a buffer
+// another job writes) the observed rows are gathered before any is written.
+template <typename R>
+bool rows_apart(ms_plan* p, int njobs, const void* const* obs, void* const* out) {
+  const size_t len = sizeof(C2<R>) * (size_t)p->d.nvis;
+  std::vector<std::pair<uintptr_t, int>> outs(njobs);
+  for (int j = 0; j < njobs; ++j) outs[j] = {(uintptr_t)out[j], j};
+  std::sort(outs.begin(), outs.end());
+  for (int j = 0; j < njobs; ++j) {
+    const uintptr_t a = (uintptr_t)obs[j];
+    // the outs that start in (a - len, a + len)
+    auto it = std::upper_bound(outs.begin(), outs.end(),
+                               std::make_pair(a > len ? a - len : 0, njobs));
+    for (; it != outs.end() && it->first < a + len; ++it)
+      if (it->second != j || it->first != a) return false;
+  }
+  return true;
 }
 
 // sorted visibilities -> image = Re(D Z^H F^H G^H y) / sum(w); the gridding
@@ -712,12 +735,13 @@ void grid_sorted(ms_plan* p, PartDev& pd, const void* vis_sorted, void* image, T
   launch_crop<R>((const C2<R>*)p->grid, (const R*)p->psi, p->N, p->Ng, sc, (R*)image, p->ps);
 }
 
-// i~ = A^H (obs - A model) / sum(w), obs already sorted
+// i~ = A^H (obs - A model) / sum(w), obs in plan order (obs_idx NULL) or in the
+// caller's (obs_idx = pd.idx)
 template <typename R>
-void residual_sorted(ms_plan* p, PartDev& pd, const void* obs_sorted, const void* model,
-                     void* out, Timer* tm) {
+void residual_rows(ms_plan* p, PartDev& pd, const void* obs, const int32_t* obs_idx,
+                   const void* model, void* out, Timer* tm) {
   image_to_grid<R>(p, model, tm);
-  degrid_sorted<R>(p, pd, obs_sorted, p->vis_b, tm);
+  degrid_rows<R>(p, pd, obs, obs_idx, p->vis_b, nullptr, tm);
   grid_sorted<R>(p, pd, p->vis_b, out, tm);
 }
 
@@ -736,7 +760,7 @@ template <typename R> void psf_image(ms_plan* p, PartDev& pd, void* out) {
   ck(cudaMemsetAsync(delta, 0, sizeof(R) * N * N, p->ps), "memset");
   impulse_kernel<<<1, 1, 0, p->ps>>>(delta, N, sizeof(R) == 8);
   image_to_grid<R>(p, delta, nullptr);
-  degrid_sorted<R>(p, pd, nullptr, p->vis_b, nullptr);
+  degrid_rows<R>(p, pd, nullptr, nullptr, p->vis_b, nullptr, nullptr);
   grid_sorted<R>(p, pd, p->vis_b, out, nullptr);
 }
 
@@ -1271,7 +1295,7 @@ void run_step(ms_plan* p, int step, int chan, const ms_recon_opts& o, const void
   const double coef = step == MS_STEP_LOW ? o.lambda_low
                       : step == MS_STEP_FULL ? o.lambda_full : o.lambda_single;
   for (int n = 1; n <= o.n_major; ++n) {
-    residual_sorted<R>(p, pd, p->vis_a, model, res, &tm);
+    residual_rows<R>(p, pd, p->vis_a, nullptr, model, res, &tm);
     launch_image_norms<R>(res, n2, p->parts, p->ctl, p->tickets + 5, p->ps);
     if (n == 1) {
       init_ctl_kernel<<<1, 1, 0, p->ps>>>(p->ctl, o.fista_iters, o.rel_tol, 0.0, 0,
@@ -1312,7 +1336,7 @@ void run_step(ms_plan* p, int step, int chan, const ms_recon_opts& o, const void
       st->gridded_vis += pd.n;
     }
   }
-  residual_sorted<R>(p, pd, p->vis_a, model, res, &tm);   // i~_{N+1}
+  residual_rows<R>(p, pd, p->vis_a, nullptr, model, res, &tm);   // i~_{N+1}
   if (st) st->gridded_vis += pd.n;
   launch_axpby<R>(res, model, (R*)image_out, 1.0, 1.0, n2, p->ps);
   fill_stats<R>(p, st, true);
@@ -2007,14 +2031,12 @@ void degrid_batch(ms_plan* p, int njobs, const int32_t* chans, const int32_t* pa
   batch_reserve<R>(p, sh);
   batch_upload<R>(p, sh, jobs);
   const BatchJob<R>* jd = (const BatchJob<R>*)p->batch.jobs;
-  if (vis_obs) launch_batch_gather<R>(jd, njobs, sh.max_n, p->ps);
+  const bool gather = vis_obs && !rows_apart<R>(p, njobs, vis_obs, vis_out);
+  if (gather) launch_batch_gather<R>(jd, njobs, sh.max_n, p->ps);
   batch_fft<R>(p, jd, njobs, true);
-  {
-    KSpan k(p, MS_K_DEGRID);
-    launch_degrid_batch<R>(&p->batch.tmap, jd, p->batch.job_of, (int)sh.items, vis_obs != nullptr,
-                           p->Ng, p->T, p->ntx, p->es, p->err, p->ps);
-  }
-  launch_batch_scatter<R>(jd, njobs, sh.max_n, p->ps);
+  KSpan k(p, MS_K_DEGRID);
+  launch_degrid_batch<R>(&p->batch.tmap, jd, p->batch.job_of, (int)sh.items, vis_obs != nullptr,
+                         gather, true, p->Ng, p->T, p->ntx, p->es, p->err, p->ps);
 }
 
 // ------------------------------------------------- batched minor cycles
@@ -2276,12 +2298,11 @@ void residual_batch(ms_plan* p, int njobs, const int32_t* chans, const int32_t* 
   batch_reserve<R>(p, sh);
   batch_upload<R>(p, sh, jobs);
   const BatchJob<R>* jd = (const BatchJob<R>*)p->batch.jobs;
-  launch_batch_gather<R>(jd, njobs, sh.max_n, p->ps);
   batch_fft<R>(p, jd, njobs, true);
   {
     KSpan k(p, MS_K_DEGRID);
-    launch_degrid_batch<R>(&p->batch.tmap, jd, p->batch.job_of, (int)sh.items, true, p->Ng,
-                           p->T, p->ntx, p->es, p->err, p->ps);
+    launch_degrid_batch<R>(&p->batch.tmap, jd, p->batch.job_of, (int)sh.items, true, false, false,
+                           p->Ng, p->T, p->ntx, p->es, p->err, p->ps);
   }
   // grid the residual rows obs - A x where the degridding left them
   for (auto& b : jobs) std::swap(b.sorted_in, b.sorted_out);
@@ -2420,8 +2441,7 @@ void interleaved_seq(ms_plan* p, int chan, const void* vis, const ms_recon_opts*
   auto residuals = [&]() {
     for (int j = 0; j < 2; ++j) {
       PartDev& pd = part_of(p, parts[j], chan);
-      launch_gather_vis<R>(pd.idx, pd.n, (const C2<R>*)vis, (C2<R>*)p->vis_a, p->ps);
-      residual_sorted<R>(p, pd, p->vis_a, model + j * n2, res + j * n2, nullptr);
+      residual_rows<R>(p, pd, vis, pd.idx, model + j * n2, res + j * n2, nullptr);
     }
   };
   for (int n = 1; n <= o->n_major; ++n) {
@@ -2861,11 +2881,15 @@ ms_status ms_degrid(ms_plan* p, int32_t part, int32_t chan, const void* image,
     arg(image && vis_out, "image and vis_out are required");
     Scope sc(p, stream);
     DISPATCH(p, {
-      if (vis_obs)
+      const void* obs = vis_obs;
+      const int32_t* obs_idx = pd.idx;
+      if (vis_obs && !rows_apart<R>(p, 1, &vis_obs, &vis_out)) {
         launch_gather_vis<R>(pd.idx, pd.n, (const C2<R>*)vis_obs, (C2<R>*)p->vis_a, p->ps);
+        obs = p->vis_a;
+        obs_idx = nullptr;
+      }
       image_to_grid<R>(p, image, nullptr);
-      degrid_sorted<R>(p, pd, vis_obs ? p->vis_a : nullptr, p->vis_b, nullptr);
-      launch_scatter_vis<R>(pd.idx, pd.n, (const C2<R>*)p->vis_b, (C2<R>*)vis_out, p->ps);
+      degrid_rows<R>(p, pd, obs, obs_idx, vis_out, pd.idx, nullptr);
     });
     check_device_error(p);
     sc.finish();
@@ -2893,8 +2917,7 @@ ms_status ms_residual_image(ms_plan* p, int32_t part, int32_t chan, const void* 
     arg(vis_obs && model && out, "vis_obs, model and out are required");
     Scope sc(p, stream);
     DISPATCH(p, {
-      launch_gather_vis<R>(pd.idx, pd.n, (const C2<R>*)vis_obs, (C2<R>*)p->vis_a, p->ps);
-      residual_sorted<R>(p, pd, p->vis_a, model, out, nullptr);
+      residual_rows<R>(p, pd, vis_obs, pd.idx, model, out, nullptr);
     });
     check_device_error(p);
     sc.finish();

@@ -16,7 +16,7 @@
 // + Ng / 2) cost no pass of their own.  A complex transform of the whole grid (2-D cuFFT between a padding
 // and a cropping pass) moves 4 to 9 times the bytes.  Measured, both
 // directions (own | cuFFT with the passes): N = 128 FP64 23 | 75 us, N = 1024
-// FP32 53 | 91, 16 grids of it 485 | 1166, N = 4096 862 | 1290.
+// FP32 42 | 91, 16 grids of it 395 | 1166, N = 4096 697 | 1290.
 //
 // A sequence of 2^LOGN elements is held by 2^(LOGN - LE) threads, 2^LE
 // elements each, through Stockham stages of radix up to 2^LE: inputs of the
@@ -51,10 +51,22 @@ __device__ __forceinline__ void run_stages(C2<R> (&v)[1 << LE], C2<R>* buf,
     for (int r = 0; r < Rd; ++r) w[r] = v[q * Rd + r];
     if (NS > 1) {
       const int unit = js * (N / (NS * Rd)) * tw_step;
+      // W^r: the powers of two from the table, the others products of two
+      // smaller ones (a gather of 15 entries took longer than the butterfly:
+      // N = 4096 row transforms 166 -> 117 and 124 -> 80 us)
+      C2<R> pw[Rd];
 #pragma unroll
       for (int r = 1; r < Rd; ++r) {
-        C2<R> z = tw[r * unit];
-        if (INV) z.y = -z.y;
+        const int top = r >= 8 ? 8 : (r >= 4 ? 4 : (r >= 2 ? 2 : 1));
+        if (r == top) {
+          pw[r] = tw[r * unit];
+          if (INV) pw[r].y = -pw[r].y;
+        } else {
+          const C2<R> x = pw[top], y = pw[r - top];
+          pw[r].x = x.x * y.x - x.y * y.y;
+          pw[r].y = x.x * y.y + x.y * y.x;
+        }
+        const C2<R> z = pw[r];
         const C2<R> x = w[r];
         w[r].x = x.x * z.x - x.y * z.y;
         w[r].y = x.x * z.y + x.y * z.x;

@@ -325,23 +325,9 @@ __global__ void gather_vis_kernel(const int32_t* __restrict__ idx, int64_t n,
 }
 
 template <typename R>
-__global__ void scatter_vis_kernel(const int32_t* __restrict__ idx, int64_t n,
-                                   const C2<R>* __restrict__ src, C2<R>* __restrict__ dst) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-       k += (int64_t)gridDim.x * blockDim.x)
-    dst[idx[k]] = src[k];
-}
-
-template <typename R>
 void launch_gather_vis(const int32_t* idx, int64_t n, const C2<R>* src, C2<R>* dst,
                        cudaStream_t s) {
   if (n > 0) gather_vis_kernel<R><<<grid_for(n, 256), 256, 0, s>>>(idx, n, src, dst);
-}
-
-template <typename R>
-void launch_scatter_vis(const int32_t* idx, int64_t n, const C2<R>* src, C2<R>* dst,
-                        cudaStream_t s) {
-  if (n > 0) scatter_vis_kernel<R><<<grid_for(n, 256), 256, 0, s>>>(idx, n, src, dst);
 }
 
 // psi(a) = int phi(t) cos(2 pi a t / Ng) dt over |t| <= W/2.  With
@@ -379,9 +365,5 @@ template void launch_gather_vis<float>(const int32_t*, int64_t, const float2*, f
                                        cudaStream_t);
 template void launch_gather_vis<double>(const int32_t*, int64_t, const double2*, double2*,
                                         cudaStream_t);
-template void launch_scatter_vis<float>(const int32_t*, int64_t, const float2*, float2*,
-                                        cudaStream_t);
-template void launch_scatter_vis<double>(const int32_t*, int64_t, const double2*, double2*,
-                                         cudaStream_t);
 
 }  // namespace ms
