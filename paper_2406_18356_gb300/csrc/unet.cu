@@ -19,8 +19,8 @@
 // and stored activations (after ReLU, after pooling) are rounded to bfloat16,
 // and so is every pre-activation gradient before it enters a product.
 //
-// Measured (6 levels, width 6): forward pass at 1024 x 1024 481 us, forward
-// and backward pass with the gradients at 512 x 512 982 us; before, with the
+// Measured (6 levels, width 6): forward pass at 1024 x 1024 418 us, forward
+// and backward pass with the gradients at 512 x 512 866 us; before, with the
 // windows written out (im2col, 9 times the activations, and a transposed copy
 // for the weight gradients) and one general product kernel: 4166 and 5449 us.
 #include <cuda_bf16.h>
@@ -29,6 +29,7 @@
 #include <cmath>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -108,30 +109,46 @@ int act_vec(const Act& x) {
   return g % 8 == 0 ? 8 : (g % 2 == 0 ? 2 : 1);
 }
 
-// Stages channels [c0, c0 + n) (at most xc) of the (rows x cols) pixels from
-// (y0, x0) on (rows and columns outside the image, and channels past xc:
-// zero) into dst [rows cols][stride], nst >= n values of each pixel written.
-// VEC as act_vec (n, nst and c0 multiples of it).  The copies of VEC > 1 are
-// asynchronous (the caller commits and waits).
-template <int VEC, class At>
+// Stages channels [c0, c0 + n) of the (rows x cols) pixels from (y0, x0) on
+// into dst [rows cols][stride], nst >= n values of each pixel written (zeros
+// for rows and columns outside the image, and from n on).  VEC as act_vec (n,
+// nst and c0 multiples of it).  The copies of VEC > 1 are asynchronous (the
+// caller commits and waits).  A thread keeps its column and channels and goes
+// down the rows, so the quotients and the choice of the source are taken once
+// and a copy costs an add and a compare (element by element the index
+// arithmetic took more instructions than the products: forward pass at
+// 1024 px 481 -> 418 us with the other changes beside it, dw_kernel at 512 px
+// 207 -> 136 with them).
+template <int VEC>
 __device__ __forceinline__ void stage_pixels(bf16* dst, int stride, int rows, int cols, int y0,
                                              int x0, int H, int W, int c0, int n, int nst,
-                                             const At& at, const bf16* any) {
-  const int nv = nst / VEC;
-  const float inv_nv = 1.0f / (float)nv, inv_cols = 1.0f / (float)cols;
-  for (int e = threadIdx.x; e < rows * cols * nv; e += blockDim.x) {
-    // exact quotients (e < 2^22, see div_small of the wavelet kernels)
-    const int pix = (int)(((float)e + 0.5f) * inv_nv), v = (e - pix * nv) * VEC;
-    const int py = (int)(((float)pix + 0.5f) * inv_cols), px = pix - py * cols;
-    const int y = y0 + py, x = x0 + px;
-    const bool ok = y >= 0 && y < H && x >= 0 && x < W && v < n;
-    bf16* d = dst + pix * stride + v;
-    if constexpr (VEC == 8) {
-      cpz<16>(d, ok ? at(y, x, c0 + v) : any, ok);
-    } else if constexpr (VEC == 2) {
-      cpz<4>(d, ok ? at(y, x, c0 + v) : any, ok);
+                                             const Act& src) {
+  const int nv = nst / VEC, len = cols * nv, nt = blockDim.x;
+  // rows side by side where one takes fewer copies than there are threads
+  const int par = len < nt ? nt / len : 1;
+  const int r0 = len < nt ? (int)threadIdx.x / len : 0;
+  if (r0 >= par) return;
+  for (int e = threadIdx.x - r0 * len; e < len; e += nt) {
+    const int px = e / nv, v = (e - px * nv) * VEC, x = x0 + px, c = c0 + v;
+    const bool okx = x >= 0 && x < W && v < n;
+    const bool up = src.cb != 0 && c < src.ca;
+    const bf16* g;
+    int64_t row;
+    if (src.cb == 0 || up) {
+      g = src.a + (int64_t)(up ? x >> 1 : x) * src.ca + c;
+      row = (int64_t)(up ? W >> 1 : W) * src.ca;
     } else {
-      *d = ok ? *at(y, x, c0 + v) : __float2bfloat16_rn(0.0f);
+      g = src.b + (int64_t)x * src.cb + (c - src.ca);
+      row = (int64_t)W * src.cb;
+    }
+    bf16* d = dst + (r0 * cols + px) * stride + v;
+    for (int r = r0; r < rows; r += par, d += par * cols * stride) {
+      const int y = y0 + r;
+      const bool ok = okx && y >= 0 && y < H;
+      const bf16* q = ok ? g + (up ? y >> 1 : y) * row : src.a;
+      if constexpr (VEC == 8) cpz<16>(d, q, ok);
+      else if constexpr (VEC == 2) cpz<4>(d, q, ok);
+      else *d = ok ? *q : __float2bfloat16_rn(0.0f);
     }
   }
 }
@@ -204,8 +221,7 @@ __global__ void __launch_bounds__(128) conv_kernel(const ConvArgs p) {
   for (int c0 = 0; c0 < p.ci; c0 += p.ck) {
     const int ck = min(p.ck, p.ci - c0), kl = pad16(9 * ck);
     if (c0) __syncthreads();
-    const auto at = [&](int y, int x, int c) { return act_at(p.x, p.W, y, x, c); };
-    stage_pixels<VEC>(sx, CS, TL::R, TL::R, y0 - 1, x0 - 1, p.H, p.W, c0, ck, ck, at, p.x.a);
+    stage_pixels<VEC>(sx, CS, TL::R, TL::R, y0 - 1, x0 - 1, p.H, p.W, c0, ck, ck, p.x);
     if (ck == p.ci) {   // whole packed rows (kl = kp, a multiple of 16)
       const int nv = kl / 8;
       const float inv = 1.0f / (float)nv;
@@ -245,7 +261,9 @@ __global__ void __launch_bounds__(128) conv_kernel(const ConvArgs p) {
     const unsigned zero_a = sx_a + 2u * zero_off;
     // B rows: matrix lane / 8 = (n8 tile of the pair, k half)
     const unsigned b_a = sw_a + 2u * (((lane >> 4) * 8 + (lane & 7)) * KS + ((lane >> 3) & 1) * 8);
-    for (int k0 = 0; k0 < kl; k0 += 16) {
+    // one k step; PAD: it may hold k >= 9 ck
+    const auto k_step = [&](int k0, auto last) {
+      constexpr bool PAD = decltype(last)::value;
       unsigned b[NT][2];
 #pragma unroll
       for (int j = 0; j + 1 < NT; j += 2) {
@@ -264,7 +282,7 @@ __global__ void __launch_bounds__(128) conv_kernel(const ConvArgs p) {
 #pragma unroll
         for (int i = 0; i < MT; ++i) {
           unsigned a[4];
-          ldsm4(a, ko >= 0 ? sx_a + 2u * (base[i] + ko) : zero_a);
+          ldsm4(a, !PAD || ko >= 0 ? sx_a + 2u * (base[i] + ko) : zero_a);
 #pragma unroll
           for (int j = 0; j < NT; ++j) mma16816(acc[i][j], a, b[j][0], b[j][1]);
         }
@@ -274,10 +292,10 @@ __global__ void __launch_bounds__(128) conv_kernel(const ConvArgs p) {
 #pragma unroll
         for (int i = 0; i < MT; ++i) {
           unsigned a[4];
-          const bf16* q = sx + (k_lo >= 0 ? base[i] + k_lo : zero_off);
-          const bf16* q1 = sx + (k_lo >= 0 ? base[i] + dy + k_lo : zero_off);
-          const bf16* h = sx + (k_hi >= 0 ? base[i] + k_hi : zero_off);
-          const bf16* h1 = sx + (k_hi >= 0 ? base[i] + dy + k_hi : zero_off);
+          const bf16* q = sx + (!PAD || k_lo >= 0 ? base[i] + k_lo : zero_off);
+          const bf16* q1 = sx + (!PAD || k_lo >= 0 ? base[i] + dy + k_lo : zero_off);
+          const bf16* h = sx + (!PAD || k_hi >= 0 ? base[i] + k_hi : zero_off);
+          const bf16* h1 = sx + (!PAD || k_hi >= 0 ? base[i] + dy + k_hi : zero_off);
           a[0] = *reinterpret_cast<const unsigned*>(q);
           a[1] = *reinterpret_cast<const unsigned*>(q1);
           a[2] = *reinterpret_cast<const unsigned*>(h);
@@ -297,16 +315,18 @@ __global__ void __launch_bounds__(128) conv_kernel(const ConvArgs p) {
             const int row = base[i] + (f & 1) * TL::R * CS;
             const int e0 = ko[2 * (f >> 1)], e1 = ko[2 * (f >> 1) + 1];
             const unsigned short l0 =
-                *reinterpret_cast<const unsigned short*>(sx + (e0 >= 0 ? row + e0 : zero_off));
+                *reinterpret_cast<const unsigned short*>(sx + (!PAD || e0 >= 0 ? row + e0 : zero_off));
             const unsigned short l1 =
-                *reinterpret_cast<const unsigned short*>(sx + (e1 >= 0 ? row + e1 : zero_off));
+                *reinterpret_cast<const unsigned short*>(sx + (!PAD || e1 >= 0 ? row + e1 : zero_off));
             a[f] = (unsigned)l0 | ((unsigned)l1 << 16);
           }
 #pragma unroll
           for (int j = 0; j < NT; ++j) mma16816(acc[i][j], a, b[j][0], b[j][1]);
         }
       }
-    }
+    };
+    for (int k0 = 0; k0 < kl - 16; k0 += 16) k_step(k0, std::false_type());
+    k_step(kl - 16, std::true_type());
   }
 
   // acc[.][.][q]: pixel row q / 2 of the m-tile's two, column gid, channel
@@ -419,8 +439,8 @@ __global__ void __launch_bounds__(BIG ? 256 : 128) dx_kernel(const DxArgs p) {
   for (int c0 = 0; c0 < p.co; c0 += p.ck) {
     const int ck = min(p.ck, p.co - c0), kl = pad16(ck);
     if (c0) __syncthreads();
-    const auto at = [&](int y, int x, int c) { return p.dz + ((int64_t)y * p.W + x) * p.co + c; };
-    stage_pixels<VEC>(sz, KS, TL::R, TL::R, y0 - 1, x0 - 1, p.H, p.W, c0, ck, kl, at, p.dz);
+    stage_pixels<VEC>(sz, KS, TL::R, TL::R, y0 - 1, x0 - 1, p.H, p.W, c0, ck, kl,
+                      Act{p.dz, nullptr, p.co, 0});
     const int nv = kl / 8;
     const float inv = 1.0f / (float)nv;
     for (int e = tid; e < 9 * NT * 8 * nv; e += NW * 32) {
@@ -537,6 +557,8 @@ __global__ void __launch_bounds__(BIG ? 256 : 128) dx_kernel(const DxArgs p) {
 // taps: the same staged pixels serve them) and a range of 8 x 16 pixel tiles,
 // whose four warps take 32 pixels of each tile.  The pixel sums of a block go to its slice of
 // the partial sums; sum_partials_kernel adds a layer's slices in order.
+// The sums' exchange shares the staging buffers, so four blocks fit an SM
+// (registers; three before, 33 KB of shared memory each).
 // A unit of 8 input channels (rather than more) leaves enough units at the
 // coarse levels, where a layer has 256 pixels and up to 192 x 1728 weights.
 constexpr int kMaxConvs = 24;   // 4 levels - 1 at most 6 levels
@@ -564,21 +586,26 @@ constexpr int kWZS = 24;                              // row stride of a staged 
 
 template <int VEC>
 __device__ __forceinline__ void w_stage_x(bf16* dst, const WLayer& l, int y0, int x0, int c0) {
-  const auto at = [&](int y, int x, int c) { return act_at(l.x, l.W, y, x, c); };
   stage_pixels<VEC>(dst, 8, kWTileY + 2, kWTileX + 2, y0 - 1, x0 - 1, l.H, l.W, c0,
-                    min(8, l.ci - c0), 8, at, l.x.a);
+                    min(8, l.ci - c0), 8, l.x);
 }
 template <int VEC>
 __device__ __forceinline__ void w_stage_z(bf16* dst, const WLayer& l, int y0, int x0, int c0) {
-  const auto at = [&](int y, int x, int c) { return l.dz + ((int64_t)y * l.W + x) * l.co + c; };
-  stage_pixels<VEC>(dst, kWZS, kWTileY, kWTileX, y0, x0, l.H, l.W, c0, min(16, l.co - c0), 16, at,
-                    l.dz);
+  stage_pixels<VEC>(dst, kWZS, kWTileY, kWTileX, y0, x0, l.H, l.W, c0, min(16, l.co - c0), 16,
+                    Act{l.dz, nullptr, l.co, 0});
 }
 
-__global__ void __launch_bounds__(128) dw_kernel(const __grid_constant__ WArgs p) {
-  __shared__ __align__(16) bf16 sx[2][kWXP * 8];
-  __shared__ __align__(16) bf16 sz[2][kWTileY * kWTileX * kWZS];
-  __shared__ float red[3][10][32][4];
+__global__ void __launch_bounds__(128, 4) dw_kernel(const __grid_constant__ WArgs p) {
+  struct Stage {
+    bf16 x[2][kWXP * 8], z[2][kWTileY * kWTileX * kWZS];
+  };
+  __shared__ __align__(16) union {
+    Stage st;
+    float red[3][10][32][4];   // the warps' sums, once the tiles are done
+  } sm;
+  auto& sx = sm.st.x;
+  auto& sz = sm.st.z;
+  auto& red = sm.red;
   int li = 0;
   while (li + 1 < p.n && (int)blockIdx.x >= p.l[li + 1].first) ++li;
   const WLayer& l = p.l[li];
@@ -676,7 +703,8 @@ __global__ void sum_partials_kernel(const __grid_constant__ WArgs p) {
     const int64_t n = (int64_t)l.co * (9 * l.ci + 1);
     const float* q = p.parts + l.part + (e - l.woff);
     float a = 0.0f;
-    for (int s = 0; s < l.splits; ++s) a += q[s * n];
+#pragma unroll 16
+    for (int s = 0; s < l.splits; ++s) a += q[s * n];   // (loads ahead of the sum)
     p.grad[e] = a;
   }
 }
@@ -698,15 +726,26 @@ struct PackLayer {
 struct PackArgs {
   PackLayer l[kMaxConvs];
 };
-__global__ void pack_weights_kernel(const __grid_constant__ PackArgs p) {
+__global__ void __launch_bounds__(kT) pack_weights_kernel(const __grid_constant__ PackArgs p) {
+  // 32 x 32 tiles, turned in shared memory: both copies are written by rows
+  __shared__ bf16 t[32][33];
   const PackLayer& l = p.l[blockIdx.y];
-  const int64_t total = (int64_t)l.kp * l.cop;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int co = (int)(e / l.kp), k = (int)(e - (int64_t)co * l.kp);
-    const bf16 v = __float2bfloat16_rn(co < l.co && k < l.k9 ? l.w[(int64_t)co * l.k9 + k] : 0.0f);
-    if (co < l.co) l.wb[e] = v;
-    if (k < l.k9) l.wt[(int64_t)k * l.cop + co] = v;
+  const int tk = (l.kp + 31) / 32, tiles = tk * ((l.cop + 31) / 32);
+  const int lx = threadIdx.x & 31, ly = threadIdx.x >> 5;
+  for (int i = blockIdx.x; i < tiles; i += gridDim.x) {
+    const int co0 = i / tk * 32, k0 = i % tk * 32;
+    __syncthreads();
+    for (int r = ly; r < 32; r += kT / 32) {
+      const int co = co0 + r, k = k0 + lx;
+      const bf16 v = __float2bfloat16_rn(co < l.co && k < l.k9 ? l.w[(int64_t)co * l.k9 + k] : 0.0f);
+      if (co < l.co && k < l.kp) l.wb[(int64_t)co * l.kp + k] = v;
+      t[r][lx] = v;
+    }
+    __syncthreads();
+    for (int r = ly; r < 32; r += kT / 32) {
+      const int co = co0 + lx, k = k0 + r;
+      if (k < l.k9 && co < l.cop) l.wt[(int64_t)k * l.cop + co] = t[lx][r];
+    }
   }
 }
 
@@ -845,8 +884,9 @@ constexpr size_t kSmemBig = 110 * 1024;
 // Tile side, n8 tiles per block and channels staged at a time of one layer
 // (n output channels of the product, c channels staged, smem(big, ck, nt)).
 // 16 x 16 pixels where two waves of them fill the SMs, else 8 x 8; then the
-// most n8 tiles (fewest re-reads of the pixels) that divide the layer's and
-// leave a block per SM.
+// most n8 tiles (fewest re-reads of the pixels) that divide the layer's, leave
+// a block per SM and whose weights fit beside the pixels (288 -> 96 channels at
+// 64 px: 3 n8 tiles a block 34.9 us, one 41).
 struct Shape {
   bool big;
   int nt, ck;
@@ -855,17 +895,15 @@ template <class F> Shape pick_shape(int H, int W, int n, int c, F smem) {
   const int n8 = (n + 7) / 8;
   const int64_t tb = (int64_t)((H + 15) / 16) * ((W + 15) / 16);
   const int64_t ts = (int64_t)((H + 7) / 8) * ((W + 7) / 8);
-  auto nt_for = [&](int64_t tiles) {
+  auto nt_for = [&](bool big, int64_t tiles, size_t limit) {
     for (int nt : {4, 3, 2})
-      if (n8 % nt == 0 && tiles * (n8 / nt) >= sm_count()) return nt;
+      if (n8 % nt == 0 && tiles * (n8 / nt) >= sm_count() && smem(big, c, nt) <= limit) return nt;
     return 1;
   };
-  Shape s{true, nt_for(tb), c};
+  Shape s{true, nt_for(true, tb, kSmemBig), c};
   if (tb * (n8 / s.nt) >= 2 * sm_count() && smem(true, c, s.nt) <= kSmemBig) return s;
-  s = Shape{false, nt_for(ts), c};
+  s = Shape{false, nt_for(false, ts, kSmemMax), c};
   if (smem(false, c, s.nt) <= kSmemMax) return s;
-  s.nt = 1;
-  s.ck = c;
   while (smem(false, s.ck, 1) > kSmemMax) s.ck = (s.ck - 1) / 16 * 16;   // (16 channels fit)
   return s;
 }
@@ -977,9 +1015,10 @@ void pack(ms_unet* u, cudaStream_t s) {
   for (size_t i = 0; i < u->L.size(); ++i) {
     const Layer& l = u->L[i];
     p.l[i] = PackLayer{u->master + l.woff, l.co, 9 * l.ci, l.kp, l.cop, l.Wb, l.Wt};
-    most = std::max(most, (int64_t)l.kp * l.cop);
+    most = std::max(most, (int64_t)((l.kp + 31) / 32) * ((l.cop + 31) / 32));
   }
-  pack_weights_kernel<<<dim3(blocks(most, 512), (unsigned)u->L.size()), kT, 0, s>>>(p);
+  pack_weights_kernel<<<dim3((unsigned)std::min<int64_t>(most, 1024), (unsigned)u->L.size()), kT,
+                        0, s>>>(p);
 }
 
 // out = net(in) [H][W] (FP32)
