@@ -243,6 +243,8 @@ void launch_count_tiles(const uint32_t* keys, int64_t n, int shift, int32_t* cou
 void launch_exclusive_scan(const int32_t* in, int32_t* out, int n, cudaStream_t s);
 void launch_chunks_per_tile(const int32_t* counts, int ntiles, int chunk, int32_t* nchunks,
                             cudaStream_t s);
+// *most = max(in[0..n))
+void launch_max(const int32_t* in, int n, int32_t* most, cudaStream_t s);
 void launch_make_items(const int32_t* counts, const int32_t* tile_start,
                        const int32_t* item_start, int ntiles, int chunk, WorkItem* items,
                        cudaStream_t s);
@@ -273,10 +275,12 @@ template <typename R, bool KAHAN>
 void launch_grid(const WorkItem* items, int nitems, const uint32_t* cell, const C2<R>* frac,
                  const C2<R>* vis, void* scratch, int Ng, int tile, int ntx, const EsKernel& es,
                  cudaStream_t s);
-// (ext: cells within +-ext of the origin only, Ng / 2 = all)
+// ext: cells within +-ext of the origin only (Ng / 2 = all); longest: the most
+// items of one tile (some of the tiles in scratch are summed in place)
 template <typename R, bool KAHAN>
-void launch_fold(const void* scratch, const int32_t* tile_items, int Ng, int tile, int ntx, int ext,
-                 C2<R>* grid, cudaStream_t s);
+void launch_fold(void* scratch, const WorkItem* items, int nitems, int longest,
+                 const int32_t* tile_items, int Ng, int tile, int ntx, int ext, C2<R>* grid,
+                 cudaStream_t s);
 size_t grid_scratch_cell_bytes(int precision);
 // batched form (all launches take the device job table)
 template <typename R>
@@ -288,8 +292,9 @@ template <typename R, bool KAHAN>
 void launch_grid_batch(const BatchJob<R>* jobs, const int32_t* job_of, int total_items,
                        void* scratch, int tile, int ntx, const EsKernel& es, cudaStream_t s);
 template <typename R, bool KAHAN>
-void launch_fold_batch(const BatchJob<R>* jobs, int njobs, const void* scratch, int Ng,
-                       int tile, int ntx, int ext, cudaStream_t s);
+void launch_fold_batch(const BatchJob<R>* jobs, int njobs, const int32_t* job_of, int total_items,
+                       int longest, void* scratch, int Ng, int tile, int ntx, int ext,
+                       cudaStream_t s);
 // observed values from user_in, or (gathered) sorted_in; results to user_out
 // (user_order) or sorted_out
 template <typename R>

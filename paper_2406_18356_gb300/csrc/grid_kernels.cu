@@ -11,6 +11,7 @@ namespace ms {
 
 namespace {
 constexpr int kThreads = 256;
+constexpr int kFoldThreads = 128;
 
 __device__ __forceinline__ unsigned smem_addr(const void* p) {
   return (unsigned)__cvta_generic_to_shared(p);
@@ -921,75 +922,144 @@ void launch_grid(const WorkItem* items, int nitems, const uint32_t* cell, const 
 // order, the scratch tiles of all work items of the (up to four) tiles whose
 // footprint region covers it: its own tile and, within W - 1 cells of a tile
 // edge, the tiles to the left and above (periodically).  Each cell is written
-// once, so the grid needs no clearing.  A thread per cell, a block per 256
-// cells of a row (a row of cells shares its tile row, so the branch on it is
-// uniform); a cell's items are read 16 (8) or 4 at a time (independent loads
-// in flight) and added in item order.  Bound by the latency of the tile and
-// scratch loads: the densest tile of a 9.27M-row observation has hundreds of
-// work items.
-template <typename R, bool KAHAN>
-__device__ __forceinline__ void fold_cell(const typename ScratchOf<R, KAHAN>::T* __restrict__ scratch,
-                                          const int32_t* __restrict__ tile_items, int Ng, int T,
-                                          int ntx, int first, int side, C2<R>* __restrict__ grid) {
+// once, so the grid needs no clearing.  Bound by the latency of its dependent
+// loads (a tile's items, then their cells), so a thread takes Q = 4 cells of a
+// row (they share both; one cell each where the grid is too small to occupy
+// the SMs that way: 128 px 32 | 13 us), reads the four tiles' item ranges
+// together and several items at a time; and where a tile has more than kFoldList items
+// (dense cores: hundreds) groups of kFoldGroup are first added up in parallel
+// into their first item's tile (fold_groups_kernel), so that no cell's chain
+// is long.  Measured (before | now): 1024 px, 9.27M rows 57 | 32 us;
+// 16 jobs at 1024 px 224 | 118; 4096 px, compensated 297 | 140.
+constexpr int kFoldList = 32, kFoldGroup = 16;
+
+// Q consecutive scratch cells (Q = 4: an even offset, 16-byte aligned)
+__device__ __forceinline__ void load_cells(const float2* p, float2 (&a)[4]) {
+  const float4 x = *reinterpret_cast<const float4*>(p), y = *reinterpret_cast<const float4*>(p + 2);
+  a[0] = make_float2(x.x, x.y);
+  a[1] = make_float2(x.z, x.w);
+  a[2] = make_float2(y.x, y.y);
+  a[3] = make_float2(y.z, y.w);
+}
+template <typename A, int Q> __device__ __forceinline__ void load_cells(const A* p, A (&a)[Q]) {
+#pragma unroll
+  for (int q = 0; q < Q; ++q) a[q] = p[q];
+}
+
+// scratch: the job's first item's tile; item i of the job's tile_items
+template <typename R, bool KAHAN, int Q>
+__device__ __forceinline__ void fold_cells(const typename ScratchOf<R, KAHAN>::T* __restrict__ scratch,
+                                           const int32_t* __restrict__ tile_items, int Ng, int T,
+                                           int ntx, int first, int side, C2<R>* __restrict__ grid) {
   using Acc = typename ScratchOf<R, KAHAN>::T;
+  constexpr int U = (sizeof(Acc) == 8 ? 16 : 8) / Q;   // items in flight
   const int S = T + kW - 1;
   const int cells = S * S;
   const int lt = __ffs(T) - 1;   // T is a power of two
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= side) return;
-  const int cu = first + x, cv = first + blockIdx.y;
+  const int x = Q * (blockIdx.x * blockDim.x + threadIdx.x);
+  if (x >= side + (first & (Q - 1))) return;
+  const int cu = (first & ~(Q - 1)) + x, cv = first + blockIdx.y;
   const int tx = cu >> lt, ty = cv >> lt, ou = cu & (T - 1), ov = cv & (T - 1);
-  constexpr int U = sizeof(Acc) == 8 ? 16 : 8;   // loads in flight of a long item list
-  Acc sum{};
+  int lo[4], hi[4];
 #pragma unroll
-  for (int dy = 0; dy < 2; ++dy) {
-    if (dy && ov >= kW - 1) break;
+  for (int q = 0; q < 4; ++q) {
+    const int dy = q >> 1, dx = q & 1;
+    lo[q] = hi[q] = 0;
+    if ((dy && ov >= kW - 1) || (dx && ou >= kW - 1)) continue;
+    int stx = tx - dx, sty = ty - dy;
+    stx += stx < 0 ? ntx : 0;
+    sty += sty < 0 ? ntx : 0;
+    lo[q] = tile_items[sty * ntx + stx];
+    hi[q] = tile_items[sty * ntx + stx + 1];
+  }
+  Acc sum[Q] = {};
 #pragma unroll
-    for (int dx = 0; dx < 2; ++dx) {
-      if (dx && ou >= kW - 1) break;
-      int stx = tx - dx, sty = ty - dy;
-      stx += stx < 0 ? ntx : 0;
-      sty += sty < 0 ? ntx : 0;
-      const int t = sty * ntx + stx;
-      const int off = (ov + dy * T) * S + (ou + dx * T);
-      const int e = tile_items[t + 1];
-      int i = tile_items[t];
-      for (; i + U <= e; i += U) {
-        Acc a[U];
+  for (int q = 0; q < 4; ++q) {
+    const int dy = q >> 1, dx = q & 1;
+    const Acc* base = scratch + (ov + dy * T) * S + (ou + dx * T);
+    // of the left tile only columns up to S - 1 (T + 6 cells) exist
+    const int live = dx ? min(Q, kW - 1 - ou) : Q;
+    const int step = hi[q] - lo[q] > kFoldList ? kFoldGroup : 1;
+    int i = lo[q];
+    if (live == Q) {
+      for (; i + (U - 1) * step < hi[q]; i += U * step) {
+        Acc a[U][Q];
 #pragma unroll
-        for (int u = 0; u < U; ++u) a[u] = scratch[(int64_t)(i + u) * cells + off];
+        for (int u = 0; u < U; ++u) load_cells(base + (int64_t)(i + u * step) * cells, a[u]);
 #pragma unroll
-        for (int u = 0; u < U; ++u) cell_sum(sum, a[u]);
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int c = 0; c < Q; ++c) cell_sum(sum[c], a[u][c]);
       }
-      for (; i + 4 <= e; i += 4) {
-        Acc a[4];
+    }
+    for (; i < hi[q]; i += step) {
+      const Acc* p = base + (int64_t)i * cells;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) a[u] = scratch[(int64_t)(i + u) * cells + off];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) cell_sum(sum, a[u]);
-      }
-      for (; i < e; ++i) cell_sum(sum, scratch[(int64_t)i * cells + off]);
+      for (int c = 0; c < Q; ++c)
+        if (c < live) cell_sum(sum[c], p[c]);
     }
   }
-  grid[(int64_t)cv * Ng + cu] = cell_value(sum);
+  C2<R>* g = grid + (int64_t)cv * Ng + cu;   // (Ng a multiple of 4: all exist)
+#pragma unroll
+  for (int c = 0; c < Q; ++c) g[c] = cell_value(sum[c]);
 }
 
-template <typename R, bool KAHAN>
-__global__ void fold_kernel(const typename ScratchOf<R, KAHAN>::T* __restrict__ scratch,
-                            const int32_t* __restrict__ tile_items, int Ng, int T, int ntx,
-                            int first, int side, C2<R>* __restrict__ grid) {
-  fold_cell<R, KAHAN>(scratch, tile_items, Ng, T, ntx, first, side, grid);
+template <typename R, bool KAHAN, int Q>
+__global__ void __launch_bounds__(kFoldThreads)
+    fold_kernel(const typename ScratchOf<R, KAHAN>::T* __restrict__ scratch,
+                const int32_t* __restrict__ tile_items, int Ng, int T, int ntx, int first,
+                int side, C2<R>* __restrict__ grid) {
+  fold_cells<R, KAHAN, Q>(scratch, tile_items, Ng, T, ntx, first, side, grid);
 }
 
 // stacked form: blockIdx.z = job (its tiles start at its first item)
-template <typename R, bool KAHAN>
-__global__ void fold_batch_kernel(const BatchJob<R>* __restrict__ jobs,
-                                  const typename ScratchOf<R, KAHAN>::T* __restrict__ scratch,
-                                  int Ng, int T, int ntx, int first, int side) {
+template <typename R, bool KAHAN, int Q>
+__global__ void __launch_bounds__(kFoldThreads)
+    fold_batch_kernel(const BatchJob<R>* __restrict__ jobs,
+                      const typename ScratchOf<R, KAHAN>::T* __restrict__ scratch, int Ng, int T,
+                      int ntx, int first, int side) {
   const BatchJob<R>& jb = jobs[blockIdx.z];
   const int S = T + kW - 1;
-  fold_cell<R, KAHAN>(scratch + jb.item_base * (int64_t)(S * S), jb.tile_items, Ng, T, ntx, first,
-                      side, jb.grid);
+  fold_cells<R, KAHAN, Q>(scratch + jb.item_base * (int64_t)(S * S), jb.tile_items, Ng, T, ntx, first,
+                       side, jb.grid);
+}
+
+// Work item `it` (index `item` of its job's), if it leads a group of a long
+// list: its tile becomes the group's sum, in item order.
+template <typename Acc>
+__device__ __forceinline__ void fold_group(Acc* scratch, const int32_t* tile_items,
+                                           const WorkItem& it, int item, int cells) {
+  const int lo = tile_items[it.tile], hi = tile_items[it.tile + 1];
+  if (hi - lo <= kFoldList || (item - lo) % kFoldGroup) return;
+  const int n = min(kFoldGroup, hi - item);
+  Acc* dst = scratch + (int64_t)item * cells;
+  for (int c = threadIdx.x; c < cells; c += blockDim.x) {
+    Acc a[kFoldGroup];
+#pragma unroll
+    for (int u = 0; u < kFoldGroup; ++u)
+      if (u < n) a[u] = dst[(int64_t)u * cells + c];
+    Acc s = a[0];
+#pragma unroll
+    for (int u = 1; u < kFoldGroup; ++u)
+      if (u < n) cell_sum(s, a[u]);
+    dst[c] = s;
+  }
+}
+template <typename R, bool KAHAN>
+__global__ void __launch_bounds__(128)
+    fold_groups_kernel(typename ScratchOf<R, KAHAN>::T* __restrict__ scratch,
+                       const WorkItem* __restrict__ items, const int32_t* __restrict__ tile_items,
+                       int cells) {
+  fold_group(scratch, tile_items, items[blockIdx.x], blockIdx.x, cells);
+}
+template <typename R, bool KAHAN>
+__global__ void __launch_bounds__(128)
+    fold_groups_batch_kernel(const BatchJob<R>* __restrict__ jobs,
+                             const int32_t* __restrict__ job_of,
+                             typename ScratchOf<R, KAHAN>::T* __restrict__ scratch, int cells) {
+  const BatchJob<R>& jb = jobs[job_of[blockIdx.x]];
+  const int item = (int)(blockIdx.x - jb.item_base);
+  fold_group(scratch + jb.item_base * cells, jb.tile_items, jb.items[item], item, cells);
 }
 
 namespace {
@@ -998,16 +1068,35 @@ void fold_region(int Ng, int ext, int* first, int* side) {
   *first = ext >= Ng / 2 ? 0 : Ng / 2 - ext;
   *side = ext >= Ng / 2 ? Ng : 2 * ext + 1;
 }
+// four cells a thread where that is still a thread for half of what the SMs
+// hold (1024 threads each), else one
+bool fold_quads(int side, int jobs) {
+  return (int64_t)side * side * jobs / 4 >= (int64_t)sm_count() * 1024;
+}
+dim3 fold_grid(int first, int side, int jobs, int Q) {
+  const int n = ((first & (Q - 1)) + side + Q - 1) / Q;
+  return dim3((n + kFoldThreads - 1) / kFoldThreads, side, jobs);
+}
 }  // namespace
 
 template <typename R, bool KAHAN>
-void launch_fold(const void* scratch, const int32_t* tile_items, int Ng, int tile, int ntx, int ext,
-                 C2<R>* grid, cudaStream_t s) {
+void launch_fold(void* scratch, const WorkItem* items, int nitems, int longest,
+                 const int32_t* tile_items, int Ng, int tile, int ntx, int ext, C2<R>* grid,
+                 cudaStream_t s) {
+  using Acc = typename ScratchOf<R, KAHAN>::T;
+  const int S = tile + kW - 1;
+  if (longest > kFoldList)
+    fold_groups_kernel<R, KAHAN><<<nitems, 128, 0, s>>>(static_cast<Acc*>(scratch), items,
+                                                        tile_items, S * S);
   int first, side;
   fold_region(Ng, ext, &first, &side);
-  fold_kernel<R, KAHAN><<<dim3((side + kThreads - 1) / kThreads, side), kThreads, 0, s>>>(
-      reinterpret_cast<const typename ScratchOf<R, KAHAN>::T*>(scratch), tile_items, Ng, tile,
-      ntx, first, side, grid);
+  const auto go = [&](auto* k, int Q) {
+    k<<<fold_grid(first, side, 1, Q), kFoldThreads, 0, s>>>(static_cast<const Acc*>(scratch),
+                                                            tile_items, Ng, tile, ntx, first, side,
+                                                            grid);
+  };
+  if (fold_quads(side, 1)) go(fold_kernel<R, KAHAN, 4>, 4);
+  else go(fold_kernel<R, KAHAN, 1>, 1);
 }
 
 // ---------------------------------------------------------------- instances
@@ -1101,14 +1190,22 @@ void launch_grid_batch(const BatchJob<R>* jobs, const int32_t* job_of, int total
 }
 
 template <typename R, bool KAHAN>
-void launch_fold_batch(const BatchJob<R>* jobs, int njobs, const void* scratch, int Ng,
-                       int tile, int ntx, int ext, cudaStream_t s) {
+void launch_fold_batch(const BatchJob<R>* jobs, int njobs, const int32_t* job_of, int total_items,
+                       int longest, void* scratch, int Ng, int tile, int ntx, int ext,
+                       cudaStream_t s) {
+  using Acc = typename ScratchOf<R, KAHAN>::T;
+  const int S = tile + kW - 1;
+  if (longest > kFoldList && total_items > 0)
+    fold_groups_batch_kernel<R, KAHAN>
+        <<<total_items, 128, 0, s>>>(jobs, job_of, static_cast<Acc*>(scratch), S * S);
   int first, side;
   fold_region(Ng, ext, &first, &side);
-  fold_batch_kernel<R, KAHAN>
-      <<<dim3((side + kThreads - 1) / kThreads, side, njobs), kThreads, 0, s>>>(
-          jobs, reinterpret_cast<const typename ScratchOf<R, KAHAN>::T*>(scratch), Ng, tile, ntx,
-          first, side);
+  const auto go = [&](auto* k, int Q) {
+    k<<<fold_grid(first, side, njobs, Q), kFoldThreads, 0, s>>>(
+        jobs, static_cast<const Acc*>(scratch), Ng, tile, ntx, first, side);
+  };
+  if (fold_quads(side, njobs)) go(fold_batch_kernel<R, KAHAN, 4>, 4);
+  else go(fold_batch_kernel<R, KAHAN, 1>, 1);
 }
 
 template <typename R>
@@ -1162,12 +1259,12 @@ template void launch_grid_batch<float, true>(const BatchJob<float>*, const int32
                                              int, int, const EsKernel&, cudaStream_t);
 template void launch_grid_batch<double, false>(const BatchJob<double>*, const int32_t*, int,
                                                void*, int, int, const EsKernel&, cudaStream_t);
-template void launch_fold_batch<float, false>(const BatchJob<float>*, int, const void*, int, int,
-                                              int, int, cudaStream_t);
-template void launch_fold_batch<float, true>(const BatchJob<float>*, int, const void*, int, int,
-                                              int, int, cudaStream_t);
-template void launch_fold_batch<double, false>(const BatchJob<double>*, int, const void*, int, int,
-                                              int, int, cudaStream_t);
+template void launch_fold_batch<float, false>(const BatchJob<float>*, int, const int32_t*, int, int, void*,
+                                              int, int, int, int, cudaStream_t);
+template void launch_fold_batch<float, true>(const BatchJob<float>*, int, const int32_t*, int, int, void*,
+                                              int, int, int, int, cudaStream_t);
+template void launch_fold_batch<double, false>(const BatchJob<double>*, int, const int32_t*, int, int, void*,
+                                              int, int, int, int, cudaStream_t);
 
 template void launch_pad<float>(const float*, const float*, int, int, float2*, cudaStream_t);
 template void launch_pad<double>(const double*, const double*, int, int, double2*,
@@ -1191,11 +1288,11 @@ template void launch_grid<float, true>(const WorkItem*, int, const uint32_t*, co
 template void launch_grid<double, false>(const WorkItem*, int, const uint32_t*, const double2*,
                                          const double2*, void*, int, int, int, const EsKernel&,
                                          cudaStream_t);
-template void launch_fold<float, false>(const void*, const int32_t*, int, int, int, int, float2*,
-                                        cudaStream_t);
-template void launch_fold<float, true>(const void*, const int32_t*, int, int, int, int, float2*,
-                                       cudaStream_t);
-template void launch_fold<double, false>(const void*, const int32_t*, int, int, int, int, double2*,
-                                         cudaStream_t);
+template void launch_fold<float, false>(void*, const WorkItem*, int, int, const int32_t*, int, int, int,
+                                        int, float2*, cudaStream_t);
+template void launch_fold<float, true>(void*, const WorkItem*, int, int, const int32_t*, int, int, int,
+                                        int, float2*, cudaStream_t);
+template void launch_fold<double, false>(void*, const WorkItem*, int, int, const int32_t*, int, int, int,
+                                        int, double2*, cudaStream_t);
 
 }  // namespace ms

@@ -304,6 +304,7 @@ struct PartDev {
   void* frac = nullptr;
   WorkItem* items = nullptr;
   int nitems = 0;
+  int longest = 0;                 // the most items of one tile
   int32_t* tile_items = nullptr;
   void* Hhat = nullptr;
   bool have_psf = false;
@@ -702,8 +703,8 @@ void grid_sorted(ms_plan* p, PartDev& pd, const void* vis_sorted, void* image, T
                                p->es, p->ps);
     }
     KSpan k(p, MS_K_FOLD);
-    launch_fold<float, true>(scratch, pd.tile_items, p->Ng, p->T, p->ntx, p->ext, (float2*)p->grid,
-                             p->ps);
+    launch_fold<float, true>(scratch, pd.items, pd.nitems, pd.longest, pd.tile_items, p->Ng, p->T,
+                             p->ntx, p->ext, (float2*)p->grid, p->ps);
   } else {
     {
       KSpan k(p, MS_K_GRID);
@@ -712,8 +713,8 @@ void grid_sorted(ms_plan* p, PartDev& pd, const void* vis_sorted, void* image, T
                             p->ps);
     }
     KSpan k(p, MS_K_FOLD);
-    launch_fold<R, false>(scratch, pd.tile_items, p->Ng, p->T, p->ntx, p->ext, (C2<R>*)p->grid,
-                          p->ps);
+    launch_fold<R, false>(scratch, pd.items, pd.nitems, pd.longest, pd.tile_items, p->Ng, p->T,
+                          p->ntx, p->ext, (C2<R>*)p->grid, p->ps);
   }
   int b = tm ? tm->mark() : 0;
   if (tm) tm->spans[0].push_back({a, b});
@@ -1514,7 +1515,7 @@ template <typename R> void build_plan(ms_plan* p, const ms_plan_desc* d) {
   while ((1u << bits) <= (unsigned)p->ntiles) ++bits;
   bits = ((bits + 2 * lg_t + 7) / 8) * 8;
   const uint32_t sentinel = (uint32_t)p->ntiles << (2 * lg_t);
-  int32_t* d_ext = dalloc<int32_t>(1, "extent");
+  int32_t* d_ext = dalloc<int32_t>(2, "extent");   // and a tile's longest item list
   ck(cudaMemsetAsync(d_ext, 0, sizeof(int32_t), s), "memset");
   const uint8_t masks[3] = {4 | 1, 4 | 2, 4};
   p->ch.resize(d->nchan);
@@ -1547,6 +1548,9 @@ template <typename R> void build_plan(ms_plan* p, const ms_plan_desc* d) {
       launch_chunks_per_tile(counts, p->ntiles, p->chunk, nch, s);
       pd.tile_items = p->alloc<int32_t>(p->ntiles + 1, "tile items");
       launch_exclusive_scan(nch, pd.tile_items, p->ntiles, s);
+      launch_max(nch, p->ntiles, d_ext + 1, s);
+      ck(cudaMemcpyAsync(&pd.longest, d_ext + 1, sizeof(int32_t), cudaMemcpyDeviceToHost, s),
+         "copy");
       int32_t nitems = 0;
       ck(cudaMemcpyAsync(&nitems, pd.tile_items + p->ntiles, sizeof(int32_t),
                          cudaMemcpyDeviceToHost, s),
@@ -1831,7 +1835,7 @@ void destroy(ms_plan* p) {
 struct BatchShape {
   int njobs = 0;
   int64_t items = 0, rows = 0, max_n = 0;
-  int max_items = 0;
+  int max_items = 0, longest = 0;
 };
 
 template <typename R>
@@ -1859,6 +1863,7 @@ BatchShape batch_jobs(ms_plan* p, int njobs, const int32_t* chans, const int32_t
     sh.rows += pd.n;
     sh.max_n = std::max(sh.max_n, pd.n);
     sh.max_items = std::max(sh.max_items, pd.nitems);
+    sh.longest = std::max(sh.longest, pd.longest);
   }
   arg(sh.items < (int64_t)1 << 31, "too many work items for one launch");
   return sh;
@@ -2006,11 +2011,12 @@ void grid_batch(ms_plan* p, int njobs, const int32_t* chans, const int32_t* part
   {
     KSpan k(p, MS_K_FOLD);
     if (p->prec == MS_FP32_KAHAN)
-      launch_fold_batch<float, true>((const BatchJob<float>*)jd, njobs, p->batch.scratch, p->Ng,
-                                     p->T, p->ntx, p->ext, p->ps);
+      launch_fold_batch<float, true>((const BatchJob<float>*)jd, njobs, p->batch.job_of,
+                                     (int)sh.items, sh.longest, p->batch.scratch, p->Ng, p->T,
+                                     p->ntx, p->ext, p->ps);
     else
-      launch_fold_batch<R, false>(jd, njobs, p->batch.scratch, p->Ng, p->T, p->ntx, p->ext,
-                                  p->ps);
+      launch_fold_batch<R, false>(jd, njobs, p->batch.job_of, (int)sh.items, sh.longest,
+                                  p->batch.scratch, p->Ng, p->T, p->ntx, p->ext, p->ps);
   }
   batch_fft<R>(p, jd, njobs, false);
 }
@@ -2321,11 +2327,12 @@ void residual_batch(ms_plan* p, int njobs, const int32_t* chans, const int32_t* 
   {
     KSpan k(p, MS_K_FOLD);
     if (p->prec == MS_FP32_KAHAN)
-      launch_fold_batch<float, true>((const BatchJob<float>*)jd, njobs, p->batch.scratch, p->Ng,
-                                     p->T, p->ntx, p->ext, p->ps);
+      launch_fold_batch<float, true>((const BatchJob<float>*)jd, njobs, p->batch.job_of,
+                                     (int)sh.items, sh.longest, p->batch.scratch, p->Ng, p->T,
+                                     p->ntx, p->ext, p->ps);
     else
-      launch_fold_batch<R, false>(jd, njobs, p->batch.scratch, p->Ng, p->T, p->ntx, p->ext,
-                                  p->ps);
+      launch_fold_batch<R, false>(jd, njobs, p->batch.job_of, (int)sh.items, sh.longest,
+                                  p->batch.scratch, p->Ng, p->T, p->ntx, p->ext, p->ps);
   }
   batch_fft<R>(p, jd, njobs, false);
 }

@@ -265,6 +265,20 @@ void launch_chunks_per_tile(const int32_t* counts, int ntiles, int chunk, int32_
   chunks_kernel<<<(ntiles + 255) / 256, 256, 0, s>>>(counts, ntiles, chunk, nchunks);
 }
 
+__global__ void max_kernel(const int32_t* __restrict__ in, int n, int32_t* __restrict__ most) {
+  int m = 0;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+    m = max(m, in[i]);
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_down_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(most, m);
+}
+
+void launch_max(const int32_t* in, int n, int32_t* most, cudaStream_t s) {
+  cudaMemsetAsync(most, 0, sizeof(int32_t), s);
+  max_kernel<<<grid_for(n, 256), 256, 0, s>>>(in, n, most);
+}
+
+
 __global__ void make_items_kernel(const int32_t* __restrict__ counts,
                                   const int32_t* __restrict__ tile_start,
                                   const int32_t* __restrict__ item_start, int ntiles, int chunk,

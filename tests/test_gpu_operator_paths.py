@@ -90,3 +90,30 @@ def test_degridding_into_its_observed_rows(ms, precision):
     for p in "LH":   # rows of both partitions get the same value from either
         assert torch.equal(shared[rows[p]], apart[p][rows[p]])
     plan.close()
+
+
+# work items of one tile around the fold's limits (lists up to 32 are summed
+# by the cell, longer ones in groups of 16 first), the other tiles with few, on
+# a grid summed one cell a thread and one summed four
+@pytest.mark.parametrize("items", [1, 31, 32, 33, 48, 49, 70])
+@pytest.mark.parametrize("N,tile", [(48, 16), (48, 32), (448, 16)])
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "fp32_kahan"])
+def test_long_item_lists(ms, precision, N, tile, items):
+    import torch
+    rng = np.random.default_rng(items)
+    dl, chunk = 1e-3, 16
+    n = items * chunk - 5
+    u = rng.uniform(2.0, tile - 3.0, n) / (2 * N * dl)   # inside the tile at the origin
+    v = rng.uniform(2.0, tile - 3.0, n) / (2 * N * dl)
+    u2, v2 = synth.random_uv(200, N, dl, rng)
+    u, v = np.concatenate([u, u2]), np.concatenate([v, v2])
+    vis = rng.standard_normal(len(u)) + 1j * rng.standard_normal(len(u))
+    A = og.GriddedOperator(u, v, N, dl)
+    plan = ms.Plan(u, v, N, dl, 9.0, 2.0, precision=precision, levels=2, tile=tile, chunk=chunk)
+    d = torch.from_numpy(vis).to("cuda", plan.complex_dtype)
+    got = plan.grid("ALL", d).cpu().numpy()
+    assert rel(got, A.dirty(vis)) <= TOL[precision]
+    both = plan.grid_batch([(0, "ALL"), (0, "L")], [d, d])
+    np.testing.assert_array_equal(both[0].cpu().numpy(), got)
+    assert torch.equal(both[1], plan.grid("L", d))
+    plan.close()
