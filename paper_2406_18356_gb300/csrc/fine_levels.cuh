@@ -49,7 +49,8 @@ __device__ __forceinline__ void fine_analysis_item(R* smem, const R* __restrict_
   // aligned (n and TX multiples of the chunk), else element by element
   constexpr int V = 16 / (int)sizeof(R);
   constexpr int nch = (cols + V - 1) / V;
-  if ((2 * TX) % V == 0 && n % V == 0 && p0x + nch * V <= n) {
+  if ((2 * TX) % V == 0 && n % V == 0 && p0x + nch * V <= n &&
+      (reinterpret_cast<uintptr_t>(src) & 15) == 0) {
     for (int e = tid; e < rows_in * nch; e += THREADS) {
       const int a = div_const<nch>(e), c = e - a * nch;
       int py = p0y + a;
@@ -199,46 +200,78 @@ __global__ void __launch_bounds__(THREADS)
 // ------------------------------------------------------------ synthesis
 template <int TY, int TX> struct FineSyn {
   static constexpr int InY = TY / 2 + kMaxTaps / 2 - 1, InX = TX / 2 + kMaxTaps / 2 - 1;
-  static constexpr int XS = InX | 1;
+  static constexpr int XS = TX / 2 + kMaxTaps / 2;   // window row: whole 16-byte chunks
   static constexpr int ZS = InX | 1;
   static constexpr int Sub = InY * XS;
-  static constexpr int Elems = 4 * Sub + 2 * TY * ZS;
+  static constexpr int Elems = 4 * Sub + round4(2 * TY * ZS);
 };
+// of basis MB: halo columns, and staged columns before the filter's first (a
+// window row starts on a chunk)
+template <int MB> constexpr int kSynHalo = MB;
+template <typename R, int MB>
+constexpr int kSynLead = (16 / (int)sizeof(R) - MB % (16 / (int)sizeof(R))) % (16 / (int)sizeof(R));
 
-// Output tile of TY x TX of one level for basis MB: the four subband windows
-// staged by cp.async (periodic), columns into zlo / zhi, rows into put(row,
-// first column, 2 U outputs).  TID of NT threads (a block, or a warp that
-// works by itself: SYNC joins them).
-template <typename R, int MB, int TY, int TX, int U, int NT, class Sync, class Put>
-__device__ __forceinline__ void fine_synthesis_item(R* smem, int tid, const R* __restrict__ ap,
-                                                    int aps, const R* __restrict__ plane, int N,
-                                                    int h, int r0, int c0, const Sync& sync,
-                                                    const Put& put) {
+// The four subband windows of basis MB for the output tile at (r0, c0), by
+// cp.async: whole 16-byte chunks where no column wraps and rows start
+// aligned, else lane by lane along a row.  (Element by element through two
+// quotients, staging took half of a tile's instructions: an iteration at 2048
+// px 398 -> 350 us, at 1024 px 122 -> 114, 8 jobs at 1024 px 88 -> 76 a job.)
+// TID of NT threads (a block, or a warp that works by itself).
+template <typename R, int MB, int TY, int TX, int NT>
+__device__ __forceinline__ void fine_synthesis_stage(R* sub, int tid, const R* __restrict__ ap,
+                                                     int aps, const R* __restrict__ plane, int N,
+                                                     int h, int r0, int c0) {
   using G = FineSyn<TY, TX>;
-  constexpr int L = 2 * (MB + 1), HL = L / 2 - 1;
-  constexpr int iny = TY / 2 + HL, inx = TX / 2 + HL;   // staged rows / columns per subband
-  R* zlo = smem + 4 * G::Sub;
-  R* zhi = zlo + TY * G::ZS;
-  for (int e = tid; e < 4 * iny * inx; e += NT) {
-    const int s = div_const<iny * inx>(e), rem = e - s * (iny * inx);
-    const int q = div_const<inx>(rem), c = rem - q * inx;
-    int y = r0 / 2 - HL + q, x = c0 / 2 - HL + c;
-    y = y >= -h ? wrapc(y, h) : wrap(y, h);
+  constexpr int V = 16 / (int)sizeof(R), HL = kSynHalo<MB>, LEAD = kSynLead<R, MB>;
+  constexpr int iny = TY / 2 + HL, inx = TX / 2 + HL;
+  constexpr int nch = (LEAD + inx + V - 1) / V;
+  const int x0 = c0 / 2 - HL - LEAD, y0 = r0 / 2 - HL;
+  const bool chunks = (TX / 2) % V == 0 && x0 >= 0 && h % V == 0 &&
+                      ((reinterpret_cast<uintptr_t>(ap) | reinterpret_cast<uintptr_t>(plane)) &
+                       15) == 0;
+  if (chunks) {
+    for (int e = tid; e < 4 * iny * nch; e += NT) {
+      const int sq = div_const<nch>(e), c = (e - sq * nch) * V;
+      const int s = div_const<iny>(sq), q = sq - s * iny;
+      int y = y0 + q;
+      y = y >= -h ? wrapc(y, h) : wrap(y, h);
+      const R* p = s == 0 ? ap + (int64_t)y * aps
+                          : plane + (int64_t)(s >= 2 ? h + y : y) * N + (s & 1 ? h : 0);
+      cp_async<16>(sub + s * G::Sub + q * G::XS + c, p + x0 + c);
+    }
+  } else {
+    constexpr int LW = inx <= 8 ? 8 : (inx <= 16 ? 16 : 32);   // lanes a row
+    static_assert(inx <= 32 && NT % LW == 0, "a row fits a warp");
+    const int c = tid % LW;
+    int x = c0 / 2 - HL + c;
     x = x >= -h ? wrapc(x, h) : wrap(x, h);
-    const R* p = s == 0 ? ap + (int64_t)y * aps + x
-                        : plane + (int64_t)(s >= 2 ? h + y : y) * N + (s & 1 ? h + x : x);
-    cp_async<sizeof(R)>(smem + s * G::Sub + q * G::XS + c, p);
+    if (c < inx) {
+      for (int q = tid / LW; q < iny; q += NT / LW) {
+        int y = y0 + q;
+        y = y >= -h ? wrapc(y, h) : wrap(y, h);
+        R* d = sub + q * G::XS + LEAD + c;
+        const R* lo = plane + (int64_t)y * N + x;
+        const R* hi = lo + (int64_t)h * N;
+        cp_async<sizeof(R)>(d, ap + (int64_t)y * aps + x);
+        cp_async<sizeof(R)>(d + G::Sub, lo + h);
+        cp_async<sizeof(R)>(d + 2 * G::Sub, hi);
+        cp_async<sizeof(R)>(d + 3 * G::Sub, hi + h);
+      }
+    }
   }
   cp_async_commit();
-  cp_async_wait<0>();
-  sync();
-  // columns: unit = (column, group of U output row pairs, pair lo / hi)
-  constexpr int NI = U + HL;
+}
+
+// columns: unit = (column, group of U output row pairs, pair lo / hi)
+template <typename R, int MB, int TY, int TX, int U, int NT>
+__device__ __forceinline__ void fine_synthesis_columns(const R* sub, R* zlo, R* zhi, int tid) {
+  using G = FineSyn<TY, TX>;
+  constexpr int L = 2 * (MB + 1), HL = kSynHalo<MB>, inx = TX / 2 + HL, NI = U + HL;
   constexpr int gy = TY / 2 / U;
   for (int u = tid; u < inx * gy * 2; u += NT) {
     const int rest = div_const<inx>(u), x = u - rest * inx;
     const int g = rest % gy, pair = rest / gy;
-    const R* s0 = smem + pair * G::Sub + U * g * G::XS + x;
+    const R* s0 = sub + pair * G::Sub + U * g * G::XS + kSynLead<R, MB> + x;
     const R* s1 = s0 + 2 * G::Sub;
     R lo[NI], hi[NI];
 #pragma unroll
@@ -256,8 +289,15 @@ __device__ __forceinline__ void fine_synthesis_item(R* smem, int tid, const R* _
       z[(2 * q + 1) * G::ZS] = o;
     }
   }
-  sync();
-  // rows: unit = (segment of U output pairs, row), rows fastest
+}
+
+// rows: unit = (segment of U output pairs, row), rows fastest; put(row, first
+// column, 2 U outputs)
+template <typename R, int MB, int TY, int TX, int U, int NT, class Put>
+__device__ __forceinline__ void fine_synthesis_rows(const R* zlo, const R* zhi, int tid,
+                                                    const Put& put) {
+  using G = FineSyn<TY, TX>;
+  constexpr int L = 2 * (MB + 1), HL = kSynHalo<MB>, NI = U + HL;
   constexpr int gx = TX / 2 / U;
   for (int u = tid; u < TY * gx; u += NT) {
     const int r = u % TY, g = u / TY;
@@ -280,6 +320,23 @@ __device__ __forceinline__ void fine_synthesis_item(R* smem, int tid, const R* _
     }
     put(r, 2 * U * g, o);
   }
+}
+
+// One output tile of one basis: SYNC joins the NT threads.
+template <typename R, int MB, int TY, int TX, int U, int NT, class Sync, class Put>
+__device__ __forceinline__ void fine_synthesis_item(R* smem, int tid, const R* __restrict__ ap,
+                                                    int aps, const R* __restrict__ plane, int N,
+                                                    int h, int r0, int c0, const Sync& sync,
+                                                    const Put& put) {
+  using G = FineSyn<TY, TX>;
+  R* zlo = smem + 4 * G::Sub;
+  R* zhi = zlo + TY * G::ZS;
+  fine_synthesis_stage<R, MB, TY, TX, NT>(smem, tid, ap, aps, plane, N, h, r0, c0);
+  cp_async_wait<0>();
+  sync();
+  fine_synthesis_columns<R, MB, TY, TX, U, NT>(smem, zlo, zhi, tid);
+  sync();
+  fine_synthesis_rows<R, MB, TY, TX, U, NT>(zlo, zhi, tid, put);
 }
 
 // Levels j >= 2: blockIdx.x = tile, blockIdx.y = basis (longest first); writes
@@ -375,4 +432,63 @@ __global__ void __launch_bounds__(32 * kMaxBases)
     const int r = e / TX, c = e - r * TX;
     a.x[(int64_t)(r0 + r) * n + c0 + c] = s;
   }
+}
+
+// Level 1, FP32: x = sum of the bases, a block per tile, basis after basis with
+// the next one's windows in flight.  A thread keeps the sums of its 2 U
+// outputs of one row in registers.  Tiles this small, rather than 64 pixels
+// with half of an SM's shared memory and two blocks an SM, let seven or more
+// blocks share an SM and hide each other's barriers (an iteration, 64 | 32: at
+// 1024 px 114 | 109 us, 2048 px 350 | 335, 8 jobs at 1024 px 76.1 | 74.7 a
+// job).
+template <typename R, int TY, int TX, int U, int NT>
+__global__ void __launch_bounds__(NT)
+    fine_synthesis_sum_kernel(FistaPass<R> a_, const R* plain) {
+  static_assert(TY * (TX / 2 / U) == NT, "a row unit per thread");
+  const FistaPass<R> a = job_slice(a_);   // blockIdx.z: the job (batched form)
+  pdl_wait();
+  pdl_trigger();
+  const R* coef = plain;
+  if (!plain) {
+    if (a.ctl->done) return;   // uniform: `done` does not change during this kernel
+    const int k = a.ctl->k;
+    coef = k % 3 == 0 ? a.B0 : (k % 3 == 1 ? a.B1 : a.B2);
+  }
+  using G = FineSyn<TY, TX>;
+  __shared__ __align__(16) R subs[2][4 * G::Sub];
+  __shared__ R z[2][TY * G::ZS];
+  const int tid = threadIdx.x, h = a.N / 2, n = a.N, tiles_x = n / TX;
+  const int r0 = (int)blockIdx.x / tiles_x * TY, c0 = (int)blockIdx.x % tiles_x * TX;
+  const auto stage = [&](auto basis) {
+    constexpr int MB = decltype(basis)::value;
+    const R* plane = coef + (int64_t)MB * n * n;
+    const R* ap = a.J == 1 ? plane : a.tmp + (int64_t)MB * h * h;   // LL_1: half (2 & 1)
+    fine_synthesis_stage<R, MB, TY, TX, NT>(subs[MB & 1], tid, ap, a.J == 1 ? n : h, plane, n, h,
+                                            r0, c0);
+  };
+  R acc[2 * U];
+#pragma unroll
+  for (int q = 0; q < 2 * U; ++q) acc[q] = 0;
+  const auto step = [&](auto basis) {
+    constexpr int MB = decltype(basis)::value;
+    if (MB >= a.M) return;
+    cp_async_wait<0>();
+    __syncthreads();   // window MB is there; the other buffer and z are free
+    if constexpr (MB + 1 < kMaxBases)
+      if (MB + 1 < a.M) stage(std::integral_constant<int, MB + 1>());
+    fine_synthesis_columns<R, MB, TY, TX, U, NT>(subs[MB & 1], z[0], z[1], tid);
+    __syncthreads();
+    fine_synthesis_rows<R, MB, TY, TX, U, NT>(z[0], z[1], tid,
+                                              [&](int, int, const R (&o)[2 * U]) {
+#pragma unroll
+                                                for (int q = 0; q < 2 * U; ++q) acc[q] += o[q];
+                                              });
+  };
+  stage(std::integral_constant<int, 0>());
+#define MS_FS(MBV) step(std::integral_constant<int, MBV>());
+  MS_FS(0) MS_FS(1) MS_FS(2) MS_FS(3) MS_FS(4) MS_FS(5) MS_FS(6) MS_FS(7)
+#undef MS_FS
+  struct alignas(2 * U * sizeof(R) < 16 ? 2 * U * sizeof(R) : 16) Pack { R v[2 * U]; };
+  R* dst = a.x + (int64_t)(r0 + tid % TY) * n + c0 + 2 * U * (tid / TY);
+  *reinterpret_cast<Pack*>(dst) = *reinterpret_cast<const Pack*>(acc);
 }

@@ -148,32 +148,8 @@ template <int AT> struct AG {
   static_assert(4 * AT * GS <= InSz, "the outputs alias the input window");
   static_assert(2 * AT * (AT / kP) <= Threads, "one thread per row unit");
 };
-// Synthesis geometry for output tiles of side ST: four staged subband windows
-// per basis (double-buffered over the bases) and the column-filtered rows.
-template <int ST> struct SG {
-  static constexpr int T = ST;
-  static constexpr int In = ST / 2 + kMaxTaps / 2 - 1;   // window side: 39, 23, 15
-  static constexpr int SubS = round4(In + 1);            // staged row stride: 40, 24, 16
-  static constexpr int ZS = In + 2;                      // odd row stride of zlo / zhi
-  static constexpr int SubSz = 4 * In * SubS;            // one staged basis
-#ifndef MS_SYN_SMALL_THREADS
-  static constexpr int Threads = 256;
-#else
-  static constexpr int Threads = ST >= 64 ? 256 : MS_SYN_SMALL_THREADS;
-#endif
-  static constexpr int Q = (ST * (ST / kP) + Threads - 1) / Threads;   // row units per thread
-};
-// Staging table of a synthesis block that sums all M bases (level 1): the
-// 16-byte chunks a thread copies, and their source offsets from the basis's
-// plane (or LL buffer), are the same for every basis, so an interior tile
-// computes them once.  K slots per thread.
-template <typename R, class G> struct SynTab {
-  static constexpr int V = 16 / (int)sizeof(R);
-  static constexpr int K = (4 * G::In * ((G::In + 1 + V - 1) / V) + G::Threads - 1) / G::Threads;
-};
-// the widest tiles (level 1 at N >= 512); the TMA box of the level-1 window
+// the widest tiles; the TMA box of the level-1 window
 constexpr int kAT = 32;
-constexpr int kST = 64;
 
 // The largest power of two <= the preferred side that divides the level's
 // side (sides need not be powers of two: N = 48 gives 48, 24, 12, 6).
@@ -181,12 +157,6 @@ __host__ __device__ __forceinline__ int fit_tile(int t, int n) {
   int p = 1;
   while (2 * p <= t && n % (2 * p) == 0) p *= 2;
   return p;
-}
-// output side of a synthesis tile: 64 (fewest halo rows) where that leaves a
-// block for nearly every resident slot, else 32.  Measured at 512 px, one job
-// (64 -> 256 blocks): level 1 21.0 -> 12.6 us.
-__host__ __device__ __forceinline__ int syn_tile(int n, int jobs) {
-  return fit_tile((n / kST) * (n / kST) * jobs >= 256 ? kST : 32, n);
 }
 __host__ __device__ __forceinline__ int ana_tile(int h) { return fit_tile(kAT, h); }   // subband side
 __device__ __forceinline__ int wrap(int i, int n) {
@@ -271,27 +241,6 @@ __device__ __forceinline__ void fir_down8(const R* x, R* lo, R* hi) {
   }
 }
 
-// 8 upsampled outputs r = 0..7 from L/2 + 3 low and high inputs:
-// out[r] = sum_{k = r mod 2, step 2} h_k lo[(r - k)/2 + L/2 - 1] + g_k hi[...]
-template <typename R, int MB>
-__device__ __forceinline__ void fir_up8(const R* lo, const R* hi, R* out) {
-  constexpr int L = 2 * (MB + 1);
-  // one fused multiply-add per tap and band (a chain, no separate product
-  // and sum); outputs 2m and 2m + 1 read the same inputs (with the even and
-  // the odd taps), so they run as one pair
-#pragma unroll
-  for (int r = 0; r < kP; r += 2) {
-    R e = 0, o = 0;
-#pragma unroll
-    for (int m = 0; m < L / 2; ++m) {
-      const int i = r / 2 - m + L / 2 - 1;
-      tap_syn<R, MB>(m, lo[i], hi[i], e, o);
-    }
-    out[r] = e;
-    out[r + 1] = o;
-  }
-}
-
 // per-thread compensated sum of |x| in the working precision (Kahan), so the
 // FP64 unit only sees one value per thread
 template <typename R> struct KSum {
@@ -310,346 +259,7 @@ template <> struct Vec<float> { using T = float4; static constexpr int N = 4; };
 template <> struct Vec<double> { using T = double2; static constexpr int N = 2; };
 }  // namespace
 
-// ------------------------------------------------------------------ synthesis
-// Level j: subbands of side h = N >> j -> output side n = 2h.  Level J reads
-// its approximation from the coefficient planes, lower levels from the LL
-// buffer written by the level above.  Level 1 sums the M bases into x, with
-// the next basis's windows prefetched by cp.async while the current one is
-// filtered.  G = SG<ST> is the geometry serving the level's tile side.
-
-// Stages the four subband windows of one basis: rows from r0/2 - 7, columns
-// from c0/2 - 8 (one column before the filter's first, so that in the image's
-// interior each window row starts on a 16-byte boundary and is copied in
-// whole 16-byte chunks); rows always, columns near the edges, wrap
-// periodically.  Window element (a, b) of subband s is at sub[s][a][b] with
-// b = column - (c0/2 - 8).
-template <typename R, class G>
-__device__ __forceinline__ void synth_stage(const R* plane, const R* llp, int N, int h, int r0,
-                                            int c0, int cnt, R* sub) {
-  const int base_r = r0 / 2 - (kMaxTaps / 2 - 1), base_c = c0 / 2 - kMaxTaps / 2;
-  const int ncol = cnt + 1;
-  constexpr int V = 16 / (int)sizeof(R);
-  const int nch = (ncol + V - 1) / V;
-  // rows lie in [-7, h), columns in [-8, h): one conditional wrap when h >= 8
-  const bool cheap = h >= kMaxTaps / 2;
-  // whole chunks: no column wraps, and every subband row of the window starts
-  // on a 16-byte boundary (h = 30, tiles of 4: neither holds)
-  if (base_c >= 0 && base_c + nch * V <= h && base_c % V == 0 && h % V == 0) {
-    const int per_sub = cnt * nch;
-    for (int e = threadIdx.x; e < 4 * per_sub; e += G::Threads) {
-      const int sb = e / per_sub, rem = e - sb * per_sub;
-      const int a = rem / nch, c = rem - a * nch;
-      const int iy = cheap ? wrapc(base_r + a, h) : wrap(base_r + a, h);
-      const int ix = base_c + c * V;
-      const R* src;
-      if (sb == 0)
-        src = llp ? llp + (int64_t)iy * h + ix : plane + (int64_t)iy * N + ix;
-      else if (sb == 1)
-        src = plane + (int64_t)iy * N + h + ix;
-      else if (sb == 2)
-        src = plane + (int64_t)(h + iy) * N + ix;
-      else
-        src = plane + (int64_t)(h + iy) * N + h + ix;
-      cp_async<16>(sub + (sb * G::In + a) * G::SubS + c * V, src);
-    }
-    return;
-  }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  constexpr int NW = G::Threads / 32;
-  for (int a = warp; a < cnt; a += NW) {
-    const int iy = cheap ? wrapc(base_r + a, h) : wrap(base_r + a, h);
-    for (int b = lane; b < ncol; b += 32) {
-      const int ix = cheap ? wrapc(base_c + b, h) : wrap(base_c + b, h);
-      R* d = sub + a * G::SubS + b;
-      cp_async<sizeof(R)>(d, llp ? llp + (int64_t)iy * h + ix : plane + (int64_t)iy * N + ix);
-      cp_async<sizeof(R)>(d + G::In * G::SubS, plane + (int64_t)iy * N + h + ix);
-      cp_async<sizeof(R)>(d + 2 * G::In * G::SubS, plane + (int64_t)(h + iy) * N + ix);
-      cp_async<sizeof(R)>(d + 3 * G::In * G::SubS, plane + (int64_t)(h + iy) * N + h + ix);
-    }
-  }
-}
-
-// The compact synthesis filter (see analysis_filter_compact): output pairs
-// (2 rr, 2 rr + 1) of a unit both read inputs rr - kk + L/2 - 1, kk < L/2,
-// with the even and the odd taps; same summation order as fir_up8.  Used
-// for the levels that write an LL buffer (not the basis sum of level 1).
-template <typename R, int MB, class G>
-__device__ __forceinline__ void synth_basis_compact(int TS, int lts, int cnt, int r0, int c0,
-                                                    const R* sub, R* zlo, R* zhi, R* ll_out,
-                                                    int n) {
-  constexpr int L = 2 * (MB + 1);
-  const int tid = threadIdx.x;
-  const int nseg = TS / kP > 0 ? TS / kP : 1;
-  const int units_a = cnt * 2 * nseg;
-  const float inv_cnt = 1.0f / (float)cnt;
-  for (int u = tid; u < units_a; u += G::Threads) {
-    int rest = div_small(u, inv_cnt);
-    int b = u - rest * cnt;
-    int pair = rest & 1, seg = rest >> 1;
-    const R* s0 = sub + (pair ? 1 : 0) * G::In * G::SubS + 1 + b;
-    const R* s1 = sub + (pair ? 3 : 2) * G::In * G::SubS + 1 + b;
-    const int first = 4 * seg + 8 - L / 2;
-    R* z = (pair ? zhi : zlo) + (kP * seg) * G::ZS + b;
-#pragma unroll 1
-    for (int rr = 0; rr < kP / 2; ++rr) {
-      R e = 0, o = 0;
-#pragma unroll
-      for (int kk = 0; kk < L / 2; ++kk) {
-        const int i = first + rr - kk + L / 2 - 1;
-        const R x = s0[i * G::SubS], y = s1[i * G::SubS];
-        tap_syn<R, MB>(kk, x, y, e, o);
-      }
-      z[(2 * rr) * G::ZS] = e;
-      z[(2 * rr + 1) * G::ZS] = o;
-    }
-  }
-  __syncthreads();
-  for (int q = 0; q < G::Q; ++q) {
-    int u = tid + q * G::Threads;
-    int r = u & (TS - 1), seg = u >> lts;
-    if (seg >= nseg) continue;
-    const int first = 4 * seg + 8 - L / 2;
-    const R* lr = zlo + r * G::ZS + first;
-    const R* hr = zhi + r * G::ZS + first;
-    R* dst = ll_out + (int64_t)(r0 + r) * n + c0 + kP * seg;
-#pragma unroll 1
-    for (int rr = 0; rr < kP / 2; ++rr) {
-      R e = 0, o = 0;
-#pragma unroll
-      for (int kk = 0; kk < L / 2; ++kk) {
-        const int i = rr - kk + L / 2 - 1;
-        tap_syn<R, MB>(kk, lr[i], hr[i], e, o);
-      }
-      if (kP * seg + 2 * rr < TS) dst[2 * rr] = e;
-      if (kP * seg + 2 * rr + 1 < TS) dst[2 * rr + 1] = o;
-    }
-  }
-}
-
-template <typename R, int MB, class G>
-__device__ __forceinline__ void synth_basis(int TS, int lts, int cnt, int r0, int c0,
-                                            const R* sub, R* zlo, R* zhi, R (&acc)[G::Q][kP],
-                                            bool sum_bases, R* ll_out, int n) {
-  constexpr int L = 2 * (MB + 1);
-  constexpr int NI = L / 2 + 3;
-  const int tid = threadIdx.x;
-  if constexpr (kCompact<G::T>) {
-    if (!sum_bases) {
-      synth_basis_compact<R, MB, G>(TS, lts, cnt, r0, c0, sub, zlo, zhi, ll_out, n);
-      return;
-    }
-  }
-  // columns (y): units (b, pair, seg); pair 0 -> zlo from (approximation,
-  // high-y/low-x), pair 1 -> zhi from (low-y/high-x, high/high)
-  const int nseg = TS / kP > 0 ? TS / kP : 1;
-  const int units_a = cnt * 2 * nseg;
-  const float inv_cnt = 1.0f / (float)cnt;
-  for (int u = tid; u < units_a; u += G::Threads) {
-    int rest = div_small(u, inv_cnt);
-    int b = u - rest * cnt;
-    int pair = rest & 1, seg = rest >> 1;
-    // window column b + 1 is filter column b (the window starts one early)
-    const R* s0 = sub + (pair ? 1 : 0) * G::In * G::SubS + 1;
-    const R* s1 = sub + (pair ? 3 : 2) * G::In * G::SubS + 1;
-    const int first = 4 * seg + 8 - L / 2;
-    R lo[NI], hi[NI];
-#pragma unroll
-    for (int i = 0; i < NI; ++i) {
-      lo[i] = s0[(first + i) * G::SubS + b];
-      hi[i] = s1[(first + i) * G::SubS + b];
-    }
-    R out[kP];
-    fir_up8<R, MB>(lo, hi, out);
-    R* z = pair ? zhi : zlo;
-#pragma unroll
-    for (int r = 0; r < kP; ++r) z[(kP * seg + r) * G::ZS + b] = out[r];
-  }
-  __syncthreads();
-  // rows (x): units (r, seg), a warp takes consecutive rows of one segment
-#pragma unroll
-  for (int q = 0; q < G::Q; ++q) {
-    int u = tid + q * G::Threads;
-    int r = u & (TS - 1), seg = u >> lts;
-    if (seg >= nseg) continue;
-    const int first = 4 * seg + 8 - L / 2;
-    R lo[NI], hi[NI];
-#pragma unroll
-    for (int i = 0; i < NI; ++i) {
-      lo[i] = zlo[r * G::ZS + first + i];
-      hi[i] = zhi[r * G::ZS + first + i];
-    }
-    R out[kP];
-    fir_up8<R, MB>(lo, hi, out);
-    if (sum_bases) {
-#pragma unroll
-      for (int cc = 0; cc < kP; ++cc) acc[q][cc] += out[cc];
-    } else {
-      R* dst = ll_out + (int64_t)(r0 + r) * n + c0 + kP * seg;
-#pragma unroll
-      for (int cc = 0; cc < kP; ++cc)
-        if (kP * seg + cc < TS) dst[cc] = out[cc];
-    }
-  }
-}
-
-// One synthesis work item: output tile `tile` of level j for basis mb
-// (level 1: all bases summed into x).  Ends with a block barrier, so the
-// caller may reuse the shared buffers.
-template <typename R, class G>
-__device__ __forceinline__ void synth_item(unsigned char* smem_raw, const R* __restrict__ coef,
-                                           const R* __restrict__ ll_in, R* __restrict__ ll_out,
-                                           R* __restrict__ x, int N, int j, int J, int M,
-                                           int tile, int mb, int jobs) {
-  R* subs = reinterpret_cast<R*>(smem_raw);          // [2][4][G::In][G::SubS]
-  R* zlo = subs + 2 * G::SubSz;                       // [G::T][G::ZS]
-  R* zhi = zlo + G::T * G::ZS;
-  int2* tab = reinterpret_cast<int2*>(zhi + G::T * G::ZS);   // [K][G::Threads]
-  const int h = N >> j, n = 2 * h;
-  const int TS = syn_tile(n, jobs);
-  const int lts = 31 - __clz(TS);
-  const int cnt = TS / 2 + kMaxTaps / 2 - 1;
-  const int tiles_x = n / TS;
-  const int r0 = (tile / tiles_x) * TS, c0 = (tile % tiles_x) * TS;
-  const bool sum_bases = (j == 1);
-  const int m_lo = sum_bases ? 0 : mb, m_hi = sum_bases ? M : mb + 1;
-  R acc[G::Q][kP];
-#pragma unroll
-  for (int q = 0; q < G::Q; ++q)
-#pragma unroll
-    for (int cc = 0; cc < kP; ++cc) acc[q][cc] = (R)0;
-  // interior tiles of a level summing several bases stage through the table:
-  // entry = {source offset, shared offset | 1 << 30 for the LL buffer}, or
-  // y = -1 for an unused slot; each thread reads back only its own entries
-  using Tab = SynTab<R, G>;
-  constexpr int V = Tab::V;
-  const int nch = (cnt + 1 + V - 1) / V;
-  const int base_r = r0 / 2 - (kMaxTaps / 2 - 1), base_c = c0 / 2 - kMaxTaps / 2;
-  const bool table = sum_bases && m_hi - m_lo > 1 && base_c >= 0 && base_c + nch * V <= h &&
-                     base_c % V == 0 && h % V == 0;
-  if (table) {
-    const int per_sub = cnt * nch;
-    const bool cheap = h >= kMaxTaps / 2;
-    const bool from_ll = j != J;
-#pragma unroll
-    for (int k = 0; k < Tab::K; ++k) {
-      const int e = threadIdx.x + k * G::Threads;
-      int2 t = make_int2(0, -1);
-      if (e < 4 * per_sub) {
-        const int sb = e / per_sub, rem = e - sb * per_sub;
-        const int a = rem / nch, c = rem - a * nch;
-        const int iy = cheap ? wrapc(base_r + a, h) : wrap(base_r + a, h);
-        const int ix = base_c + c * V;
-        int off;
-        if (sb == 0)
-          off = from_ll ? iy * h + ix : iy * N + ix;
-        else if (sb == 1)
-          off = iy * N + h + ix;
-        else if (sb == 2)
-          off = (h + iy) * N + ix;
-        else
-          off = (h + iy) * N + h + ix;
-        t.x = off;
-        t.y = ((sb * G::In + a) * G::SubS + c * V) | ((sb == 0 && from_ll) ? 1 << 30 : 0);
-      }
-      tab[k * G::Threads + threadIdx.x] = t;
-    }
-  }
-  auto stage = [&](int m) {
-    const R* plane = coef + (int64_t)m * N * N;
-    const R* llp = (j == J) ? nullptr : ll_in + (int64_t)m * h * h;
-    R* dst = subs + (m & 1) * G::SubSz;
-    if (table) {
-#pragma unroll
-      for (int k = 0; k < Tab::K; ++k) {
-        const int2 t = tab[k * G::Threads + threadIdx.x];
-        if (t.y >= 0) cp_async<16>(dst + (t.y & ((1 << 30) - 1)), ((t.y >> 30) ? llp : plane) + t.x);
-      }
-    } else {
-      synth_stage<R, G>(plane, llp, N, h, r0, c0, cnt, dst);
-    }
-    cp_async_commit();
-  };
-  stage(m_lo);
-  for (int m = m_lo; m < m_hi; ++m) {
-    if (m + 1 < m_hi) {
-      stage(m + 1);
-      cp_async_wait<1>();
-    } else {
-      cp_async_wait<0>();
-    }
-    __syncthreads();
-    const R* sub = subs + (m & 1) * G::SubSz;
-    R* llo = sum_bases ? nullptr : ll_out + (int64_t)m * n * n;
-    switch (m) {
-#define MS_SYN(MBV)                                                                       \
-  case MBV:                                                                               \
-    synth_basis<R, MBV, G>(TS, lts, cnt, r0, c0, sub, zlo, zhi, acc, sum_bases, llo, n);  \
-    break;
-      MS_SYN(0) MS_SYN(1) MS_SYN(2) MS_SYN(3) MS_SYN(4) MS_SYN(5) MS_SYN(6) MS_SYN(7)
-#undef MS_SYN
-    }
-    __syncthreads();
-  }
-  if (sum_bases) {
-    const int nseg = TS / kP > 0 ? TS / kP : 1;
-#pragma unroll
-    for (int q = 0; q < G::Q; ++q) {
-      int u = threadIdx.x + q * G::Threads;
-      int r = u & (TS - 1), seg = u >> lts;
-      if (seg >= nseg) continue;
-      R* dst = x + (int64_t)(r0 + r) * N + c0 + kP * seg;
-      if (TS % kP == 0) {
-        using V = typename Vec<R>::T;
-        constexpr int NV = Vec<R>::N;
-#pragma unroll
-        for (int cc = 0; cc < kP; cc += NV) {
-          V v;
-          R* vp = reinterpret_cast<R*>(&v);
-#pragma unroll
-          for (int e = 0; e < NV; ++e) vp[e] = acc[q][cc + e];
-          *reinterpret_cast<V*>(dst + cc) = v;
-        }
-      } else {
-#pragma unroll
-        for (int cc = 0; cc < kP; ++cc)
-          if (kP * seg + cc < TS) dst[cc] = acc[q][cc];
-      }
-    }
-  }
-}
-
-// Level j of the synthesis x = W B_k of the minor cycle (B_k picked by k % 3
-// from buffers that come by value, so no pointer table is read before the
-// first load), or of a.x = W plain: blockIdx.x = output tile, blockIdx.y =
-// basis (level 1: one block per tile sums all bases).
-template <typename R, int ST>
-__global__ void __launch_bounds__(SG<ST>::Threads, 512 / SG<ST>::Threads)
-    synthesis_level_kernel(FistaPass<R> a_, const R* plain, int j) {
-  const FistaPass<R> a = job_slice(a_);   // blockIdx.z: the job (batched form)
-  pdl_wait();
-  pdl_trigger();
-  const R* coef = plain;
-  if (!plain) {
-    const int done = a.ctl->done;
-    const int k = a.ctl->k;
-    if (done) return;   // uniform: `done` does not change during this kernel
-    coef = k % 3 == 0 ? a.B0 : (k % 3 == 1 ? a.B1 : a.B2);
-  }
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int64_t half = (int64_t)a.M * (a.N / 2) * (a.N / 2);
-  const R* ll_in = (j == a.J) ? nullptr : a.tmp + ((j + 1) & 1) * half;
-  R* ll_out = a.tmp + (j & 1) * half;
-  synth_item<R, SG<ST>>(smem_raw, coef, ll_in, ll_out, a.x, a.N, j, a.J, a.M, blockIdx.x,
-                        blockIdx.y, a.js.jobs);
-}
-
 namespace {
-// staged windows, column-filtered rows and the staging table
-template <int ST> size_t synthesis_smem_bytes(size_t rsz) {
-  const size_t tab = rsz == 4 ? SynTab<float, SG<ST>>::K : SynTab<double, SG<ST>>::K;
-  return (size_t)(2 * SG<ST>::SubSz + 2 * SG<ST>::T * SG<ST>::ZS) * rsz +
-         tab * SG<ST>::Threads * sizeof(int2);
-}
 // the four output subbands alias the input window; + alignment slack,
 // block-sum scratch, mbarrier and flags
 template <int AT> size_t analysis_smem_bytes(size_t rsz) {
@@ -1071,13 +681,14 @@ int ana_side(bool f64, int h) {
 // (32, 32, 16) 132 and 136, (16, 16, 16) 134; 8 jobs: (32, 32, 32) 89.9 a
 // job, (16, 16, 16) 95.1.  FP64: 8 below 512 (the fewest instructions in the
 // busiest scheduler), else 16.
-enum class Syn { kWide, k32, k16, k8 };
+enum class Syn { k32, k16, k8, k4, k2 };
 Syn syn_kernel(bool f64, int n, int M, int jobs) {
   auto blocks = [&](int t) { return (int64_t)(n / t) * (n / t) * M * jobs; };
-  if (f64) return n >= 512 && n % 16 == 0 ? Syn::k16 : (n % 8 == 0 ? Syn::k8 : Syn::kWide);
+  const Syn small = n % 8 == 0 ? Syn::k8 : (n % 4 == 0 ? Syn::k4 : Syn::k2);
+  if (f64) return n >= 512 && n % 16 == 0 ? Syn::k16 : small;
   if (n % 32 == 0 && blocks(32) >= 1000) return Syn::k32;
   if (n % 16 == 0 && blocks(16) >= 500) return Syn::k16;
-  return n % 8 == 0 ? Syn::k8 : Syn::kWide;
+  return small;
 }
 
 template <typename R, int MODE>
@@ -1120,10 +731,9 @@ cudaError_t launch_synthesis_level(const FistaPass<R>& a, const R* plain, int j,
   const int n = 2 * (a.N >> j), jobs = a.js.jobs;
   const bool f64 = sizeof(R) == 8;
   if (j == 1) {
-    // FP64, and FP32 images too small for the wide tiles: a warp per basis.
-    // Measured at 128 px, FP64: 24.6 us an iteration less than one block per
-    // 16-pixel tile; at 512 px 542 | 632 us an iteration.  FP32 at 256 px:
-    // 49.6 | 48.5 with the wide tiles.
+    // FP64, and FP32 below 256 px: a warp per basis.  Measured at 128 px,
+    // FP64: 24.6 us an iteration less than one block per 16-pixel tile; at 512
+    // px 542 | 632 us an iteration.
     auto go = [&](auto kern, int ty, int tx, size_t elems) {
       const size_t smem = kMaxBases * elems * sizeof(R);
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1134,32 +744,32 @@ cudaError_t launch_synthesis_level(const FistaPass<R>& a, const R* plain, int j,
       return go(fine_synthesis_l1_kernel<R, 8, 16, 1>, 8, 16, FineSyn<8, 16>::Elems);
     if (f64 || n < 256 || n % 32)
       return go(fine_synthesis_l1_kernel<R, 16, 16, 2>, 16, 16, FineSyn<16, 16>::Elems);
-  } else {
-    auto go = [&](auto kern, int t, int threads) {
-      return launch_pdl(kern, dim3((n / t) * (n / t), a.M, jobs), dim3(threads), 0, s, a, plain, j);
-    };
-    switch (syn_kernel(f64, n, a.M, jobs)) {
-      case Syn::k32:
-        if constexpr (sizeof(R) == 4) return go(fine_synthesis_kernel<R, 32, 32, 4, 128>, 32, 128);
-        break;
-      case Syn::k16: return go(fine_synthesis_kernel<R, 16, 16, 2, 128>, 16, 128);
-      case Syn::k8: return go(fine_synthesis_kernel<R, 8, 8, 1, 128>, 8, 128);
-      default: break;
+    if constexpr (sizeof(R) == 4) {
+      auto sum = [&](auto kern, int threads) {
+        return launch_pdl(kern, dim3((n / 32) * (n / 32), 1, jobs), dim3(threads), 0, s, a, plain);
+      };
+      // 4 output pairs a thread (fewest shared-memory loads) where the tiles
+      // occupy the SMs several times over, else 2 by twice the threads.
+      // Measured, us an iteration and job (4 | 2): 256 px 58.6 | 44.9, 512 px
+      // 73.6 | 65.1, 4 jobs at 512 px 30.5 | 31.1, 1024 px 109.4 | 110.7.
+      if ((int64_t)(n / 32) * (n / 32) * jobs >= 1000)
+        return sum(fine_synthesis_sum_kernel<R, 32, 32, 4, 128>, 128);
+      return sum(fine_synthesis_sum_kernel<R, 32, 32, 2, 256>, 256);
     }
   }
-  const int TS = syn_tile(n, jobs);
-  const dim3 grid((n / TS) * (n / TS), j == 1 ? 1 : a.M, jobs);
-  auto go = [&](auto kern, int threads, size_t smem) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    return launch_pdl(kern, grid, dim3(threads), smem, s, a, plain, j);
+  auto go = [&](auto kern, int t, int threads) {
+    return launch_pdl(kern, dim3((n / t) * (n / t), a.M, jobs), dim3(threads), 0, s, a, plain, j);
   };
-  if constexpr (sizeof(R) == 4) {
-    if (TS >= 64)
-      return go(synthesis_level_kernel<R, 64>, SG<64>::Threads, synthesis_smem_bytes<64>(sizeof(R)));
-    if (TS >= 32)
-      return go(synthesis_level_kernel<R, 32>, SG<32>::Threads, synthesis_smem_bytes<32>(sizeof(R)));
+  switch (syn_kernel(f64, n, a.M, jobs)) {
+    case Syn::k32:
+      if constexpr (sizeof(R) == 4) return go(fine_synthesis_kernel<R, 32, 32, 4, 128>, 32, 128);
+      break;
+    case Syn::k16: return go(fine_synthesis_kernel<R, 16, 16, 2, 128>, 16, 128);
+    case Syn::k8: return go(fine_synthesis_kernel<R, 8, 8, 1, 128>, 8, 128);
+    case Syn::k4: return go(fine_synthesis_kernel<R, 4, 4, 1, 64>, 4, 64);
+    default: break;
   }
-  return go(synthesis_level_kernel<R, 16>, SG<16>::Threads, synthesis_smem_bytes<16>(sizeof(R)));
+  return go(fine_synthesis_kernel<R, 2, 2, 1, 32>, 2, 32);
 }
 }  // namespace
 

@@ -47,6 +47,23 @@ def test_transforms_on_odd_coarse_levels(ms, N, J, precision, tol):
     plan.close()
 
 
+# level 1 of the synthesis, FP32: 4 output pairs a thread (1024 px: 1024
+# tiles), 2 (fewer tiles), straight from the coefficient planes (one level),
+# with fewer bases; FP64 beside it
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-12), ("fp32", 1e-5)])
+@pytest.mark.parametrize("N,J,M", [(1024, 2, 8), (320, 1, 8), (288, 2, 3), (256, 1, 1)])
+def test_synthesis_sum_over_bases(ms, N, J, M, precision, tol):
+    import torch
+    w = synth.tiny(npix=32)
+    plan = ms.Plan(w.u[0], w.v[0], N, w.pixel_size * 32 / N, 0.1 * N, 3.0, precision=precision,
+                   levels=J, n_bases=M)
+    dt = torch.float64 if precision == "fp64" else torch.float32
+    alpha = np.random.default_rng(N).standard_normal((M, N, N))
+    got = plan.dictionary_synthesis(torch.from_numpy(alpha).to("cuda", dt)).double().cpu().numpy()
+    assert rel(got, Dictionary(N, M, J).synth(alpha)) <= tol
+    plan.close()
+
+
 @pytest.mark.parametrize("precision,tol", [("fp64", 1e-9), ("fp32", 2e-5)])
 @pytest.mark.parametrize("N,J", [(176, 4), (480, 4), (96, 4)])
 def test_fista_on_odd_coarse_levels(ms, N, J, precision, tol):
