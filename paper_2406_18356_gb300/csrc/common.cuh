@@ -468,7 +468,7 @@ template <typename R>
 void launch_dot(const R* x, const R* y, int64_t n, double* parts, double* out, int32_t* ticket,
                 cudaStream_t s);
 template <typename R>
-void launch_normalize(R* x, int64_t n, const double* den, cudaStream_t s);
+void launch_normalize(const R* x, R* y, int64_t n, const double* den, double gain, cudaStream_t s);
 template <typename R>
 void launch_hash_fill(R* x, int64_t n, uint64_t seed, cudaStream_t s);
 // the linear PSF operator of the minor cycle (2N x 2N zero padding)

@@ -1296,18 +1296,20 @@ void launch_dot(const R* x, const R* y, int64_t n, double* parts, double* out, i
   reduce_kernel<R, 1><<<nparts_for(n), kThreads, 0, s>>>(x, y, n, parts, out, ticket);
 }
 
-// x <- x / sqrt(*den)
+// y = gain x / sqrt(*den) (y may be x)
 template <typename R>
-__global__ void normalize_kernel(R* __restrict__ x, int64_t n, const double* __restrict__ den) {
-  const double sc = 1.0 / sqrt(*den);
+__global__ void normalize_kernel(const R* x, R* y, int64_t n, const double* __restrict__ den,
+                                 double gain) {
+  const double sc = gain / sqrt(*den);
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
        k += (int64_t)gridDim.x * blockDim.x)
-    x[k] = (R)((double)x[k] * sc);
+    y[k] = (R)((double)x[k] * sc);
 }
 
 template <typename R>
-void launch_normalize(R* x, int64_t n, const double* den, cudaStream_t s) {
-  normalize_kernel<R><<<nparts_for(n), kThreads, 0, s>>>(x, n, den);
+void launch_normalize(const R* x, R* y, int64_t n, const double* den, double gain,
+                      cudaStream_t s) {
+  normalize_kernel<R><<<nparts_for(n), kThreads, 0, s>>>(x, y, n, den, gain);
 }
 
 // deterministic pseudo-random start vector in [-1, 1] (splitmix64 of the index)
@@ -1654,7 +1656,8 @@ void launch_lin_theta(const R* H2, int N, const R* gl2, const R* gh2, int M, dou
   template void launch_l1<R>(const R*, int64_t, double*, double*, int32_t*, cudaStream_t);       \
   template void launch_dot<R>(const R*, const R*, int64_t, double*, double*, int32_t*,           \
                               cudaStream_t);                                                     \
-  template void launch_normalize<R>(R*, int64_t, const double*, cudaStream_t);                   \
+  template void launch_normalize<R>(const R*, R*, int64_t, const double*, double,                 \
+                                    cudaStream_t);                   \
   template void launch_hash_fill<R>(R*, int64_t, uint64_t, cudaStream_t);                       \
   template void launch_lin_pad<R>(const R*, R*, int, const FistaCtl*, cudaStream_t);            \
   template void launch_lin_mul<R>(C2<R>*, const R*, int, const FistaCtl*, cudaStream_t);        \
