@@ -83,6 +83,21 @@ template <typename R> struct OpFftArgs {
   int ext;              // cells beyond +-ext are neither written nor read (<= Ng / 2)
 };
 
+struct FistaCtl;
+// Operands of the linear PSF operator's own transforms (operator_fft.cu):
+// out = scale (H in + add), images of side N.
+template <typename R> struct LinFftArgs {
+  const R* in;
+  R* out;
+  const R* add;         // or nullptr
+  C2<R>* half;          // N rows of the half plane, `pitch` values each
+  const R* H;           // spectrum by columns, over L^2
+  const C2<R>* tw;      // exp(-2 pi i m / L), m < L
+  const FistaCtl* ctl;  // or nullptr
+  int N, pitch;
+  R scale;
+};
+
 // Device-side state of a minor cycle, one per plan.  Read and written only by
 // the library's kernels; the host reads it back after a cycle.
 struct FistaCtl {
@@ -314,6 +329,14 @@ int op_fft_pitch(int N);
 template <typename R>
 cudaError_t launch_op_fft(const OpFftArgs<R>& a, bool forward, int njobs, cudaStream_t s);
 
+int lin_fft_length(int N, size_t rsz);
+template <typename R> cudaError_t launch_lin_fft(const LinFftArgs<R>& a, int L, cudaStream_t s);
+template <typename R> void launch_lin_spectrum(const R* H2, R* H, int L, cudaStream_t s);
+template <typename R> void launch_lin_widen(const R* H2, double2* out, int64_t n, cudaStream_t s);
+void launch_lin_embed(const double* psf, double* out, int N, int L, cudaStream_t s);
+template <typename R>
+void launch_lin_spectrum_of(const double2* spec, R* H, int L, cudaStream_t s);
+
 // wavelet_kernels.cu
 void set_wavelet_filters(const double* h, const int* len, int nbases);   // host -> __constant__
 struct WaveletGeom {
@@ -480,11 +503,11 @@ template <typename R>
 void launch_lin_crop(const R* q, const R* add, R* out, int N, double scale, const FistaCtl* ctl,
                      cudaStream_t s);
 template <typename R>
-void launch_lin_low_step(const R* q, const R* res, R* ycur, const R* yprev, R* rp, int N,
+void launch_lin_low_step(const R* q, const R* res, R* ycur, const R* yprev, R* rp, int N, int P,
                          double* parts, FistaCtl* ctl, double* trace, int32_t* ticket,
                          const double* l1_parts, int n_l1, cudaStream_t s);
 template <typename R>
-void launch_lin_full_diff(const R* q, const R* res, const R* x, const R* l, R* de, int N,
+void launch_lin_full_diff(const R* q, const R* res, const R* x, const R* l, R* de, int N, int P,
                           const FistaCtl* ctl, cudaStream_t s);
 template <typename R>
 void launch_lin_full_spec(const C2<R>* dek, const C2<R>* dep, const R* gl2, const R* gh2,

@@ -309,6 +309,7 @@ struct PartDev {
   void* Hhat = nullptr;
   bool have_psf = false;
   void* Hhat2 = nullptr;   // real spectrum of the PSF on the 2N x 2N field (linear operator)
+  void* Hlin = nullptr;    // ... by columns at the length of the own transforms
 };
 
 // Batched minor cycles: each job's FISTA state as one slice of these arrays
@@ -416,6 +417,10 @@ struct ms_plan {
   // spectra by pass parity, the filtered spectra [U^; V^] and their images
   int conv = MS_CONV_CIRCULAR;
   void *lp = nullptr, *lq = nullptr, *ls = nullptr, *lh2 = nullptr;
+  // with the own transforms (length lin_L, else 0) instead: the half plane, the
+  // current problem's H^ and the twiddles
+  int lin_L = 0;
+  void *lhalf = nullptr, *lH = nullptr, *ltw = nullptr;
   void *lres = nullptr, *ll = nullptr, *ly[2] = {};
   void *lde = nullptr, *ldes[2] = {}, *luvs = nullptr, *luv = nullptr;
   cufftHandle r2c2 = 0, c2r2 = 0, r2cb = 0, c2rb = 0;
@@ -590,6 +595,20 @@ template <typename R> void fft_c2c(ms_plan* p, int dir) {
         "Z2Z");
   else
     ckf(cufftExecC2C(p->c2c, (cufftComplex*)p->grid, (cufftComplex*)p->grid, dir), "C2C");
+}
+
+// row pitch of the linear operator's half plane: whole 32-byte sectors
+int lin_pitch(int L) { return L / 2 + 4; }
+
+// tw[m] = exp(-2 pi i m / n), m < n, formed in FP64
+template <typename R> void upload_twiddles(void* dst, int n) {
+  std::vector<C2<R>> tw(n);
+  for (int m = 0; m < n; ++m) {
+    const double ang = -2.0 * M_PI * (double)m / (double)n;
+    tw[m].x = (R)std::cos(ang);
+    tw[m].y = (R)std::sin(ang);
+  }
+  ck(cudaMemcpy(dst, tw.data(), sizeof(C2<R>) * n, cudaMemcpyHostToDevice), "twiddles");
 }
 
 template <typename R> void fft_r2c(ms_plan* p, const void* in, void* out) {
@@ -921,6 +940,30 @@ template <typename R> void linear_psf(ms_plan* p, const R* x, const FistaCtl* ct
   exec_c2r<R>(p->c2r2, p->ls, p->lq);
 }
 
+// out = scale (H x + add) for images of side N
+template <typename R>
+void linear_image(ms_plan* p, const R* x, const R* add, R* out, double scale, const FistaCtl* ctl) {
+  if (!p->lin_L) {
+    linear_psf<R>(p, x, ctl);
+    KSpan k(p, MS_K_LINEAR_PSF);
+    launch_lin_crop<R>((const R*)p->lq, add, out, p->N, scale, ctl, p->ps);
+    return;
+  }
+  KSpan k(p, MS_K_LINEAR_PSF);
+  LinFftArgs<R> a{};
+  a.in = x;
+  a.out = out;
+  a.add = add;
+  a.half = (C2<R>*)p->lhalf;
+  a.H = (const R*)p->lH;
+  a.tw = (const C2<R>*)p->ltw;
+  a.ctl = ctl;
+  a.N = p->N;
+  a.pitch = lin_pitch(p->lin_L);
+  a.scale = (R)scale;
+  ck(launch_lin_fft<R>(a, p->lin_L, p->ps), "linear operator transforms");
+}
+
 // One FISTA iteration with the linear PSF operator (the pass of
 // record_fista_pass with the smooth part evaluated in the image domain; the
 // pass parity selects the ring slots of y_k / [D^_k; E^_k] as there).
@@ -928,35 +971,48 @@ template <typename R> void record_linear_pass(ms_plan* p, int parity, bool full)
   const FistaPass<R> a = fista_pass_args<R>(p);
   const int N = p->N;
   const int64_t n2 = (int64_t)N * N;
+  const R* x = (const R*)p->xwork;
+  const int P = p->lin_L ? N : 2 * N;   // side of H x_k as the next step reads it
   record_synthesis<R>(p, a);
-  linear_psf<R>(p, (const R*)p->xwork, p->ctl);   // y_k = H x_k
   if (!full) {
+    // y_k = H x_k, r, gradient image 2 H r
+    R *y = (R*)p->ly[parity], *r = (R*)(p->lin_L ? p->luv : p->lp);
+    if (p->lin_L)
+      linear_image<R>(p, x, nullptr, y, 1.0, p->ctl);
+    else
+      linear_psf<R>(p, x, p->ctl);
     {
       KSpan k(p, MS_K_SPEC_MUL);
-      launch_lin_low_step<R>((const R*)p->lq, (const R*)p->lres, (R*)p->ly[parity],
-                             (const R*)p->ly[parity ^ 1], (R*)p->lp, N, p->parts, p->ctl,
-                             p->trace, p->tickets + 0, p->l1parts, p->n_l1, p->ps);
+      launch_lin_low_step<R>(p->lin_L ? y : (const R*)p->lq, (const R*)p->lres, y,
+                             (const R*)p->ly[parity ^ 1], r, N, P, p->parts, p->ctl, p->trace,
+                             p->tickets + 0, p->l1parts, p->n_l1, p->ps);
     }
-    KSpan k(p, MS_K_LINEAR_PSF);   // gradient image 2 H r
-    exec_r2c<R>(p->r2c2, p->lp, p->ls);
-    launch_lin_mul<R>((C2<R>*)p->ls, (const R*)p->lh2, N, p->ctl, p->ps);
-    exec_c2r<R>(p->c2r2, p->ls, p->lq);
-    launch_lin_crop<R>((const R*)p->lq, nullptr, (R*)p->ywork, N, 2.0, p->ctl, p->ps);
+    if (p->lin_L) {
+      linear_image<R>(p, r, nullptr, (R*)p->ywork, 2.0, p->ctl);
+    } else {
+      KSpan k(p, MS_K_LINEAR_PSF);
+      exec_r2c<R>(p->r2c2, p->lp, p->ls);
+      launch_lin_mul<R>((C2<R>*)p->ls, (const R*)p->lh2, N, p->ctl, p->ps);
+      exec_c2r<R>(p->c2r2, p->ls, p->lq);
+      launch_lin_crop<R>((const R*)p->lq, nullptr, (R*)p->ywork, N, 2.0, p->ctl, p->ps);
+    }
   } else {
+    R* uv = (R*)p->luv;
+    if (p->lin_L)
+      linear_image<R>(p, x, nullptr, uv, 1.0, p->ctl);
+    else
+      linear_psf<R>(p, x, p->ctl);
     {
       KSpan k(p, MS_K_SPEC_MUL);
-      launch_lin_full_diff<R>((const R*)p->lq, (const R*)p->lres, (const R*)p->xwork,
-                              (const R*)p->ll, (R*)p->lde, N, p->ctl, p->ps);
+      launch_lin_full_diff<R>(p->lin_L ? uv : (const R*)p->lq, (const R*)p->lres, x,
+                              (const R*)p->ll, (R*)p->lde, N, P, p->ctl, p->ps);
       exec_r2c<R>(p->r2cb, p->lde, p->ldes[parity]);
       launch_lin_full_spec<R>((const C2<R>*)p->ldes[parity], (const C2<R>*)p->ldes[parity ^ 1],
                               (const R*)p->gl2, (const R*)p->gh2, (C2<R>*)p->luvs, N, p->parts,
                               p->ctl, p->trace, p->tickets + 0, p->l1parts, p->n_l1, p->ps);
       exec_c2r<R>(p->c2rb, p->luvs, p->luv);   // [u; v] = [G_H^2 D_z; G_L^2 E_z]
     }
-    linear_psf<R>(p, (const R*)p->luv, p->ctl);
-    KSpan k(p, MS_K_LINEAR_PSF);   // gradient image 2 (H u + v)
-    launch_lin_crop<R>((const R*)p->lq, (const R*)p->luv + n2, (R*)p->ywork, N, 2.0, p->ctl,
-                       p->ps);
+    linear_image<R>(p, uv, uv + n2, (R*)p->ywork, 2.0, p->ctl);   // 2 (H u + v)
   }
   record_analysis<R>(p, a, p->have_grad_map ? &p->grad_map : nullptr);
 }
@@ -1030,15 +1086,14 @@ template <typename R> void dict_analysis(ms_plan* p, const R* x, R* alpha) {
 template <typename R> void linear_normal(ms_plan* p, bool full, const R* x, R* out) {
   const int N = p->N;
   const int64_t n2 = (int64_t)N * N;
-  linear_psf<R>(p, x, nullptr);
+  R* uv = (R*)p->luv;
   if (!full) {
-    launch_lin_crop<R>((const R*)p->lq, nullptr, (R*)p->luv, N, 1.0, nullptr, p->ps);
-    linear_psf<R>(p, (const R*)p->luv, nullptr);
-    launch_lin_crop<R>((const R*)p->lq, nullptr, out, N, 1.0, nullptr, p->ps);
+    linear_image<R>(p, x, nullptr, uv, 1.0, nullptr);
+    linear_image<R>(p, uv, nullptr, out, 1.0, nullptr);
     return;
   }
   // [H x; x] -> spectra -> [G_H^2 H x; G_L^2 x] -> images
-  launch_lin_crop<R>((const R*)p->lq, nullptr, (R*)p->lde, N, 1.0, nullptr, p->ps);
+  linear_image<R>(p, x, nullptr, (R*)p->lde, 1.0, nullptr);
   ck(cudaMemcpyAsync((R*)p->lde + n2, x, sizeof(R) * n2, cudaMemcpyDeviceToDevice, p->ps),
      "copy");
   exec_r2c<R>(p->r2cb, p->lde, p->ldes[0]);
@@ -1046,8 +1101,7 @@ template <typename R> void linear_normal(ms_plan* p, bool full, const R* x, R* o
                           (C2<R>*)p->luvs, N, nullptr, nullptr, nullptr, nullptr, nullptr, 0,
                           p->ps);
   exec_c2r<R>(p->c2rb, p->luvs, p->luv);
-  linear_psf<R>(p, (const R*)p->luv, nullptr);
-  launch_lin_crop<R>((const R*)p->lq, (const R*)p->luv + n2, out, N, 1.0, nullptr, p->ps);
+  linear_image<R>(p, uv, uv + n2, out, 1.0, nullptr);
 }
 
 // y = K x with the plan's K (the circular operator's K^, or the linear normal
@@ -1117,7 +1171,9 @@ template <typename R> void build_normal(ms_plan* p, int step, PartDev& pd, doubl
   ensure_psf<R>(p, pd);
   if (p->conv == MS_CONV_LINEAR) {
     // the problem's H2^ into the buffer the captured passes read
-    ck(cudaMemcpyAsync(p->lh2, pd.Hhat2, sizeof(R) * 2 * p->N * (p->N + 1),
+    const int L = p->lin_L;
+    ck(cudaMemcpyAsync(L ? p->lH : p->lh2, L ? pd.Hlin : pd.Hhat2,
+                       sizeof(R) * (L ? (size_t)L * (L / 2 + 1) : (size_t)2 * p->N * (p->N + 1)),
                        cudaMemcpyDeviceToDevice, p->ps),
        "copy");
     const bool full = step_full(step);
@@ -1129,7 +1185,7 @@ template <typename R> void build_normal(ms_plan* p, int step, PartDev& pd, doubl
     // the bound (and c0 = 0), then the step size itself: the operator is not
     // circulant, so the closed form is only a bound; power iteration from
     // the fixed start as for the IUWT
-    launch_lin_theta<R>((const R*)p->lh2, p->N, full ? (const R*)p->gl2 : nullptr,
+    launch_lin_theta<R>((const R*)pd.Hhat2, p->N, full ? (const R*)p->gl2 : nullptr,
                         full ? (const R*)p->gh2 : nullptr, p->M, p->parts, p->ctl,
                         p->tickets + 2, p->ps);
     power_theta<R>(p, kPowerIterations, full);
@@ -1652,14 +1708,8 @@ template <typename R> void build_plan(ms_plan* p, const ms_plan_desc* d) {
   p->own_fft = op_fft_supported(N);
   if (p->own_fft) {
     p->half = p->alloc<C2<R>>((size_t)N * op_fft_pitch(N), "half plane");
-    std::vector<C2<R>> tw(Ng);   // exp(-2 pi i m / Ng) in FP64
-    for (int m = 0; m < Ng; ++m) {
-      const double ang = -2.0 * M_PI * (double)m / (double)Ng;
-      tw[m].x = (R)std::cos(ang);
-      tw[m].y = (R)std::sin(ang);
-    }
     p->otw = p->alloc<C2<R>>(Ng, "twiddles");
-    ck(cudaMemcpy(p->otw, tw.data(), sizeof(C2<R>) * Ng, cudaMemcpyHostToDevice), "twiddles");
+    upload_twiddles<R>(p->otw, Ng);
   } else {
     p->ext = Ng / 2;   // cuFFT transforms the whole grid
     ckf(cufftPlan2d(&p->c2c, Ng, Ng, tc), "plan C2C");
@@ -1669,11 +1719,21 @@ template <typename R> void build_plan(ms_plan* p, const ms_plan_desc* d) {
   ckf(cufftPlan2d(&p->c2r, N, N, ti), "plan C2R");
   for (cufftHandle h : {p->r2c, p->c2r}) ckf(cufftSetStream(h, s), "set stream");
   if (p->conv == MS_CONV_LINEAR) {
-    const int64_t n4 = 4 * n2, s2 = (int64_t)2 * N * (N + 1);
-    p->lp = p->alloc<R>(n4, "linear pad");
-    p->lq = p->alloc<R>(n4, "linear product");
-    p->ls = p->alloc<C2<R>>(s2, "linear spectrum");
-    p->lh2 = p->alloc<R>(s2, "linear PSF spectrum");
+    const int L = p->lin_L = lin_fft_length(N, sizeof(R));
+    if (L) {
+      p->lhalf = p->alloc<C2<R>>((size_t)N * lin_pitch(L), "linear half plane");
+      p->lH = p->alloc<R>((size_t)L * (L / 2 + 1), "linear PSF spectrum");
+      p->ltw = p->alloc<C2<R>>(L, "twiddles");
+      upload_twiddles<R>(p->ltw, L);
+    } else {
+      const int64_t n4 = 4 * n2, s2 = (int64_t)2 * N * (N + 1);
+      p->lp = p->alloc<R>(n4, "linear pad");
+      p->lq = p->alloc<R>(n4, "linear product");
+      p->ls = p->alloc<C2<R>>(s2, "linear spectrum");
+      p->lh2 = p->alloc<R>(s2, "linear PSF spectrum");
+      ckf(cufftPlan2d(&p->r2c2, 2 * N, 2 * N, tr), "plan R2C 2N");
+      ckf(cufftPlan2d(&p->c2r2, 2 * N, 2 * N, ti), "plan C2R 2N");
+    }
     p->lres = p->alloc<R>(n2, "image");
     p->ll = p->alloc<R>(n2, "image");
     for (auto& y : p->ly) y = p->alloc<R>(n2, "image");
@@ -1681,13 +1741,11 @@ template <typename R> void build_plan(ms_plan* p, const ms_plan_desc* d) {
     for (auto& q : p->ldes) q = p->alloc<C2<R>>(2 * nspec, "spectrum");
     p->luvs = p->alloc<C2<R>>(2 * nspec, "spectrum");
     p->luv = p->alloc<R>(2 * n2, "image");
-    ckf(cufftPlan2d(&p->r2c2, 2 * N, 2 * N, tr), "plan R2C 2N");
-    ckf(cufftPlan2d(&p->c2r2, 2 * N, 2 * N, ti), "plan C2R 2N");
     int nn[2] = {N, N};   // two stacked N x N transforms, contiguous
     ckf(cufftPlanMany(&p->r2cb, 2, nn, nullptr, 1, 0, nullptr, 1, 0, tr, 2), "plan R2C x2");
     ckf(cufftPlanMany(&p->c2rb, 2, nn, nullptr, 1, 0, nullptr, 1, 0, ti, 2), "plan C2R x2");
     for (cufftHandle h : {p->r2c2, p->c2r2, p->r2cb, p->c2rb})
-      ckf(cufftSetStream(h, s), "set stream");
+      if (h) ckf(cufftSetStream(h, s), "set stream");
   }
   {
     int dev_smem = 0;
@@ -2753,6 +2811,47 @@ void* static_grid_scratch(int dev) {
 
 }  // namespace
 
+// The FP64 buffers and plans of build_linear_spectrum, made on first use and
+// shared by a plan's channels and partitions.
+struct LinearEmbedding {
+  void *img = nullptr, *emb = nullptr, *spec = nullptr;
+  cufftHandle inv = 0, fwd = 0;
+  void init(int P, int L, cudaStream_t s) {
+    if (fwd) return;
+    ck(cudaMalloc(&img, sizeof(double) * P * P), "linear PSF image");
+    ck(cudaMalloc(&emb, sizeof(double) * L * L), "linear PSF image");
+    ck(cudaMalloc(&spec, sizeof(double2) * L * (L / 2 + 1)), "linear PSF spectrum");
+    ckf(cufftPlan2d(&inv, P, P, CUFFT_Z2D), "plan Z2D");
+    ckf(cufftPlan2d(&fwd, L, L, CUFFT_D2Z), "plan D2Z");
+    for (cufftHandle h : {inv, fwd}) ckf(cufftSetStream(h, s), "set stream");
+  }
+  ~LinearEmbedding() {
+    for (cufftHandle h : {inv, fwd})
+      if (h) cufftDestroy(h);
+    for (void* q : {img, emb, spec})
+      if (q) cudaFree(q);
+  }
+};
+
+// pd.Hlin, H2^ as the own transforms of length lin_L read it, on stream s.
+// For lin_L > 2N the PSF goes through its image, in FP64.
+template <typename R>
+void build_linear_spectrum(ms_plan* p, PartDev& pd, LinearEmbedding& w, cudaStream_t s) {
+  const int N = p->N, P = 2 * N, L = p->lin_L;
+  pd.Hlin = p->alloc<R>((size_t)L * (L / 2 + 1), "linear PSF spectrum");
+  if (L == P) {
+    launch_lin_spectrum<R>((const R*)pd.Hhat2, (R*)pd.Hlin, L, s);
+  } else {
+    w.init(P, L, s);
+    launch_lin_widen<R>((const R*)pd.Hhat2, (double2*)w.spec, (int64_t)P * (N + 1), s);
+    exec_c2r<double>(w.inv, w.spec, w.img);
+    launch_lin_embed((const double*)w.img, (double*)w.emb, N, L, s);
+    exec_r2c<double>(w.fwd, w.emb, w.spec);
+    launch_lin_spectrum_of<R>((const double2*)w.spec, (R*)pd.Hlin, L, s);
+  }
+  ck(cudaGetLastError(), "linear PSF spectrum");
+}
+
 // H2^ of every channel and partition for the linear PSF operator: the real
 // spectrum of the PSF on a 2N x 2N field with the same pixel size, from a
 // temporary plan of side 2N whose partition bounds are 2 ell, 2 delta (the
@@ -2775,6 +2874,7 @@ template <typename R> void build_linear_psf(ms_plan* p, const ms_plan_desc* d) {
   const size_t bytes = sizeof(R) * 2 * p->N * (p->N + 1);
   try {
     ck(cudaSetDevice(q->dev), "set device");
+    LinearEmbedding embedding;
     for (size_t c = 0; c < p->ch.size(); ++c)
       for (int pt = 0; pt < 3; ++pt) {
         PartDev& qd = q->ch[c].part[pt];
@@ -2782,6 +2882,7 @@ template <typename R> void build_linear_psf(ms_plan* p, const ms_plan_desc* d) {
         PartDev& pd = p->ch[c].part[pt];
         pd.Hhat2 = p->alloc<R>(bytes / sizeof(R), "linear PSF spectrum");
         ck(cudaMemcpyAsync(pd.Hhat2, qd.Hhat, bytes, cudaMemcpyDeviceToDevice, q->ps), "copy");
+        if (p->lin_L) build_linear_spectrum<R>(p, pd, embedding, q->ps);
         ck(cudaStreamSynchronize(q->ps), "synchronize");
       }
   } catch (...) {

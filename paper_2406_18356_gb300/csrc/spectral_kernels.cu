@@ -1340,9 +1340,10 @@ void launch_set_lambda(FistaCtl* ctl, int rule, double coef, int n, int first, c
 //   H x = P F2^-1( H2^ . F2( P^T x ) ),
 // P^T the zero padding to 2N x 2N, P the restriction to the first N x N,
 // F2 the 2N x 2N DFT and H2^ the real spectrum of the PSF on the 2N x 2N
-// field (offsets up to +-N, so no product wraps).  The transforms are
-// cuFFT's; these kernels pad, multiply, restrict and run the iteration
-// control.  With it the smooth parts are no longer diagonal in the N x N
+// field (offsets up to +-N, so no product wraps).  H x is
+// one call of operator_fft.cu's kernels where those serve the side, else the
+// kernels here pad, multiply and restrict around cuFFT transforms; the
+// iteration control is here.  With it the smooth parts are no longer diagonal in the N x N
 // Fourier basis, so a FISTA pass evaluates them in the image domain:
 //   LOW:  y_k = H x_k, f = ||y_k - i~||^2, gradient image 2 H r,
 //         r = (1 + t_k) y_k - t_k y_k-1 - i~ (= H z - i~ at the extrapolated
@@ -1416,11 +1417,11 @@ template <typename R> __device__ __forceinline__ void kahan_add(R& s, R& c, R y)
 
 // LOW / SINGLE: y_k = P q into ycur, f = ||y_k - i~||^2 (with ||B_k||_1 the
 // iteration control, in the last block), and r = (1 + t_k) y_k - t_k y_k-1 - i~
-// zero-padded into rp
+// into rp; q and rp of side P >= N, zero beyond N (q may be ycur)
 template <typename R>
-__global__ void lin_low_step_kernel(const R* __restrict__ q, const R* __restrict__ res,
-                                    R* __restrict__ ycur, const R* __restrict__ yprev,
-                                    R* __restrict__ rp, int N, double* __restrict__ parts,
+__global__ void lin_low_step_kernel(const R* q, const R* __restrict__ res, R* ycur,
+                                    const R* __restrict__ yprev, R* __restrict__ rp, int N, int P,
+                                    double* __restrict__ parts,
                                     FistaCtl* __restrict__ ctl, double* __restrict__ trace,
                                     int32_t* ticket, const double* __restrict__ l1_parts,
                                     int n_l1) {
@@ -1428,18 +1429,17 @@ __global__ void lin_low_step_kernel(const R* __restrict__ q, const R* __restrict
   const int kit = ctl->k;
   const R t = ctl_t<R>(ctl, kit & 1);
   const R a = (R)1 + t;
-  const int N2 = 2 * N;
   const double l1s = lin_l1_share(l1_parts, n_l1);
   R s0 = 0, c0 = 0;
-  for (int row = blockIdx.x; row < N2; row += gridDim.x) {
-    R* out = rp + (int64_t)row * N2;
+  for (int row = blockIdx.x; row < P; row += gridDim.x) {
+    R* out = rp + (int64_t)row * P;
     if (row >= N) {
-      for (int c = threadIdx.x; c < N2; c += blockDim.x) out[c] = (R)0;
+      for (int c = threadIdx.x; c < P; c += blockDim.x) out[c] = (R)0;
       continue;
     }
-    const R* qr = q + (int64_t)row * N2;
+    const R* qr = q + (int64_t)row * P;
     const int64_t o = (int64_t)row * N;
-    for (int c = threadIdx.x; c < N2; c += blockDim.x) {
+    for (int c = threadIdx.x; c < P; c += blockDim.x) {
       if (c >= N) {
         out[c] = (R)0;
         continue;
@@ -1449,7 +1449,7 @@ __global__ void lin_low_step_kernel(const R* __restrict__ q, const R* __restrict
       const R d = y - b;
       kahan_add<R>(s0, c0, d * d);
       out[c] = a * y - t * yprev[o + c] - b;
-      ycur[o + c] = y;
+      if (P != N) ycur[o + c] = y;
     }
   }
   double v[3];
@@ -1465,16 +1465,16 @@ __global__ void lin_low_step_kernel(const R* __restrict__ q, const R* __restrict
   }
 }
 
-// FULL: D_k = P q - i~ and E_k = x_k - l, stacked [D; E] (N x N each)
+// FULL: D_k = P q - i~ (q of side P) and E_k = x_k - l, stacked [D; E] (N x N each)
 template <typename R>
 __global__ void lin_full_diff_kernel(const R* __restrict__ q, const R* __restrict__ res,
                                      const R* __restrict__ x, const R* __restrict__ l,
-                                     R* __restrict__ de, int N, const FistaCtl* __restrict__ ctl) {
+                                     R* __restrict__ de, int N, int P,
+                                     const FistaCtl* __restrict__ ctl) {
   if (ctl && ctl->done) return;
-  const int N2 = 2 * N;
   const int64_t n2 = (int64_t)N * N;
   for (int row = blockIdx.x; row < N; row += gridDim.x) {
-    const R* qr = q + (int64_t)row * N2;
+    const R* qr = q + (int64_t)row * P;
     const int64_t o = (int64_t)row * N;
     for (int c = threadIdx.x; c < N; c += blockDim.x) {
       de[o + c] = qr[c] - res[o + c];
@@ -1598,16 +1598,16 @@ void launch_lin_crop(const R* q, const R* add, R* out, int N, double scale, cons
   lin_crop_kernel<R><<<lin_rows_grid(N), kThreads, 0, s>>>(q, add, out, N, (R)scale, ctl);
 }
 template <typename R>
-void launch_lin_low_step(const R* q, const R* res, R* ycur, const R* yprev, R* rp, int N,
+void launch_lin_low_step(const R* q, const R* res, R* ycur, const R* yprev, R* rp, int N, int P,
                          double* parts, FistaCtl* ctl, double* trace, int32_t* ticket,
                          const double* l1_parts, int n_l1, cudaStream_t s) {
-  lin_low_step_kernel<R><<<std::min(2 * N, sm_count() * 4), kThreads, 0, s>>>(
-      q, res, ycur, yprev, rp, N, parts, ctl, trace, ticket, l1_parts, n_l1);
+  lin_low_step_kernel<R><<<std::min(P, sm_count() * 4), kThreads, 0, s>>>(
+      q, res, ycur, yprev, rp, N, P, parts, ctl, trace, ticket, l1_parts, n_l1);
 }
 template <typename R>
-void launch_lin_full_diff(const R* q, const R* res, const R* x, const R* l, R* de, int N,
+void launch_lin_full_diff(const R* q, const R* res, const R* x, const R* l, R* de, int N, int P,
                           const FistaCtl* ctl, cudaStream_t s) {
-  lin_full_diff_kernel<R><<<lin_rows_grid(N), kThreads, 0, s>>>(q, res, x, l, de, N, ctl);
+  lin_full_diff_kernel<R><<<lin_rows_grid(N), kThreads, 0, s>>>(q, res, x, l, de, N, P, ctl);
 }
 template <typename R>
 void launch_lin_full_spec(const C2<R>* dek, const C2<R>* dep, const R* gl2, const R* gh2,
@@ -1663,10 +1663,10 @@ void launch_lin_theta(const R* H2, int N, const R* gl2, const R* gh2, int M, dou
   template void launch_lin_mul<R>(C2<R>*, const R*, int, const FistaCtl*, cudaStream_t);        \
   template void launch_lin_crop<R>(const R*, const R*, R*, int, double, const FistaCtl*,        \
                                    cudaStream_t);                                                \
-  template void launch_lin_low_step<R>(const R*, const R*, R*, const R*, R*, int, double*,      \
+  template void launch_lin_low_step<R>(const R*, const R*, R*, const R*, R*, int, int, double*, \
                                        FistaCtl*, double*, int32_t*, const double*, int,         \
                                        cudaStream_t);                                            \
-  template void launch_lin_full_diff<R>(const R*, const R*, const R*, const R*, R*, int,        \
+  template void launch_lin_full_diff<R>(const R*, const R*, const R*, const R*, R*, int, int,   \
                                         const FistaCtl*, cudaStream_t);                          \
   template void launch_lin_full_spec<R>(const C2<R>*, const C2<R>*, const R*, const R*, C2<R>*, \
                                         int, double*, FistaCtl*, double*, int32_t*,              \

@@ -11,15 +11,12 @@
 // rows [h,n) x cols [0,h) high-y/low-x, [h,n)^2 high/high, h = n/2.
 // Synthesis is the transpose X = T^T Y T.
 //
-// Most levels run in small tiles, one block per (tile, basis)
-// (fine_levels.cuh).  The kernels of this file serve what is left: level 1 of
-// the FP32 synthesis (a block sums the bases of a 32 or 64 pixel tile, the
-// next basis's subband windows prefetched while the current one is filtered),
-// the analysis levels of FP64 images of more than 512 pixels, and subbands
-// whose side is no multiple of four.  They are register-blocked: a thread
-// slides over 8 outputs of one row or column with its inputs held in
-// registers.  Each basis is a separate template instance so the filter taps
-// are compile-time constant-bank operands.
+// Nearly every level runs in small tiles (fine_levels.cuh).  The kernel of
+// this file serves what is left: the analysis levels of FP64 images of more
+// than 512 pixels, and subbands whose side is no multiple of four.  It is
+// register-blocked: a thread slides over 8 outputs of one row or column with
+// its inputs held in registers.  Each basis is a separate template instance so
+// the filter taps are compile-time constant-bank operands.
 //
 // The analysis kernel of the minor cycle also does FISTA's step (Algorithm 1):
 // its level-1 input is the gradient image 2 (K W alpha_k - b) of the
