@@ -489,9 +489,9 @@ void launch_l1(const R* x, int64_t n, double* parts, double* out, int32_t* ticke
                cudaStream_t s);
 template <typename R>
 void launch_dot(const R* x, const R* y, int64_t n, double* parts, double* out, int32_t* ticket,
-                cudaStream_t s);
+                double gain, cudaStream_t s);
 template <typename R>
-void launch_normalize(const R* x, R* y, int64_t n, const double* den, double gain, cudaStream_t s);
+void launch_scale(const R* x, R* y, int64_t n, const double* factor, cudaStream_t s);
 template <typename R>
 void launch_hash_fill(R* x, int64_t n, uint64_t seed, cudaStream_t s);
 // the linear PSF operator of the minor cycle (2N x 2N zero padding)

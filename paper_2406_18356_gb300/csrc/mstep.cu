@@ -1131,31 +1131,33 @@ template <typename R> void power_theta(ms_plan* p, int iters, bool full) {
   R* w = (R*)p->B[1];
   R *x = (R*)p->xwork, *y = (R*)p->ywork;
   double* sc = p->scal;
-  auto dot = [&](const R* a, const R* b, int64_t n, double* out, int ticket) {
-    launch_dot<R>(a, b, n, p->parts, out, p->tickets + ticket, p->ps);
+  auto dot = [&](const R* a, const R* b, int64_t n, double* out, int ticket, double gain) {
+    launch_dot<R>(a, b, n, p->parts, out, p->tickets + ticket, gain, p->ps);
+  };
+  // b = gain a / ||a||
+  auto normalize = [&](const R* a, R* b, int64_t n, double gain) {
+    dot(a, a, n, sc + 3, 7, gain);
+    launch_scale<R>(a, b, n, sc + 4, p->ps);
   };
   launch_hash_fill<R>(v, ncoef, 12345, p->ps);
   if (p->dict == MS_DICT_IUWT) {
     for (int it = 0; it < iters; ++it) {
-      dot(v, v, ncoef, sc + 0, 7);
-      launch_normalize<R>(v, v, ncoef, sc + 0, 1.0, p->ps);
+      normalize(v, v, ncoef, 1.0);
       dict_synthesis<R>(p, v, x);
       normal_image<R>(p, full, x, y);
       dict_analysis<R>(p, y, w);
-      dot(v, w, ncoef, sc + 1, 8);
+      dot(v, w, ncoef, sc + 1, 8, 0.0);
       ck(cudaMemcpyAsync(v, w, sizeof(R) * ncoef, cudaMemcpyDeviceToDevice, p->ps), "copy");
     }
   } else {
-    dot(v, v, ncoef, sc + 0, 7);
-    launch_normalize<R>(v, v, ncoef, sc + 0, 1.0, p->ps);
+    normalize(v, v, ncoef, 1.0);
     dict_synthesis<R>(p, v, x);
     for (int it = 0; it < iters; ++it) {
       normal_image<R>(p, full, x, y);
       if (it + 1 == iters) {
-        dot(x, y, n2, sc + 1, 8);
+        dot(x, y, n2, sc + 1, 8, 0.0);
       } else {
-        dot(y, y, n2, sc + 0, 7);
-        launch_normalize<R>(y, x, n2, sc + 0, std::sqrt((double)p->M), p->ps);
+        normalize(y, x, n2, std::sqrt((double)p->M));
       }
     }
   }

@@ -535,17 +535,19 @@ template cudaError_t launch_op_fft<float>(const OpFftArgs<float>&, bool, int, cu
 template cudaError_t launch_op_fft<double>(const OpFftArgs<double>&, bool, int, cudaStream_t);
 
 // The transform length of the linear PSF operator's own kernels for image
-// side N, or 0: cuFFT on the 2N x 2N field.  2N itself, or in FP32 the next
-// power of two up to 4/3 of it: the extra columns cost less than the launches
-// and passes saved.  Measured, step size and a minor cycle of 30 iterations,
-// ms (own | cuFFT): FP32 128 px 5.8 | 10.0, 384 px (L = 4/3 of 2N) 8.6 | 13.4,
-// 448 px 9.5 | 16.2, 1024 px 15.5 | 23.8; FP64 128 px 10.5 | 23.1, 256 px 19.1
-// | 43.4, 512 px 55 | 109, 1024 px 199 | 330.
+// side N, or 0: cuFFT on the 2N x 2N field.  The next power of two where the
+// extra columns cost less than the launches and passes saved: up to 8/5 of 2N
+// in FP32, 4/3 in FP64.  Measured, step size and a minor cycle of 30
+// iterations, ms (own | cuFFT): FP32 128 px 5.8 | 10.0, 320 px (L = 8/5 of 2N)
+// 7.9 | 12.9, 384 px (4/3) 8.0 | 13.3, 448 px 9.5 | 16.2, 640 px (8/5) 12.1 |
+// 21.6, 1024 px 15.5 | 23.8; FP64 128 px 10.5 | 23.1, 192 px (4/3) 17.3 | 37,
+// 384 px (4/3) 46 | 65, 512 px 55 | 109, 640 px (8/5) 162 | 138, 1024 px 199 |
+// 330.
 int lin_fft_length(int N, size_t rsz) {
   int L = 32;
   while (L < 2 * N) L *= 2;
   if (N % 2 || L > 8192) return 0;
-  return rsz == 8 ? (L == 2 * N ? L : 0) : (3 * L <= 8 * N ? L : 0);
+  return (rsz == 8 ? 3 * L <= 8 * N : 5 * L <= 16 * N) ? L : 0;
 }
 
 template <typename R> cudaError_t launch_lin_fft(const LinFftArgs<R>& a, int L, cudaStream_t s) {

@@ -7,11 +7,11 @@ import synth
 pytestmark = pytest.mark.gpu
 
 
-# L = 2N, L > 2N by up to 4/3, and sides that keep cuFFT (FP32: 80; FP64:
-# every side that is no power of two)
+# L = 2N, L > 2N by up to 8/5 (FP32) or 4/3 (FP64), and sides that keep cuFFT
+# (FP32: 144, 272; FP64 also 80)
 @pytest.mark.parametrize("precision,sides", [
-    ("fp32", (16, 32, 48, 80, 96, 112, 128, 192, 256, 448, 512, 1024, 2048, 4096)),
-    ("fp64", (16, 48, 64, 128, 256, 448, 512, 1024)),
+    ("fp32", (16, 32, 48, 80, 96, 112, 128, 144, 192, 256, 272, 448, 512, 1024, 2048, 4096)),
+    ("fp64", (16, 48, 64, 80, 128, 192, 256, 448, 512, 1024)),
     ("fp32_kahan", (32, 96, 256)),
 ])
 def test_first_iteration_is_the_convolved_residual(precision, sides):
