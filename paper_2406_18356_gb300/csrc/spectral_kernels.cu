@@ -587,6 +587,8 @@ template <typename R, int LOGN> struct ColCfg {
   static constexpr int TPS = fft_threads(LOGN, LRAD);
   static constexpr int THREADS = CB * TPS < 32 ? 32 : CB * TPS;
   static constexpr size_t SMEM = col_smem_c(N, CB, CBY, PF);
+  static constexpr size_t SMEM2 = col_smem_c(N, CB, CBY, false);   // without the prefetch
+  static constexpr int BLOCKS = (N / 2 + 1 + CB - 1) / CB;
   static_assert(THREADS <= 1024 && THREADS % 32 == 0, "column block");
 };
 
@@ -617,9 +619,15 @@ template <typename R> __device__ __forceinline__ float2 fp32_pair(R hi, R lo) {
 // warp leaves its sums of the objective terms in parts[i W + warp] (W warps
 // in all; i = <x,Kx>, <b,x>, the l1 partials); the inverse row transform
 // kernel gathers them and runs the iteration control, so this kernel has no
-// grid-wide tail.
-template <typename R, int LOGN>
-__global__ void __launch_bounds__(ColCfg<R, LOGN>::THREADS, 1) spec_col_kernel(
+// grid-wide tail.  MANY, for launches of more blocks than SMs: no prefetch,
+// whose shared memory leaves one block an SM; two blocks then copy and
+// transform beside each other (8 jobs at 1024 px 32.0 -> 31.3 ms a minor cycle
+// of 50, 4 jobs at 512 px 6.8 -> 6.5, one image at 2048 px 9.56 -> 9.28 ms a
+// cycle of 25).  Where one wave does it (1024 px: 129 blocks) the prefetch is
+// the faster form.
+template <typename R, int LOGN, bool MANY>
+__global__ void __launch_bounds__(ColCfg<R, LOGN>::THREADS,
+                                  MANY && ColCfg<R, LOGN>::THREADS <= 512 ? 2 : 1) spec_col_kernel(
     C2<R>* __restrict__ Z, C2<R>* __restrict__ Xk, const C2<R>* __restrict__ Xprev,
     const R* __restrict__ Ks, const C2<R>* __restrict__ Bs, const C2<R>* __restrict__ tw_g,
     double* __restrict__ parts, const FistaCtl* __restrict__ ctl,
@@ -637,7 +645,7 @@ __global__ void __launch_bounds__(ColCfg<R, LOGN>::THREADS, 1) spec_col_kernel(
     l1_parts += z * js.l1;
   }
   constexpr int N = Cfg::N, CB = Cfg::CB, T = Cfg::THREADS, P = seq_pitch(N);
-  constexpr bool PF = Cfg::PF;
+  constexpr bool PF = Cfg::PF && !MANY;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2<R>* b0 = reinterpret_cast<C2<R>*>(smem_raw);   // [CB][P]
   C2<R>* b1 = b0 + CB * P;                           // [CB][P]
@@ -1047,16 +1055,17 @@ template <typename R> struct ColLaunch {
                           const C2<R>* tw, double* parts, const FistaCtl* ctl,
                           const double* l1_parts, int n_l1, cudaStream_t s, JobStride js) {
       using Cfg = ColCfg<R, LOGN>;
-      return launch_fft(spec_col_kernel<R, LOGN>,
-                        dim3((Cfg::N / 2 + 1 + Cfg::CB - 1) / Cfg::CB, 1, js.jobs),
-                        dim3(Cfg::THREADS), Cfg::SMEM, s, Z, Xk, Xprev, Ks, Bs, tw, parts, ctl,
+      const bool many = Cfg::PF && Cfg::BLOCKS * js.jobs > sm_count();
+      return launch_fft(many ? spec_col_kernel<R, LOGN, true> : spec_col_kernel<R, LOGN, false>,
+                        dim3(Cfg::BLOCKS, 1, js.jobs), dim3(Cfg::THREADS),
+                        many ? Cfg::SMEM2 : Cfg::SMEM, s, Z, Xk, Xprev, Ks, Bs, tw, parts, ctl,
                         l1_parts, n_l1, js);
     }
   };
   template <int LOGN> struct Info {
     static cudaError_t go(int* blocks, size_t* smem, int* warps) {
       using Cfg = ColCfg<R, LOGN>;
-      *blocks = (Cfg::N / 2 + 1 + Cfg::CB - 1) / Cfg::CB;
+      *blocks = Cfg::BLOCKS;
       *smem = Cfg::SMEM;
       *warps = Cfg::THREADS / 32;
       return cudaSuccess;
