@@ -19,8 +19,8 @@
 // and stored activations (after ReLU, after pooling) are rounded to bfloat16,
 // and so is every pre-activation gradient before it enters a product.
 //
-// Measured (6 levels, width 6): forward pass at 1024 x 1024 418 us, forward
-// and backward pass with the gradients at 512 x 512 866 us; before, with the
+// Measured (6 levels, width 6): forward pass at 1024 x 1024 360 us, forward
+// and backward pass with the gradients at 512 x 512 750 us; before, with the
 // windows written out (im2col, 9 times the activations, and a transposed copy
 // for the weight gradients) and one general product kernel: 4166 and 5449 us.
 #include <cuda_bf16.h>
@@ -39,6 +39,18 @@ namespace ms {
 namespace {
 using bf16 = __nv_bfloat16;
 constexpr int kT = 256;
+
+// The network's kernels after the packing of the weights are launched early
+// (programmatic dependent launch): a block stages its weights and computes
+// its offsets while the layer before finishes, and waits here before it reads
+// or writes anything else.  The next kernel is let go only after the wait, so
+// when a kernel starts all kernels but its predecessor have completed: the
+// packed weights, two or more launches back, may be read before the wait.
+// (Forward pass at 1024 px 421 -> 360 us, gradients at 512 px 870 -> 750.)
+__device__ __forceinline__ void after_predecessor() {
+  pdl_wait();
+  pdl_trigger();
+}
 
 int blocks(int64_t n, int cap = 0) {
   if (cap <= 0) cap = sm_count() * 16;
@@ -221,7 +233,12 @@ __global__ void __launch_bounds__(128) conv_kernel(const ConvArgs p) {
   for (int c0 = 0; c0 < p.ci; c0 += p.ck) {
     const int ck = min(p.ck, p.ci - c0), kl = pad16(9 * ck);
     if (c0) __syncthreads();
-    stage_pixels<VEC>(sx, CS, TL::R, TL::R, y0 - 1, x0 - 1, p.H, p.W, c0, ck, ck, p.x);
+    if (tid < 16) sx[zero_off + tid] = __float2bfloat16_rn(0.0f);
+    for (int k = tid * VEC; k < kl; k += 128 * VEC) {
+      const int tap = k / ck, c = k - tap * ck;
+      // (k >= 9 ck: the padding reads zeros, whatever the window holds)
+      koff[k / VEC] = tap < 9 ? ((tap / 3) * TL::R + tap % 3) * CS + c : -1;
+    }
     if (ck == p.ci) {   // whole packed rows (kl = kp, a multiple of 16)
       const int nv = kl / 8;
       const float inv = 1.0f / (float)nv;
@@ -230,7 +247,9 @@ __global__ void __launch_bounds__(128) conv_kernel(const ConvArgs p) {
         const bool ok = n0 + r < p.co;
         cpz<16>(sw + r * KS + v, ok ? p.w + (int64_t)(n0 + r) * p.kp + v : p.w, ok);
       }
+      after_predecessor();
     } else {
+      if (c0 == 0) after_predecessor();
       for (int e = tid; e < NT * 8 * kl; e += 128) {
         const int r = e / kl, k = e - r * kl, tap = k / ck;
         const bool ok = n0 + r < p.co && tap < 9;
@@ -238,13 +257,8 @@ __global__ void __launch_bounds__(128) conv_kernel(const ConvArgs p) {
                             : __float2bfloat16_rn(0.0f);
       }
     }
+    stage_pixels<VEC>(sx, CS, TL::R, TL::R, y0 - 1, x0 - 1, p.H, p.W, c0, ck, ck, p.x);
     asm volatile("cp.async.commit_group;" ::: "memory");
-    if (tid < 16) sx[zero_off + tid] = __float2bfloat16_rn(0.0f);
-    for (int k = tid * VEC; k < kl; k += 128 * VEC) {
-      const int tap = k / ck, c = k - tap * ck;
-      // (k >= 9 ck: the padding reads zeros, whatever the window holds)
-      koff[k / VEC] = tap < 9 ? ((tap / 3) * TL::R + tap % 3) * CS + c : -1;
-    }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
 
@@ -439,8 +453,6 @@ __global__ void __launch_bounds__(BIG ? 256 : 128) dx_kernel(const DxArgs p) {
   for (int c0 = 0; c0 < p.co; c0 += p.ck) {
     const int ck = min(p.ck, p.co - c0), kl = pad16(ck);
     if (c0) __syncthreads();
-    stage_pixels<VEC>(sz, KS, TL::R, TL::R, y0 - 1, x0 - 1, p.H, p.W, c0, ck, kl,
-                      Act{p.dz, nullptr, p.co, 0});
     const int nv = kl / 8;
     const float inv = 1.0f / (float)nv;
     for (int e = tid; e < 9 * NT * 8 * nv; e += NW * 32) {
@@ -449,6 +461,9 @@ __global__ void __launch_bounds__(BIG ? 256 : 128) dx_kernel(const DxArgs p) {
       const bool ok = c < p.ci;
       cpz<16>(sw + r * KS + v, ok ? p.wt + (int64_t)(tap * p.ci + c) * p.cop + c0 + v : p.wt, ok);
     }
+    if (c0 == 0) after_predecessor();
+    stage_pixels<VEC>(sz, KS, TL::R, TL::R, y0 - 1, x0 - 1, p.H, p.W, c0, ck, kl,
+                      Act{p.dz, nullptr, p.co, 0});
     asm volatile("cp.async.commit_group;" ::: "memory");
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
@@ -603,6 +618,7 @@ __global__ void __launch_bounds__(128, 4) dw_kernel(const __grid_constant__ WArg
     Stage st;
     float red[3][10][32][4];   // the warps' sums, once the tiles are done
   } sm;
+  after_predecessor();
   auto& sx = sm.st.x;
   auto& sz = sm.st.z;
   auto& red = sm.red;
@@ -695,6 +711,7 @@ __global__ void __launch_bounds__(128, 4) dw_kernel(const __grid_constant__ WArg
 // the flat gradient (each layer's weights [co][9 ci], then its bias): a
 // layer's slices added in order
 __global__ void sum_partials_kernel(const __grid_constant__ WArgs p) {
+  after_predecessor();
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < p.nparams;
        e += (int64_t)gridDim.x * blockDim.x) {
     int li = 0;
@@ -711,6 +728,7 @@ __global__ void sum_partials_kernel(const __grid_constant__ WArgs p) {
 
 // ------------------------------------------------------------- small passes
 __global__ void to_bf16_kernel(const float* __restrict__ in, int64_t n, bf16* __restrict__ out) {
+  after_predecessor();
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
        e += (int64_t)gridDim.x * blockDim.x)
     out[e] = __float2bfloat16_rn(in[e]);
@@ -763,8 +781,9 @@ __global__ void cat_kernel(Act x, int H, int W, bf16* __restrict__ cat) {
 
 // the head's pre-activation gradient bf16(2 (y - t) / P) and per-block partial
 // sums of (y - t)^2 in FP64
-__global__ void mse_kernel(const float* __restrict__ y, const float* __restrict__ t, int64_t P,
+__global__ void mse_kernel(const float* y, const float* t, int64_t P,
                            bf16* __restrict__ dz, double* __restrict__ parts) {
+  after_predecessor();
   __shared__ double red[kT / 32];
   double s = 0.0;
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < P;
@@ -913,7 +932,7 @@ void launch(K kern, dim3 grid, int threads, size_t smem, const A& p, cudaStream_
   if (smem > 48 * 1024)
     ck(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
        "shared memory");
-  kern<<<grid, threads, smem, s>>>(p);
+  ck(launch_pdl(kern, grid, dim3(threads), smem, s, p), "launch");
 }
 #define MS_BY_NT(NTV, CALL)              \
   switch (NTV) {                         \
@@ -1030,7 +1049,8 @@ void forward(ms_unet* u, const float* in, int H, int W, float* out, cudaStream_t
   u->last_h = H;
   u->last_w = W;
   const int Lv = u->levels;
-  to_bf16_kernel<<<blocks((int64_t)H * W * 2), kT, 0, s>>>(in, (int64_t)H * W * 2, u->xin);
+  ck(launch_pdl(to_bf16_kernel, dim3(blocks((int64_t)H * W * 2)), dim3(kT), 0, s, in,
+                (int64_t)H * W * 2, u->xin), "launch");
   size_t li = 0;
   Act x{u->xin, nullptr, 2, 0};
   int h = H, w = W;
@@ -1069,7 +1089,8 @@ int backward(ms_unet* u, const float* target, int H, int W, const float* out, cu
   const int nb = blocks(P, 1024);
   const int Lv = u->levels;
   int li = (int)u->L.size() - 1;
-  mse_kernel<<<nb, kT, 0, s>>>(out, target, P, u->L[li].dz, u->parts);
+  ck(launch_pdl(mse_kernel, dim3(nb), dim3(kT), 0, s, out, target, P, u->L[li].dz, u->parts),
+     "launch");
   auto through = [&](Layer& prev) {   // the input is prev's output
     DxArgs p{};
     p.mode = 0;
@@ -1115,8 +1136,8 @@ int backward(ms_unet* u, const float* target, int H, int W, const float* out, cu
   int64_t np = 0;
   const WArgs a = weight_args(u, H, W, &wb, &np);
   arg(np <= u->wparts_n, "weight-gradient partial sums");
-  dw_kernel<<<wb, 128, 0, s>>>(a);
-  sum_partials_kernel<<<blocks(a.nparams), kT, 0, s>>>(a);
+  launch(dw_kernel, dim3(wb), 128, 0, a, s);
+  launch(sum_partials_kernel, dim3(blocks(a.nparams)), kT, 0, a, s);
   if (u->keep) u->kept = true;
   return nb;
 }
