@@ -13,10 +13,11 @@
 //             cropped, deapodized and scaled as they are written.
 // Each grid cell is written or read once, by lanes that cover 32-byte sectors;
 // padding, cropping, deapodization and the grid's centring (cell k at index k
-// + Ng / 2) cost no pass of their own.  A complex transform of the whole grid (2-D cuFFT between a padding
-// and a cropping pass) moves 4 to 9 times the bytes.  Measured, both
-// directions (own | cuFFT with the passes): N = 128 FP64 23 | 75 us, N = 1024
-// FP32 42 | 91, 16 grids of it 395 | 1166, N = 4096 697 | 1290.
+// + Ng / 2) cost no pass of their own.  A complex transform of the whole grid
+// (2-D cuFFT between a padding and a cropping pass) moves 4 to 9 times the
+// bytes.  Measured, both directions (own | cuFFT with the passes): N = 128 FP64
+// 23 | 75 us, N = 1024 FP32 42 | 91, 16 grids of it 395 | 1166, N = 4096 697 |
+// 1290.
 //
 // A sequence of 2^LOGN elements is held by 2^(LOGN - LE) threads, 2^LE
 // elements each, through Stockham stages of radix up to 2^LE: inputs of the
@@ -26,6 +27,12 @@
 // columns fit a block).  LE is 4 for long FP32 sequences (fewest exchanges);
 // FP64, bound by the FP64 instructions of its busiest warp at short lengths,
 // spreads them over more threads (see fft_lrad of the spectral kernels).
+//
+// The kernels are launched with programmatic dependent launch and wait first
+// of all: chains of short launches (the linear operator's six an iteration, a
+// small image's four) then overlap each launch with its predecessor's end.
+// 448 px linear minor cycle 10.65 -> 9.23 ms, residual image at 128 px, FP64, 143
+// -> 137 us.
 #include <algorithm>
 
 #include "common.cuh"
@@ -161,6 +168,8 @@ template <typename R> __device__ __forceinline__ OpFftJob<R> pick_job(const OpFf
 // image row p, deapodized and centred -> its half-plane spectrum 0..ext
 template <typename R, int LOGM>
 __global__ void __launch_bounds__(RowBlock<R, LOGM>::THREADS) op_row_forward_kernel(OpFftArgs<R> a) {
+  pdl_wait();
+  pdl_trigger();
   using B = RowBlock<R, LOGM>;
   using S = typename B::S;
   constexpr int M = 1 << LOGM, N = M, H = N / 2;
@@ -202,6 +211,8 @@ __global__ void __launch_bounds__(RowBlock<R, LOGM>::THREADS) op_row_forward_ker
 // columns u of the half plane -> grid columns u and -u, rows -ext..ext
 template <typename R, int LOGG>
 __global__ void __launch_bounds__(ColBlock<R, LOGG>::THREADS) op_col_forward_kernel(OpFftArgs<R> a) {
+  pdl_wait();
+  pdl_trigger();
   using B = ColBlock<R, LOGG>;
   using S = typename B::S;
   constexpr int Ng = 1 << LOGG, N = Ng / 2, H = N / 2;
@@ -235,6 +246,8 @@ __global__ void __launch_bounds__(ColBlock<R, LOGG>::THREADS) op_col_forward_ker
 // N image rows of the column's inverse transform
 template <typename R, int LOGG>
 __global__ void __launch_bounds__(ColBlock<R, LOGG>::THREADS) op_col_adjoint_kernel(OpFftArgs<R> a) {
+  pdl_wait();
+  pdl_trigger();
   using B = ColBlock<R, LOGG>;
   using S = typename B::S;
   constexpr int Ng = 1 << LOGG, N = Ng / 2, H = N / 2;
@@ -267,6 +280,8 @@ __global__ void __launch_bounds__(ColBlock<R, LOGG>::THREADS) op_col_adjoint_ker
 // half-plane row p (0..ext) -> image row p: cropped, deapodized, scaled
 template <typename R, int LOGM>
 __global__ void __launch_bounds__(RowBlock<R, LOGM>::THREADS) op_row_adjoint_kernel(OpFftArgs<R> a) {
+  pdl_wait();
+  pdl_trigger();
   using B = RowBlock<R, LOGM>;
   using S = typename B::S;
   constexpr int M = 1 << LOGM, N = M, H = N / 2;
@@ -314,8 +329,7 @@ cudaError_t go(const OpFftArgs<R>& a, bool forward, int njobs, cudaStream_t s) {
           cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
     }
-    kern<<<dim3(blocks, njobs), threads, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(kern, dim3(blocks, njobs), dim3(threads), smem, s, a);
   };
   const int rows = W::N / W::RB, cols = a.ext / C::CB + 1;
   cudaError_t e;
@@ -339,6 +353,8 @@ cudaError_t go(const OpFftArgs<R>& a, bool forward, int njobs, cudaStream_t s) {
 // transforms of the whole L x L field take ten launches and move some 20 N L.
 template <typename R, int LOGM>
 __global__ void __launch_bounds__(RowBlock<R, LOGM>::THREADS) lin_row_forward_kernel(LinFftArgs<R> a) {
+  pdl_wait();
+  pdl_trigger();
   using B = RowBlock<R, LOGM>;
   using S = typename B::S;
   constexpr int M = 1 << LOGM;
@@ -376,6 +392,8 @@ __global__ void __launch_bounds__(RowBlock<R, LOGM>::THREADS) lin_row_forward_ke
 
 template <typename R, int LOGL>
 __global__ void __launch_bounds__(ColBlock<R, LOGL>::THREADS) lin_col_kernel(LinFftArgs<R> a) {
+  pdl_wait();
+  pdl_trigger();
   using B = ColBlock<R, LOGL>;
   using S = typename B::S;
   constexpr int L = 1 << LOGL, M = L / 2;
@@ -413,6 +431,8 @@ __global__ void __launch_bounds__(ColBlock<R, LOGL>::THREADS) lin_col_kernel(Lin
 
 template <typename R, int LOGM>
 __global__ void __launch_bounds__(RowBlock<R, LOGM>::THREADS) lin_row_inverse_kernel(LinFftArgs<R> a) {
+  pdl_wait();
+  pdl_trigger();
   using B = RowBlock<R, LOGM>;
   using S = typename B::S;
   constexpr int M = 1 << LOGM;
@@ -465,8 +485,7 @@ template <typename R, int LOGL> cudaError_t go_linear(const LinFftArgs<R>& a, cu
           cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
     }
-    kern<<<blocks, threads, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(kern, dim3(blocks), dim3(threads), smem, s, a);
   };
   const int rows = (a.N + W::RB - 1) / W::RB, cols = W::N / C::CB + 1;
   cudaError_t e = run(lin_row_forward_kernel<R, LOGL - 1>, rows, W::THREADS, W::SMEM);
