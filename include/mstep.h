@@ -225,7 +225,7 @@ ms_status ms_grid_static_scratch(ms_plan* plan, int32_t part, int32_t chan, cons
 
 /* Gridding of several (channel, partition) jobs at once: the work items of
  * all jobs go through one gridding launch and one fold launch, the grids
- * through one batched inverse FFT and one crop.  chans, parts, vis, dirty are
+ * through one batched inverse transform.  chans, parts, vis, dirty are
  * HOST arrays of njobs entries; vis[j] is a dev complex [nvis] array of
  * channel chans[j] in original row order, dirty[j] a dev N*N real image that
  * receives A^H y / sum(w) of the rows of parts[j] (as ms_grid would).  The
@@ -488,7 +488,7 @@ ms_status ms_warm_start_coefficients(ms_plan* plan, ms_unet* net, const void* lo
  * (for N a power of two: the row transforms, the inverse one with the
  * iteration control) and SPEC_MUL its spectral step (for N a power of two:
  * fused with the column transforms).  LINEAR_PSF is the 2N x 2N linear
- * PSF operator of the minor cycle (padding, transforms, multiply, crop) when
+ * PSF operator of the minor cycle (with its padding, product and crop) when
  * the plan uses MS_CONV_LINEAR; its objective and control kernels count as
  * SPEC_MUL. */
 typedef enum {
