@@ -266,16 +266,17 @@ void launch_crop(const C2<R>* grid, const R* psi, int npix, int Ng, double scale
 // thread interpolates visibilities: V = sum_j phi_v[j] sum_i phi_u[i] G[..].
 // One degridding work item `it` of a grid whose TMA descriptor row of the
 // grid's first row is tma_y0 (0 for one grid; job * Ng for stacked grids).
+// obs may be out (rows_apart: each row is read, then written, by one thread),
+// so neither is __restrict__.
 template <typename R, bool HAS_OBS>
 __device__ __forceinline__ void degrid_item(const CUtensorMap* tmap, int tma_y0,
                                             const C2<R>* __restrict__ grid, const WorkItem it,
                                             const uint32_t* __restrict__ cell,
                                             const C2<R>* __restrict__ frac,
-                                            const C2<R>* __restrict__ obs,
-                                            const int32_t* __restrict__ obs_idx,
-                                            C2<R>* __restrict__ out,
-                                            const int32_t* __restrict__ out_idx, int Ng, int T,
-                                            int ntx, R beta, const double* __restrict__ es_tab,
+                                            const C2<R>* obs, const int32_t* __restrict__ obs_idx,
+                                            C2<R>* out, const int32_t* __restrict__ out_idx, int Ng,
+                                            int T, int ntx, R beta,
+                                            const double* __restrict__ es_tab,
                                             int32_t* __restrict__ err) {
   // the tile sits at a 128-byte-aligned shared address (TMA destination rule),
   // the mbarrier and a flag after it, all in the dynamic allocation
@@ -389,8 +390,8 @@ template <typename R, bool HAS_OBS>
 __global__ void __launch_bounds__(degrid_threads<R>())
     degrid_kernel(const __grid_constant__ CUtensorMap tmap, const C2<R>* __restrict__ grid,
                   const WorkItem* __restrict__ items, const uint32_t* __restrict__ cell,
-                  const C2<R>* __restrict__ frac, const C2<R>* __restrict__ obs,
-                  const int32_t* __restrict__ obs_idx, C2<R>* __restrict__ out,
+                  const C2<R>* __restrict__ frac, const C2<R>* obs,
+                  const int32_t* __restrict__ obs_idx, C2<R>* out,
                   const int32_t* __restrict__ out_idx, int Ng, int T, int ntx, R beta,
                   const double* __restrict__ es_tab, int32_t* __restrict__ err) {
   degrid_item<R, HAS_OBS>(&tmap, 0, grid, items[blockIdx.x], cell, frac, obs, obs_idx, out,
