@@ -886,15 +886,30 @@ FAMILY_SOURCE = {"synth": "wavelet_kernels.cu", "synth_l1": "wavelet_kernels.cu"
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "dram_traffic_1024px_fp32.json")
 
 
+def kernel_sources(name):
+    """A kernel source and the csrc headers that it includes, directly or
+    through one another."""
+    import re
+    csrc = os.path.join(ROOT, "paper_2406_18356_gb300", "csrc")
+    found, todo = [], [name]
+    while todo:
+        f = todo.pop()
+        path = os.path.join(csrc, f)
+        if f in found or not os.path.exists(path):   # (include/mstep.h has no kernels)
+            continue
+        found.append(f)
+        with open(path) as fh:
+            todo += re.findall(r'^\s*#\s*include\s+"([^"]+)"', fh.read(), re.M)
+    return [os.path.join(csrc, f) for f in sorted(found)]
+
+
 def kernel_source_digest(fam):
-    """sha256 of the source that defines a family's kernels plus the shared
-    header: a recorded DRAM traffic is valid only for the same kernels."""
+    """sha256 of the sources that define a family's kernels, headers included:
+    a recorded DRAM traffic is valid only for the same kernels."""
     import hashlib
     h = hashlib.sha256()
-    csrc = os.path.join(ROOT, "paper_2406_18356_gb300", "csrc")
-    extra = ("fine_levels.cuh",) if FAMILY_SOURCE[fam] == "wavelet_kernels.cu" else ()
-    for f in (FAMILY_SOURCE[fam], "common.cuh") + extra:
-        with open(os.path.join(csrc, f), "rb") as fh:
+    for path in kernel_sources(FAMILY_SOURCE[fam]):
+        with open(path, "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()
 
