@@ -809,10 +809,12 @@ def fused_spectral_step(N, rsz):
     return N & (N - 1) == 0 and 16 <= N <= (8192 if rsz == 4 else 4096)
 
 
-def family_bytes(fam, N, M, J, rsz, plan):
+def family_bytes(fam, N, M, J, rsz, plan, ext=None):
     """Algorithmic HBM bytes of one span of a kernel family (what the
     operation must move at least once; per minor-cycle pass for the FISTA
-    families, per call for the operator families).  rsz = bytes of a real.
+    families, per call for the operator families).  rsz = bytes of a real,
+    ext: only the (2 ext + 1)^2 grid cells around the origin are in use (None
+    or N: all (2N)^2).
 
       analysis_l1  read the gradient image, read B_k and B_k-1 and write B_k+1
                    over the level-1 detail subbands (3 M (N/2)^2 each), write
@@ -831,14 +833,16 @@ def family_bytes(fam, N, M, J, rsz, plan):
       fft_r2c /    (our row transforms, N a power of two) read N^2 reals, write
       fft_c2r      the N (N/2 + 1) half-plane values, or the reverse.
       degrid       per row: packed cell (4 B) + offsets (2 rsz) + observed and
-                   residual value (2 x 2 rsz), plus one read of the (2N)^2
-                   complex grid.
+                   residual value (2 x 2 rsz), plus one read of the complex
+                   grid's cells in use.
       grid         per row: packed cell + offsets + value (4 + 4 rsz), plus one
-                   write of the (2N)^2 complex grid.
+                   write of the complex grid's cells in use.
       fold         (the design's reduction of the gridding tiles) every work
-                   item's scratch tile read once, the grid written once.
+                   item's scratch tile read once, the grid's cells in use
+                   written once.
     """
     q = lambda j: (N >> j) ** 2   # subband side^2 at level j
+    grid = 2 * rsz * (4 * N * N if ext is None or ext >= N else (2 * ext + 1) ** 2)
     if fam == "analysis_l1":
         return (N * N + 9 * M * q(1) + M * q(1)) * rsz
     if fam == "analysis":
@@ -860,20 +864,19 @@ def family_bytes(fam, N, M, J, rsz, plan):
     if fam == "degrid":
         counts = plan.partition_counts()
         rows = (counts["L"] + counts["H"]) / 2.0
-        return rows * (4 + 2 * rsz + 4 * rsz) + 4 * N * N * 2 * rsz
+        return rows * (4 + 2 * rsz + 4 * rsz) + grid
     if fam == "grid":
-        # per row: packed cell (4 B) + offsets (2 rsz) + value (2 rsz); one
-        # write of the (2N)^2 complex grid
+        # per row: packed cell (4 B) + offsets (2 rsz) + value (2 rsz)
         counts = plan.partition_counts()
         rows = (counts["L"] + counts["H"]) / 2.0
-        return rows * (4 + 4 * rsz) + 4 * N * N * 2 * rsz
+        return rows * (4 + 4 * rsz) + grid
     if fam == "fold":
         # the design's reduction: read every work item's scratch tile, write
-        # the grid once (mean of the two partitions' calls)
+        # the cells in use once (mean of the two partitions' calls)
         b = 0.0
         for part in ("L", "H"):
             items, cells, cell_bytes = plan.partition_layout(part)
-            b += items * cells * cell_bytes + 4 * N * N * 2 * rsz
+            b += items * cells * cell_bytes + grid
         return b / 2.0
     return None
 
@@ -939,16 +942,17 @@ def roofline_of(prof, w, plan, args):
     hbm, kind = _peaks()
     rsz = 4 if args.precision != "fp64" else 8
     N, M, J = w.npix, 8, 4
+    ext = plan.grid_extent() if plan is not None else None
     ours_fft = fused_spectral_step(N, rsz)   # else the FISTA transforms are cuFFT's
     mine = {k: v for k, v in prof.items()
             if (ours_fft or not k.startswith("fft")) and k != "fft_grid" and v[0] > 0}
     fam = max(mine, key=lambda k: mine[k][1])
     launches, total_ms = mine[fam]
     avg_s = total_ms / launches / 1000.0
-    bytes_ = family_bytes(fam, N, M, J, rsz, plan)
+    bytes_ = family_bytes(fam, N, M, J, rsz, plan, ext)
     others = {}
     for k, (n, t) in mine.items():
-        b = family_bytes(k, N, M, J, rsz, plan)
+        b = family_bytes(k, N, M, J, rsz, plan, ext)
         if b:
             others[k] = round(b / (t / n / 1000.0) / 1e9 / hbm, 4)
     if bytes_ is None:

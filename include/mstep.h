@@ -181,6 +181,10 @@ ms_status ms_partition_counts(ms_plan* plan, int32_t chan, int64_t out[4]);
  * scratch cell (8 for FP32, 16 for FP64 and the compensated FP32 form). */
 ms_status ms_partition_layout(ms_plan* plan, int32_t part, int32_t chan, int64_t out[3]);
 
+/* The cells of the 2N x 2N grid in use: those within +-*cells of the origin in
+ * both axes (N: the whole grid). */
+ms_status ms_grid_extent(ms_plan* plan, int32_t* cells);
+
 /* The rows of partition `part` in the plan's sorted (tile) order, copied to
  * host `rows` [count]; count = ms_partition_counts of that partition. */
 ms_status ms_partition_rows(ms_plan* plan, int32_t part, int32_t chan, int32_t* rows);

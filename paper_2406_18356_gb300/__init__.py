@@ -90,6 +90,7 @@ _SIGNATURES = {
     "ms_partition_counts": [_P, _I32, ctypes.POINTER(_I64)],
     "ms_partition_rows": [_P, _I32, _I32, _P],
     "ms_partition_layout": [_P, _I32, _I32, ctypes.POINTER(_I64)],
+    "ms_grid_extent": [_P, ctypes.POINTER(_I32)],
     "ms_degrid": [_P, _I32, _I32, _P, _P, _P, _P],
     "ms_grid": [_P, _I32, _I32, _P, _P, _P],
     "ms_grid_static_scratch": [_P, _I32, _I32, _P, _P, _P],
@@ -325,6 +326,12 @@ class Plan:
         out = (_I64 * 3)()
         self._check(self._lib.ms_partition_layout(self._h, PARTS[part], chan, out))
         return int(out[0]), int(out[1]), int(out[2])
+
+    def grid_extent(self) -> int:
+        """cells of the 2N grid beyond +- this of its origin are not used"""
+        out = _I32()
+        self._check(self._lib.ms_grid_extent(self._h, ctypes.byref(out)))
+        return out.value
 
     def partition_rows(self, part: str, chan: int = 0) -> np.ndarray:
         n = self.partition_counts(chan)[part]
@@ -645,6 +652,10 @@ def ms_partition_counts(plan: Plan, chan: int = 0):
 
 def ms_partition_layout(plan: Plan, part: str, chan: int = 0):
     return plan.partition_layout(part, chan)
+
+
+def ms_grid_extent(plan: Plan):
+    return plan.grid_extent()
 
 
 def ms_partition_rows(plan: Plan, part: str, chan: int = 0):

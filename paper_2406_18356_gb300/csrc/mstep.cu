@@ -3003,6 +3003,13 @@ ms_status ms_partition_layout(ms_plan* p, int32_t part, int32_t chan, int64_t ou
   });
 }
 
+ms_status ms_grid_extent(ms_plan* p, int32_t* cells) {
+  return guarded(p, [&] {
+    arg(cells != nullptr, "cells is NULL");
+    *cells = p->ext;
+  });
+}
+
 ms_status ms_partition_rows(ms_plan* p, int32_t part, int32_t chan, int32_t* rows) {
   return guarded(p, [&] {
     PartDev& pd = part_of(p, part, chan);

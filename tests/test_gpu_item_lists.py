@@ -29,8 +29,8 @@ def tile_of(gu, gv, Ng, tile):
 def observation(N, tile, items):
     """u, v whose longest list has `items` work items of CHUNK rows (the last
     one five rows short): all its rows anchor in one tile near the origin, no
-    other tile has more than one item; the outermost footprint reaches cell 439
-    / 512 N."""
+    other tile has more than one item; at 512 px the outermost footprint reaches
+    cell 439."""
     rng = np.random.default_rng(items)
     Ng = 2 * N
     corner = (Ng // 2 // tile) * tile - Ng // 2   # grid cell of the tile's first anchor
@@ -77,4 +77,18 @@ def test_fold_of_long_lists(precision, N, tile, items):
     both = plan.grid_batch([(0, "ALL"), (0, "L")], [d, d])
     np.testing.assert_array_equal(both[0].cpu().numpy(), got)
     assert torch.equal(both[1], plan.grid("L", d))
+    plan.close()
+
+
+# (48: cuFFT sides use the whole grid)
+@pytest.mark.gpu
+@pytest.mark.parametrize("N,want", [(48, 48), (64, 58), (512, 439)])
+def test_grid_extent(N, want):
+    import paper_2406_18356_gb300 as ms
+    u, v = observation(N, 16, 2)
+    plan = ms.Plan(u, v, N, DL, 9.0, 2.0, levels=2)
+    A = og.GriddedOperator(u, v, N, DL)
+    if N != 48:
+        assert want == max(np.abs(c).max() for a in (A.c0u, A.c0v) for c in (a, a + 6))
+    assert plan.grid_extent() == want
     plan.close()
