@@ -332,10 +332,10 @@ cudaError_t launch_op_fft(const OpFftArgs<R>& a, bool forward, int njobs, cudaSt
 int lin_fft_length(int N, size_t rsz);
 template <typename R> cudaError_t launch_lin_fft(const LinFftArgs<R>& a, int L, cudaStream_t s);
 template <typename R> void launch_lin_spectrum(const R* H2, R* H, int L, cudaStream_t s);
-template <typename R> void launch_lin_widen(const R* H2, double2* out, int64_t n, cudaStream_t s);
-void launch_lin_embed(const double* psf, double* out, int N, int L, cudaStream_t s);
+// half: 2N - 1 rows of `pitch` values; tw: exp(-2 pi i m / L), m < L
 template <typename R>
-void launch_lin_spectrum_of(const double2* spec, R* H, int L, cudaStream_t s);
+cudaError_t launch_lin_psf(const R* psf, C2<R>* half, R* H, const C2<R>* tw, int N, int L,
+                           int pitch, cudaStream_t s);
 
 // wavelet_kernels.cu
 void set_wavelet_filters(const double* h, const int* len, int nbases);   // host -> __constant__

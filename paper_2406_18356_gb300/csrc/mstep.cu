@@ -2813,44 +2813,23 @@ void* static_grid_scratch(int dev) {
 
 }  // namespace
 
-// The FP64 buffers and plans of build_linear_spectrum, made on first use and
-// shared by a plan's channels and partitions.
-struct LinearEmbedding {
-  void *img = nullptr, *emb = nullptr, *spec = nullptr;
-  cufftHandle inv = 0, fwd = 0;
-  void init(int P, int L, cudaStream_t s) {
-    if (fwd) return;
-    ck(cudaMalloc(&img, sizeof(double) * P * P), "linear PSF image");
-    ck(cudaMalloc(&emb, sizeof(double) * L * L), "linear PSF image");
-    ck(cudaMalloc(&spec, sizeof(double2) * L * (L / 2 + 1)), "linear PSF spectrum");
-    ckf(cufftPlan2d(&inv, P, P, CUFFT_Z2D), "plan Z2D");
-    ckf(cufftPlan2d(&fwd, L, L, CUFFT_D2Z), "plan D2Z");
-    for (cufftHandle h : {inv, fwd}) ckf(cufftSetStream(h, s), "set stream");
-  }
-  ~LinearEmbedding() {
-    for (cufftHandle h : {inv, fwd})
-      if (h) cufftDestroy(h);
-    for (void* q : {img, emb, spec})
-      if (q) cudaFree(q);
-  }
-};
-
-// pd.Hlin, H2^ as the own transforms of length lin_L read it, on stream s.
-// For lin_L > 2N the PSF goes through its image, in FP64.
+// pd.Hlin, H2^ as the own transforms of length lin_L read it, from the PSF
+// that ensure_psf has just left in q (the 2N x 2N plan) as spectrum and image:
+// the same values for L = 2N; else the image on the longer field, transformed
+// in q's grid buffer (16 N^2 complex values; 2N rows of L / 2 + 4 take less).
+// (Built at 448 px, FP32, with one and four channels: 16.9 and 24.1 ms; through
+// the PSF's spectrum, two FP64 cuFFT plans and their transforms 19.4 and 29.6,
+// with the spectrum of the 2N x 2N field alone 17.6 and 23.5.)
 template <typename R>
-void build_linear_spectrum(ms_plan* p, PartDev& pd, LinearEmbedding& w, cudaStream_t s) {
-  const int N = p->N, P = 2 * N, L = p->lin_L;
+void build_linear_spectrum(ms_plan* p, PartDev& pd, ms_plan* q, PartDev& qd) {
+  const int N = p->N, L = p->lin_L;
   pd.Hlin = p->alloc<R>((size_t)L * (L / 2 + 1), "linear PSF spectrum");
-  if (L == P) {
-    launch_lin_spectrum<R>((const R*)pd.Hhat2, (R*)pd.Hlin, L, s);
-  } else {
-    w.init(P, L, s);
-    launch_lin_widen<R>((const R*)pd.Hhat2, (double2*)w.spec, (int64_t)P * (N + 1), s);
-    exec_c2r<double>(w.inv, w.spec, w.img);
-    launch_lin_embed((const double*)w.img, (double*)w.emb, N, L, s);
-    exec_r2c<double>(w.fwd, w.emb, w.spec);
-    launch_lin_spectrum_of<R>((const double2*)w.spec, (R*)pd.Hlin, L, s);
-  }
+  if (L == 2 * N)
+    launch_lin_spectrum<R>((const R*)qd.Hhat, (R*)pd.Hlin, L, q->ps);
+  else
+    ck(launch_lin_psf<R>((const R*)q->img[5], (C2<R>*)q->grid, (R*)pd.Hlin, (const C2<R>*)p->ltw, N,
+                         L, lin_pitch(L), q->ps),
+       "linear PSF spectrum");
   ck(cudaGetLastError(), "linear PSF spectrum");
 }
 
@@ -2876,7 +2855,6 @@ template <typename R> void build_linear_psf(ms_plan* p, const ms_plan_desc* d) {
   const size_t bytes = sizeof(R) * 2 * p->N * (p->N + 1);
   try {
     ck(cudaSetDevice(q->dev), "set device");
-    LinearEmbedding embedding;
     for (size_t c = 0; c < p->ch.size(); ++c)
       for (int pt = 0; pt < 3; ++pt) {
         PartDev& qd = q->ch[c].part[pt];
@@ -2884,7 +2862,7 @@ template <typename R> void build_linear_psf(ms_plan* p, const ms_plan_desc* d) {
         PartDev& pd = p->ch[c].part[pt];
         pd.Hhat2 = p->alloc<R>(bytes / sizeof(R), "linear PSF spectrum");
         ck(cudaMemcpyAsync(pd.Hhat2, qd.Hhat, bytes, cudaMemcpyDeviceToDevice, q->ps), "copy");
-        if (p->lin_L) build_linear_spectrum<R>(p, pd, embedding, q->ps);
+        if (p->lin_L) build_linear_spectrum<R>(p, pd, q, qd);
         ck(cudaStreamSynchronize(q->ps), "synchronize");
       }
   } catch (...) {

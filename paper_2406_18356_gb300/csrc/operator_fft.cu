@@ -165,6 +165,24 @@ template <typename R> __device__ __forceinline__ OpFftJob<R> pick_job(const OpFf
   return o;
 }
 
+// The spectrum out[0..last] of a real row of 2M elements from buf, the M-point
+// transform of z_n = x_2n + i x_2n+1: X_k = E_k + W^k O_k, E, O the transforms
+// of the even and odd elements (thread t of tps).
+template <typename R, int M>
+__device__ __forceinline__ void unpack_real_row(const C2<R>* buf, const C2<R>* __restrict__ tw,
+                                                C2<R>* out, int last, int t, int tps) {
+  for (int k = t; k <= last; k += tps) {
+    const C2<R> zk = buf[padi(k == M ? 0 : k)], zm = buf[padi(k == 0 ? 0 : M - k)];
+    const R ex = (R)0.5 * (zk.x + zm.x), ey = (R)0.5 * (zk.y - zm.y);
+    const R ox = (R)0.5 * (zk.y + zm.y), oy = (R)-0.5 * (zk.x - zm.x);
+    const C2<R> w = tw[k];
+    C2<R> X;
+    X.x = ex + (w.x * ox - w.y * oy);
+    X.y = ey + (w.x * oy + w.y * ox);
+    out[k] = X;
+  }
+}
+
 // image row p, deapodized and centred -> its half-plane spectrum 0..ext
 template <typename R, int LOGM>
 __global__ void __launch_bounds__(RowBlock<R, LOGM>::THREADS) op_row_forward_kernel(OpFftArgs<R> a) {
@@ -194,18 +212,7 @@ __global__ void __launch_bounds__(RowBlock<R, LOGM>::THREADS) op_row_forward_ker
   auto keep = [&](int k, C2<R> z) { buf[padi(k)] = z; };
   transform<R, LOGM, S::LE, false>(buf, a.tw, 2, t, load, keep);
   __syncthreads();
-  // X_k = E_k + W^k O_k, E, O the transforms of the even and odd elements
-  C2<R>* out = jb.half + (int64_t)p * a.pitch;
-  for (int k = t; k <= a.ext; k += S::TPS) {
-    const C2<R> zk = buf[padi(k == M ? 0 : k)], zm = buf[padi(k == 0 ? 0 : M - k)];
-    const R ex = (R)0.5 * (zk.x + zm.x), ey = (R)0.5 * (zk.y - zm.y);
-    const R ox = (R)0.5 * (zk.y + zm.y), oy = (R)-0.5 * (zk.x - zm.x);
-    const C2<R> w = a.tw[k];
-    C2<R> X;
-    X.x = ex + (w.x * ox - w.y * oy);
-    X.y = ey + (w.x * oy + w.y * ox);
-    out[k] = X;
-  }
+  unpack_real_row<R, M>(buf, a.tw, jb.half + (int64_t)p * a.pitch, a.ext, t, S::TPS);
 }
 
 // columns u of the half plane -> grid columns u and -u, rows -ext..ext
@@ -376,18 +383,7 @@ __global__ void __launch_bounds__(RowBlock<R, LOGM>::THREADS) lin_row_forward_ke
   transform<R, LOGM, S::LE, false>(buf, a.tw, 2, t, load, keep);
   __syncthreads();
   if (!live) return;
-  // X_k = E_k + W^k O_k, E, O the transforms of the even and odd elements
-  C2<R>* out = a.half + (int64_t)p * a.pitch;
-  for (int k = t; k <= M; k += S::TPS) {
-    const C2<R> zk = buf[padi(k == M ? 0 : k)], zm = buf[padi(k == 0 ? 0 : M - k)];
-    const R ex = (R)0.5 * (zk.x + zm.x), ey = (R)0.5 * (zk.y - zm.y);
-    const R ox = (R)0.5 * (zk.y + zm.y), oy = (R)-0.5 * (zk.x - zm.x);
-    const C2<R> w = a.tw[k];
-    C2<R> X;
-    X.x = ex + (w.x * ox - w.y * oy);
-    X.y = ey + (w.x * oy + w.y * ox);
-    out[k] = X;
-  }
+  unpack_real_row<R, M>(buf, a.tw, a.half + (int64_t)p * a.pitch, M, t, S::TPS);
 }
 
 template <typename R, int LOGL>
@@ -494,37 +490,94 @@ template <typename R, int LOGL> cudaError_t go_linear(const LinFftArgs<R>& a, cu
   return e;
 }
 
-// H^ of the L x L field as lin_col_kernel reads it, from the DFT of the
-// re-embedded PSF (or from the real spectrum of the 2N x 2N field, L = 2N)
-template <typename R, typename T>
-__global__ void lin_spectrum_kernel(const T* __restrict__ in, int step, R* __restrict__ H, int L) {
+// H^ as lin_col_kernel reads it from H2, the real spectrum on the 2N x 2N
+// field (L = 2N)
+template <typename R>
+__global__ void lin_spectrum_kernel(const R* __restrict__ H2, R* __restrict__ H, int L) {
   const int nc = L / 2 + 1;
   const double inv = 1.0 / ((double)L * L);
   const int64_t total = (int64_t)L * nc;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < total;
        k += (int64_t)gridDim.x * blockDim.x) {
     const int64_t u = k / L, v = k - u * L;
-    H[k] = (R)((double)in[(v * nc + u) * step] * inv);
+    H[k] = (R)((double)H2[v * nc + u] * inv);
   }
 }
-template <typename R>
-__global__ void lin_widen_kernel(const R* __restrict__ in, double2* __restrict__ out, int64_t n) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-       k += (int64_t)gridDim.x * blockDim.x)
-    out[k] = make_double2((double)in[k], 0.0);
+
+// H^ of the L x L field from the PSF image (plan time): rows, then columns, as
+// the operator's transforms, whose tables and block shapes serve.  The image
+// has side P = 2N and its origin at (0, 0); of the L-field only rows and
+// columns at offsets below +-N are not zero, 2N - 1 of each.
+template <typename R, int LOGM>
+__global__ void __launch_bounds__(RowBlock<R, LOGM>::THREADS)
+    lin_psf_row_kernel(const R* __restrict__ psf, C2<R>* __restrict__ half,
+                       const C2<R>* __restrict__ tw, int N, int pitch) {
+  using B = RowBlock<R, LOGM>;
+  using S = typename B::S;
+  constexpr int M = 1 << LOGM, L = 2 * M;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int rr = threadIdx.x / S::TPS, t = threadIdx.x - rr * S::TPS;
+  const int p = blockIdx.x * B::RB + rr;
+  const bool live = p < 2 * N - 1;
+  C2<R>* buf = reinterpret_cast<C2<R>*>(smem_raw) + rr * S::P;
+  // row p: offset p, or p - (2N - 1) from N on
+  const R* row = psf + (int64_t)(p < N ? p : p + 1) * (2 * N);
+  auto at = [&](int x) {
+    return live && (x < N || x > L - N) ? row[x < N ? x : x - L + 2 * N] : (R)0;
+  };
+  auto load = [&](int n) {
+    C2<R> z;
+    z.x = at(2 * n);
+    z.y = at(2 * n + 1);
+    return z;
+  };
+  auto keep = [&](int k, C2<R> z) { buf[padi(k)] = z; };
+  transform<R, LOGM, S::LE, false>(buf, tw, 2, t, load, keep);
+  __syncthreads();
+  if (live) unpack_real_row<R, M>(buf, tw, half + (int64_t)p * pitch, M, t, S::TPS);
 }
-// the PSF at offsets below +-N of the P x P field, on the L x L field
-__global__ void lin_embed_kernel(const double* __restrict__ in, double* __restrict__ out, int N,
-                                 int L) {
-  const int P = 2 * N;
-  const double inv = 1.0 / ((double)P * P);
-  const int64_t total = (int64_t)L * L;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < total;
-       k += (int64_t)gridDim.x * blockDim.x) {
-    const int y = (int)(k / L), x = (int)(k - (int64_t)y * L);
-    const int sy = y < N ? y : y - L + P, sx = x < N ? x : x - L + P;
-    out[k] = (y < N || sy > N) && (x < N || sx > N) ? in[(int64_t)sy * P + sx] * inv : 0.0;
-  }
+
+template <typename R, int LOGL>
+__global__ void __launch_bounds__(ColBlock<R, LOGL>::THREADS)
+    lin_psf_col_kernel(const C2<R>* __restrict__ half, R* __restrict__ H,
+                       const C2<R>* __restrict__ tw, int N, int pitch) {
+  using B = ColBlock<R, LOGL>;
+  using S = typename B::S;
+  constexpr int L = 1 << LOGL;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int c = threadIdx.x % B::CB, t = threadIdx.x / B::CB;
+  const int u = blockIdx.x * B::CB + c;
+  const bool live = u <= L / 2;
+  C2<R>* buf = reinterpret_cast<C2<R>*>(smem_raw) + c * S::P;
+  auto load = [&](int n) {
+    C2<R> z;
+    z.x = z.y = (R)0;
+    if (live && (n < N || n > L - N))
+      z = half[(int64_t)(n < N ? n : n - L + 2 * N - 1) * pitch + u];
+    return z;
+  };
+  auto store = [&](int v, C2<R> z) {   // (L^2: a power of two)
+    if (live) H[(int64_t)u * L + v] = z.x * ((R)1 / ((R)L * (R)L));
+  };
+  transform<R, LOGL, S::LE, false>(buf, tw, 1, t, load, store);
+}
+
+template <typename R, int LOGL>
+cudaError_t go_psf(const R* psf, C2<R>* half, R* H, const C2<R>* tw, int N, int pitch,
+                   cudaStream_t s) {
+  using C = ColBlock<R, LOGL>;
+  using W = RowBlock<R, LOGL - 1>;
+  auto rows = lin_psf_row_kernel<R, LOGL - 1>;
+  auto cols = lin_psf_col_kernel<R, LOGL>;
+  cudaError_t e = cudaSuccess;
+  if (W::SMEM > 48 * 1024)
+    e = cudaFuncSetAttribute(rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W::SMEM);
+  if (e == cudaSuccess && C::SMEM > 48 * 1024)
+    e = cudaFuncSetAttribute(cols, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+  if (e != cudaSuccess) return e;
+  rows<<<(2 * N - 1 + W::RB - 1) / W::RB, W::THREADS, W::SMEM, s>>>(psf, half, tw, N, pitch);
+  cols<<<W::N / C::CB + 1, C::THREADS, C::SMEM, s>>>(half, H, tw, N, pitch);
+  return cudaGetLastError();
 }
 }  // namespace
 
@@ -584,29 +637,29 @@ template <typename R> cudaError_t launch_lin_fft(const LinFftArgs<R>& a, int L, 
   }
 }
 
-// H from H2, the real spectrum on the 2N x 2N field: directly (L = 2N), or
-// through the PSF's image in FP64 (widen, inverse transform, embed, transform,
-// spectrum_of)
 template <typename R>
 void launch_lin_spectrum(const R* H2, R* H, int L, cudaStream_t s) {
-  lin_spectrum_kernel<R, R><<<1024, 256, 0, s>>>(H2, 1, H, L);
-}
-template <typename R> void launch_lin_widen(const R* H2, double2* out, int64_t n, cudaStream_t s) {
-  lin_widen_kernel<R><<<1024, 256, 0, s>>>(H2, out, n);
-}
-void launch_lin_embed(const double* psf, double* out, int N, int L, cudaStream_t s) {
-  lin_embed_kernel<<<1024, 256, 0, s>>>(psf, out, N, L);
+  lin_spectrum_kernel<R><<<1024, 256, 0, s>>>(H2, H, L);
 }
 template <typename R>
-void launch_lin_spectrum_of(const double2* spec, R* H, int L, cudaStream_t s) {
-  lin_spectrum_kernel<R, double>
-      <<<1024, 256, 0, s>>>(reinterpret_cast<const double*>(spec), 2, H, L);
+cudaError_t launch_lin_psf(const R* psf, C2<R>* half, R* H, const C2<R>* tw, int N, int L,
+                           int pitch, cudaStream_t s) {
+  switch (L) {
+    case 128: return go_psf<R, 7>(psf, half, H, tw, N, pitch, s);
+    case 256: return go_psf<R, 8>(psf, half, H, tw, N, pitch, s);
+    case 512: return go_psf<R, 9>(psf, half, H, tw, N, pitch, s);
+    case 1024: return go_psf<R, 10>(psf, half, H, tw, N, pitch, s);
+    case 2048: return go_psf<R, 11>(psf, half, H, tw, N, pitch, s);
+    case 4096: return go_psf<R, 12>(psf, half, H, tw, N, pitch, s);
+    case 8192: return go_psf<R, 13>(psf, half, H, tw, N, pitch, s);
+    default: return cudaErrorInvalidValue;
+  }
 }
 #define MS_INST(R)                                                                       \
   template cudaError_t launch_lin_fft<R>(const LinFftArgs<R>&, int, cudaStream_t);       \
   template void launch_lin_spectrum<R>(const R*, R*, int, cudaStream_t);                 \
-  template void launch_lin_widen<R>(const R*, double2*, int64_t, cudaStream_t);          \
-  template void launch_lin_spectrum_of<R>(const double2*, R*, int, cudaStream_t);
+  template cudaError_t launch_lin_psf<R>(const R*, C2<R>*, R*, const C2<R>*, int, int,   \
+                                         int, cudaStream_t);
 MS_INST(float)
 MS_INST(double)
 #undef MS_INST
