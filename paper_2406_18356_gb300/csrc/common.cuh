@@ -6,6 +6,8 @@
 #include <cufft.h>
 #include <stdint.h>
 
+#include "es_tables.h"
+
 namespace ms {
 
 template <typename R> struct CplxOf;
@@ -13,25 +15,9 @@ template <> struct CplxOf<float> { using T = float2; };
 template <> struct CplxOf<double> { using T = double2; };
 template <typename R> using C2 = typename CplxOf<R>::T;
 
-constexpr int kW = 7;          // ES kernel support in cells
-constexpr int kHalfW = 3;      // (W - 1) / 2
 constexpr int kMaxBases = 8;   // db1 .. db8
 constexpr int kMaxTaps = 16;   // db8 has 16 taps
 constexpr int kMaxLevels = 8;
-
-// The gridding kernel: its shape and, for FP64 plans, the device tables of
-// its taps' weights (nullptr: evaluated directly): kEsSegs segments of the
-// inner taps (5 x 7 polynomial coefficients, the segment's centre, one pad),
-// then of the outer taps (9 coefficients, the centre, one pad).  Odd strides,
-// so that lanes in different segments read different banks.
-struct EsKernel {
-  double beta = 0;
-  const double* tab = nullptr;
-};
-constexpr int kEsSegs = 64, kEsInner = 37, kEsOuter = 11;
-constexpr int kEsTable = kEsSegs * (kEsInner + kEsOuter);
-constexpr double kEsOuterRange = 0.7;   // of v = sqrt(1 - z^2) at |z| >= 5/7
-constexpr double kEsMaxBeta = 32.0;     // the tables' accuracy holds up to here
 
 // One unit of (de)gridding work: `count` sorted rows starting at `start`
 // that all anchor in grid tile `tile`.

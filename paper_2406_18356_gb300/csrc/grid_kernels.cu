@@ -123,44 +123,6 @@ __device__ __forceinline__ void es_weights<float>(float f, float beta, float* w)
   }
 }
 
-// FP64 weights from the plan's tables (EsKernel): the inner five taps are
-// degree-6 polynomials of f on 64 segments of its range, the outer two
-// exp(beta (v - 1)), a degree-8 polynomial on 64 segments of v = sqrt(1 - z^2)
-// in [0, 0.7) (smooth there; in f they have a square-root end point).  Their
-// errors are below 1e-16 of the kernel's peak.  A scheduler issues one FP64
-// instruction per 76 cycles, and the library's exp, sqrt and division spend
-// most of the operator's on the 14 weights of a row: some 170 of them this
-// way.  Measured at 128 px, 31,744 rows (with the smaller work items): the
-// residual image 374 -> 203 us, degridding 20.9 and gridding 30.9 us of it;
-// 5.9M rows 16.1 -> 9.0 ms.
-__device__ __forceinline__ void es_weights_tab(double f, const double* tab, double* w) {
-  const int seg = min(max((int)(((float)f + 0.5f) * kEsSegs), 0), kEsSegs - 1);
-  const double* c = tab + seg * kEsInner;
-  const double x = f - c[kEsInner - 2];
-#pragma unroll
-  for (int i = 1; i < kW - 1; ++i) {
-    const double* q = c + (i - 1) * 7;
-    double a = q[6];
-#pragma unroll
-    for (int k = 5; k >= 0; --k) a = fma(a, x, q[k]);
-    w[i] = a;
-  }
-#pragma unroll
-  for (int i = 0; i < kW; i += kW - 1) {
-    const double t = f + (double)(kHalfW - i);
-    double s = fma(t * (-4.0 / (kW * kW)), t, 1.0);
-    s = s > 0.0 ? s : 0.0;
-    const double v = sqrt(s);
-    const double* q = tab + kEsSegs * kEsInner +
-                      min((int)((float)v * (float)(kEsSegs / kEsOuterRange)), kEsSegs - 1) * kEsOuter;
-    const double y = v - q[kEsOuter - 2];
-    double a = q[8];
-#pragma unroll
-    for (int k = 7; k >= 0; --k) a = fma(a, y, q[k]);
-    w[i] = a;
-  }
-}
-
 // the weights of one axis: FP64 from the tables where the plan has them
 // (staged in shared memory), else directly
 template <typename R> struct EsWeights {

@@ -150,75 +150,6 @@ void gauss_legendre(int n, std::vector<double>& x, std::vector<double>& w) {
   }
 }
 
-// Matrix [n][n] from the values of a function at the n Chebyshev nodes x_i =
-// cos(pi (2i + 1) / 2n) of [-1, 1] to the monomial coefficients of its
-// interpolating polynomial (Newton's divided differences of unit vectors).
-std::vector<double> chebyshev_fit(int n, std::vector<double>* nodes) {
-  const long double pi = 3.141592653589793238462643383279502884L;
-  std::vector<long double> x(n);
-  for (int i = 0; i < n; ++i) x[i] = std::cos(pi * (2 * i + 1) / (2.0L * n));
-  if (n % 2) x[n / 2] = 0.0L;
-  nodes->assign(x.begin(), x.end());
-  std::vector<double> m(n * n);
-  for (int u = 0; u < n; ++u) {
-    std::vector<long double> d(n, 0.0L), p(n, 0.0L);
-    d[u] = 1.0L;
-    for (int k = 1; k < n; ++k)
-      for (int i = n - 1; i >= k; --i) d[i] = (d[i] - d[i - 1]) / (x[i] - x[i - k]);
-    for (int i = n - 1; i >= 0; --i) {   // p <- p (x - x_i) + d_i
-      for (int k = n - 1; k >= 1; --k) p[k] = p[k - 1] - x[i] * p[k];
-      p[0] = d[i] - x[i] * p[0];
-    }
-    for (int k = 0; k < n; ++k) m[k * n + u] = (double)p[k];
-  }
-  return m;
-}
-
-// The FP64 weight tables (see EsKernel) of the ES kernel with shape beta.  A
-// segment's polynomial interpolates the differences from its centre value
-// (relative to it, through expm1, so that they keep their digits); the inner
-// taps i and 6 - i mirror each other, and the outer function's segments are
-// one polynomial of exp(beta x) times their centre values.
-std::vector<double> es_tables(double beta) {
-  std::vector<double> t(kEsTable, 0.0), x7, x9;
-  const std::vector<double> f7 = chebyshev_fit(7, &x7), f9 = chebyshev_fit(9, &x9);
-  const double c2 = 4.0 / (kW * kW), h = 0.5 / kEsSegs, ho = 0.5 * kEsOuterRange / kEsSegs;
-  // out[k] = a c_k / h^k, c the fit of d (d = 0 at the centre), out[0] = a
-  auto put = [](const std::vector<double>& fit, int n, const double* d, double a, double h,
-                double* out) {
-    double hk = 1.0;
-    out[0] = a;
-    for (int k = 1; k < n; ++k) {
-      double s = 0.0;
-      hk *= h;
-      for (int i = 0; i < n; ++i) s += fit[k * n + i] * d[i];
-      out[k] = a * s / hk;
-    }
-  };
-  double d9[9];
-  for (int i = 0; i < 9; ++i) d9[i] = std::expm1(beta * ho * x9[i]);
-  for (int g = 0; g < kEsSegs; ++g) {
-    const double c = -0.5 + (2 * g + 1) * h;
-    double* q = &t[g * kEsInner];
-    q[kEsInner - 2] = c;
-    for (int i = 1; i <= kHalfW; ++i) {
-      const double tc = c + (kHalfW - i), z2 = tc * tc * c2, sc = std::sqrt(1.0 - z2);
-      double d[7];
-      for (int n = 0; n < 7; ++n) {
-        const double x = h * x7[n], ds = -c2 * x * (2.0 * tc + x);   // s(tc + x) - s(tc)
-        d[n] = std::expm1(beta * ds / (std::sqrt(1.0 - z2 + ds) + sc));
-      }
-      put(f7, 7, d, std::exp(-beta * z2 / (1.0 + sc)), h, q + (i - 1) * 7);
-      double* mirror = &t[(kEsSegs - 1 - g) * kEsInner] + (kW - 2 - i) * 7;
-      for (int k = 0; k < 7 && i < kHalfW; ++k) mirror[k] = (k & 1 ? -1 : 1) * q[(i - 1) * 7 + k];
-    }
-    double* o = &t[kEsSegs * kEsInner + g * kEsOuter];
-    o[kEsOuter - 2] = (2 * g + 1) * ho;
-    put(f9, 9, d9, std::exp(beta * (o[kEsOuter - 2] - 1.0)), ho, o);
-  }
-  return t;
-}
-
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
                                   const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
                                   const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
