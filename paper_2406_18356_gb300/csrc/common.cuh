@@ -500,7 +500,10 @@ void launch_lin_full_spec(const C2<R>* dek, const C2<R>* dep, const R* gl2, cons
                           C2<R>* uv, int N, double* parts, FistaCtl* ctl, double* trace,
                           int32_t* ticket, const double* l1_parts, int n_l1, cudaStream_t s);
 template <typename R>
-void launch_lin_theta(const R* H2, int N, const R* gl2, const R* gh2, int M, double* parts,
+void launch_lin_peak(const R* H2, int64_t n, double* parts, double* out, int32_t* ticket,
+                     cudaStream_t s);
+template <typename R>
+void launch_lin_theta(const double* peak, int N, const R* gl2, const R* gh2, int M, double* parts,
                       FistaCtl* ctl, int32_t* ticket, cudaStream_t s);
 
 }  // namespace ms

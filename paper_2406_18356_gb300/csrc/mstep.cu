@@ -239,8 +239,11 @@ struct PartDev {
   int32_t* tile_items = nullptr;
   void* Hhat = nullptr;
   bool have_psf = false;
-  void* Hhat2 = nullptr;   // real spectrum of the PSF on the 2N x 2N field (linear operator)
-  void* Hlin = nullptr;    // ... by columns at the length of the own transforms
+  // linear operator: the PSF's real spectrum as its transforms read it (on the
+  // 2N x 2N field, or by columns at the length of the own ones), and the
+  // largest square of that on the 2N x 2N field
+  void* Hhat2 = nullptr;
+  double* h2_peak = nullptr;
 };
 
 // Batched minor cycles: each job's FISTA state as one slice of these arrays
@@ -530,6 +533,22 @@ template <typename R> void fft_c2c(ms_plan* p, int dir) {
 
 // row pitch of the linear operator's half plane: whole 32-byte sectors
 int lin_pitch(int L) { return L / 2 + 4; }
+// values of the linear operator's spectrum (L: the own transforms' length)
+size_t lin_spectrum_values(int N, int L) {
+  return L ? (size_t)L * (L / 2 + 1) : (size_t)2 * N * (N + 1);
+}
+size_t lin_spectrum_values(const ms_plan* p) { return lin_spectrum_values(p->N, p->lin_L); }
+
+// The length of a linear plan's own transforms, or 0 (cuFFT).  The spectra of
+// every channel and partition at a length above 2N take up to 2.6 times those
+// of the 2N x 2N field: only where that is at most 4 GiB more, so that a plan
+// of many channels fits wherever it would with cuFFT (whose work fields of 14
+// N^2 values and plans are larger than the own transforms' of 5 to 8).
+int lin_length(int N, size_t rsz, int nchan) {
+  const int L = lin_fft_length(N, rsz);
+  const int64_t more = (int64_t)lin_spectrum_values(N, L) - (int64_t)lin_spectrum_values(N, 0);
+  return 3 * nchan * more * (int64_t)rsz > (int64_t)4 << 30 ? 0 : L;
+}
 
 // tw[m] = exp(-2 pi i m / n), m < n, formed in FP64
 template <typename R> void upload_twiddles(void* dst, int n) {
@@ -1104,9 +1123,7 @@ template <typename R> void build_normal(ms_plan* p, int step, PartDev& pd, doubl
   ensure_psf<R>(p, pd);
   if (p->conv == MS_CONV_LINEAR) {
     // the problem's H2^ into the buffer the captured passes read
-    const int L = p->lin_L;
-    ck(cudaMemcpyAsync(L ? p->lH : p->lh2, L ? pd.Hlin : pd.Hhat2,
-                       sizeof(R) * (L ? (size_t)L * (L / 2 + 1) : (size_t)2 * p->N * (p->N + 1)),
+    ck(cudaMemcpyAsync(p->lin_L ? p->lH : p->lh2, pd.Hhat2, sizeof(R) * lin_spectrum_values(p),
                        cudaMemcpyDeviceToDevice, p->ps),
        "copy");
     const bool full = step_full(step);
@@ -1118,7 +1135,7 @@ template <typename R> void build_normal(ms_plan* p, int step, PartDev& pd, doubl
     // the bound (and c0 = 0), then the step size itself: the operator is not
     // circulant, so the closed form is only a bound; power iteration from
     // the fixed start as for the IUWT
-    launch_lin_theta<R>((const R*)pd.Hhat2, p->N, full ? (const R*)p->gl2 : nullptr,
+    launch_lin_theta<R>(pd.h2_peak, p->N, full ? (const R*)p->gl2 : nullptr,
                         full ? (const R*)p->gh2 : nullptr, p->M, p->parts, p->ctl,
                         p->tickets + 2, p->ps);
     power_theta<R>(p, kPowerIterations, full);
@@ -1652,7 +1669,7 @@ template <typename R> void build_plan(ms_plan* p, const ms_plan_desc* d) {
   ckf(cufftPlan2d(&p->c2r, N, N, ti), "plan C2R");
   for (cufftHandle h : {p->r2c, p->c2r}) ckf(cufftSetStream(h, s), "set stream");
   if (p->conv == MS_CONV_LINEAR) {
-    const int L = p->lin_L = lin_fft_length(N, sizeof(R));
+    const int L = p->lin_L = lin_length(N, sizeof(R), d->nchan);
     if (L) {
       p->lhalf = p->alloc<C2<R>>((size_t)N * lin_pitch(L), "linear half plane");
       p->lH = p->alloc<R>((size_t)L * (L / 2 + 1), "linear PSF spectrum");
@@ -2744,22 +2761,26 @@ void* static_grid_scratch(int dev) {
 
 }  // namespace
 
-// pd.Hlin, H2^ as the own transforms of length lin_L read it, from the PSF
-// that ensure_psf has just left in q (the 2N x 2N plan) as spectrum and image:
-// the same values for L = 2N; else the image on the longer field, transformed
-// in q's grid buffer (16 N^2 complex values; 2N rows of L / 2 + 4 take less).
-// (Built at 448 px, FP32, with one and four channels: 16.9 and 24.1 ms; through
-// the PSF's spectrum, two FP64 cuFFT plans and their transforms 19.4 and 29.6,
-// with the spectrum of the 2N x 2N field alone 17.6 and 23.5.)
+// pd.Hhat2 and its peak from the PSF that ensure_psf has just left in q (the
+// 2N x 2N plan) as spectrum and image.  For the own transforms: the same values
+// for L = 2N; else the image on the longer field, transformed in q's grid
+// buffer (16 N^2 complex values; 2N rows of L / 2 + 4 take less).  (Built at 448
+// px, FP32, with one and four channels: 16.8 and 23.7 ms; through the PSF's
+// spectrum, two FP64 cuFFT plans and their transforms 19.4 and 29.6, with the
+// spectrum of the 2N x 2N field alone 17.6 and 23.5 to 23.9.)
 template <typename R>
 void build_linear_spectrum(ms_plan* p, PartDev& pd, ms_plan* q, PartDev& qd) {
   const int N = p->N, L = p->lin_L;
-  pd.Hlin = p->alloc<R>((size_t)L * (L / 2 + 1), "linear PSF spectrum");
-  if (L == 2 * N)
-    launch_lin_spectrum<R>((const R*)qd.Hhat, (R*)pd.Hlin, L, q->ps);
+  const size_t n2 = lin_spectrum_values(N, 0);
+  pd.Hhat2 = p->alloc<R>(lin_spectrum_values(p), "linear PSF spectrum");
+  launch_lin_peak<R>((const R*)qd.Hhat, (int64_t)n2, q->parts, pd.h2_peak, q->tickets + 2, q->ps);
+  if (L == 0)
+    ck(cudaMemcpyAsync(pd.Hhat2, qd.Hhat, sizeof(R) * n2, cudaMemcpyDeviceToDevice, q->ps), "copy");
+  else if (L == 2 * N)
+    launch_lin_spectrum<R>((const R*)qd.Hhat, (R*)pd.Hhat2, L, q->ps);
   else
-    ck(launch_lin_psf<R>((const R*)q->img[5], (C2<R>*)q->grid, (R*)pd.Hlin, (const C2<R>*)p->ltw, N,
-                         L, lin_pitch(L), q->ps),
+    ck(launch_lin_psf<R>((const R*)q->img[5], (C2<R>*)q->grid, (R*)pd.Hhat2, (const C2<R>*)p->ltw,
+                         N, L, lin_pitch(L), q->ps),
        "linear PSF spectrum");
   ck(cudaGetLastError(), "linear PSF spectrum");
 }
@@ -2783,17 +2804,16 @@ template <typename R> void build_linear_psf(ms_plan* p, const ms_plan_desc* d) {
   ms_plan* q = nullptr;
   const ms_status st = ms_plan_create(&d2, &q);
   if (st != MS_OK) throw Fail{st, "linear PSF operator: the 2N x 2N plan could not be built"};
-  const size_t bytes = sizeof(R) * 2 * p->N * (p->N + 1);
   try {
     ck(cudaSetDevice(q->dev), "set device");
+    double* peaks = p->alloc<double>(3 * p->ch.size(), "linear PSF peaks");
     for (size_t c = 0; c < p->ch.size(); ++c)
       for (int pt = 0; pt < 3; ++pt) {
         PartDev& qd = q->ch[c].part[pt];
         ensure_psf<R>(q, qd);
         PartDev& pd = p->ch[c].part[pt];
-        pd.Hhat2 = p->alloc<R>(bytes / sizeof(R), "linear PSF spectrum");
-        ck(cudaMemcpyAsync(pd.Hhat2, qd.Hhat, bytes, cudaMemcpyDeviceToDevice, q->ps), "copy");
-        if (p->lin_L) build_linear_spectrum<R>(p, pd, q, qd);
+        pd.h2_peak = peaks + 3 * c + pt;
+        build_linear_spectrum<R>(p, pd, q, qd);
         ck(cudaStreamSynchronize(q->ps), "synchronize");
       }
   } catch (...) {

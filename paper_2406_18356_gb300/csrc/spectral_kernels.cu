@@ -1560,30 +1560,43 @@ __global__ void lin_full_spec_kernel(const C2<R>* __restrict__ dek, const C2<R>*
 // ||P H P^T|| <= max |H2^|, so theta = 2 M max H2^2 (LOW / SINGLE) or
 // 2 M (max g_H^2 max H2^2 + max g_L^2) (FULL).  Also c0 = 0 (the objective
 // is evaluated directly in the image domain).
+// *out = max H2^2 over a spectrum (plan time)
 template <typename R>
-__global__ void lin_theta_kernel(const R* __restrict__ H2, int64_t n2, const R* __restrict__ gl2,
-                                 const R* __restrict__ gh2, int64_t nspec, int M,
-                                 double* __restrict__ parts, FistaCtl* __restrict__ ctl,
-                                 int32_t* ticket) {
-  double v[3] = {0.0, 0.0, 0.0};
-  const bool mx[3] = {true, true, true};
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  for (int64_t k = first; k < n2; k += stride) {
+__global__ void lin_peak_kernel(const R* __restrict__ H2, int64_t n2, double* __restrict__ parts,
+                                double* __restrict__ out, int32_t* ticket) {
+  double v[1] = {0.0};
+  const bool mx[1] = {true};
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n2;
+       k += (int64_t)gridDim.x * blockDim.x) {
     const double h = (double)H2[k];
     v[0] = fmax(v[0], h * h);
   }
+  block_reduce<1>(v, mx);
+  if (publish_partials<1>(v, parts, ticket)) {
+    double o[1];
+    gather_partials<1>(o, parts, mx, ticket);
+    if (threadIdx.x == 0) out[0] = o[0];
+  }
+}
+template <typename R>
+__global__ void lin_theta_kernel(const double* __restrict__ peak, const R* __restrict__ gl2,
+                                 const R* __restrict__ gh2, int64_t nspec, int M,
+                                 double* __restrict__ parts, FistaCtl* __restrict__ ctl,
+                                 int32_t* ticket) {
+  double v[2] = {0.0, 0.0};
+  const bool mx[2] = {true, true};
   if (gl2)
-    for (int64_t k = first; k < nspec; k += stride) {
-      v[1] = fmax(v[1], (double)gh2[k]);
-      v[2] = fmax(v[2], (double)gl2[k]);
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nspec;
+         k += (int64_t)gridDim.x * blockDim.x) {
+      v[0] = fmax(v[0], (double)gh2[k]);
+      v[1] = fmax(v[1], (double)gl2[k]);
     }
-  block_reduce<3>(v, mx);
-  if (publish_partials<3>(v, parts, ticket)) {
-    double o[3];
-    gather_partials<3>(o, parts, mx, ticket);
+  block_reduce<2>(v, mx);
+  if (publish_partials<2>(v, parts, ticket)) {
+    double o[2];
+    gather_partials<2>(o, parts, mx, ticket);
     if (threadIdx.x == 0) {
-      const double kmax = gl2 ? o[1] * o[0] + o[2] : o[0];
+      const double kmax = gl2 ? o[0] * *peak + o[1] : *peak;
       ctl->kmax = kmax;
       ctl->theta = 2.0 * M * kmax;
       ctl->inv_theta = kmax > 0 ? 1.0 / (2.0 * M * kmax) : 0.0;
@@ -1631,11 +1644,16 @@ void launch_lin_full_spec(const C2<R>* dek, const C2<R>* dep, const R* gl2, cons
       dek, dep, gl2, gh2, uv, N, parts, ctl, trace, ticket, l1_parts, n_l1);
 }
 template <typename R>
-void launch_lin_theta(const R* H2, int N, const R* gl2, const R* gh2, int M, double* parts,
+void launch_lin_peak(const R* H2, int64_t n, double* parts, double* out, int32_t* ticket,
+                     cudaStream_t s) {
+  lin_peak_kernel<R><<<nparts_for(n), kThreads, 0, s>>>(H2, n, parts, out, ticket);
+}
+template <typename R>
+void launch_lin_theta(const double* peak, int N, const R* gl2, const R* gh2, int M, double* parts,
                       FistaCtl* ctl, int32_t* ticket, cudaStream_t s) {
-  const int64_t n2 = (int64_t)2 * N * (N + 1);
-  lin_theta_kernel<R><<<nparts_for(n2), kThreads, 0, s>>>(
-      H2, n2, gl2, gh2, (int64_t)N * (N / 2 + 1), M, parts, ctl, ticket);
+  const int64_t n = (int64_t)N * (N / 2 + 1);
+  lin_theta_kernel<R><<<gl2 ? nparts_for(n) : 1, kThreads, 0, s>>>(peak, gl2, gh2, n, M, parts, ctl,
+                                                                  ticket);
 }
 
 #define MS_INST(R)                                                                               \
@@ -1684,8 +1702,10 @@ void launch_lin_theta(const R* H2, int N, const R* gl2, const R* gh2, int M, dou
   template void launch_lin_full_spec<R>(const C2<R>*, const C2<R>*, const R*, const R*, C2<R>*, \
                                         int, double*, FistaCtl*, double*, int32_t*,              \
                                         const double*, int, cudaStream_t);                       \
-  template void launch_lin_theta<R>(const R*, int, const R*, const R*, int, double*, FistaCtl*, \
-                                    int32_t*, cudaStream_t);
+  template void launch_lin_peak<R>(const R*, int64_t, double*, double*, int32_t*,              \
+                                   cudaStream_t);                                               \
+  template void launch_lin_theta<R>(const double*, int, const R*, const R*, int, double*,       \
+                                    FistaCtl*, int32_t*, cudaStream_t);
 
 MS_INST(float)
 MS_INST(double)
