@@ -434,12 +434,12 @@ __global__ void __launch_bounds__(32 * kMaxBases)
   }
 }
 
-// Level 1, FP32: x = sum of the bases, a block per tile, basis after basis with
-// the next one's windows in flight.  A thread keeps the sums of its 2 U
-// outputs of one row in registers.  Tiles this small, rather than 64 pixels
+// Level 1 of larger images: x = sum of the bases, a block per tile, basis after
+// basis with the next one's windows in flight.  A thread keeps the sums of its
+// 2 U outputs of one row in registers.  Tiles this small, rather than 64 pixels
 // with half of an SM's shared memory and two blocks an SM, let seven or more
-// blocks share an SM and hide each other's barriers (an iteration, 64 | 32: at
-// 1024 px 114 | 109 us, 2048 px 350 | 335, 8 jobs at 1024 px 76.1 | 74.7 a
+// blocks share an SM and hide each other's barriers (an FP32 iteration, 64 | 32:
+// at 1024 px 114 | 109 us, 2048 px 350 | 335, 8 jobs at 1024 px 76.1 | 74.7 a
 // job).
 template <typename R, int TY, int TX, int U, int NT>
 __global__ void __launch_bounds__(NT)

@@ -655,16 +655,21 @@ namespace {
 // against 133 per iteration at 1024 px with both directions' coarse levels
 // replaced; FP64, an iteration at 128 px with h = 64..8: 155 | 219, at 256
 // px 301 | 337 with tiles of 16, at 1024 px with h = 512 wide 1549 | 1715
-// with tiles of 16.
+// with tiles of 16.  The plain FP64 transform has no prox operands in flight:
+// tiles of 8 below h = 256 (8 bases, h = 192: 62 | 80 with 16; 256: 101 | 96),
+// then of 16 (h = 384: 197 | 203 wide, 512: 346 | 352) until some 4500 wide
+// tiles keep the SMs evenly busy (h = 768: 740 wide | 772; 4 bases 211 | 203).
 enum class Ana { kWide, k16, k8, k4 };
-Ana ana_kernel(bool f64, int h) {
+Ana ana_kernel(bool f64, bool plain, int h, int M) {
+  if (f64 && plain && h % 8 == 0 && h < 256) return Ana::k8;
+  if (f64 && plain && h % 16 == 0 && (int64_t)h * h * M < 4500 * 32 * 32) return Ana::k16;
   if (f64 && h > 256) return h % 16 == 0 ? Ana::kWide : (h % 4 == 0 ? Ana::k4 : Ana::kWide);
   if (h % 16 == 0 && h >= (f64 ? 129 : 64)) return Ana::k16;
   if (h % 8 == 0) return Ana::k8;
   return h % 4 == 0 ? Ana::k4 : Ana::kWide;
 }
-int ana_side(bool f64, int h) {
-  switch (ana_kernel(f64, h)) {
+int ana_side(bool f64, bool plain, int h, int M) {
+  switch (ana_kernel(f64, plain, h, M)) {
     case Ana::k16: return 16;
     case Ana::k8: return 8;
     case Ana::k4: return 4;
@@ -676,12 +681,15 @@ int ana_side(bool f64, int h) {
 // make some 1000 or 500 blocks, else of 8.  Measured at 1024 px, FP32, one
 // job, us an iteration: (n = 512, 256, 128) in tiles of (32, 16, 16) 128,
 // (32, 32, 16) 132 and 136, (16, 16, 16) 134; 8 jobs: (32, 32, 32) 89.9 a
-// job, (16, 16, 16) 95.1.  FP64: 8 below 512 (the fewest instructions in the
-// busiest scheduler), else 16.
+// job, (16, 16, 16) 95.1.  FP64: 32 (2 pairs, 256 threads) from 512 blocks on
+// (8 bases, us a level, 32 | 16 | 8: n = 384 48 | 60 | 75, 512 81 | 103 | 132,
+// 8 jobs at 128 54 | 62 | 71; n = 256, 512 blocks, 36 | 37 | 35), else 16 from
+// 512 on and 8 below (the fewest instructions in the busiest scheduler).
 enum class Syn { k32, k16, k8, k4, k2 };
 Syn syn_kernel(bool f64, int n, int M, int jobs) {
   auto blocks = [&](int t) { return (int64_t)(n / t) * (n / t) * M * jobs; };
   const Syn small = n % 8 == 0 ? Syn::k8 : (n % 4 == 0 ? Syn::k4 : Syn::k2);
+  if (f64 && n % 32 == 0 && blocks(32) >= 512) return Syn::k32;
   if (f64) return n >= 512 && n % 16 == 0 ? Syn::k16 : small;
   if (n % 32 == 0 && blocks(32) >= 1000) return Syn::k32;
   if (n % 16 == 0 && blocks(16) >= 500) return Syn::k16;
@@ -691,9 +699,9 @@ Syn syn_kernel(bool f64, int n, int M, int jobs) {
 template <typename R, int MODE>
 cudaError_t launch_analysis_level(const FistaPass<R>& a, R* plain, const CUtensorMap* grad_map,
                                   int j, int part_base, cudaStream_t s) {
-  const int h = a.N >> j, T = ana_side(sizeof(R) == 8, h);
+  const int h = a.N >> j, T = ana_side(sizeof(R) == 8, MODE == 0, h, a.M);
   const dim3 grid((h / T) * (h / T), a.M, a.js.jobs);
-  switch (ana_kernel(sizeof(R) == 8, h)) {
+  switch (ana_kernel(sizeof(R) == 8, MODE == 0, h, a.M)) {
     case Ana::k16:
       return launch_pdl(fine_analysis_kernel<R, MODE, 16, 16, 4, 128>, grid, dim3(128), 0, s, a,
                         plain, j, part_base);
@@ -728,9 +736,12 @@ cudaError_t launch_synthesis_level(const FistaPass<R>& a, const R* plain, int j,
   const int n = 2 * (a.N >> j), jobs = a.js.jobs;
   const bool f64 = sizeof(R) == 8;
   if (j == 1) {
-    // FP64, and FP32 below 256 px: a warp per basis.  Measured at 128 px,
-    // FP64: 24.6 us an iteration less than one block per 16-pixel tile; at 512
-    // px 542 | 632 us an iteration.
+    // FP32 below 256 px, and FP64 below some 218 tiles of 32 pixels: a warp per
+    // basis (at 128 px, FP64: 24.6 us an iteration less than one block per
+    // 16-pixel tile).  FP64 above: the sum kernel, an output pair a thread (us
+    // a level, 8 bases, warps | sum: 320 px 49 | 54, 448 px 90 | 100, 512 px
+    // 118 | 100, 768 px 235 | 197, 2048 px 1595 | 1312; one basis at 1024 px 36
+    // | 13; 8 jobs at 512 px 806 | 681).
     auto go = [&](auto kern, int ty, int tx, size_t elems) {
       const size_t smem = kMaxBases * elems * sizeof(R);
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -739,18 +750,20 @@ cudaError_t launch_synthesis_level(const FistaPass<R>& a, const R* plain, int j,
     };
     if (f64 && (int64_t)(n / 8) * (n / 16) * jobs < 256)
       return go(fine_synthesis_l1_kernel<R, 8, 16, 1>, 8, 16, FineSyn<8, 16>::Elems);
-    if (f64 || n < 256 || n % 32)
+    const int64_t tiles = (int64_t)(n / 32) * (n / 32) * jobs;
+    if (n < 256 || n % 32 || (f64 && tiles < 218))
       return go(fine_synthesis_l1_kernel<R, 16, 16, 2>, 16, 16, FineSyn<16, 16>::Elems);
-    if constexpr (sizeof(R) == 4) {
-      auto sum = [&](auto kern, int threads) {
-        return launch_pdl(kern, dim3((n / 32) * (n / 32), 1, jobs), dim3(threads), 0, s, a, plain);
-      };
+    auto sum = [&](auto kern, int threads) {
+      return launch_pdl(kern, dim3((n / 32) * (n / 32), 1, jobs), dim3(threads), 0, s, a, plain);
+    };
+    if constexpr (sizeof(R) == 8) {
+      return sum(fine_synthesis_sum_kernel<R, 32, 32, 1, 512>, 512);
+    } else {
       // 4 output pairs a thread (fewest shared-memory loads) where the tiles
       // occupy the SMs several times over, else 2 by twice the threads.
       // Measured, us an iteration and job (4 | 2): 256 px 58.6 | 44.9, 512 px
       // 73.6 | 65.1, 4 jobs at 512 px 30.5 | 31.1, 1024 px 109.4 | 110.7.
-      if ((int64_t)(n / 32) * (n / 32) * jobs >= 1000)
-        return sum(fine_synthesis_sum_kernel<R, 32, 32, 4, 128>, 128);
+      if (tiles >= 1000) return sum(fine_synthesis_sum_kernel<R, 32, 32, 4, 128>, 128);
       return sum(fine_synthesis_sum_kernel<R, 32, 32, 2, 256>, 256);
     }
   }
@@ -760,7 +773,7 @@ cudaError_t launch_synthesis_level(const FistaPass<R>& a, const R* plain, int j,
   switch (syn_kernel(f64, n, a.M, jobs)) {
     case Syn::k32:
       if constexpr (sizeof(R) == 4) return go(fine_synthesis_kernel<R, 32, 32, 4, 128>, 32, 128);
-      break;
+      else return go(fine_synthesis_kernel<R, 32, 32, 2, 256>, 32, 256);
     case Syn::k16: return go(fine_synthesis_kernel<R, 16, 16, 2, 128>, 16, 128);
     case Syn::k8: return go(fine_synthesis_kernel<R, 8, 8, 1, 128>, 8, 128);
     case Syn::k4: return go(fine_synthesis_kernel<R, 4, 4, 1, 64>, 4, 64);
@@ -773,7 +786,7 @@ cudaError_t launch_synthesis_level(const FistaPass<R>& a, const R* plain, int j,
 int analysis_prox_partials(WaveletGeom g, size_t rsz) {
   int total = 0;
   for (int j = 1; j <= g.J; ++j) {
-    const int h = g.N >> j, T = ana_side(rsz == 8, h);
+    const int h = g.N >> j, T = ana_side(rsz == 8, false, h, g.M);
     total += (h / T) * (h / T) * g.M;
   }
   return total;
@@ -835,7 +848,7 @@ cudaError_t launch_analysis_pass(const FistaPass<R>& a, const CUtensorMap* grad_
                                  cudaStream_t s, int only_level) {
   int part_base = 0;
   for (int j = 1; j <= a.J; ++j) {
-    const int h = a.N >> j, T = ana_side(sizeof(R) == 8, h);
+    const int h = a.N >> j, T = ana_side(sizeof(R) == 8, false, h, a.M);
     if (only_level == 0 || j == only_level || (only_level < 0 && j > 1)) {
       const cudaError_t e = launch_analysis_level<R, 1>(a, nullptr, grad_map, j, part_base, s);
       if (e != cudaSuccess) return e;
