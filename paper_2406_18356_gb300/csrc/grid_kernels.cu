@@ -889,11 +889,17 @@ void launch_grid(const WorkItem* items, int nitems, const uint32_t* cell, const 
 // loads (a tile's items, then their cells), so a thread takes Q = 4 cells of a
 // row (they share both; one cell each where the grid is too small to occupy
 // the SMs that way: 128 px 32 | 13 us), reads the four tiles' item ranges
-// together and several items at a time; and where a tile has more than kFoldList items
-// (dense cores: hundreds) groups of kFoldGroup are first added up in parallel
-// into their first item's tile (fold_groups_kernel), so that no cell's chain
-// is long.  Measured (before | now): 1024 px, 9.27M rows 57 | 32 us;
-// 16 jobs at 1024 px 224 | 118; 4096 px, compensated 297 | 140.
+// together and several items at a time (one cell a thread: 16 or 8, then four,
+// then one by one; a dozen items one by one took a small, dense grid's fold
+// from 12 to 23 us); and where a tile has more than kFoldList items (dense
+// cores: hundreds) groups of kFoldGroup are first added up in parallel into
+// their first item's tile (fold_groups_kernel), so that no cell's chain is
+// long.  Measured (before | now): 1024 px, 9.27M rows 57 | 32 us; 16 jobs at 1024
+// px 224 | 118; 4096 px, compensated 297 | 140; 128 px, 1M rows 12.0 | 12.5.
+// Both kernels are launched early and wait first of all, which hides 2 us of
+// each launch; neither lets the next one go before its end, whose blocks would
+// wait in the SMs that this one's need (gridding at 128 px, 30,000 rows, us:
+// 28.5 without, 33.9 with, 26.5 so).
 constexpr int kFoldList = 32, kFoldGroup = 16;
 
 // Q consecutive scratch cells (Q = 4: an even offset, 16-byte aligned)
@@ -955,6 +961,15 @@ __device__ __forceinline__ void fold_cells(const typename ScratchOf<R, KAHAN>::T
           for (int c = 0; c < Q; ++c) cell_sum(sum[c], a[u][c]);
       }
     }
+    if constexpr (Q == 1) {
+      for (; i + 3 * step < hi[q]; i += 4 * step) {
+        Acc a[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) a[u] = base[(int64_t)(i + u * step) * cells];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) cell_sum(sum[0], a[u]);
+      }
+    }
     for (; i < hi[q]; i += step) {
       const Acc* p = base + (int64_t)i * cells;
 #pragma unroll
@@ -972,6 +987,7 @@ __global__ void __launch_bounds__(kFoldThreads)
     fold_kernel(const typename ScratchOf<R, KAHAN>::T* __restrict__ scratch,
                 const int32_t* __restrict__ tile_items, int Ng, int T, int ntx, int first,
                 int side, C2<R>* __restrict__ grid) {
+  pdl_wait();
   fold_cells<R, KAHAN, Q>(scratch, tile_items, Ng, T, ntx, first, side, grid);
 }
 
@@ -1013,6 +1029,7 @@ __global__ void __launch_bounds__(128)
     fold_groups_kernel(typename ScratchOf<R, KAHAN>::T* __restrict__ scratch,
                        const WorkItem* __restrict__ items, const int32_t* __restrict__ tile_items,
                        int cells) {
+  pdl_wait();
   fold_group(scratch, tile_items, items[blockIdx.x], blockIdx.x, cells);
 }
 template <typename R, bool KAHAN>
@@ -1049,14 +1066,13 @@ void launch_fold(void* scratch, const WorkItem* items, int nitems, int longest,
   using Acc = typename ScratchOf<R, KAHAN>::T;
   const int S = tile + kW - 1;
   if (longest > kFoldList)
-    fold_groups_kernel<R, KAHAN><<<nitems, 128, 0, s>>>(static_cast<Acc*>(scratch), items,
-                                                        tile_items, S * S);
+    launch_pdl(fold_groups_kernel<R, KAHAN>, dim3(nitems), dim3(128), 0, s,
+               static_cast<Acc*>(scratch), items, tile_items, S * S);
   int first, side;
   fold_region(Ng, ext, &first, &side);
   const auto go = [&](auto* k, int Q) {
-    k<<<fold_grid(first, side, 1, Q), kFoldThreads, 0, s>>>(static_cast<const Acc*>(scratch),
-                                                            tile_items, Ng, tile, ntx, first, side,
-                                                            grid);
+    launch_pdl(k, fold_grid(first, side, 1, Q), dim3(kFoldThreads), 0, s,
+               static_cast<const Acc*>(scratch), tile_items, Ng, tile, ntx, first, side, grid);
   };
   if (fold_quads(side, 1)) go(fold_kernel<R, KAHAN, 4>, 4);
   else go(fold_kernel<R, KAHAN, 1>, 1);
