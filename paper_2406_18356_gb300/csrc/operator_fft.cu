@@ -11,7 +11,8 @@
 //             of column -u are added as they are read, transformed, and the N
 //             image rows of the result kept; N real rows from the half plane,
 //             cropped, deapodized and scaled as they are written.
-// Each grid cell is written or read once, by lanes that cover 32-byte sectors;
+// Each grid cell is written or read once, 8 to 32 bytes of a row by each block
+// (ColBlock; blocks that share a sector run side by side and meet in L2);
 // padding, cropping, deapodization and the grid's centring (cell k at index k
 // + Ng / 2) cost no pass of their own.  A complex transform of the whole grid
 // (2-D cuFFT between a padding and a cropping pass) moves 4 to 9 times the
@@ -116,15 +117,27 @@ __device__ __forceinline__ void transform(C2<R>* buf, const C2<R>* __restrict__ 
   run_stages<R, LOGN, LE, 0, INV>(v, buf, tw, tw_step, t, store);
 }
 
-// log2 of the elements per thread of a sequence of length 2^logn
+// log2 of the elements per thread of a sequence of length 2^logn.  Measured,
+// the operator's forward + adjoint transforms, us (rows N, columns 2N long):
+// FP32 N = 1024 with 16 a thread from length 2048 on 25.4 + 23.8, with 8 28.8 +
+// 27.6; N = 4096 388 + 302 | 463 + 378; N = 512 with 8 15.7 + 14.6, with 16 16.1
+// + 16.6, with 4 16.8 + 14.8 (N = 64 to 256 would take 0.5 to 1.5 less with 4).
+// FP64 with the elements below | twice | half: N = 128 16.3 + 14.6 | 18.4 + 18.0
+// | -, N = 512 80 + 96 | 77 + 79 | 84 + 99, N = 1024 258 + 264 | 266 + 273 | 248
+// + 250, N = 2048 984 + 1017 | 975 + 1018 | 999 + 1037 (two columns a block).
 constexpr int elems_log(size_t rsz, int logn) {
   return rsz == 4 ? (logn >= 11 ? 4 : (logn >= 6 ? 3 : 2))
                   : (logn <= 9 ? 1 : (logn <= 11 ? 2 : 3));
 }
-// sequences of length 2^logn of a block and its shared memory.  Columns: a
-// 32-byte sector of each row, fewer for short columns (a block per SM) and
-// where 1024 threads or the shared memory set the limit.  Rows: some 256
-// threads, at most N / 128 rows.
+// Sequences of length 2^logn of a block and its shared memory.  Rows: some 256
+// threads, at most N / 128 rows.  Columns, as far as 1024 threads and the
+// shared memory go: FP32 a 32-byte sector of each row from length 2048 on (N =
+// 2048, 4 | 2 columns: 74 + 64 | 83 + 71 us), two at 1024 (N = 512, 2 | 1: 15.7
+// + 14.6 | 17.9 + 14.1), else one, so that short columns make a block for each
+// SM; FP64 one (N = 512, 1 | 2: 70 + 70 | 80 + 96, N = 1024 228 + 236 | 258 +
+// 264; linear operator, 20 iterations and the step size, at 512 px 43.6 | 46.3
+// ms, 1024 px 137 | 147), two at 4096 (2 | 1: 984 + 1017 | 963 + 977 us, but the
+// linear operator at 2048 px 568 | 572 ms).
 template <typename R, int LOGN> struct Seq {
   static constexpr int LE = elems_log(sizeof(R), LOGN);
   static constexpr int TPS = 1 << (LOGN - LE);
@@ -133,7 +146,7 @@ template <typename R, int LOGN> struct Seq {
 template <typename R, int LOGN> struct ColBlock {
   using S = Seq<R, LOGN>;
   static constexpr int kWant = sizeof(R) == 4 ? (LOGN >= 11 ? 4 : (LOGN == 10 ? 2 : 1))
-                                              : (LOGN >= 10 ? 2 : 1);
+                                              : (LOGN >= 12 ? 2 : 1);
   static constexpr int kMax = 1024 / S::TPS;
   static constexpr int CB0 = kWant < kMax ? kWant : kMax;
   static constexpr int CB = S::TPS * CB0 < 32 ? 32 / S::TPS : CB0;
@@ -614,12 +627,18 @@ template cudaError_t launch_op_fft<double>(const OpFftArgs<double>&, bool, int, 
 // 7.9 | 12.9, 384 px (4/3) 8.0 | 13.3, 448 px 9.5 | 16.2, 640 px (8/5) 12.1 |
 // 21.6, 1024 px 15.5 | 23.8; FP64 128 px 10.5 | 23.1, 192 px (4/3) 17.3 | 37,
 // 384 px (4/3) 46 | 65, 512 px 55 | 109, 640 px (8/5) 162 | 138, 1024 px 199 |
-// 330.
+// 330.  Larger sides, the step size and 30 iterations of one basis: FP32 1280 px
+// (8/5) 30 | 37, 2048 px 37 | 67, 2560 px (8/5, L = 8192) 151 | 137, 2624 px
+// 152 | 266, 2816 px (16/11) 155 | 156, 3072 px (4/3) 161 | 203, 4096 px 187 |
+// 246; FP64 1408 px (16/11) 547 | 518, 1536 px (4/3) 563 | 661, 2048 px 617 |
+// 1200, 3072 px (4/3) 2379 | 2753, 4096 px 2611 | 4219.  So 8192 serves FP32
+// below 8/5 only.
 int lin_fft_length(int N, size_t rsz) {
   int L = 32;
   while (L < 2 * N) L *= 2;
   if (N % 2 || L > 8192) return 0;
-  return (rsz == 8 ? 3 * L <= 8 * N : 5 * L <= 16 * N) ? L : 0;
+  if (rsz == 8) return 3 * L <= 8 * N ? L : 0;
+  return 5 * L < 16 * N + (L < 8192) ? L : 0;
 }
 
 template <typename R> cudaError_t launch_lin_fft(const LinFftArgs<R>& a, int L, cudaStream_t s) {
