@@ -270,8 +270,8 @@ void launch_crop(const C2<R>* grid, const R* psi, int npix, int Ng, double scale
 template <typename R>
 void launch_degrid(const CUtensorMap* tmap, const C2<R>* grid, const WorkItem* items,
                    int nitems, const uint32_t* cell, const C2<R>* frac, const C2<R>* obs,
-                   const int32_t* obs_idx, C2<R>* out, const int32_t* out_idx, int Ng, int tile, int ntx, const EsKernel& es, int32_t* err,
-                   cudaStream_t s);
+                   const int32_t* obs_idx, C2<R>* out, const int32_t* out_idx, int Ng, int tile,
+                   int ntx, const EsKernel& es, int32_t* err, cudaStream_t s);
 template <typename R, bool KAHAN>
 void launch_grid(const WorkItem* items, int nitems, const uint32_t* cell, const C2<R>* frac,
                  const C2<R>* vis, void* scratch, int Ng, int tile, int ntx, const EsKernel& es,
@@ -301,7 +301,8 @@ void launch_fold_batch(const BatchJob<R>* jobs, int njobs, const int32_t* job_of
 template <typename R>
 void launch_degrid_batch(const CUtensorMap* tmap, const BatchJob<R>* jobs,
                          const int32_t* job_of, int total_items, bool has_obs, bool gathered,
-                         bool user_order, int Ng, int tile, int ntx, const EsKernel& es, int32_t* err, cudaStream_t s);
+                         bool user_order, int Ng, int tile, int ntx, const EsKernel& es,
+                         int32_t* err, cudaStream_t s);
 template <typename R>
 void launch_pad_batch(const BatchJob<R>* jobs, int njobs, const R* psi, int npix, int Ng,
                       cudaStream_t s);

@@ -380,8 +380,8 @@ __global__ void __launch_bounds__(degrid_threads<R>())
 template <typename R>
 void launch_degrid(const CUtensorMap* tmap, const C2<R>* grid, const WorkItem* items,
                    int nitems, const uint32_t* cell, const C2<R>* frac, const C2<R>* obs,
-                   const int32_t* obs_idx, C2<R>* out, const int32_t* out_idx, int Ng, int tile, int ntx, const EsKernel& es, int32_t* err,
-                   cudaStream_t s) {
+                   const int32_t* obs_idx, C2<R>* out, const int32_t* out_idx, int Ng, int tile,
+                   int ntx, const EsKernel& es, int32_t* err, cudaStream_t s) {
   if (nitems <= 0) return;
   const int S = tile + kW - 1;
   // tile + alignment slack + mbarrier + flag + tables
@@ -895,7 +895,7 @@ void launch_grid(const WorkItem* items, int nitems, const uint32_t* cell, const 
 // cores: hundreds) groups of kFoldGroup are first added up in parallel into
 // their first item's tile (fold_groups_kernel), so that no cell's chain is
 // long.  Measured (before | now): 1024 px, 9.27M rows 57 | 32 us; 16 jobs at 1024
-// px 224 | 118; 4096 px, compensated 297 | 140; 128 px, 1M rows 12.0 | 12.5.
+// px 224 | 118; 4096 px, compensated 297 | 140; 128 px, 1M rows 12 | 15.
 // Both kernels are launched early and wait first of all, which hides 2 us of
 // each launch; neither lets the next one go before its end, whose blocks would
 // wait in the SMs that this one's need (gridding at 128 px, 30,000 rows, us:
@@ -917,9 +917,10 @@ template <typename A, int Q> __device__ __forceinline__ void load_cells(const A*
 
 // scratch: the job's first item's tile; item i of the job's tile_items
 template <typename R, bool KAHAN, int Q>
-__device__ __forceinline__ void fold_cells(const typename ScratchOf<R, KAHAN>::T* __restrict__ scratch,
-                                           const int32_t* __restrict__ tile_items, int Ng, int T,
-                                           int ntx, int first, int side, C2<R>* __restrict__ grid) {
+__device__ __forceinline__ void fold_cells(
+    const typename ScratchOf<R, KAHAN>::T* __restrict__ scratch,
+    const int32_t* __restrict__ tile_items, int Ng, int T, int ntx, int first, int side,
+    C2<R>* __restrict__ grid) {
   using Acc = typename ScratchOf<R, KAHAN>::T;
   constexpr int U = (sizeof(Acc) == 8 ? 16 : 8) / Q;   // items in flight
   const int S = T + kW - 1;
@@ -999,8 +1000,8 @@ __global__ void __launch_bounds__(kFoldThreads)
                       int ntx, int first, int side) {
   const BatchJob<R>& jb = jobs[blockIdx.z];
   const int S = T + kW - 1;
-  fold_cells<R, KAHAN, Q>(scratch + jb.item_base * (int64_t)(S * S), jb.tile_items, Ng, T, ntx, first,
-                       side, jb.grid);
+  fold_cells<R, KAHAN, Q>(scratch + jb.item_base * (int64_t)(S * S), jb.tile_items, Ng, T, ntx,
+                          first, side, jb.grid);
 }
 
 // Work item `it` (index `item` of its job's), if it leads a group of a long
@@ -1148,7 +1149,8 @@ int blocks_for(int64_t n, int cap) {
 template <typename R>
 void launch_job_of(const BatchJob<R>* jobs, int njobs, int max_items, int32_t* job_of,
                    cudaStream_t s) {
-  job_of_kernel<R><<<dim3(blocks_for(max_items, sm_count()), njobs), kThreads, 0, s>>>(jobs, job_of);
+  const dim3 grid(blocks_for(max_items, sm_count()), njobs);
+  job_of_kernel<R><<<grid, kThreads, 0, s>>>(jobs, job_of);
 }
 
 template <typename R>
@@ -1190,27 +1192,29 @@ void launch_fold_batch(const BatchJob<R>* jobs, int njobs, const int32_t* job_of
 template <typename R>
 void launch_degrid_batch(const CUtensorMap* tmap, const BatchJob<R>* jobs,
                          const int32_t* job_of, int total_items, bool has_obs, bool gathered,
-                         bool user_order, int Ng, int tile, int ntx, const EsKernel& es, int32_t* err, cudaStream_t s) {
+                         bool user_order, int Ng, int tile, int ntx, const EsKernel& es,
+                         int32_t* err, cudaStream_t s) {
   if (total_items <= 0) return;
   const int S = tile + kW - 1;
   const size_t smem = (size_t)S * S * sizeof(C2<R>) + 128 + 16 + es_smem<R>(es);
   if (has_obs) {
     auto k = degrid_batch_kernel<R, true>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<total_items, degrid_threads<R>(), smem, s>>>(*tmap, jobs, job_of, gathered, user_order, Ng, tile,
-                                                     ntx, (R)es.beta, es.tab, err);
+    k<<<total_items, degrid_threads<R>(), smem, s>>>(*tmap, jobs, job_of, gathered, user_order, Ng,
+                                                     tile, ntx, (R)es.beta, es.tab, err);
   } else {
     auto k = degrid_batch_kernel<R, false>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<total_items, degrid_threads<R>(), smem, s>>>(*tmap, jobs, job_of, gathered, user_order, Ng, tile,
-                                                     ntx, (R)es.beta, es.tab, err);
+    k<<<total_items, degrid_threads<R>(), smem, s>>>(*tmap, jobs, job_of, gathered, user_order, Ng,
+                                                     tile, ntx, (R)es.beta, es.tab, err);
   }
 }
 
 template <typename R>
 void launch_pad_batch(const BatchJob<R>* jobs, int njobs, const R* psi, int npix, int Ng,
                       cudaStream_t s) {
-  pad_batch_kernel<R><<<dim3(blocks_for((int64_t)Ng * Ng, sm_count() * 8), njobs), kThreads, 0, s>>>(
+  const dim3 blocks(blocks_for((int64_t)Ng * Ng, sm_count() * 8), njobs);
+  pad_batch_kernel<R><<<blocks, kThreads, 0, s>>>(
       jobs, psi, npix, Ng);
 }
 
@@ -1238,12 +1242,12 @@ template void launch_grid_batch<float, true>(const BatchJob<float>*, const int32
                                              int, int, const EsKernel&, cudaStream_t);
 template void launch_grid_batch<double, false>(const BatchJob<double>*, const int32_t*, int,
                                                void*, int, int, const EsKernel&, cudaStream_t);
-template void launch_fold_batch<float, false>(const BatchJob<float>*, int, const int32_t*, int, int, void*,
-                                              int, int, int, int, cudaStream_t);
-template void launch_fold_batch<float, true>(const BatchJob<float>*, int, const int32_t*, int, int, void*,
-                                              int, int, int, int, cudaStream_t);
-template void launch_fold_batch<double, false>(const BatchJob<double>*, int, const int32_t*, int, int, void*,
-                                              int, int, int, int, cudaStream_t);
+template void launch_fold_batch<float, false>(const BatchJob<float>*, int, const int32_t*, int, int,
+                                              void*, int, int, int, int, cudaStream_t);
+template void launch_fold_batch<float, true>(const BatchJob<float>*, int, const int32_t*, int, int,
+                                             void*, int, int, int, int, cudaStream_t);
+template void launch_fold_batch<double, false>(const BatchJob<double>*, int, const int32_t*, int,
+                                               int, void*, int, int, int, int, cudaStream_t);
 
 template void launch_pad<float>(const float*, const float*, int, int, float2*, cudaStream_t);
 template void launch_pad<double>(const double*, const double*, int, int, double2*,
@@ -1254,10 +1258,12 @@ template void launch_crop<double>(const double2*, const double*, int, int, doubl
                                   cudaStream_t);
 template void launch_degrid<float>(const CUtensorMap*, const float2*, const WorkItem*, int,
                                    const uint32_t*, const float2*, const float2*, const int32_t*,
-                                   float2*, const int32_t*, int, int, int, const EsKernel&, int32_t*, cudaStream_t);
+                                   float2*, const int32_t*, int, int, int, const EsKernel&,
+                                   int32_t*, cudaStream_t);
 template void launch_degrid<double>(const CUtensorMap*, const double2*, const WorkItem*, int,
-                                    const uint32_t*, const double2*, const double2*,
-                                    const int32_t*, double2*, const int32_t*, int, int, int, const EsKernel&, int32_t*, cudaStream_t);
+                                    const uint32_t*, const double2*, const double2*, const int32_t*,
+                                    double2*, const int32_t*, int, int, int, const EsKernel&,
+                                    int32_t*, cudaStream_t);
 template void launch_grid<float, false>(const WorkItem*, int, const uint32_t*, const float2*,
                                         const float2*, void*, int, int, int, const EsKernel&,
                                         cudaStream_t);
@@ -1267,11 +1273,11 @@ template void launch_grid<float, true>(const WorkItem*, int, const uint32_t*, co
 template void launch_grid<double, false>(const WorkItem*, int, const uint32_t*, const double2*,
                                          const double2*, void*, int, int, int, const EsKernel&,
                                          cudaStream_t);
-template void launch_fold<float, false>(void*, const WorkItem*, int, int, const int32_t*, int, int, int,
-                                        int, float2*, cudaStream_t);
-template void launch_fold<float, true>(void*, const WorkItem*, int, int, const int32_t*, int, int, int,
-                                        int, float2*, cudaStream_t);
-template void launch_fold<double, false>(void*, const WorkItem*, int, int, const int32_t*, int, int, int,
-                                        int, double2*, cudaStream_t);
+template void launch_fold<float, false>(void*, const WorkItem*, int, int, const int32_t*, int, int,
+                                        int, int, float2*, cudaStream_t);
+template void launch_fold<float, true>(void*, const WorkItem*, int, int, const int32_t*, int, int,
+                                       int, int, float2*, cudaStream_t);
+template void launch_fold<double, false>(void*, const WorkItem*, int, int, const int32_t*, int, int,
+                                         int, int, double2*, cudaStream_t);
 
 }  // namespace ms

@@ -1,10 +1,10 @@
 // libmstep: plan object, C ABI and the orchestration of the method.
 //
 // Host code only sequences kernels: every step of the path (partitioning,
-// sorting, gridding, the operator's FFTs through cuFFT, wavelets, FISTA with
-// its own spectral-step transforms, reductions) runs on the device.  All work of a call is issued on a plan-owned stream
-// that is ordered after the caller's stream at entry, and the caller's stream
-// is ordered after it at exit.
+// sorting, gridding, the operator's and FISTA's transforms, own or cuFFT's by
+// the side, wavelets, reductions) runs on the device.  All work of a call is
+// issued on a plan-owned stream that is ordered after the caller's stream at
+// entry, and the caller's stream is ordered after it at exit.
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <cufft.h>
@@ -1734,7 +1734,8 @@ template <typename R> void build_plan(ms_plan* p, const ms_plan_desc* d) {
     cuuint32_t box[2] = {(cuuint32_t)(2 * p->S), (cuuint32_t)p->S};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = ((EncodeTiledFn)fn)(
-        &p->tmap, sizeof(R) == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
+        &p->tmap,
+        sizeof(R) == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
         2, p->grid, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
         CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -1748,9 +1749,8 @@ template <typename R> void build_plan(ms_plan* p, const ms_plan_desc* d) {
       cuuint64_t gs[1] = {(cuuint64_t)N * sizeof(R)};
       cuuint32_t gb[2] = {bc, br};
       r = ((EncodeTiledFn)fn)(
-          &p->grad_map,
-          sizeof(R) == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
-          p->ywork, gd, gs, gb, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+          &p->grad_map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2, p->ywork, gd, gs, gb, estr,
+          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
       if (r != CUDA_SUCCESS) throw Fail{MS_ERR_CUDA, "cuTensorMapEncodeTiled failed (gradient)"};
       p->have_grad_map = true;
@@ -1837,8 +1837,8 @@ void destroy(ms_plan* p) {
     if (h) cufftDestroy(h);
   for (void* a : p->allocs) cudaFree(a);
   if (p->batch.fft) cufftDestroy(p->batch.fft);
-  for (void* a : {p->batch.jobs, (void*)p->batch.job_of, p->batch.grids, p->batch.half, p->batch.scratch,
-                  p->batch.rows_a, p->batch.rows_b})
+  for (void* a : {p->batch.jobs, (void*)p->batch.job_of, p->batch.grids, p->batch.half,
+                  p->batch.scratch, p->batch.rows_a, p->batch.rows_b})
     if (a) cudaFree(a);
   for (auto e : p->tev) cudaEventDestroy(e);
   for (auto e : p->evpool) cudaEventDestroy(e);
@@ -2112,10 +2112,10 @@ template <typename R> void ensure_fista_batch(ms_plan* p, int jobs, int max_iter
   ck(cudaMemset(F.ctl, 0, sizeof(FistaCtl) * cap), "memset");
   F.cap = cap;
   F.trace_cap = tcap;
-  // the stacked gradient images for the level-1 analysis's TMA window loads
-  unsigned bc = 0, br = 0;
-  analysis_window_box(&bc, &br);
-  if (p->have_grad_map && (unsigned)N >= bc) {
+  // the stacked gradient images for the level-1 analysis's TMA window loads (FP64)
+  if (p->have_grad_map) {
+    unsigned bc = 0, br = 0;
+    analysis_window_box(&bc, &br);
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult q;
     ck(cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault,
@@ -2127,8 +2127,8 @@ template <typename R> void ensure_fista_batch(ms_plan* p, int jobs, int max_iter
     cuuint32_t gb[2] = {bc, br};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = ((EncodeTiledFn)fn)(
-        &F.gmap, sizeof(R) == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
-        2, F.y, gd, gs, gb, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+        &F.gmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2, F.y, gd, gs, gb, estr,
+        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
         CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) throw Fail{MS_ERR_CUDA, "cuTensorMapEncodeTiled failed (batch)"};
     F.have_gmap = true;

@@ -198,7 +198,8 @@ __device__ __forceinline__ void unpack_real_row(const C2<R>* buf, const C2<R>* _
 
 // image row p, deapodized and centred -> its half-plane spectrum 0..ext
 template <typename R, int LOGM>
-__global__ void __launch_bounds__(RowBlock<R, LOGM>::THREADS) op_row_forward_kernel(OpFftArgs<R> a) {
+__global__ void __launch_bounds__(RowBlock<R, LOGM>::THREADS)
+    op_row_forward_kernel(OpFftArgs<R> a) {
   pdl_wait();
   pdl_trigger();
   using B = RowBlock<R, LOGM>;
@@ -230,7 +231,8 @@ __global__ void __launch_bounds__(RowBlock<R, LOGM>::THREADS) op_row_forward_ker
 
 // columns u of the half plane -> grid columns u and -u, rows -ext..ext
 template <typename R, int LOGG>
-__global__ void __launch_bounds__(ColBlock<R, LOGG>::THREADS) op_col_forward_kernel(OpFftArgs<R> a) {
+__global__ void __launch_bounds__(ColBlock<R, LOGG>::THREADS)
+    op_col_forward_kernel(OpFftArgs<R> a) {
   pdl_wait();
   pdl_trigger();
   using B = ColBlock<R, LOGG>;
@@ -265,7 +267,8 @@ __global__ void __launch_bounds__(ColBlock<R, LOGG>::THREADS) op_col_forward_ker
 // grid columns u and -u (their Hermitian part, doubled), rows -ext..ext -> the
 // N image rows of the column's inverse transform
 template <typename R, int LOGG>
-__global__ void __launch_bounds__(ColBlock<R, LOGG>::THREADS) op_col_adjoint_kernel(OpFftArgs<R> a) {
+__global__ void __launch_bounds__(ColBlock<R, LOGG>::THREADS)
+    op_col_adjoint_kernel(OpFftArgs<R> a) {
   pdl_wait();
   pdl_trigger();
   using B = ColBlock<R, LOGG>;
@@ -299,7 +302,8 @@ __global__ void __launch_bounds__(ColBlock<R, LOGG>::THREADS) op_col_adjoint_ker
 
 // half-plane row p (0..ext) -> image row p: cropped, deapodized, scaled
 template <typename R, int LOGM>
-__global__ void __launch_bounds__(RowBlock<R, LOGM>::THREADS) op_row_adjoint_kernel(OpFftArgs<R> a) {
+__global__ void __launch_bounds__(RowBlock<R, LOGM>::THREADS)
+    op_row_adjoint_kernel(OpFftArgs<R> a) {
   pdl_wait();
   pdl_trigger();
   using B = RowBlock<R, LOGM>;
@@ -372,7 +376,8 @@ cudaError_t go(const OpFftArgs<R>& a, bool forward, int njobs, cudaStream_t s) {
 // 4 N (N + M) values; padding, product and cropping as passes between cuFFT
 // transforms of the whole L x L field take ten launches and move some 20 N L.
 template <typename R, int LOGM>
-__global__ void __launch_bounds__(RowBlock<R, LOGM>::THREADS) lin_row_forward_kernel(LinFftArgs<R> a) {
+__global__ void __launch_bounds__(RowBlock<R, LOGM>::THREADS)
+    lin_row_forward_kernel(LinFftArgs<R> a) {
   pdl_wait();
   pdl_trigger();
   using B = RowBlock<R, LOGM>;
@@ -400,7 +405,8 @@ __global__ void __launch_bounds__(RowBlock<R, LOGM>::THREADS) lin_row_forward_ke
 }
 
 template <typename R, int LOGL>
-__global__ void __launch_bounds__(ColBlock<R, LOGL>::THREADS) lin_col_kernel(LinFftArgs<R> a) {
+__global__ void __launch_bounds__(ColBlock<R, LOGL>::THREADS)
+    lin_col_kernel(LinFftArgs<R> a) {
   pdl_wait();
   pdl_trigger();
   using B = ColBlock<R, LOGL>;
@@ -439,7 +445,8 @@ __global__ void __launch_bounds__(ColBlock<R, LOGL>::THREADS) lin_col_kernel(Lin
 }
 
 template <typename R, int LOGM>
-__global__ void __launch_bounds__(RowBlock<R, LOGM>::THREADS) lin_row_inverse_kernel(LinFftArgs<R> a) {
+__global__ void __launch_bounds__(RowBlock<R, LOGM>::THREADS)
+    lin_row_inverse_kernel(LinFftArgs<R> a) {
   pdl_wait();
   pdl_trigger();
   using B = RowBlock<R, LOGM>;

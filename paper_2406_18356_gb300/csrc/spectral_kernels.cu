@@ -282,7 +282,8 @@ __global__ void b_spectrum_kernel(const C2<R>* __restrict__ Ihat, const C2<R>* _
       double gh = (double)gh2[k], gl = (double)gl2[k];
       br = gh * h * I.x + gl * Lv.x;
       bi = gh * h * I.y + gl * Lv.y;
-      c = gh * ((double)I.x * I.x + (double)I.y * I.y) + gl * ((double)Lv.x * Lv.x + (double)Lv.y * Lv.y);
+      c = gh * ((double)I.x * I.x + (double)I.y * I.y) +
+          gl * ((double)Lv.x * Lv.x + (double)Lv.y * Lv.y);
     } else {
       br = h * I.x;
       bi = h * I.y;
@@ -413,11 +414,12 @@ __device__ void spec_finish(R s0, R c0, R s1, R c1, double l1s, bool has_l1, dou
 
 
 template <typename R>
-__global__ void __launch_bounds__(kThreads, 4) spec_mul_kernel(const C2<R>* __restrict__ Xk, C2<R>* __restrict__ Xprev,
-                                const R* __restrict__ Ks, const C2<R>* __restrict__ Bs, int N,
-                                double* __restrict__ parts, FistaCtl* __restrict__ ctl,
-                                double* __restrict__ trace, int32_t* ticket,
-                                const double* __restrict__ l1_parts, int n_l1) {
+__global__ void __launch_bounds__(kThreads, 4)
+    spec_mul_kernel(const C2<R>* __restrict__ Xk, C2<R>* __restrict__ Xprev,
+                    const R* __restrict__ Ks, const C2<R>* __restrict__ Bs, int N,
+                    double* __restrict__ parts, FistaCtl* __restrict__ ctl,
+                    double* __restrict__ trace, int32_t* ticket,
+                    const double* __restrict__ l1_parts, int n_l1) {
   pdl_wait();
   pdl_trigger();
   if (ctl->done) return;
@@ -476,9 +478,10 @@ __global__ void __launch_bounds__(kThreads, 4) spec_mul_kernel(const C2<R>* __re
 
 // ------------------------------------------------- shared-memory transforms
 // Complex FFTs of length N = 2^LOGN (a compile-time constant) held in shared
-// memory, one sequence per N/8 threads, as a mixed-radix Stockham autosort
-// transform (natural order in and out, ping-pong between two buffers):
-// radix-8 stages, then one radix-2 or radix-4 stage for what is left.  Stage
+// memory, one sequence per N / 2^fft_lrad threads, as a mixed-radix Stockham
+// autosort transform (natural order in and out, ping-pong between two buffers):
+// stages of radix 2^fft_lrad (8 in FP32; 2, 4 or 8 in FP64), then one of a
+// smaller radix for what is left.  Stage
 // with radix Rd after sub-transforms of size Ns: for j < N/Rd, the Rd inputs
 // a[j + r N/Rd] are twiddled by W_N^(r (j mod Ns) N/(Ns Rd)), transformed by
 // an Rd-point DFT in registers and written to
@@ -487,23 +490,23 @@ __global__ void __launch_bounds__(kThreads, 4) spec_mul_kernel(const C2<R>* __re
 // twiddle table tw[pad(m)] = W_N^m (m < N), which keeps the strided accesses
 // of every stage within a few shared-memory wavefronts.
 
-// one Stockham stage (radix Rd after sub-transforms of size NS) of the
-// calling thread's sequence; src / dst already offset to the sequence
 // threads of one sequence of length 2^LOGN at radix 2^LRAD
 __host__ __device__ constexpr int fft_threads(int logn, int lrad) {
   return logn > lrad ? 1 << (logn - lrad) : 1;
 }
 // log2 of the largest radix.  FP32: 8 (fewest stages).  FP64: a warp
-// instruction holds its scheduler's FP64 pipe (2 lanes a cycle per SM) for 64
-// cycles, so the time of a short transform is the instructions of its busiest
-// warp: radix 2 spreads them over 4 times the warps up to length 256, radix 4
-// over twice as many above (its stages take about as many operations per
-// point as radix 8's); radix 8 where a sequence would pass 1024 threads.
-// Measured at 128 px, FP64 (with the blocks per launch below): row R2C 36.8 ->
-// 5.3 us, column step 22.8 -> 11.5 us, row C2R 34.2 -> 5.0 us.
+// instruction holds its scheduler's FP64 pipe for 64 cycles (76 with all four
+// schedulers at it, measured), so the time of a short transform is the
+// instructions of its busiest warp: radix 2 spreads them over 4 times the warps
+// up to length 256, radix 4 over twice as many above (its stages take about as
+// many operations per point as radix 8's); radix 8 where a sequence would pass
+// 1024 threads.  Measured at 128 px, FP64 (with the blocks per launch below):
+// row R2C 36.8 -> 5.3 us, column step 22.8 -> 11.5 us, row C2R 34.2 -> 5.0 us.
 __host__ __device__ constexpr int fft_lrad(size_t rsz, int logn) {
   return rsz == 4 ? 3 : (logn <= 8 ? 1 : (logn <= 11 ? 2 : 3));
 }
+// one Stockham stage (radix Rd after sub-transforms of size NS) of the
+// calling thread's sequence; src / dst already offset to the sequence
 template <typename R, int LOGN, int Rd, int NS, int TPS, bool INV>
 __device__ __forceinline__ void stage_ct(const C2<R>* src, C2<R>* dst, const C2<R>* tw, int tid) {
   constexpr int N = 1 << LOGN, nj = N / Rd;
@@ -872,8 +875,8 @@ __global__ void __launch_bounds__(RowCfg<R, LOGN>::THREADS) row_r2c_kernel(
   cp_async_wait<0>();
   __syncthreads();
   int cur = 0;
-  stages_ct<R, LOGN - 1, Cfg::LRAD, 0, false>(b0 + (active ? rr : 0) * P, b1 + (active ? rr : 0) * P, cur,
-                                   tw, t, active);
+  stages_ct<R, LOGN - 1, Cfg::LRAD, 0, false>(b0 + (active ? rr : 0) * P,
+                                              b1 + (active ? rr : 0) * P, cur, tw, t, active);
   if (!active) return;
   const C2<R>* Zs = (cur ? b1 : b0) + rr * P;
   C2<R>* out = Z + (int64_t)(row0 + rr) * nc;
@@ -1005,8 +1008,8 @@ __global__ void __launch_bounds__(RowCfg<R, LOGN>::THREADS) row_c2r_kernel(
   }
   __syncthreads();
   int cur = 0;
-  stages_ct<R, LOGN - 1, Cfg::LRAD, 0, true>(b0 + (active ? rr : 0) * P, b1 + (active ? rr : 0) * P, cur,
-                                  tw, t, active);
+  stages_ct<R, LOGN - 1, Cfg::LRAD, 0, true>(b0 + (active ? rr : 0) * P,
+                                             b1 + (active ? rr : 0) * P, cur, tw, t, active);
   if (!active) return;
   const C2<R>* zs = (cur ? b1 : b0) + rr * P;
   C2<R>* xo = reinterpret_cast<C2<R>*>(x) + (int64_t)(row0 + rr) * M;

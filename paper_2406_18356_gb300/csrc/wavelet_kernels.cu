@@ -155,7 +155,9 @@ __host__ __device__ __forceinline__ int fit_tile(int t, int n) {
   while (2 * p <= t && n % (2 * p) == 0) p *= 2;
   return p;
 }
-__host__ __device__ __forceinline__ int ana_tile(int h) { return fit_tile(kAT, h); }   // subband side
+__host__ __device__ __forceinline__ int ana_tile(int h) {   // subband side
+  return fit_tile(kAT, h);
+}
 __device__ __forceinline__ int wrap(int i, int n) {
   i %= n;
   return i < 0 ? i + n : i;
