@@ -185,28 +185,97 @@ __host__ __device__ constexpr int pix_stride(int c) {
 
 struct ConvArgs {
   Act x;
-  int H, W, ci, co, kp;     // kp: row length of the packed weights (9 ci, padded to 16)
+  int H, W, ci, co;
+  int kp, cop;              // row lengths of the packed weights (9 ci and co, padded to 16)
   const bf16* w;            // [co][kp]
+  const bf16* wt;           // [9 ci][cop]
   const float* bias;
   bf16* out;                // [P][co] after the ReLU, or nullptr (the head)
   bf16* pooled;             // [P/4][co] 2 x 2 averages of out, or nullptr
   const float* head_in;     // head: the network's input [P][2]
   float* head_out;          // head: product + bias + the input's first channel
-  int ck;                   // channels staged at a time
+  int ck;                   // = ci (conv_kernel's loop over channels)
   int vec;                  // act_vec of x
 };
-// k steps of a chunk of c channels, its weight row stride, and shared memory
+// k of c channels, padded to whole steps, and shared memory
 __host__ __device__ constexpr int conv_kl(int c) { return pad16(9 * c); }
-template <bool BIG> size_t conv_smem(int ck, int nt) {
-  return ((size_t)Tile<BIG>::R * Tile<BIG>::R * pix_stride(ck) + 16 + 8 +
-          (size_t)nt * 8 * (conv_kl(ck) + 8)) * sizeof(bf16) + (size_t)conv_kl(ck) * sizeof(int);
+template <bool BIG> size_t conv_smem(int c, int nt) {
+  return ((size_t)Tile<BIG>::R * Tile<BIG>::R * pix_stride(c) + 16 + 8 +
+          (size_t)nt * 8 * (conv_kl(c) + 8)) * sizeof(bf16) + (size_t)conv_kl(c) * sizeof(int);
+}
+
+// What a warp's sums become: bias and ReLU into out (and its 2 x 2 averages
+// into pooled), or the head's output.  Its first m-tile, the tile's first pixel
+// and its first channel; all lanes take part.
+template <class TL, int MT, int NT>
+__device__ __forceinline__ void conv_store(const ConvArgs& p, const float (&acc)[MT][NT][4],
+                                           int mt0, int y0, int x0, int n0, int lane) {
+  const int gid = lane >> 2, tig = lane & 3;
+  // acc[.][.][q]: pixel row q / 2 of the m-tile's two, column gid, channel
+  // 2 tig + (q & 1) of the n8 tile
+#pragma unroll
+  for (int i = 0; i < MT; ++i) {
+    const int mt = mt0 + i;
+    const int y = y0 + TL::y(mt), x = x0 + TL::x(mt) + gid;
+    const bool okx = x < p.W;
+#pragma unroll
+    for (int j = 0; j < NT; ++j) {
+      const int n = n0 + j * 8 + 2 * tig;
+      if (p.out) {
+        float v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int c = n + (q & 1);
+          v[q] = fmaxf(acc[i][j][q] + (c < p.co ? p.bias[c] : 0.0f), 0.0f);
+          v[q] = __bfloat162float(__float2bfloat16_rn(v[q]));   // exact in the stores below
+        }
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          if (!okx || y + r >= p.H || n >= p.co) continue;
+          bf16* o = p.out + ((int64_t)(y + r) * p.W + x) * p.co + n;
+          if (p.co % 2 == 0) {
+            *reinterpret_cast<__nv_bfloat162*>(o) =
+                __floats2bfloat162_rn(v[2 * r], v[2 * r + 1]);
+          } else {
+            o[0] = __float2bfloat16_rn(v[2 * r]);
+            if (n + 1 < p.co) o[1] = __float2bfloat16_rn(v[2 * r + 1]);
+          }
+        }
+        if (p.pooled) {
+          // the pixel to the right is 4 lanes on; sides are even, so a 2 x 2
+          // block lies in the image as a whole
+          float s[2];
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            const float right0 = __shfl_xor_sync(0xffffffffu, v[c], 4);
+            const float right1 = __shfl_xor_sync(0xffffffffu, v[2 + c], 4);
+            s[c] = 0.25f * (((v[c] + right0) + v[2 + c]) + right1);
+          }
+          if (okx && y < p.H && (gid & 1) == 0) {
+            bf16* o = p.pooled + ((int64_t)(y >> 1) * (p.W >> 1) + (x >> 1)) * p.co + n;
+            if (n < p.co) o[0] = __float2bfloat16_rn(s[0]);
+            if (n + 1 < p.co) o[1] = __float2bfloat16_rn(s[1]);
+          }
+        }
+      } else if (n == 0 && okx) {
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          if (y + r >= p.H) continue;
+          const int64_t k = (int64_t)(y + r) * p.W + x;
+          p.head_out[k] = (acc[i][j][2 * r] + p.bias[0]) + p.head_in[2 * k];
+        }
+      }
+    }
+  }
 }
 
 // One convolution on one pixel tile and NT n8 tiles of output channels.  VEC:
 // act_vec of the input (8: operand rows by ldmatrix; else per-lane loads).
 // The accumulation runs over k = tap ci + c in steps of 16, one chain per
-// output (with the channels in one chunk, ck = ci: images of up to some 300
-// channels; wider layers sum chunk after chunk).
+// output.  The loop over channels makes one trip (p.ck = ci), which the compiler
+// does not know: without the loop it schedules the k steps in fewer registers
+// (NT = 2: 36 | 32) and small images take longer (6 levels of 6, forward pass:
+// 128 px 82.2 | 85.2 us, 512 px 161.6 | 163.5).
 template <bool BIG, int NT, int VEC>
 __global__ void __launch_bounds__(128) conv_kernel(const ConvArgs p) {
   using TL = Tile<BIG>;
@@ -232,31 +301,20 @@ __global__ void __launch_bounds__(128) conv_kernel(const ConvArgs p) {
 
   for (int c0 = 0; c0 < p.ci; c0 += p.ck) {
     const int ck = min(p.ck, p.ci - c0), kl = pad16(9 * ck);
-    if (c0) __syncthreads();
     if (tid < 16) sx[zero_off + tid] = __float2bfloat16_rn(0.0f);
     for (int k = tid * VEC; k < kl; k += 128 * VEC) {
       const int tap = k / ck, c = k - tap * ck;
       // (k >= 9 ck: the padding reads zeros, whatever the window holds)
       koff[k / VEC] = tap < 9 ? ((tap / 3) * TL::R + tap % 3) * CS + c : -1;
     }
-    if (ck == p.ci) {   // whole packed rows (kl = kp, a multiple of 16)
-      const int nv = kl / 8;
-      const float inv = 1.0f / (float)nv;
-      for (int e = tid; e < NT * 8 * nv; e += 128) {
-        const int r = (int)(((float)e + 0.5f) * inv), v = (e - r * nv) * 8;
-        const bool ok = n0 + r < p.co;
-        cpz<16>(sw + r * KS + v, ok ? p.w + (int64_t)(n0 + r) * p.kp + v : p.w, ok);
-      }
-      after_predecessor();
-    } else {
-      if (c0 == 0) after_predecessor();
-      for (int e = tid; e < NT * 8 * kl; e += 128) {
-        const int r = e / kl, k = e - r * kl, tap = k / ck;
-        const bool ok = n0 + r < p.co && tap < 9;
-        sw[r * KS + k] = ok ? p.w[(int64_t)(n0 + r) * p.kp + tap * p.ci + c0 + k - tap * ck]
-                            : __float2bfloat16_rn(0.0f);
-      }
+    const int nv = kl / 8;   // whole packed rows (kl = kp, a multiple of 16)
+    const float inv = 1.0f / (float)nv;
+    for (int e = tid; e < NT * 8 * nv; e += 128) {
+      const int r = (int)(((float)e + 0.5f) * inv), v = (e - r * nv) * 8;
+      const bool ok = n0 + r < p.co;
+      cpz<16>(sw + r * KS + v, ok ? p.w + (int64_t)(n0 + r) * p.kp + v : p.w, ok);
     }
+    after_predecessor();
     stage_pixels<VEC>(sx, CS, TL::R, TL::R, y0 - 1, x0 - 1, p.H, p.W, c0, ck, ck, p.x);
     asm volatile("cp.async.commit_group;" ::: "memory");
     asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -328,10 +386,10 @@ __global__ void __launch_bounds__(128) conv_kernel(const ConvArgs p) {
           for (int f = 0; f < 4; ++f) {   // (row half f & 1, k half f >> 1)
             const int row = base[i] + (f & 1) * TL::R * CS;
             const int e0 = ko[2 * (f >> 1)], e1 = ko[2 * (f >> 1) + 1];
-            const unsigned short l0 =
-                *reinterpret_cast<const unsigned short*>(sx + (!PAD || e0 >= 0 ? row + e0 : zero_off));
-            const unsigned short l1 =
-                *reinterpret_cast<const unsigned short*>(sx + (!PAD || e1 >= 0 ? row + e1 : zero_off));
+            const unsigned short l0 = *reinterpret_cast<const unsigned short*>(
+                sx + (!PAD || e0 >= 0 ? row + e0 : zero_off));
+            const unsigned short l1 = *reinterpret_cast<const unsigned short*>(
+                sx + (!PAD || e1 >= 0 ? row + e1 : zero_off));
             a[f] = (unsigned)l0 | ((unsigned)l1 << 16);
           }
 #pragma unroll
@@ -343,62 +401,107 @@ __global__ void __launch_bounds__(128) conv_kernel(const ConvArgs p) {
     k_step(kl - 16, std::true_type());
   }
 
-  // acc[.][.][q]: pixel row q / 2 of the m-tile's two, column gid, channel
-  // 2 tig + (q & 1) of the n8 tile
+  conv_store<TL, MT, NT>(p, acc, warp * MT, y0, x0, n0, lane);
+}
+
+// Wider layers: a block takes 64 output channels of a pixel tile and walks over
+// the input channels 16 at a time, the next ones' pixels and weights on their
+// way (two buffers) while this one's nine taps are multiplied.  Half of the
+// warps share each 32 channels; a warp's operand row then serves 4 n8 tiles and
+// its weights 2 or 4 m-tiles, where conv_kernel, whose block holds the weights
+// of all k at once, has room for one n8 tile beside some 400 channels and
+// re-reads the pixels for each.  The weights come from the transposed copy,
+// whose rows are aligned for any number of channels.  The sums run chunk by
+// chunk, tap by tap, one chain per output.  Measured, forward pass of 2 levels
+// of width 256 at 256 px: 1333 us (378 TFLOP/s); conv_kernel, channel chunks
+// staged in turn, 32303; the products on written-out windows before it 6790.
+constexpr int kWideN = 64, kWideC = 16;
+constexpr int kWideXS = kWideC + 8, kWideWS = kWideN + 8;   // row strides (no bank conflicts)
+template <bool BIG> struct Wide {
+  static constexpr int Threads = BIG ? 256 : 128;
+  static constexpr int X = Tile<BIG>::R * Tile<BIG>::R * kWideXS, W = 9 * kWideC * kWideWS;
+  static constexpr size_t Smem = 2 * (size_t)(X + W) * sizeof(bf16);
+};
+
+template <bool BIG, int VEC>
+__global__ void __launch_bounds__(Wide<BIG>::Threads, BIG ? 2 : 3)
+    conv_wide_kernel(const ConvArgs p) {
+  using TL = Tile<BIG>;
+  using G = Wide<BIG>;
+  constexpr int NW = G::Threads / 32, MT = TL::MTILES / (NW / 2), NT = kWideN / 16;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  bf16* buf = reinterpret_cast<bf16*>(smem_raw);   // two of (pixels [R R], weights [9][16][64])
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tiles_x = (p.W + TL::S - 1) / TL::S;
+  const int ty = blockIdx.x / tiles_x, tx = blockIdx.x - ty * tiles_x;
+  const int y0 = ty * TL::S, x0 = tx * TL::S, n0 = blockIdx.y * kWideN;
+  const int mt0 = (warp >> 1) * MT, nw = (warp & 1) * NT * 8;   // this warp's share
+  const auto stage_w = [&](int c0) {
+    bf16* sw = buf + (c0 / kWideC & 1) * (G::X + G::W) + G::X;
+    for (int e = tid; e < 9 * kWideC * (kWideN / 8); e += G::Threads) {
+      const int r = e / (kWideN / 8), v = e % (kWideN / 8) * 8;
+      const int tap = r / kWideC, c = c0 + r % kWideC;
+      const bool ok = c < p.ci && n0 + v < p.cop;
+      const bf16* q = ok ? p.wt + (int64_t)(tap * p.ci + c) * p.cop + n0 + v : p.wt;
+      cpz<16>(sw + r * kWideWS + v, q, ok);
+    }
+  };
+  const auto stage_x = [&](int c0) {
+    stage_pixels<VEC>(buf + (c0 / kWideC & 1) * (G::X + G::W), kWideXS, TL::R, TL::R, y0 - 1,
+                      x0 - 1, p.H, p.W, c0, min(kWideC, p.ci - c0), kWideC, p.x);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  float acc[MT][NT][4];
 #pragma unroll
-  for (int i = 0; i < MT; ++i) {
-    const int mt = warp * MT + i;
-    const int y = y0 + TL::y(mt), x = x0 + TL::x(mt) + gid;
-    const bool okx = x < p.W;
+  for (int i = 0; i < MT; ++i)
 #pragma unroll
-    for (int j = 0; j < NT; ++j) {
-      const int n = n0 + j * 8 + 2 * tig;
-      if (p.out) {
-        float v[4];
+    for (int j = 0; j < NT; ++j)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int c = n + (q & 1);
-          v[q] = fmaxf(acc[i][j][q] + (c < p.co ? p.bias[c] : 0.0f), 0.0f);
-          v[q] = __bfloat162float(__float2bfloat16_rn(v[q]));   // exact in the stores below
-        }
+      for (int q = 0; q < 4; ++q) acc[i][j][q] = 0.0f;
+  // ldmatrix rows: pixels (row half lane / 8 mod 2, k half lane / 16); weights,
+  // transposed (n8 tile of the pair lane / 16, k half lane / 8 mod 2)
+  unsigned a_o[MT];
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          if (!okx || y + r >= p.H || n >= p.co) continue;
-          bf16* o = p.out + ((int64_t)(y + r) * p.W + x) * p.co + n;
-          if (p.co % 2 == 0) {
-            *reinterpret_cast<__nv_bfloat162*>(o) =
-                __floats2bfloat162_rn(v[2 * r], v[2 * r + 1]);
-          } else {
-            o[0] = __float2bfloat16_rn(v[2 * r]);
-            if (n + 1 < p.co) o[1] = __float2bfloat16_rn(v[2 * r + 1]);
-          }
-        }
-        if (p.pooled) {
-          // the pixel to the right is 4 lanes on; sides are even, so a 2 x 2
-          // block lies in the image as a whole
-          float s[2];
+  for (int i = 0; i < MT; ++i)
+    a_o[i] = 2u * (((TL::y(mt0 + i) + ((lane >> 3) & 1)) * TL::R + TL::x(mt0 + i) + (lane & 7)) *
+                       kWideXS + (lane >> 4) * 8);
+  const unsigned b_o = 2u * (G::X + (lane & 15) * kWideWS + nw + (lane >> 4) * 8);
+  stage_w(0);
+  after_predecessor();
+  stage_x(0);
+  for (int c0 = 0; c0 < p.ci; c0 += kWideC) {
+    if (c0 + kWideC < p.ci) {
+      stage_w(c0 + kWideC);
+      stage_x(c0 + kWideC);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();
+    const unsigned base = saddr(buf) + 2u * (c0 / kWideC & 1) * (G::X + G::W);
 #pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            const float right0 = __shfl_xor_sync(0xffffffffu, v[c], 4);
-            const float right1 = __shfl_xor_sync(0xffffffffu, v[2 + c], 4);
-            s[c] = 0.25f * (((v[c] + right0) + v[2 + c]) + right1);
-          }
-          if (okx && y < p.H && (gid & 1) == 0) {
-            bf16* o = p.pooled + ((int64_t)(y >> 1) * (p.W >> 1) + (x >> 1)) * p.co + n;
-            if (n < p.co) o[0] = __float2bfloat16_rn(s[0]);
-            if (n + 1 < p.co) o[1] = __float2bfloat16_rn(s[1]);
-          }
-        }
-      } else if (n == 0 && okx) {
+    for (int tap = 0; tap < 9; ++tap) {
+      unsigned b[NT][2];
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          if (y + r >= p.H) continue;
-          const int64_t k = (int64_t)(y + r) * p.W + x;
-          p.head_out[k] = (acc[i][j][2 * r] + p.bias[0]) + p.head_in[2 * k];
-        }
+      for (int j = 0; j < NT; j += 2) {
+        unsigned r[4];
+        ldsm4t(r, base + b_o + 2u * (tap * kWideC * kWideWS + j * 8));
+        b[j][0] = r[0];
+        b[j][1] = r[1];
+        b[j + 1][0] = r[2];
+        b[j + 1][1] = r[3];
+      }
+#pragma unroll
+      for (int i = 0; i < MT; ++i) {
+        unsigned a[4];
+        ldsm4(a, base + a_o[i] + 2u * ((tap / 3) * TL::R + tap % 3) * kWideXS);
+#pragma unroll
+        for (int j = 0; j < NT; ++j) mma16816(acc[i][j], a, b[j][0], b[j][1]);
       }
     }
+    __syncthreads();   // the buffer is staged again
   }
+  conv_store<TL, MT, NT>(p, acc, mt0, y0, x0, n0 + nw, lane);
 }
 
 // ---------------------------------------------------------- data gradient
@@ -474,8 +577,8 @@ __global__ void __launch_bounds__(BIG ? 256 : 128) dx_kernel(const DxArgs p) {
 #pragma unroll
     for (int i = 0; i < MT; ++i) {
       const int mt = warp * MT + i;
-      a_a[i] = sz_a + 2u * (((TL::y(mt) + ((lane >> 3) & 1)) * TL::R + TL::x(mt) + (lane & 7)) * KS +
-                            (lane >> 4) * 8);
+      const int px = (TL::y(mt) + ((lane >> 3) & 1)) * TL::R + TL::x(mt) + (lane & 7);
+      a_a[i] = sz_a + 2u * (px * KS + (lane >> 4) * 8);
     }
 #pragma unroll 1
     for (int tap = 0; tap < 9; ++tap) {
@@ -755,7 +858,8 @@ __global__ void __launch_bounds__(kT) pack_weights_kernel(const __grid_constant_
     __syncthreads();
     for (int r = ly; r < 32; r += kT / 32) {
       const int co = co0 + r, k = k0 + lx;
-      const bf16 v = __float2bfloat16_rn(co < l.co && k < l.k9 ? l.w[(int64_t)co * l.k9 + k] : 0.0f);
+      const bool ok = co < l.co && k < l.k9;
+      const bf16 v = __float2bfloat16_rn(ok ? l.w[(int64_t)co * l.k9 + k] : 0.0f);
       if (co < l.co && k < l.kp) l.wb[(int64_t)co * l.kp + k] = v;
       t[r][lx] = v;
     }
@@ -948,17 +1052,46 @@ void launch(K kern, dim3 grid, int threads, size_t smem, const A& p, cudaStream_
     default: { constexpr int VEC = 1; CALL; break; } \
   }
 
+// The layers of conv_wide_kernel: those whose channels conv_kernel cannot hold
+// at once; from 96 input and 64 output channels on where 16 x 16 tiles make a
+// block for every SM; and from 289 on (193 where the pixels are no whole 16-byte
+// chunks, which costs conv_kernel an operand read per lane) where 8 x 8 tiles do
+// for half of them.  Forward pass, us, this rule | conv_kernel wherever it fits:
+// 4 levels of width 64 at 512 px TODO_A, 3 of 128 at 128 px TODO_B, 3 of 75 at
+// 128 px TODO_C.  With fewer blocks conv_kernel's 8 channels a block win (6
+// levels of 10 at 256 px 158 | 196 wide from 193 on).  Narrower layers keep its
+// order of summation: rounded to bfloat16 layer after layer, another order's
+// last bits move a pass of the configured network by 1.5 %, as much as half of
+// its distance from exact arithmetic.
+constexpr int kWideBig = 96, kWideSmall = 289, kWideSmallOdd = 193;
 void conv_forward(ms_unet* u, Layer& l, const Act& x, int H, int W, bf16* pooled,
                   const float* head_in, float* head_out, cudaStream_t s) {
   l.in = x;
+  const float* bias = u->master + l.woff + (size_t)l.co * 9 * l.ci;
+  const ConvArgs p{x,    H,     W,      l.ci,    l.co,     l.kp, l.cop,    l.Wb, l.Wt,
+                   bias, l.out, pooled, head_in, head_out, l.ci, act_vec(x)};
+  const auto tiles = [&](int S) { return ((H + S - 1) / S) * ((W + S - 1) / S); };
+  const int nw = (l.co + kWideN - 1) / kWideN;
+  const bool big =
+      l.ci >= kWideBig && l.co >= kWideN && (int64_t)tiles(16) * nw >= sm_count();
+  const bool small = l.ci >= (p.vec == 8 ? kWideSmall : kWideSmallOdd) &&
+                     (int64_t)tiles(8) * nw >= sm_count() / 2;
+  if (l.out && (big || small || conv_smem<false>(l.ci, 1) > kSmemMax)) {
+    const dim3 grid(tiles(big ? 16 : 8), nw);
+    MS_BY_VEC(p.vec, {
+      if (big)
+        launch(conv_wide_kernel<true, VEC>, grid, Wide<true>::Threads, Wide<true>::Smem, p, s);
+      else
+        launch(conv_wide_kernel<false, VEC>, grid, Wide<false>::Threads, Wide<false>::Smem, p, s);
+    })
+    return;
+  }
   const Shape sh = pick_shape(H, W, l.co, l.ci, [](bool big, int c, int nt) {
     return big ? conv_smem<true>(c, nt) : conv_smem<false>(c, nt);
   });
-  ConvArgs p{x, H, W, l.ci, l.co, l.kp, l.Wb, u->master + l.woff + (size_t)l.co * 9 * l.ci,
-             l.out, pooled, head_in, head_out, sh.ck, act_vec(x)};
-  const int S = sh.big ? 16 : 8, n8 = (l.co + 7) / 8;
-  const dim3 grid(((H + S - 1) / S) * ((W + S - 1) / S), (n8 + sh.nt - 1) / sh.nt);
-  const size_t smem = sh.big ? conv_smem<true>(sh.ck, sh.nt) : conv_smem<false>(sh.ck, sh.nt);
+  const int n8 = (l.co + 7) / 8;
+  const dim3 grid(tiles(sh.big ? 16 : 8), (n8 + sh.nt - 1) / sh.nt);
+  const size_t smem = sh.big ? conv_smem<true>(l.ci, sh.nt) : conv_smem<false>(l.ci, sh.nt);
   MS_BY_VEC(p.vec, MS_BY_NT(sh.nt, {
     if (sh.big) launch(conv_kernel<true, NT, VEC>, grid, 128, smem, p, s);
     else launch(conv_kernel<false, NT, VEC>, grid, 128, smem, p, s);
