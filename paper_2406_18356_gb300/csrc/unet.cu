@@ -19,8 +19,8 @@
 // and stored activations (after ReLU, after pooling) are rounded to bfloat16,
 // and so is every pre-activation gradient before it enters a product.
 //
-// Measured (6 levels, width 6): forward pass at 1024 x 1024 360 us, forward
-// and backward pass with the gradients at 512 x 512 750 us; before, with the
+// Measured (6 levels, width 6): forward pass at 1024 x 1024 356 us, forward
+// and backward pass with the gradients at 512 x 512 746 us; before, with the
 // windows written out (im2col, 9 times the activations, and a transposed copy
 // for the weight gradients) and one general product kernel: 4166 and 5449 us.
 #include <cuda_bf16.h>
@@ -1056,13 +1056,14 @@ void launch(K kern, dim3 grid, int threads, size_t smem, const A& p, cudaStream_
 // at once; from 96 input and 64 output channels on where 16 x 16 tiles make a
 // block for every SM; and from 289 on (193 where the pixels are no whole 16-byte
 // chunks, which costs conv_kernel an operand read per lane) where 8 x 8 tiles do
-// for half of them.  Forward pass, us, this rule | conv_kernel wherever it fits:
-// 4 levels of width 64 at 512 px TODO_A, 3 of 128 at 128 px TODO_B, 3 of 75 at
-// 128 px TODO_C.  With fewer blocks conv_kernel's 8 channels a block win (6
-// levels of 10 at 256 px 158 | 196 wide from 193 on).  Narrower layers keep its
-// order of summation: rounded to bfloat16 layer after layer, another order's
-// last bits move a pass of the configured network by 1.5 %, as much as half of
-// its distance from exact arithmetic.
+// for half of them.  Forward pass, us, this rule | conv_kernel throughout, in
+// chunks of channels where it must | the products on written-out windows before
+// both: 4 levels of width 64 at 512 px 1246 | 11100 | 8790, 3 of 128 at 128 px
+// 531 | 2626 | 1430, 3 of 75 at 128 px 532 | 1039 | 884.  With fewer blocks
+// conv_kernel's 8 channels a block win (6 levels of 10 at 256 px 158 | 196 wide
+// from 193 on).  Narrower layers keep its order of summation: rounded to
+// bfloat16 layer after layer, another order's last bits move a pass of the
+// configured network by 1.5 %, half of its distance from exact arithmetic.
 constexpr int kWideBig = 96, kWideSmall = 289, kWideSmallOdd = 193;
 void conv_forward(ms_unet* u, Layer& l, const Act& x, int H, int W, bf16* pooled,
                   const float* head_in, float* head_out, cudaStream_t s) {
