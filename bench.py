@@ -378,8 +378,7 @@ def record_traffic(paths, precision):
                 b += float(r[idx[m]].replace(",", "")) * scale[units[idx[m]]]
             launches.append((name, b))
     # (one launch per level, in order)
-    syn = [b for n, b in launches
-           if "synthesis_level_kernel" in n or "fine_synthesis" in n]
+    syn = [b for n, b in launches if "fine_synthesis" in n]
     ana = [b for n, b in launches
            if "analysis_level_kernel" in n or "fine_analysis_kernel" in n]
     if syn:
@@ -483,9 +482,13 @@ def main():
     value = vis_total / grid_s
     ms_per_step = wall_ms / args.steps
     fista_rate = tot["iters"] / (tot["minor_ms"] / 1000.0)
-    kernels_per_pass = 2 * 4 + 1
+    # a pass: four levels each way and the spectral step's three kernels; a
+    # major cycle: its residual image (7) and the minor cycle's set-up and
+    # update (7); a step: the last residual image and its set-up (2344 of the
+    # launch list's at one major cycle of 100 iterations)
+    kernels_per_pass = 2 * 4 + 3
     passes_per_cycle = math.ceil((args.fista_iters + 1) / 8) * 8
-    launches_per_step = 2 * (args.n_major * (passes_per_cycle * kernels_per_pass + 5 + 8) + 5 + 2)
+    launches_per_step = 2 * (args.n_major * (passes_per_cycle * kernels_per_pass + 7 + 7) + 7 + 7)
     gpu_launches = launches_per_step * args.steps
 
     # ---- per-kernel durations: the same steps with every kernel family
